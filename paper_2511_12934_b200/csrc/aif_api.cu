@@ -481,8 +481,7 @@ int aif_item_nearline_refresh(aif_ctx *ctx, const int32_t *ids, int64_t n, const
     const bool versioned = ctx->cfg.versioned_table && !ids;
     if (versioned) AIF_CUDA(begin_full_refresh(ctx, n, as_stream(stream)));
     else AIF_CUDA(wait_table_ready(ctx, as_stream(stream)));
-    AIF_CUDA(launch_scatter_rows(ctx, ids, n, rows, bea_w, lsh_sig, as_stream(stream)));
-    AIF_CUDA(launch_row_norm_max(ctx, ctx->E, ids, n, ctx->cfg.M, ctx->e_norm, as_stream(stream)));
+    AIF_CUDA(launch_refresh_rows(ctx, ids, n, rows, bea_w, lsh_sig, ctx->e_norm, as_stream(stream)));
     if (versioned) AIF_CUDA(end_full_refresh(ctx, as_stream(stream)));
     ctx->table_version += 1;
     ctx->stats.table_version = ctx->table_version;

@@ -222,8 +222,9 @@ void timing_mark(const aif_ctx *ctx, const char *name, cudaStream_t st);
 ModelDev make_model(const aif_ctx *ctx);
 
 // aif_simt.cu
-cudaError_t launch_scatter_rows(const aif_ctx *ctx, const int32_t *ids, int64_t n, const void *rows, const void *bea_w,
-                                const uint8_t *sig, cudaStream_t st);
+// table rows ids[i] (ids == nullptr: i) = rows[i] with their sidecars; *norm_max (may be null) raised to the largest row norm
+cudaError_t launch_refresh_rows(const aif_ctx *ctx, const int32_t *ids, int64_t n, const void *rows, const void *bea_w, const uint8_t *sig,
+                                float *norm_max, cudaStream_t st);
 // *out = max(*out, largest row norm) over rows ids[0..n) of `rows` (ids == nullptr: rows 0..n); ids outside [0, M) skipped
 cudaError_t launch_row_norm_max(const aif_ctx *ctx, const void *rows, const int32_t *ids, int64_t n, int64_t M, float *out, cudaStream_t st);
 cudaError_t launch_stage_ids(const int32_t *mapped_src, int32_t *dst, int n, cudaStream_t st);

@@ -237,7 +237,7 @@ int nearline_compute(aif_ctx *ctx, const int32_t *ids, int64_t n, const void *I_
         uint8_t *sig_out = !lsh ? nullptr : ids ? pl->sig : ctx->sig + (size_t)off * c.lsh_bits / 8;
         cudaError_t e = el == 4 ? run_pass<float>(ctx, pl, m, raw, iid, mm, rows_out, bea_out, sig_out, st)
                                 : run_pass<__nv_bfloat16>(ctx, pl, m, raw, iid, mm, rows_out, bea_out, sig_out, st);
-        if (e == cudaSuccess && ids) e = launch_scatter_rows(ctx, ids + off, m, rows_out, bea_out, sig_out, st);
+        if (e == cudaSuccess && ids) e = launch_refresh_rows(ctx, ids + off, m, rows_out, bea_out, sig_out, nullptr, st);
         if (e != cudaSuccess) {
             set_last_error(cudaGetErrorString(e));
             return AIF_ERR_CUDA;
