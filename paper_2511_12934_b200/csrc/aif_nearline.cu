@@ -82,6 +82,85 @@ __global__ void __launch_bounds__(256) k_item_bridge_weights(const T *__restrict
     }
 }
 
+// The same for bf16 rows of d = 32 VJ on the warp-level matrix instructions: a warp takes 16 items, [16 x d] . [d x 8 NT]
+// with fp32 accumulation, 2 n d flop per item against 2 d bytes read: a stream over I_id, too narrow (N = n_bridge <= 16)
+// for a tensor-memory tile to pay.  The order of K inside the product is free, so a thread takes 16 contiguous bytes of its
+// two rows at a time (a quad covers 64 bytes of a row, 2 VJ independent loads in flight per thread) and the bridges' operand
+// is read in the same order, once, into registers.  Lane 4 g + t of the accumulator holds bridges 2 t, 2 t + 1 of items g and
+// g + 8: the softmax over bridges is two shuffles inside a quad.  One warp per item with a warp reduction per bridge (the form
+// above) took 217 us for 262143 items at d = 128, n = 8.
+__device__ __forceinline__ void mma_16816(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1)
+{
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+                 : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+template <int VJ, int NT>
+__global__ void __launch_bounds__(256) k_item_bridge_weights_mma(const __nv_bfloat16 *__restrict__ I_id, int64_t n, int nb,
+                                                                 const __nv_bfloat16 *__restrict__ Bm, __nv_bfloat16 *__restrict__ out)
+{
+    constexpr int D = 32 * VJ;
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    const float scale = rsqrtf((float)D);
+    uint4 b[NT][VJ];
+#pragma unroll
+    for (int j = 0; j < NT; ++j)
+#pragma unroll
+        for (int v = 0; v < VJ; ++v)
+            b[j][v] = 8 * j + g < nb ? *reinterpret_cast<const uint4 *>(Bm + (size_t)(8 * j + g) * D + 8 * (t + 4 * v)) : make_uint4(0, 0, 0, 0);
+    const int64_t n_warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t i0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 16; i0 < n; i0 += n_warps * 16) {
+        const int64_t row[2] = {i0 + g, i0 + g + 8};
+        uint4 a[2][VJ];
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int v = 0; v < VJ; ++v)
+                a[h][v] = __ldg(reinterpret_cast<const uint4 *>(I_id + (row[h] < n ? row[h] : n - 1) * D + 8 * (t + 4 * v)));
+        float c[NT][4];
+#pragma unroll
+        for (int j = 0; j < NT; ++j) {
+            c[j][0] = c[j][1] = c[j][2] = c[j][3] = 0.f;
+#pragma unroll
+            for (int v = 0; v < VJ; ++v) {
+                mma_16816(c[j], a[0][v].x, a[1][v].x, a[0][v].y, a[1][v].y, b[j][v].x, b[j][v].y);
+                mma_16816(c[j], a[0][v].z, a[1][v].z, a[0][v].w, a[1][v].w, b[j][v].z, b[j][v].w);
+            }
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            float s[2 * NT], mx = -INFINITY, den = 0.f;
+#pragma unroll
+            for (int q = 0; q < 2 * NT; ++q) {
+                s[q] = 8 * (q >> 1) + 2 * t + (q & 1) < nb ? c[q >> 1][2 * h + (q & 1)] * scale : -INFINITY;
+                mx = fmaxf(mx, s[q]);
+            }
+            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+#pragma unroll
+            for (int q = 0; q < 2 * NT; ++q) {
+                s[q] = expf(s[q] - mx);   // 0 for the columns beyond the last bridge
+                den += s[q];
+            }
+            den += __shfl_xor_sync(0xffffffffu, den, 1);
+            den += __shfl_xor_sync(0xffffffffu, den, 2);
+            if (row[h] >= n) continue;
+#pragma unroll
+            for (int j = 0; j < NT; ++j) {
+                const int k = 8 * j + 2 * t;
+                __nv_bfloat16 *o = out + row[h] * nb + k;
+                if (nb % 2 == 0) {
+                    if (k < nb) *reinterpret_cast<__nv_bfloat162 *>(o) = __floats2bfloat162_rn(s[2 * j] / den, s[2 * j + 1] / den);
+                } else {
+                    if (k < nb) o[0] = __float2bfloat16_rn(s[2 * j] / den);
+                    if (k + 1 < nb) o[1] = __float2bfloat16_rn(s[2 * j + 1] / den);
+                }
+            }
+        }
+    }
+}
+
 // eq. 5 on CUDA cores: one warp per item, 32 bits per round; eight bits per byte, first bit most significant.
 template <typename T>
 __global__ void __launch_bounds__(256) k_item_signatures(const T *__restrict__ M_mm, int64_t n, int d_mm, int bits, const T *__restrict__ W_hash,
@@ -141,8 +220,20 @@ cudaError_t run_pass(aif_ctx *ctx, NearlinePlan *pl, int64_t m, const void *I_ra
     // the table's norm bound from the rows just computed (whether or not their ids turn out to lie in the table)
     if (!(pl->tensor && pl->fused_tower) && (e = launch_row_norm_max(ctx, rows_out, nullptr, m, m, ctx->e_norm, st)) != cudaSuccess) return e;
     if (c.blocks & AIF_BLK_BEA) {
-        k_item_bridge_weights<T><<<grid_for_items(m), 256, 0, st>>>((const T *)(I_id ? I_id : rows_out), m, c.d, c.n_bridge,
-                                                                    (const T *)pl->bridges, (T *)bea_out);
+        const void *id_rows = I_id ? I_id : rows_out;
+        // matrix instructions for the d that divide into whole quads of 16-byte pieces; they read 16 bytes at a time
+        const bool mma = c.dtype == AIF_BF16 && (c.d == 64 || c.d == 128 || c.d == 256) && c.n_bridge <= 16 && (uintptr_t)id_rows % 16 == 0;
+        if (mma) {
+            using bf = __nv_bfloat16;
+            const int64_t blocks = (m + 127) / 128;
+            const int grid = (int)(blocks < 148 * 6 ? blocks : 148 * 6);
+            auto go = [&](auto kernel) { kernel<<<grid, 256, 0, st>>>((const bf *)id_rows, m, c.n_bridge, (const bf *)pl->bridges, (bf *)bea_out); };
+            const bool two = c.n_bridge > 8;
+            if (c.d == 64) two ? go(k_item_bridge_weights_mma<2, 2>) : go(k_item_bridge_weights_mma<2, 1>);
+            else if (c.d == 128) two ? go(k_item_bridge_weights_mma<4, 2>) : go(k_item_bridge_weights_mma<4, 1>);
+            else two ? go(k_item_bridge_weights_mma<8, 2>) : go(k_item_bridge_weights_mma<8, 1>);
+        } else
+            k_item_bridge_weights<T><<<grid_for_items(m), 256, 0, st>>>((const T *)id_rows, m, c.d, c.n_bridge, (const T *)pl->bridges, (T *)bea_out);
         count_launch();
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
