@@ -634,9 +634,76 @@ __global__ void __launch_bounds__(LayerCfg<MODE>::kThreads, 1) k_layer_tc(const 
     if (warp == C::kMmaWarp) tmem_dealloc(tmem_base, 512);
 }
 
+// The tile of a block in the kernels below: from the launch's tile table when it was formed on the device, else from the
+// request table.
+struct BlockTile {
+    int slot, cnt;
+    int64_t pos0;
+};
+__device__ __forceinline__ BlockTile block_tile(const ScoreLaunch &sl, int tile, int mini_batch)
+{
+    if (sl.n_tiles_dev) {
+        if (tile >= *sl.n_tiles_dev) return BlockTile{0, 0, 0};
+        const TileDev t = sl.tiles[tile];
+        return BlockTile{t.slot, t.cnt, t.pos0};
+    }
+    const ReqDev rq = find_request(sl, tile);
+    int start, cnt;
+    tile_range(tile - rq.tile_begin, rq.n, kTcTile, mini_batch, start, cnt);
+    return BlockTile{rq.slot, cnt, rq.off + start};
+}
+
+// v_bea = w^ V (Algorithm 1 line 4) for half a tile of candidates per block: n d fused multiply-adds against 2 d bytes written
+// per candidate, so memory and latency bound, and all of it independent.  V goes to shared memory once per block, the ids and
+// weight rows of the 64 candidates are fetched side by side, then a thread owns eight columns (one 16-byte store) of every
+// 2048 / d-th candidate.  A warp per candidate, its loads one after the other and in line with the other blocks of the
+// interaction kernel, took 35 us for 9877 candidates at d = 128, n = 8.
+constexpr int kBeaRows = 64;
+__global__ void __launch_bounds__(256) k_bea_x(ModelDev md, ScoreLaunch sl, __nv_bfloat16 *X, int x_stride, int col)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int d = md.d, nb = md.n_bridge, tid = threadIdx.x;
+    __nv_bfloat16 *V = reinterpret_cast<__nv_bfloat16 *>(smem_raw);          // [nb][d]
+    float *w = reinterpret_cast<float *>(smem_raw + (size_t)nb * d * 2);     // [kBeaRows][nb]
+    grid_dep_launch();
+    grid_dep_wait();
+    const BlockTile t = block_tile(sl, blockIdx.x, md.mini_batch);
+    const int first = blockIdx.y * kBeaRows, cnt = min(kBeaRows, t.cnt - first);
+    if (cnt <= 0) return;
+    const int64_t pos0 = t.pos0 + first;
+    const uint4 *Vg = reinterpret_cast<const uint4 *>(sl.slots[t.slot].V);
+    for (int i = tid; i < nb * d / 8; i += 256) reinterpret_cast<uint4 *>(V)[i] = Vg[i];
+    for (int i = tid; i < cnt * nb; i += 256) {
+        const int c = i / nb, id = sl.ids[pos0 + c];
+        const bool good = id >= 0 && (int64_t)id < md.M;   // an id outside the table: zero columns
+        w[i] = good ? to_f(reinterpret_cast<const __nv_bfloat16 *>(md.bea_w)[(size_t)id * nb + (i - c * nb)]) : 0.f;
+    }
+    __syncthreads();
+    const int per_row = d / 8;
+    for (int i = tid; i < cnt * per_row; i += 256) {
+        const int c = i / per_row, k = (i - c * per_row) * 8;
+        float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        for (int b = 0; b < nb; ++b) {
+            const float wb = w[c * nb + b];
+            const uint4 v = *reinterpret_cast<const uint4 *>(V + b * d + k);
+            const __nv_bfloat162 *h = reinterpret_cast<const __nv_bfloat162 *>(&v);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float2 f = __bfloat1622float2(h[q]);
+                acc[2 * q] = fmaf(wb, f.x, acc[2 * q]), acc[2 * q + 1] = fmaf(wb, f.y, acc[2 * q + 1]);
+            }
+        }
+        uint4 o;
+        __nv_bfloat162 *oh = reinterpret_cast<__nv_bfloat162 *>(&o);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) oh[q] = __floats2bfloat162_rn(acc[2 * q], acc[2 * q + 1]);
+        *reinterpret_cast<uint4 *>(X + (size_t)(pos0 + c) * x_stride + col + k) = o;
+    }
+}
+
 // ---- interaction blocks that feed dense columns (CUDA cores; one warp per candidate) ---------------------------
-// Writes, per candidate position, a bf16 row [ att (d) | v_bea (d) | lsh_din (d) | simtier (64, first n_tiers used) ]
-// holding only the enabled blocks.
+// Writes, per candidate position, the att, lsh_din and simtier columns of a bf16 row [ att (d) | v_bea (d) | lsh_din (d) |
+// simtier (64, first n_tiers used) ] that holds only the enabled blocks (k_bea_x writes v_bea).
 __global__ void __launch_bounds__(256) k_interact_x(ModelDev md, ScoreLaunch sl, __nv_bfloat16 *X, int x_stride, int att_done, int lsh_done)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -646,25 +713,16 @@ __global__ void __launch_bounds__(256) k_interact_x(ModelDev md, ScoreLaunch sl,
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, d = md.d, dq = d >> 5;
     grid_dep_launch();
     grid_dep_wait();
-    // the tile: from the launch's tile table when it has one that was formed on the device, else from the request table
-    int slot_index, cnt;
-    int64_t pos0;
-    if (sl.n_tiles_dev) {
-        if ((int)blockIdx.x >= *sl.n_tiles_dev) return;
-        const TileDev t = sl.tiles[blockIdx.x];
-        slot_index = t.slot, cnt = t.cnt, pos0 = t.pos0;
-    } else {
-        const ReqDev rq = find_request(sl, blockIdx.x);
-        int start;
-        tile_range(blockIdx.x - rq.tile_begin, rq.n, kTcTile, md.mini_batch, start, cnt);
-        slot_index = rq.slot, pos0 = rq.off + start;
-    }
-    const SlotDev slot = sl.slots[slot_index];
+    const BlockTile tile = block_tile(sl, blockIdx.x, md.mini_batch);
+    const int cnt = tile.cnt;
+    if (cnt <= 0) return;
+    const int64_t pos0 = tile.pos0;
+    const SlotDev slot = sl.slots[tile.slot];
     // att_done / lsh_done: those columns were already written by the tensor-core attention / LSH kernels
-    const bool has_att = md.blocks & AIF_BLK_ATT, do_att = has_att && !att_done, do_bea = md.blocks & AIF_BLK_BEA;
+    const bool has_att = md.blocks & AIF_BLK_ATT, do_att = has_att && !att_done, has_bea = md.blocks & AIF_BLK_BEA;
     const bool has_din = md.blocks & AIF_BLK_LSH_DIN, has_tier = md.blocks & AIF_BLK_SIMTIER;
     const bool do_din = has_din && !lsh_done, do_tier = has_tier && !lsh_done, do_lsh = do_din || do_tier;
-    const int col_bea = has_att ? d : 0, col_din = col_bea + (do_bea ? d : 0), col_tier = col_din + (has_din ? d : 0);
+    const int col_din = (has_att ? d : 0) + (has_bea ? d : 0), col_tier = col_din + (has_din ? d : 0);
     using T = __nv_bfloat16;
     for (int c = warp; c < cnt; c += 8) {
         const int64_t pos = pos0 + c;
@@ -675,7 +733,6 @@ __global__ void __launch_bounds__(256) k_interact_x(ModelDev md, ScoreLaunch sl,
             const __nv_bfloat16 z = __float2bfloat16_rn(0.f);
             for (int k = lane; k < d; k += 32) {
                 if (do_att) xrow[k] = z;
-                if (do_bea) xrow[col_bea + k] = z;
                 if (do_din) xrow[col_din + k] = z;
             }
             if (do_tier)
@@ -692,35 +749,22 @@ __global__ void __launch_bounds__(256) k_interact_x(ModelDev md, ScoreLaunch sl,
         if (do_att || do_lsh)
             warp_interact<T>(qv + warp * d, reinterpret_cast<const T *>(slot.S), slot.L, d, rsqrtf((float)d), do_att, do_lsh,
                              do_tier, sigq + warp * 8, slot.sigS, md.lsh_bits, md.n_tiers, tiers + warp * 16, att, din);
-        int col = 0;
         if (do_att) {
 #pragma unroll
             for (int q = 0; q < 8; ++q)
-                if (q < dq) xrow[col + lane + 32 * q] = __float2bfloat16_rn(att[q]);
-        }
-        if (has_att) col += d;
-        if (do_bea) {
-            const T *wh = reinterpret_cast<const T *>(md.bea_w) + (size_t)id * md.n_bridge;
-            const T *V = reinterpret_cast<const T *>(slot.V);
-            for (int k = lane; k < d; k += 32) {
-                float acc = 0.f;
-                for (int b = 0; b < md.n_bridge; ++b) acc = fmaf(to_f(wh[b]), to_f(V[(size_t)b * d + k]), acc);
-                xrow[col + k] = __float2bfloat16_rn(acc);
-            }
-            col += d;
+                if (q < dq) xrow[lane + 32 * q] = __float2bfloat16_rn(att[q]);
         }
         if (do_din) {
             const float nrm = md.lsh_din_norm == AIF_NORM_MEAN ? 1.0f / (float)slot.L : 1.0f;
 #pragma unroll
             for (int q = 0; q < 8; ++q)
-                if (q < dq) xrow[col + lane + 32 * q] = __float2bfloat16_rn(din[q] * nrm);
+                if (q < dq) xrow[col_din + lane + 32 * q] = __float2bfloat16_rn(din[q] * nrm);
         }
-        if (has_din) col += d;
         if (do_tier) {
             __syncwarp();
             const float nrm = md.simtier_norm == AIF_NORM_MEAN ? 1.0f / (float)slot.L : 1.0f;
             for (int k = lane; k < 64; k += 32)
-                xrow[col + k] = __float2bfloat16_rn(k < md.n_tiers ? (float)tiers[warp * 16 + k] * nrm : 0.f);
+                xrow[col_tier + k] = __float2bfloat16_rn(k < md.n_tiers ? (float)tiers[warp * 16 + k] * nrm : 0.f);
         }
         __syncwarp();
     }
@@ -1095,7 +1139,16 @@ cudaError_t launch_score_tc_scratch(const aif_ctx *ctx, const ScoreLaunch &sl_in
         if (e != cudaSuccess) return e;
     }
     const bool need_att = (c.blocks & AIF_BLK_ATT) && !att_tc, need_lsh = lsh_blocks && !lsh_tc;
-    if (pl->x_cols && (need_att || need_lsh || (c.blocks & AIF_BLK_BEA))) {
+    if (c.blocks & AIF_BLK_BEA) {
+        StageRange range("aif bea");
+        const size_t smem = (size_t)c.n_bridge * c.d * 2 + (size_t)kBeaRows * c.n_bridge * 4;
+        cudaError_t e = launch_pdl(k_bea_x, dim3(sl.n_tiles, kTcTile / kBeaRows), dim3(256), smem, st, md, sl, (__nv_bfloat16 *)sc.X, pl->x_cols,
+                                   (c.blocks & AIF_BLK_ATT) ? c.d : 0);
+        count_launch();
+        timing_mark(ctx, "bea", st);
+        if (e != cudaSuccess) return e;
+    }
+    if (need_att || need_lsh) {
         StageRange range("aif interact");
         const size_t smem = (size_t)8 * c.d * 4 + 64 * 4 + 128 * 4;
         cudaError_t e = launch_pdl(k_interact_x, dim3(sl.n_tiles), dim3(256), smem, st, md, sl, (__nv_bfloat16 *)sc.X, pl->x_cols,
