@@ -302,8 +302,7 @@ int aif_create(const aif_config *cfg, aif_ctx **out)
     TRY(dev_alloc(ctx, &ctx->Wb_t, (size_t)c.d * c.d * el, true));
     TRY(dev_alloc(ctx, &ctx->Wseq_k, (size_t)c.dU * c.d * el, true));
     TRY(dev_alloc(ctx, &ctx->Wa_k, (size_t)c.d * c.d * el, true));
-    TRY(dev_alloc(ctx, (void **)&ctx->zero_bias, 256 * 4, true));
-    if (ctx->tensor_path) TRY(dev_alloc(ctx, &ctx->ffn_rows, ((size_t)c.L_max + 128) * c.d * 2, true));
+    TRY(dev_alloc(ctx, &ctx->Wprof_k, (size_t)c.dU * c.d * el, true));
     TRY(dev_alloc(ctx, (void **)&ctx->b_a, (size_t)c.d * 4, true));
     TRY(dev_alloc(ctx, (void **)&ctx->b_b, (size_t)c.d * 4, true));
 
@@ -323,7 +322,7 @@ int aif_create(const aif_config *cfg, aif_ctx **out)
     o.pu_hl = take((size_t)c.hidden[0] * 2 * 2);
     o.prof = take((size_t)c.d * 4);
     o.partial = take((size_t)kUserPartials * c.d * 4);
-    o.ppart = take((size_t)kProfParts * (c.d + 2) * 4);
+    o.ppart = take((size_t)kProfParts * (c.d + 4) * 4);
     const bool sim = c.n_categories > 0;
     o.Sg = take(sim ? ctx->grouped_rows * c.d * el : 0);
     o.sigEg = take(sim && lsh_tc ? ctx->grouped_rows * c.lsh_bits : 0);
@@ -444,6 +443,7 @@ int aif_load_weights(aif_ctx *ctx, const aif_weights *w, aif_stream stream)
         AIF_CUDA(launch_transpose(w->W_seq, ctx->Wseq_t, c.d, c.dU, el, st));
         AIF_CUDA(launch_transpose(w->W_a, ctx->Wa_t, c.d, c.d, el, st));
         AIF_CUDA(cudaMemcpyAsync(ctx->Wseq_k, w->W_seq, (size_t)c.d * c.dU * el, cudaMemcpyDeviceToDevice, st));
+        AIF_CUDA(cudaMemcpyAsync(ctx->Wprof_k, w->W_profile, (size_t)c.d * c.dU * el, cudaMemcpyDeviceToDevice, st));
         AIF_CUDA(cudaMemcpyAsync(ctx->Wa_k, w->W_a, (size_t)c.d * c.d * el, cudaMemcpyDeviceToDevice, st));
         AIF_CUDA(launch_transpose(w->W_b, ctx->Wb_t, c.d, c.d, el, st));
         AIF_CUDA(cudaMemcpyAsync(ctx->b_a, w->b_a, (size_t)c.d * 4, cudaMemcpyDeviceToDevice, st));

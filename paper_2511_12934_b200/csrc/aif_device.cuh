@@ -43,6 +43,19 @@ __device__ __forceinline__ float warp_sum(float v)
     return v;
 }
 
+// Sixteen signature bits (two bytes, first bit = most significant bit of b0) as sixteen E4M3 bytes: +1.0 (0x38) for a set
+// bit, -1.0 (0xB8) for a clear one.
+__device__ __forceinline__ uint4 expand_sig16(uint32_t b0, uint32_t b1)
+{
+    uint32_t w[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const uint32_t nib = ~((i < 2 ? b0 : b1) >> (4 - 4 * (i & 1))) & 0xFu;   // inverted bits 4 i .. 4 i + 3, first one in bit 3
+        w[i] = 0x38383838u | ((nib & 8u) << 4) | ((nib & 4u) << 13) | ((nib & 2u) << 22) | ((nib & 1u) << 31);
+    }
+    return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
 // row (storage type, global) . q (fp32, shared), d a multiple of 8
 __device__ __forceinline__ float dot_row(const float *row, const float *q, int d)
 {
@@ -90,7 +103,7 @@ __device__ __forceinline__ float dot_row(const __nv_bfloat16 *row, const float *
 template <typename T>
 __device__ void warp_interact(const float *q, const T *S, int L, int d, float scale, bool do_att, bool do_lsh,
                               bool do_tiers, const uint32_t *sig_q, const uint8_t *sigS, int lsh_bits, int n_tiers,
-                              int *tiers, float att[8], float din[8], float *ml_out = nullptr)
+                              int *tiers, float att[8], float din[8])
 {
     const int lane = threadIdx.x & 31, dq = d >> 5, words = lsh_bits >> 5;
     float m = -INFINITY, l = 0.f;
@@ -140,13 +153,9 @@ __device__ void warp_interact(const float *q, const T *S, int L, int d, float sc
         }
     }
     if (do_att) {
-        if (ml_out) {   // partial result over a slice of the keys: left unnormalised, with its maximum and sum
-            if (lane == 0) ml_out[0] = m, ml_out[1] = l;
-        } else {
-            const float inv = 1.0f / l;
+        const float inv = 1.0f / l;
 #pragma unroll
-            for (int c = 0; c < 8; ++c) att[c] *= inv;
-        }
+        for (int c = 0; c < 8; ++c) att[c] *= inv;
     }
 }
 

@@ -106,13 +106,13 @@ struct HostSlot {
     // scratch for the user-side network
     float *prof_hat = nullptr;   // [d]
     float *partial = nullptr;    // [kUserPartials x d]
-    float *ppart = nullptr;      // [kProfParts x (d + 2)]: per key slice, unnormalised attention row, maximum, sum
+    float *ppart = nullptr;      // [kProfParts x (d + 4)]: per key slice, unnormalised attention row, maximum, sum, padding
     int32_t *cat_map = nullptr;  // [L_max]: row of every sequence item in the grouped sequence (scratch of the grouping)
     int32_t *cat_hist = nullptr; // [ceil(L_max / 1024) x n_categories]: per 1024-item block, items of every category
 };
 
-constexpr int kUserPartials = 1184;
-constexpr int kProfParts = 256;      // warps (key slices) of the profile-attention launch   // warps of the self-attention launch (148 SMs x 8)
+constexpr int kUserPartials = 1184;   // most partial sums of eq. 2's pooling (warps of the CUDA-core self-attention launch: 148 SMs x 8)
+constexpr int kProfParts = 256;       // most key slices of the profile attention
 
 // Optional per-kernel timing of the last scoring call (events on the call's stream).
 struct KernelTiming {
@@ -169,9 +169,8 @@ struct aif_ctx {
     void *w_out = nullptr;
     float *b_out = nullptr;
     void *Wprofile_t = nullptr, *Wseq_t = nullptr, *Wa_t = nullptr, *Wb_t = nullptr;
-    void *Wseq_k = nullptr, *Wa_k = nullptr;   // W_seq [d x dU], W_a [d x d] as given (K-major): operands of the tensor-core user side
-    float *zero_bias = nullptr;                // [256] zeros
-    void *ffn_rows = nullptr;                  // [L_max + 128][d] bf16: hidden FFN activations of the user state being computed
+    // W_seq, W_profile [d x dU], W_a [d x d] as given (K-major): operands of the user side's matrix products
+    void *Wseq_k = nullptr, *Wprof_k = nullptr, *Wa_k = nullptr;
     float *b_a = nullptr, *b_b = nullptr;
     bool user_weights = false;
     void *bridges = nullptr, *W_f = nullptr;   // user side of Algorithm 1: B [n_bridge x d], W_f [d x d]
@@ -225,16 +224,16 @@ ModelDev make_model(const aif_ctx *ctx);
 // table rows ids[i] (ids == nullptr: i) = rows[i] with their sidecars; *norm_max (may be null) raised to the largest row norm
 cudaError_t launch_refresh_rows(const aif_ctx *ctx, const int32_t *ids, int64_t n, const void *rows, const void *bea_w, const uint8_t *sig,
                                 float *norm_max, cudaStream_t st);
-// *out = max(*out, largest row norm) over rows ids[0..n) of `rows` (ids == nullptr: rows 0..n); ids outside [0, M) skipped
-cudaError_t launch_row_norm_max(const aif_ctx *ctx, const void *rows, const int32_t *ids, int64_t n, int64_t M, float *out, cudaStream_t st);
+// *out = max(*out, largest norm of rows 0..n)
+cudaError_t launch_row_norm_max(const aif_ctx *ctx, const void *rows, int64_t n, float *out, cudaStream_t st);
 cudaError_t launch_stage_ids(const int32_t *mapped_src, int32_t *dst, int n, cudaStream_t st);
 cudaError_t launch_gather_rows(const aif_ctx *ctx, const int32_t *ids, int64_t n, void *out, cudaStream_t st);
 cudaError_t launch_gather_sidecars(const aif_ctx *ctx, const int32_t *ids, int64_t n, void *bea_w_out, uint8_t *sig_out, cudaStream_t st);
 cudaError_t launch_transpose(const void *in, void *out, int rows, int cols, size_t el, cudaStream_t st);
 cudaError_t launch_score_simt(const aif_ctx *ctx, const ScoreLaunch &sl, cudaStream_t st);
-cudaError_t launch_user_network(const aif_ctx *ctx, HostSlot &hs, int slot_index, const aif_user_inputs *in, int L,
-                                cudaStream_t st);
 int simt_tiles_for(const aif_ctx *ctx, int n);
+// user side (aif_user.cu)
+cudaError_t launch_user_network(const aif_ctx *ctx, HostSlot &hs, int slot_index, const aif_user_inputs *in, int L, cudaStream_t st);
 
 // tensor-core path (aif_tc.cu)
 bool tc_supported(const aif_config &cfg);
@@ -252,7 +251,6 @@ cudaError_t launch_att_tc(const aif_ctx *ctx, const ScoreLaunch &sl, cudaStream_
 bool tc_lsh_supported(const aif_config &cfg);
 cudaError_t tc_lsh_prepare(aif_ctx *ctx);
 void tc_lsh_destroy(aif_ctx *ctx);
-cudaError_t launch_expand_signatures(const aif_ctx *ctx, const uint8_t *sig, int L, uint8_t *out, cudaStream_t st);
 cudaError_t launch_lsh_tc(const aif_ctx *ctx, const ScoreLaunch &sl, cudaStream_t st, void *X, int x_stride, size_t x_rows, int x_din,
                           int x_tier);
 // category sub-sequences (aif_sim.cu): the user-side grouping of a sequence, and the grouping of a launch's candidates by

@@ -218,7 +218,7 @@ cudaError_t run_pass(aif_ctx *ctx, NearlinePlan *pl, int64_t m, const void *I_ra
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     // the table's norm bound from the rows just computed (whether or not their ids turn out to lie in the table)
-    if (!(pl->tensor && pl->fused_tower) && (e = launch_row_norm_max(ctx, rows_out, nullptr, m, m, ctx->e_norm, st)) != cudaSuccess) return e;
+    if (!(pl->tensor && pl->fused_tower) && (e = launch_row_norm_max(ctx, rows_out, m, ctx->e_norm, st)) != cudaSuccess) return e;
     if (c.blocks & AIF_BLK_BEA) {
         const void *id_rows = I_id ? I_id : rows_out;
         // matrix instructions for the d that divide into whole quads of 16-byte pieces; they read 16 bytes at a time

@@ -1,7 +1,5 @@
-// CUDA-core kernels of libaif: table scatter / gather, the general scoring kernel (any storage type, all
-// interaction blocks, fp32 arithmetic) and the user-side network.  The tensor-core kernels live in aif_tc.cu.
-#include <type_traits>
-
+// CUDA-core kernels of libaif: table refresh / gather and the general scoring kernel (any storage type, all
+// interaction blocks, fp32 arithmetic).  The user-side network lives in aif_user.cu, the tensor-core kernels in aif_tc*.cu.
 #include "aif_internal.h"
 #include "aif_device.cuh"
 #include "aif_tc_ptx.cuh"
@@ -536,219 +534,18 @@ cudaError_t launch_score_simt(const aif_ctx *ctx, const ScoreLaunch &sl, cudaStr
 }
 
 // ------------------------------------------------------------------------------------------------
-// user-side network (eqs. 1-3), fp32 arithmetic on storage-type inputs
+// norm bound over a set of rows
 // ------------------------------------------------------------------------------------------------
-
-// eq. 1.  blockIdx.x < L: one sequence row -> S (storage type).  blockIdx.x == L: the profile -> prof_hat (fp32).
-template <typename T>
-__global__ void k_user_project(const T *__restrict__ seq, const T *__restrict__ profile, const T *__restrict__ Wseq_t,
-                               const T *__restrict__ Wprof_t, int L, int dU, int d, T *__restrict__ S,
-                               float *__restrict__ prof_hat)
-{
-    extern __shared__ float row[];
-    const bool is_prof = (int)blockIdx.x == L;
-    const T *src = is_prof ? profile : seq + (size_t)blockIdx.x * dU;
-    const T *W = is_prof ? Wprof_t : Wseq_t;
-    for (int k = threadIdx.x; k < dU; k += blockDim.x) row[k] = to_f(src[k]);
-    __syncthreads();
-    for (int j = threadIdx.x; j < d; j += blockDim.x) {
-        float acc = 0.f;
-        for (int k = 0; k < dU; ++k) acc = fmaf(row[k], to_f(W[(size_t)k * d + j]), acc);
-        if (is_prof) prof_hat[j] = acc;
-        else from_f(S[(size_t)blockIdx.x * d + j], acc);
-    }
-}
-
-// eq. 2.  Warp g handles rows g, g + n_warps, ...: attention over the whole sequence, FFN, and a running sum
-// for the mean pooling; partial[g] holds the warp's sum (summed later in a fixed order).  att_rows != nullptr: the
-// attention rows softmax(S S^T / sqrt(d)) S were already computed by the tensor-core attention kernel.
-template <typename T>
-__global__ void __launch_bounds__(256) k_user_self(const T *__restrict__ S, int L, int d, const T *__restrict__ Wa_t,
-                                                   const float *__restrict__ b_a, const T *__restrict__ Wb_t,
-                                                   const float *__restrict__ b_b, float *__restrict__ partial,
-                                                   int n_warps, const T *__restrict__ att_rows)
-{
-    extern __shared__ float sm[];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = blockIdx.x * 8 + warp, dq = d >> 5;
-    float *q = sm + (size_t)warp * 3 * d, *ctx = q + d;
-    float pooled[8];
-#pragma unroll
-    for (int c = 0; c < 8; ++c) pooled[c] = 0.f;
-    const float scale = rsqrtf((float)d);
-    for (int i = g; i < L; i += n_warps) {
-        if (att_rows) {
-            for (int k = lane; k < d; k += 32) ctx[k] = to_f(att_rows[(size_t)i * d + k]);
-        } else {
-            for (int k = lane; k < d; k += 32) q[k] = to_f(S[(size_t)i * d + k]);
-            __syncwarp();
-            float att[8], din[8];
-            warp_interact<T>(q, S, L, d, scale, true, false, false, nullptr, nullptr, 0, 0, nullptr, att, din);
-#pragma unroll
-            for (int c = 0; c < 8; ++c)
-                if (c < dq) ctx[lane + 32 * c] = att[c];
-        }
-        __syncwarp();
-#pragma unroll
-        for (int c = 0; c < 8; ++c)
-            if (c < dq) {
-                const int j = lane + 32 * c;
-                float acc = b_a[j];
-                for (int k = 0; k < d; ++k) acc = fmaf(ctx[k], to_f(Wa_t[(size_t)k * d + j]), acc);
-                // the second FFN layer is linear, so it commutes with the mean pooling: pool the hidden activations
-                // here and apply W_b once, in k_user_finish
-                pooled[c] += fmaxf(acc, 0.f);
-            }
-        __syncwarp();
-    }
-    if (g < n_warps) {
-#pragma unroll
-        for (int c = 0; c < 8; ++c)
-            if (c < dq) partial[(size_t)g * d + lane + 32 * c] = pooled[c];
-    }
-}
-
-// eq. 3 in slices: warp g attends the profile query to keys [g * slice, (g + 1) * slice) and leaves its unnormalised
-// output row with the slice's maximum and sum; k_user_finish merges the slices.
-template <typename T>
-__global__ void __launch_bounds__(256) k_user_prof(const T *__restrict__ S, int L, int d, const float *__restrict__ prof_hat,
-                                                   int slice, float *__restrict__ ppart)
-{
-    __shared__ float q[256];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = blockIdx.x * 8 + warp, dq = d >> 5;
-    for (int k = threadIdx.x; k < d; k += 256) q[k] = prof_hat[k];
-    __syncthreads();
-    float *out = ppart + (size_t)g * (d + 2);
-    const int start = g * slice, len = min(slice, L - start);
-    if (len <= 0) {
-        if (lane == 0) out[d] = -INFINITY, out[d + 1] = 0.f;
-        return;
-    }
-    float att[8], din[8];
-    warp_interact<T>(q, S + (size_t)start * d, len, d, rsqrtf((float)d), true, false, false, nullptr, nullptr, 0, 0, nullptr, att,
-                     din, out + d);
-#pragma unroll
-    for (int c = 0; c < 8; ++c)
-        if (c < dq) out[lane + 32 * c] = att[c];
-}
-
-// eq. 3, the combined vector, and the cached first-layer partial product p_u = W1[:, 0:d] u + b1.
-// raw = 1: u = mean-pooled self-attention + profile attention.  raw = 0: u is given (u_in, storage type).
-template <typename T>
-__global__ void __launch_bounds__(256) k_user_finish(int raw, const T *__restrict__ S, int L, int d,
-                                                     const float *__restrict__ prof_hat,
-                                                     const float *__restrict__ partial, int n_warps,
-                                                     const T *__restrict__ u_in, T *__restrict__ u_out,
-                                                     float *__restrict__ u32, const T *__restrict__ W1t,
-                                                     const float *__restrict__ b1, int H1, float *__restrict__ p_u,
-                                                     __nv_bfloat16 *__restrict__ pu_hl, const T *__restrict__ Wb_t, const float *__restrict__ b_b,
-                                                     const float *__restrict__ ppart)
-{
-    __shared__ float q[256], uprof[256], us[256], wgt[kProfParts], red[256];
-    static_assert(kProfParts == 256, "one thread per key slice");
-    const int tid = threadIdx.x;
-    if (raw) {
-        // merge the key slices of the profile attention: softmax over all keys from per-slice maxima and sums.  One
-        // thread per slice for the weights 2^(m_g - m) (kProfParts = blockDim), then one thread per output column.
-        {
-            const float m_g = ppart[(size_t)tid * (d + 2) + d], l_g = ppart[(size_t)tid * (d + 2) + d + 1];
-            red[tid] = l_g > 0.f ? m_g : -INFINITY;
-            __syncthreads();
-            for (int o = 128; o > 0; o >>= 1) {
-                if (tid < o) red[tid] = fmaxf(red[tid], red[tid + o]);
-                __syncthreads();
-            }
-            const float m_all = red[0];
-            __syncthreads();
-            const float w = l_g > 0.f ? expf(m_g - m_all) : 0.f;
-            wgt[tid] = w;
-            red[tid] = w * l_g;
-            __syncthreads();
-            for (int o = 128; o > 0; o >>= 1) {   // fixed tree: the same sum in every run
-                if (tid < o) red[tid] += red[tid + o];
-                __syncthreads();
-            }
-            const float den = red[0];
-            for (int k = tid; k < d; k += 256) {
-                float n4[4] = {0.f, 0.f, 0.f, 0.f};
-                for (int g = 0; g < kProfParts; g += 4) {   // four independent loads in flight
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) n4[u] = fmaf(wgt[g + u], ppart[(size_t)(g + u) * (d + 2) + k], n4[u]);
-                }
-                uprof[k] = ((n4[0] + n4[1]) + (n4[2] + n4[3])) / den;
-            }
-        }
-        __syncthreads();
-        // mean over the sequence of the hidden FFN activations: the warps' partial sums in a fixed order, 256 / d threads
-        // per column over interleaved slices of the partials, eight loads in flight per thread
-        {
-            const int parts = 256 / d > 0 ? 256 / d : 1;
-            const int k = tid % d, part = tid / d;
-            float a8[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-            if (part < parts && k < d) {
-                int g = part;
-                for (; g + 7 * parts < n_warps; g += 8 * parts) {
-#pragma unroll
-                    for (int u = 0; u < 8; ++u) a8[u] += partial[(size_t)(g + u * parts) * d + k];
-                }
-                for (; g < n_warps; g += parts) a8[0] += partial[(size_t)g * d + k];
-            }
-            red[tid] = ((a8[0] + a8[1]) + (a8[2] + a8[3])) + ((a8[4] + a8[5]) + (a8[6] + a8[7]));
-            __syncthreads();
-            for (int kk = tid; kk < d; kk += 256) {
-                float acc = 0.f;
-                for (int pp = 0; pp < parts; ++pp) acc += red[pp * d + kk];
-                q[kk] = acc / (float)L;
-            }
-        }
-        __syncthreads();
-        // ... through the second FFN layer, plus the profile attention: the combined user vector
-        for (int k = tid; k < d; k += 256) {
-            float acc = b_b[k];
-            for (int j = 0; j < d; ++j) acc = fmaf(q[j], to_f(Wb_t[(size_t)j * d + k]), acc);
-            const float u = acc + uprof[k];
-            us[k] = u;
-            u32[k] = u;
-            from_f(u_out[k], u);
-        }
-    } else {
-        for (int k = tid; k < d; k += 256) {
-            const float u = to_f(u_in[k]);
-            us[k] = u;
-            u32[k] = u;
-        }
-    }
-    __syncthreads();
-    for (int j = tid; j < H1; j += 256) {
-        float acc = b1[j];
-        for (int k = 0; k < d; ++k) acc = fmaf(us[k], to_f(W1t[(size_t)k * H1 + j]), acc);
-        p_u[j] = acc;
-        // the same partial as two bf16 values (high part, remainder): the form in which the tensor cores add it
-        const __nv_bfloat16 hi = __float2bfloat16_rn(acc);
-        pu_hl[j] = hi;
-        pu_hl[H1 + j] = __float2bfloat16_rn(acc - __bfloat162float(hi));
-    }
-}
-
-// the slot's length, and its key-norm bound back to zero (k_row_norm_max raises it once the rows are written)
-__global__ void k_set_slot_len(SlotDev *slots, int index, int L)
-{
-    slots[index].L = L;
-    *const_cast<float *>(slots[index].k_norm) = 0.f;
-}
-
 // Largest Euclidean norm over a set of rows, one warp per row.  Norms are non-negative, so their bit patterns order like
 // integers; a NaN row yields a pattern above every finite one and stays.
 template <typename T>
-__global__ void __launch_bounds__(256) k_row_norm_max(const T *__restrict__ rows, const int32_t *__restrict__ ids, int64_t n, int64_t M, int d,
-                                                      float *__restrict__ out)
+__global__ void __launch_bounds__(256) k_row_norm_max(const T *__restrict__ rows, int64_t n, int d, float *__restrict__ out)
 {
     const int lane = threadIdx.x & 31;
     const int64_t w0 = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5), stride = (int64_t)gridDim.x * 8;
     int best = 0;
     for (int64_t i = w0; i < n; i += stride) {
-        const int64_t r = ids ? (int64_t)ids[i] : i;
-        if (r < 0 || r >= M) continue;
-        const T *row = rows + (size_t)r * d;
+        const T *row = rows + (size_t)i * d;
         float acc = 0.f;
         for (int c = lane; c < d; c += 32) {
             const float v = to_f(row[c]);
@@ -760,193 +557,15 @@ __global__ void __launch_bounds__(256) k_row_norm_max(const T *__restrict__ rows
     if (lane == 0 && best > 0) atomicMax(reinterpret_cast<int *>(out), best);
 }
 
-cudaError_t launch_row_norm_max(const aif_ctx *ctx, const void *rows, const int32_t *ids, int64_t n, int64_t M, float *out, cudaStream_t st)
+cudaError_t launch_row_norm_max(const aif_ctx *ctx, const void *rows, int64_t n, float *out, cudaStream_t st)
 {
     if (n <= 0 || !out) return cudaSuccess;
     const int64_t want = (n + 7) / 8;
     const int grid = (int)(want < 148 * 8 ? want : 148 * 8);
-    if (ctx->cfg.dtype == AIF_F32) k_row_norm_max<float><<<grid, 256, 0, st>>>((const float *)rows, ids, n, M, ctx->cfg.d, out);
-    else k_row_norm_max<__nv_bfloat16><<<grid, 256, 0, st>>>((const __nv_bfloat16 *)rows, ids, n, M, ctx->cfg.d, out);
+    if (ctx->cfg.dtype == AIF_F32) k_row_norm_max<float><<<grid, 256, 0, st>>>((const float *)rows, n, ctx->cfg.d, out);
+    else k_row_norm_max<__nv_bfloat16><<<grid, 256, 0, st>>>((const __nv_bfloat16 *)rows, n, ctx->cfg.d, out);
     count_launch();
     return cudaGetLastError();
-}
-
-// partial[g][k] = sum over rows g, g + n_parts, ... of rows[i][k] (bf16 rows, fp32 sums in a fixed order): the mean pooling of
-// eq. 2 over hidden FFN activations that a tensor-core layer has written
-__global__ void __launch_bounds__(256) k_pool_rows(const __nv_bfloat16 *__restrict__ rows, int L, int d, int n_parts, float *__restrict__ partial)
-{
-    const int lane = threadIdx.x & 31, g = blockIdx.x * 8 + (threadIdx.x >> 5), dq = d >> 5;
-    if (g >= n_parts) return;
-    float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    for (int i = g; i < L; i += n_parts) {
-#pragma unroll
-        for (int c = 0; c < 8; ++c)
-            if (c < dq) acc[c] += __bfloat162float(rows[(size_t)i * d + lane + 32 * c]);
-    }
-#pragma unroll
-    for (int c = 0; c < 8; ++c)
-        if (c < dq) partial[(size_t)g * d + lane + 32 * c] = acc[c];
-}
-
-template <typename T>
-static cudaError_t user_network_typed(const aif_ctx *ctx, HostSlot &hs, int slot_index, const aif_user_inputs *in, int L,
-                                      cudaStream_t st)
-{
-    const aif_config &c = ctx->cfg;
-    const int d = c.d, H1 = c.hidden[0];
-    cudaError_t e;
-    T *S = (T *)hs.dev.S;
-    const bool raw = in->mode == AIF_USER_RAW;
-    // Long sequences on bf16 tensor-core contexts: eq. 1's sequence projection and the first FFN layer of eq. 2 are dense
-    // layers over L rows and run through the scoring MLP's layer kernel (tcgen05); shorter ones stay on the CUDA cores,
-    // where a launch of this size is latency, not throughput.
-    const bool tc_user = raw && std::is_same<T, __nv_bfloat16>::value && ctx->tensor_path && ctx->tc_att_plan && L >= 1024 &&
-                         c.dU % 64 == 0 && d % 64 == 0;
-    if (raw && tc_user) {
-        DenseLayer lay{};
-        lay.A = in->seq, lay.W = ctx->Wseq_k, lay.bias = ctx->zero_bias, lay.out = S, lay.in_w = c.dU, lay.H = d, lay.relu = 0, lay.sign_bits = 0;
-        if ((e = tc_dense_layer(ctx, lay, L, st)) != cudaSuccess) return e;
-        // the profile row alone (block index L of the projection kernel, launched with no sequence rows)
-        k_user_project<T><<<1, 128, c.dU * sizeof(float), st>>>((const T *)in->seq, (const T *)in->profile, (const T *)ctx->Wseq_t,
-                                                                 (const T *)ctx->Wprofile_t, 0, c.dU, d, S, hs.prof_hat);
-        count_launch();
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    } else if (raw) {
-        k_user_project<T><<<L + 1, 128, c.dU * sizeof(float), st>>>((const T *)in->seq, (const T *)in->profile,
-                                                                    (const T *)ctx->Wseq_t, (const T *)ctx->Wprofile_t, L,
-                                                                    c.dU, d, S, hs.prof_hat);
-        count_launch();
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    } else {
-        if ((e = cudaMemcpyAsync(S, in->seq, (size_t)L * d * sizeof(T), cudaMemcpyDeviceToDevice, st)) != cudaSuccess) return e;
-        if ((e = cudaMemcpyAsync((void *)hs.dev.u, in->profile, (size_t)d * sizeof(T), cudaMemcpyDeviceToDevice, st)) !=
-            cudaSuccess)
-            return e;
-    }
-    {   // zero the rows between L and the end of the last 128-key block, so that block-wise readers see no stale rows
-        const int L_pad = (L + 127) / 128 * 128 < c.L_max ? (L + 127) / 128 * 128 : c.L_max;
-        if (L_pad > L && (e = cudaMemsetAsync(S + (size_t)L * d, 0, (size_t)(L_pad - L) * d * sizeof(T), st)) != cudaSuccess) return e;
-    }
-    // the slot's length is set here already: the tensor-core self-attention below reads it like any scoring launch
-    k_set_slot_len<<<1, 1, 0, st>>>(ctx->slots_dev, slot_index, L);
-    count_launch();
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if ((e = launch_row_norm_max(ctx, S, nullptr, L, L, const_cast<float *>(hs.dev.k_norm), st)) != cudaSuccess) return e;
-    if (raw) {
-        // eq. 2: the attention rows on the tensor cores where the shape allows, else inside k_user_self
-        const T *att_rows = nullptr;
-        if (std::is_same<T, __nv_bfloat16>::value && ctx->tc_att_plan) {
-            const void *rows = nullptr;
-            if ((e = launch_self_att_tc(ctx, slot_index, L, st, &rows)) != cudaSuccess) return e;
-            att_rows = static_cast<const T *>(rows);
-        }
-        const int slice = ((L + kProfParts - 1) / kProfParts + 31) / 32 * 32;
-        k_user_prof<T><<<kProfParts / 8, 256, 0, st>>>(S, L, d, hs.prof_hat, slice, hs.ppart);
-        count_launch();
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        const int n_warps = kUserPartials;
-        if (tc_user && att_rows) {
-            // hidden = ReLU(attention rows W_a^T + b_a) as a dense layer, then the pooling sums (the second FFN layer is
-            // linear and is applied once to the pooled row, in k_user_finish)
-            DenseLayer lay{};
-            lay.A = att_rows, lay.W = ctx->Wa_k, lay.bias = ctx->b_a, lay.out = ctx->ffn_rows, lay.in_w = d, lay.H = d, lay.relu = 1, lay.sign_bits = 0;
-            if ((e = tc_dense_layer(ctx, lay, L, st)) != cudaSuccess) return e;
-            k_pool_rows<<<n_warps / 8, 256, 0, st>>>((const __nv_bfloat16 *)ctx->ffn_rows, L, d, n_warps, hs.partial);
-        } else {
-            k_user_self<T><<<n_warps / 8, 256, 8 * 3 * d * sizeof(float), st>>>(S, L, d, (const T *)ctx->Wa_t, ctx->b_a,
-                                                                                (const T *)ctx->Wb_t, ctx->b_b, hs.partial,
-                                                                                n_warps, att_rows);
-        }
-        count_launch();
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
-    k_user_finish<T><<<1, 256, 0, st>>>(raw ? 1 : 0, S, L, d, hs.prof_hat, hs.partial, kUserPartials,
-                                        (const T *)in->profile, (T *)hs.dev.u, (float *)hs.dev.u32, (const T *)ctx->Wt[0],
-                                        ctx->b[0], H1, (float *)hs.dev.p_u, (__nv_bfloat16 *)hs.dev.pu_hl, (const T *)ctx->Wb_t, ctx->b_b, hs.ppart);
-    count_launch();
-    return cudaGetLastError();
-}
-
-// Algorithm 1 steps 1-2 for one user, one block: W = Softmax(B U^T / sqrt(d)) per bridge, A_k = sum_j W_kj U_j,
-// V_k = W_f A_k.  Shared memory: W [n x m] and A [n x d] in fp32.
-template <typename T>
-__global__ void __launch_bounds__(256) k_bea_user(const T *__restrict__ Bm, const T *__restrict__ U, const T *__restrict__ Wf, int n, int m,
-                                                  int d, T *__restrict__ V)
-{
-    extern __shared__ float sm_bea[];
-    float *W = sm_bea, *A = sm_bea + n * m;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const float scale = rsqrtf((float)d);
-    for (int p = warp; p < n * m; p += 8) {   // one warp per (bridge, feature) pair
-        const int k = p / m, j = p - k * m;
-        float acc = 0.f;
-        for (int c = lane; c < d; c += 32) acc = fmaf(to_f(Bm[(size_t)k * d + c]), to_f(U[(size_t)j * d + c]), acc);
-        acc = warp_sum(acc);
-        if (lane == 0) W[p] = acc * scale;
-    }
-    __syncthreads();
-    for (int k = warp; k < n; k += 8) {       // one warp per bridge: softmax over the m features
-        float mx = -INFINITY;
-        for (int j = lane; j < m; j += 32) mx = fmaxf(mx, W[k * m + j]);
-        mx = warp_max(mx);
-        float den = 0.f;
-        for (int j = lane; j < m; j += 32) den += expf(W[k * m + j] - mx);
-        den = warp_sum(den);
-        for (int j = lane; j < m; j += 32) W[k * m + j] = expf(W[k * m + j] - mx) / den;
-    }
-    __syncthreads();
-    for (int p = tid; p < n * d; p += 256) {
-        const int k = p / d, c = p - k * d;
-        float acc = 0.f;
-        for (int j = 0; j < m; ++j) acc = fmaf(W[k * m + j], to_f(U[(size_t)j * d + c]), acc);
-        A[p] = acc;
-    }
-    __syncthreads();
-    for (int p = tid; p < n * d; p += 256) {
-        const int k = p / d, r = p - k * d;
-        float acc = 0.f;
-        for (int c = 0; c < d; ++c) acc = fmaf(to_f(Wf[(size_t)r * d + c]), A[k * d + c], acc);
-        from_f(V[p], acc);
-    }
-}
-
-cudaError_t launch_user_network(const aif_ctx *ctx, HostSlot &hs, int slot_index, const aif_user_inputs *in, int L,
-                                cudaStream_t st)
-{
-    const aif_config &c = ctx->cfg;
-    cudaError_t e;
-    if (c.blocks & AIF_BLK_CROSS) {
-        e = cudaMemcpyAsync((void *)hs.dev.T, in->cross_raw, (size_t)c.F * c.B * c.dc * ctx->el, cudaMemcpyDeviceToDevice, st);
-        if (e != cudaSuccess) return e;
-    }
-    if ((c.blocks & AIF_BLK_BEA) && in->bea_V) {
-        e = cudaMemcpyAsync((void *)hs.dev.V, in->bea_V, (size_t)c.n_bridge * c.d * ctx->el, cudaMemcpyDeviceToDevice, st);
-        if (e != cudaSuccess) return e;
-    } else if (c.blocks & AIF_BLK_BEA) {
-        const size_t smem = (size_t)(c.n_bridge * in->bea_m + c.n_bridge * c.d) * 4;
-        if (smem > 48 * 1024) {   // up to 80 KB at n_bridge = 16, bea_m = 1024, d = 256: beyond the default limit of a launch
-            e = c.dtype == AIF_F32 ? cudaFuncSetAttribute(k_bea_user<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
-                                   : cudaFuncSetAttribute(k_bea_user<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return e;
-        }
-        if (c.dtype == AIF_F32)
-            k_bea_user<float><<<1, 256, smem, st>>>((const float *)ctx->bridges, (const float *)in->bea_U, (const float *)ctx->W_f, c.n_bridge,
-                                                    in->bea_m, c.d, (float *)hs.dev.V);
-        else
-            k_bea_user<__nv_bfloat16><<<1, 256, smem, st>>>((const __nv_bfloat16 *)ctx->bridges, (const __nv_bfloat16 *)in->bea_U,
-                                                            (const __nv_bfloat16 *)ctx->W_f, c.n_bridge, in->bea_m, c.d,
-                                                            (__nv_bfloat16 *)hs.dev.V);
-        count_launch();
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
-    if (c.blocks & (AIF_BLK_LSH_DIN | AIF_BLK_SIMTIER)) {
-        e = cudaMemcpyAsync((void *)hs.dev.sigS, in->seq_sig, (size_t)L * (c.lsh_bits / 8), cudaMemcpyDeviceToDevice, st);
-        if (e != cudaSuccess) return e;
-        // the form the tensor-core LSH kernel multiplies: one +-1 byte per signature bit
-        if (ctx->tc_lsh_plan && (e = launch_expand_signatures(ctx, in->seq_sig, L, const_cast<uint8_t *>(hs.dev.sigE), st)) != cudaSuccess) return e;
-    }
-    if (c.dtype == AIF_F32) return user_network_typed<float>(ctx, hs, slot_index, in, L, st);
-    return user_network_typed<__nv_bfloat16>(ctx, hs, slot_index, in, L, st);
 }
 
 }  // namespace aif

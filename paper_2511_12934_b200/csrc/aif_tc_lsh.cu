@@ -10,7 +10,7 @@
 // (and 1 / L for the mean form) is applied once, when the tile's rows are written.  eq. 9's histogram is counted from the
 // same scores in integer arithmetic, tier = min(N - 1, floor(matches N / d')), exactly as the definition has it.
 //
-// The +-1 form of the sequence signatures is written once per user state (k_expand_signatures, user side); the +-1 form
+// The +-1 form of the sequence signatures is written once per user state (k_slot_begin, user side); the +-1 form
 // of a tile's item signatures is built in shared memory by the CTA that scores the tile.
 //
 // One CTA per SM walks over the tiles blockIdx.x, blockIdx.x + gridDim.x, ...  Warps at d = 128 (512 threads; d = 256 in
@@ -110,19 +110,6 @@ __device__ __forceinline__ LshTile lsh_tile(const LshParams &p, int tile)
     t.L = p.sl.slots[rq.slot].L, t.key0 = 0;
     t.nb = (t.L + BN - 1) / BN;
     return t;
-}
-
-// Sixteen signature bits (two bytes, first bit = most significant bit of b0) as sixteen E4M3 bytes: +1.0 (0x38) for a set
-// bit, -1.0 (0xB8) for a clear one.
-__device__ __forceinline__ uint4 expand16(uint32_t b0, uint32_t b1)
-{
-    uint32_t w[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const uint32_t nib = ~((i < 2 ? b0 : b1) >> (4 - 4 * (i & 1))) & 0xFu;   // inverted bits 4 i .. 4 i + 3, first one in bit 3
-        w[i] = 0x38383838u | ((nib & 8u) << 4) | ((nib & 4u) << 13) | ((nib & 2u) << 22) | ((nib & 1u) << 31);
-    }
-    return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
 __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel)
@@ -271,7 +258,7 @@ __global__ void __launch_bounds__((LshCfg<D, BN>::kThreads), 1) k_lsh_tc(const _
             uint4 v = make_uint4(0u, 0u, 0u, 0u);   // rows beyond the tile and ids outside the table: zeros
             if (id >= 0) {
                 const uint32_t two = *reinterpret_cast<const uint16_t *>(p.sig + (size_t)id * (D / 8) + c * 16 + sub * 2);
-                v = expand16(two & 0xFFu, two >> 8);
+                v = expand_sig16(two & 0xFFu, two >> 8);
             }
             *reinterpret_cast<uint4 *>(q + c * 16384 + r * 128 + ((sub ^ (r & 7)) << 4)) = v;
         }
@@ -669,17 +656,6 @@ __global__ void __launch_bounds__((LshCfg<D, BN>::kThreads), 1) k_lsh_tc(const _
     if (warp == C::kMmaWarp) tmem_dealloc(tmem_base, 512);
 }
 
-// Sequence signatures of a user state as +-1 bytes: out[j][b] = +1.0 (E4M3) where bit b of signature j is set, else -1.0.
-__global__ void __launch_bounds__(256) k_expand_signatures(const uint8_t *__restrict__ sig, int L, int bits, uint8_t *__restrict__ out)
-{
-    const int per_row = bits >> 4;   // 16-bit pieces per signature
-    const int64_t total = (int64_t)L * per_row;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t two = *reinterpret_cast<const uint16_t *>(sig + i * 2);
-        *reinterpret_cast<uint4 *>(out + i * 16) = expand16(two & 0xFFu, two >> 8);
-    }
-}
-
 struct LshPlan {
     CUtensorMap tmap_s, tmap_g;
     CUtensorMap tmap_sg, tmap_gg;   // categories on: the same over the grouped sequences
@@ -746,21 +722,6 @@ void tc_lsh_destroy(aif_ctx *ctx)
 {
     delete reinterpret_cast<LshPlan *>(ctx->tc_lsh_plan);
     ctx->tc_lsh_plan = nullptr;
-}
-
-cudaError_t launch_expand_signatures(const aif_ctx *ctx, const uint8_t *sig, int L, uint8_t *out, cudaStream_t st)
-{
-    const int64_t total = (int64_t)L * (ctx->cfg.lsh_bits >> 4);
-    const int grid = (int)((total + 255) / 256 < 592 ? (total + 255) / 256 : 592);
-    k_expand_signatures<<<grid, 256, 0, st>>>(sig, L, ctx->cfg.lsh_bits, out);
-    count_launch();
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    // zero bytes from the sequence's end to the end of its last 128-key block: the kernel relies on a score of exactly 0
-    // for the columns beyond the sequence (rows beyond L_max are zero-filled by the tensor map)
-    const int L_pad = (L + 127) / 128 * 128 < ctx->cfg.L_max ? (L + 127) / 128 * 128 : ctx->cfg.L_max;
-    if (L_pad > L) e = cudaMemsetAsync(out + (size_t)L * ctx->cfg.lsh_bits, 0, (size_t)(L_pad - L) * ctx->cfg.lsh_bits, st);
-    return e;
 }
 
 // LSH-DIN rows into columns [x_din, x_din + d) and SimTier rows into [x_tier, x_tier + 64) of X; a negative column turns

@@ -1,0 +1,141 @@
+"""The kernels' own edges: sizes around the tiles, steps and unit widths at which a launch changes what it does, each against
+the CPU oracle or a plain numpy statement of the same operation."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import aif_oracle as orc
+from paper_2511_12934_b200 import binding as B
+from paper_2511_12934_b200 import build as libbuild
+from paper_2511_12934_b200 import serving, synth
+from tests import helpers
+
+pytestmark = pytest.mark.gpu
+
+TOL = 2e-3
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    libbuild.build()
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    B.load_library()
+
+
+def _check(got, want, tol=TOL):
+    assert np.array_equal(np.isnan(got), np.isnan(want))
+    ok = ~np.isnan(want)
+    err = np.abs(got[ok].astype(np.float64) - want[ok]).max() if ok.any() else 0.0
+    assert err <= tol, f"max |delta| = {err:.3e} > {tol}"
+
+
+@pytest.mark.parametrize("dtype,d,nb,bits", [("bf16", 128, 8, 128), ("bf16", 64, 3, 64), ("bf16", 96, 16, 32), ("bf16", 256, 5, 256),
+                                             ("f32", 64, 8, 96), ("f32", 160, 1, 160), ("f32", 256, 16, 256)])
+def test_refresh_and_gathers_at_every_row_width_and_unit(dtype, d, nb, bits):
+    """Incremental refresh and both gathers: row widths that fill a group of lanes, do not, or need two rounds of it; sidecar
+    rows moved 16, 8, 4 and 2 bytes at a time (also because the caller's sidecar starts off a 16-byte boundary); counts
+    around a warp's step; ids outside the table."""
+    dt, M = (B.F32 if dtype == "f32" else B.BF16), 3000
+    ctx = B.Aif(B.make_config(dtype=dt, M=M, d=d, L_max=8, hidden=(64,), blocks=B.BLK_BEA | B.BLK_LSH_DIN, n_bridge=nb, lsh_bits=bits))
+    g = torch.Generator().manual_seed(d + nb)
+    E, W, S = torch.zeros(M, d, dtype=ctx.torch_dtype), torch.zeros(M, nb, dtype=ctx.torch_dtype), torch.zeros(M, bits // 8, dtype=torch.uint8)
+    for n in (1, 15, 16, 17, 63, 65, 1000):
+        ids = torch.randperm(M, generator=g)[:n].to(torch.int32)
+        rows = torch.randn(n, d, generator=g).to(ctx.torch_dtype)
+        bw = torch.randn(n + 1, nb, generator=g).to(ctx.torch_dtype)
+        sg = torch.randint(0, 256, (n + 1, bits // 8), generator=g, dtype=torch.uint8)
+        if n > 16:
+            ids[3], ids[n - 1] = -1, M
+        good = (ids >= 0) & (ids < M)
+        k = n % 2    # every other count: sidecars that start one row into their buffer
+        ctx.item_nearline_refresh(ids.cuda(), rows.cuda(), bw.cuda()[k:k + n], sg.cuda()[k:k + n])
+        E[ids[good].long()], W[ids[good].long()], S[ids[good].long()] = rows[good], bw[k:k + n][good], sg[k:k + n][good]
+        assert ctx.poll_status() == (0 if good.all() else B.STATUS_BAD_ID)
+    for n in (1, 31, 32, 33, M):
+        ids = torch.randperm(M, generator=g)[:n].to(torch.int32)
+        out = torch.empty(n, d, dtype=ctx.torch_dtype, device="cuda")
+        ow = torch.empty(n + 1, nb, dtype=ctx.torch_dtype, device="cuda")
+        os_ = torch.empty(n + 1, bits // 8, dtype=torch.uint8, device="cuda")
+        ctx.gather_rows(ids.cuda(), out)
+        if nb * out.element_size() % 4 == 0:
+            ctx.gather_sidecars(ids.cuda(), ow[1:] if ow[1:].data_ptr() % 4 == 0 else ow[:n], os_[1:])
+            got = ow[1:] if ow[1:].data_ptr() % 4 == 0 else ow[:n]
+            assert torch.equal(got.cpu(), W[ids.long()])
+        else:
+            ctx.gather_sidecars(ids.cuda(), None, os_[1:])
+        assert torch.equal(out.cpu(), E[ids.long()]) and torch.equal(os_[1:].cpu(), S[ids.long()])
+    ctx.close()
+
+
+@pytest.mark.parametrize("d", [64, 128, 256])
+@pytest.mark.parametrize("nb", [1, 7, 8, 9, 16])
+def test_bridge_weights_of_the_nearline_call(d, nb):
+    """Algorithm 1 step 3 on the matrix instructions: one and two slices of eight bridges, odd numbers of them, item counts
+    around the 16 of a warp.  A weight is at most 1 and is rounded to bf16 once (2^-9)."""
+    M = 700
+    ctx = B.Aif(B.make_config(dtype=B.BF16, M=M, d=d, L_max=8, hidden=(64,), blocks=B.BLK_BEA, n_bridge=nb))
+    g = torch.Generator(device="cuda").manual_seed(nb)
+
+    def draw(*shape):
+        return torch.randn(*shape, generator=g, device="cuda").to(torch.bfloat16)
+
+    w = {"W_i0": draw(64, 64) * 0.1, "b_i0": torch.zeros(64, device="cuda"), "W_i1": draw(d, 64) * 0.1, "b_i1": torch.zeros(d, device="cuda"),
+         "bridges": draw(nb, d)}
+    ctx.load_item_weights(w)
+    for n in (1, 15, 16, 17, 257, M):
+        raw, iid = draw(n, 64), draw(n, d)
+        ctx.item_nearline_compute(None, raw, iid)
+        if nb % 2 == 0:
+            out = torch.empty(n, nb, dtype=torch.bfloat16, device="cuda")
+            ctx.gather_sidecars(torch.arange(n, dtype=torch.int32, device="cuda"), out)
+            want = orc.item_nearline(orc.BF16, I_id=iid.cpu().view(torch.int16).numpy().view(np.uint16),
+                                     bridges=w["bridges"].cpu().view(torch.int16).numpy().view(np.uint16))["w_hat"]
+            assert np.abs(out.float().cpu().numpy() - want).max() <= 2.0 ** -9
+        assert ctx.poll_status() == 0
+    ctx.close()
+
+
+@pytest.mark.parametrize("d,dU", [(128, 128), (64, 256), (256, 64), (256, 256), (128, 96)])
+def test_user_side_at_the_lengths_around_its_row_and_key_steps(d, dU):
+    """Eqs. 1-3 from raw features: sequence lengths around the 16 rows of a product, the keys of a profile step (32, 16 or 8)
+    and the 128-key blocks; widths of every product and one that takes the CUDA cores.  u and p_u carry bf16 S and attention
+    rows (2^-9 relative on values below 0.1), S one rounding."""
+    wl = helpers.MINI["c2"].with_(name=f"user_edges_{d}_{dU}", d=d, dU=dU, M=500, N=50, L=300, mini_batch=0)
+    weights = synth.make_weights(wl, zero_bias=False)
+    srv = serving.Server(wl, weights, synth.make_item_table(wl))
+    oracle = helpers.make_oracle(wl, weights, M=500)
+    W1 = synth.as_f32(weights["mlp"]["W"][0], wl.dtype).astype(np.float64)
+    for L in (1, 7, 16, 17, 33, 128, 300):
+        rq = synth.make_request(wl, L, L=L)
+        st = srv.precompute(L, srv.upload_request(rq, B.USER_RAW))
+        u, S, pu = srv.ctx.user_state_export(st, L)
+        torch.cuda.synchronize()
+        u_ref, S_ref = oracle.user_state(rq["profile"], rq["seq"])
+        assert np.abs(S.float().cpu().numpy() - S_ref).max() <= TOL
+        assert np.abs(u.cpu().numpy() - u_ref).max() <= TOL
+        assert np.abs(pu.cpu().numpy() - (W1[:, :d] @ u_ref + weights["mlp"]["b"][0])).max() <= TOL
+        st.release()
+    assert srv.ctx.poll_status() == 0
+    srv.close()
+
+
+@pytest.mark.parametrize("n_bridge", [3, 16])
+@pytest.mark.parametrize("base", ["c2", "c5"])
+def test_bridge_embedding_columns_around_half_a_tile(base, n_bridge):
+    """v = w^ V for candidate counts around the 64 of a block, one and several requests, with and without mini-batches."""
+    wl = helpers.MINI[base].with_(name=f"bea_edges_{base}_{n_bridge}", R=3, N=200, M=2000, L=40, mini_batch=70 if base == "c2" else 0,
+                                  blocks=synth.BLK_CROSS | synth.BLK_BEA, n_bridge=n_bridge)
+    weights, table = synth.make_weights(wl, zero_bias=False), synth.make_item_table(wl)
+    srv, oracle = serving.Server(wl, weights, table), helpers.make_oracle(wl, weights, M=wl.M)
+    rqs = [synth.make_request(wl, r) for r in range(3)]
+    states = [srv.precompute(r, srv.upload_request(rq, B.USER_PROJECTED)) for r, rq in enumerate(rqs)]
+    g = np.random.default_rng(9)
+    for sizes in ((1, 64, 65), (63, 128, 200)):
+        lists = [g.choice(wl.M, n, replace=False).astype(np.int32) for n in sizes]
+        lists[2][5] = wl.M
+        want = [oracle.score(table, helpers.projected_request(wl, rq), ids) for rq, ids in zip(rqs, lists)]
+        for got, w in zip(srv.score_many(states, lists), want):
+            _check(got, w)
+        _check(srv.score_ids(states[2], lists[2]), want[2])
+    assert srv.ctx.poll_status() == B.STATUS_BAD_ID
+    srv.close()
