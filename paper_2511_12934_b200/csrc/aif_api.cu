@@ -76,18 +76,28 @@ int check_config(const aif_config *c)
 cudaStream_t as_stream(aif_stream s) { return reinterpret_cast<cudaStream_t>(s); }
 
 struct DeviceGuard {
-    int prev = -1;
-    bool ok = true;
+    int prev = -1;   // the caller's device, where it is another one
     explicit DeviceGuard(int dev)
     {
-        if (cudaGetDevice(&prev) != cudaSuccess) ok = false;
-        else if (prev != dev && cudaSetDevice(dev) != cudaSuccess) ok = false;
+        int cur = -1;
+        if (cudaGetDevice(&cur) == cudaSuccess && cur != dev && cudaSetDevice(dev) == cudaSuccess) prev = cur;
     }
     ~DeviceGuard()
     {
         if (prev >= 0) cudaSetDevice(prev);
     }
 };
+
+// The device's address of page-locked host memory that is mapped into its address space, or nullptr.
+void *mapped_address(const void *host)
+{
+    cudaPointerAttributes a{};
+    if (cudaPointerGetAttributes(&a, host) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    return a.type == cudaMemoryTypeHost ? a.devicePointer : nullptr;
+}
 
 int state_check(aif_ctx *ctx, const aif_user_state *st)
 {
@@ -625,6 +635,22 @@ int aif_user_state_export_bea(aif_ctx *ctx, const aif_user_state *state, void *V
     return AIF_OK;
 }
 
+// ids_copy: the ids lie in mapped host memory and are brought here by the first kernel that needs them more than once
+static int score_one(aif_ctx *ctx, const aif_user_state *state, const int32_t *cand_ids, int32_t n, float *logits, int32_t *ids_copy,
+                     cudaStream_t st)
+{
+    const HostSlot &hs = ctx->slots[(size_t)state->index];
+    AIF_CUDA(wait_user_ready(hs, st));
+    AIF_CUDA(wait_table_ready(ctx, st));
+    ScoreLaunch sl{};
+    sl.slots = ctx->slots_dev, sl.reqs = nullptr, sl.n_req = 1;
+    sl.single = ReqDev{state->index, n, 0, 0, 0};
+    sl.n_tiles = tiles_for(ctx, n);
+    sl.total = n, sl.max_L = hs.L;
+    sl.ids = cand_ids, sl.logits = logits, sl.status = ctx->status, sl.ids_copy = ids_copy;
+    return run_score(ctx, sl, n, st);
+}
+
 int aif_score(aif_ctx *ctx, const aif_user_state *state, const int32_t *cand_ids, int32_t n, float *logits, aif_stream stream)
 {
     StageRange range("aif_score");
@@ -635,23 +661,12 @@ int aif_score(aif_ctx *ctx, const aif_user_state *state, const int32_t *cand_ids
     if (!cand_ids || !logits) return AIF_ERR_ARG;
     if ((int64_t)n > ctx->cfg.max_batch_candidates) return AIF_ERR_SHAPE;
     DeviceGuard g(ctx->device);
-    cudaStream_t st = as_stream(stream);
-    const HostSlot &hs = ctx->slots[(size_t)state->index];
-    AIF_CUDA(wait_user_ready(hs, st));
-    AIF_CUDA(wait_table_ready(ctx, st));
-    ScoreLaunch sl{};
-    sl.slots = ctx->slots_dev, sl.reqs = nullptr, sl.n_req = 1;
-    sl.single = ReqDev{state->index, n, 0, 0, 0};
-    sl.n_tiles = tiles_for(ctx, n);
-    sl.total = n, sl.max_L = hs.L;
-    sl.ids = cand_ids, sl.logits = logits, sl.status = ctx->status;
-    return run_score(ctx, sl, n, st);
+    return score_one(ctx, state, cand_ids, n, logits, nullptr, as_stream(stream));
 }
 
-int aif_score_batch(aif_ctx *ctx, int32_t n_req, const aif_user_state *const *states, const int32_t *cand_ids,
-                    const int64_t *offsets, float *logits, aif_stream stream)
+static int score_batch(aif_ctx *ctx, int32_t n_req, const aif_user_state *const *states, const int32_t *cand_ids,
+                       const int64_t *offsets, float *logits, int32_t *ids_copy, aif_stream stream)
 {
-    StageRange range("aif_score_batch");
     if (!ctx || !states || !offsets || n_req < 0) return AIF_ERR_ARG;
     if (n_req == 0) return AIF_OK;
     if (n_req > ctx->ring.capacity) return AIF_ERR_SHAPE;
@@ -689,12 +704,19 @@ int aif_score_batch(aif_ctx *ctx, int32_t n_req, const aif_user_state *const *st
     AIF_CUDA(cudaMemcpyAsync(ring.dev[slot], ring.host[slot], sizeof(ReqDev) * (size_t)n_req, cudaMemcpyHostToDevice, st));
     ScoreLaunch sl{};
     sl.slots = ctx->slots_dev, sl.reqs = ring.dev[slot], sl.n_req = n_req, sl.n_tiles = tiles, sl.total = total, sl.max_L = max_L;
-    sl.ids = cand_ids, sl.logits = logits, sl.status = ctx->status;
+    sl.ids = cand_ids, sl.logits = logits, sl.status = ctx->status, sl.ids_copy = ids_copy;
     int rc = run_score(ctx, sl, total, st);
     if (rc != AIF_OK) return rc;
     AIF_CUDA(cudaEventRecord(ring.ev[slot], st));
     ring.used[slot] = true;
     return AIF_OK;
+}
+
+int aif_score_batch(aif_ctx *ctx, int32_t n_req, const aif_user_state *const *states, const int32_t *cand_ids,
+                    const int64_t *offsets, float *logits, aif_stream stream)
+{
+    StageRange range("aif_score_batch");
+    return score_batch(ctx, n_req, states, cand_ids, offsets, logits, nullptr, stream);
 }
 
 int aif_score_host(aif_ctx *ctx, const aif_user_state *state, const int32_t *host_ids, int32_t n, float *host_logits,
@@ -708,24 +730,15 @@ int aif_score_host(aif_ctx *ctx, const aif_user_state *state, const int32_t *hos
     if (!host_ids || !host_logits) return AIF_ERR_ARG;
     DeviceGuard g(ctx->device);
     cudaStream_t st = as_stream(stream);
-    // Page-locked buffers that are mapped into the device's address space need no copy engine: a small kernel pulls
-    // the ids over, and the last scoring kernel writes the logits straight into the host buffer.
-    auto mapped = [](const void *hp) -> void * {
-        cudaPointerAttributes a{};
-        if (cudaPointerGetAttributes(&a, hp) != cudaSuccess) {
-            cudaGetLastError();
-            return nullptr;
-        }
-        return a.type == cudaMemoryTypeHost ? a.devicePointer : nullptr;
-    };
-    void *d_ids = mapped(host_ids), *d_out = mapped(host_logits);
+    // Page-locked buffers that are mapped into the device's address space need no copy engine: the first scoring kernel
+    // reads the ids across the bus, and the last one writes the logits straight into the host buffer.
+    void *d_ids = mapped_address(host_ids), *d_out = mapped_address(host_logits);
     if (d_ids && d_out) {
-        AIF_CUDA(launch_stage_ids(static_cast<const int32_t *>(d_ids), ctx->ids_stage, n, st));
-        rc = aif_score(ctx, state, ctx->ids_stage, n, static_cast<float *>(d_out), stream);
+        rc = score_one(ctx, state, static_cast<const int32_t *>(d_ids), n, static_cast<float *>(d_out), ctx->ids_stage, st);
         if (rc != AIF_OK) return rc;
     } else {
         AIF_CUDA(cudaMemcpyAsync(ctx->ids_stage, host_ids, (size_t)n * 4, cudaMemcpyHostToDevice, st));
-        rc = aif_score(ctx, state, ctx->ids_stage, n, ctx->logits_stage, stream);
+        rc = score_one(ctx, state, ctx->ids_stage, n, ctx->logits_stage, nullptr, st);
         if (rc != AIF_OK) return rc;
         AIF_CUDA(cudaMemcpyAsync(host_logits, ctx->logits_stage, (size_t)n * 4, cudaMemcpyDeviceToHost, st));
     }
@@ -745,10 +758,18 @@ int aif_score_batch_host(aif_ctx *ctx, int32_t n_req, const aif_user_state *cons
     if (!host_ids || !host_logits) return AIF_ERR_ARG;
     DeviceGuard g(ctx->device);
     cudaStream_t st = as_stream(stream);
-    AIF_CUDA(cudaMemcpyAsync(ctx->ids_stage, host_ids, (size_t)total * 4, cudaMemcpyHostToDevice, st));
-    const int rc = aif_score_batch(ctx, n_req, states, ctx->ids_stage, offsets, ctx->logits_stage, stream);
+    // Mapped buffers as in aif_score_host: the logits cross the bus while the last layer is still running instead of in a copy
+    // after it (64 requests of 10^4 candidates: 49 us).  Ids up to kMappedIds are read across the bus by the kernel that hashes
+    // them; kernels read the bus at 20 GB/s here and a copy takes 8 us plus 50 GB/s, so longer lists are copied.
+    constexpr int64_t kMappedIds = 65536;
+    void *d_ids = mapped_address(host_ids), *d_out = mapped_address(host_logits);
+    const bool direct = d_ids && d_out && total <= kMappedIds;
+    if (!direct) AIF_CUDA(cudaMemcpyAsync(ctx->ids_stage, host_ids, (size_t)total * 4, cudaMemcpyHostToDevice, st));
+    float *out = d_out ? static_cast<float *>(d_out) : ctx->logits_stage;
+    const int rc = direct ? score_batch(ctx, n_req, states, static_cast<const int32_t *>(d_ids), offsets, out, ctx->ids_stage, stream)
+                          : score_batch(ctx, n_req, states, ctx->ids_stage, offsets, out, nullptr, stream);
     if (rc != AIF_OK) return rc;
-    AIF_CUDA(cudaMemcpyAsync(host_logits, ctx->logits_stage, (size_t)total * 4, cudaMemcpyDeviceToHost, st));
+    if (!d_out) AIF_CUDA(cudaMemcpyAsync(host_logits, ctx->logits_stage, (size_t)total * 4, cudaMemcpyDeviceToHost, st));
     AIF_CUDA(cudaStreamSynchronize(st));
     return AIF_OK;
 }

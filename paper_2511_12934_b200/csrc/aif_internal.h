@@ -83,6 +83,7 @@ struct ScoreLaunch {
     int64_t total;          // candidates of the launch
     int32_t max_L;          // longest behaviour sequence among the launch's requests (host-side hint)
     const int32_t *ids;
+    int32_t *ids_copy;      // not nullptr: `ids` is mapped host memory, and a chain of kernels copies it here before it goes on
     float *logits;
     uint32_t *status;
     const TileDev *tiles;   // [n_tiles] (tensor-core tiles), or nullptr: search `reqs` per tile
@@ -226,7 +227,7 @@ cudaError_t launch_refresh_rows(const aif_ctx *ctx, const int32_t *ids, int64_t 
                                 float *norm_max, cudaStream_t st);
 // *out = max(*out, largest norm of rows 0..n)
 cudaError_t launch_row_norm_max(const aif_ctx *ctx, const void *rows, int64_t n, float *out, cudaStream_t st);
-cudaError_t launch_stage_ids(const int32_t *mapped_src, int32_t *dst, int n, cudaStream_t st);
+cudaError_t launch_stage_ids(const int32_t *mapped_src, int32_t *dst, int64_t n, cudaStream_t st);
 cudaError_t launch_gather_rows(const aif_ctx *ctx, const int32_t *ids, int64_t n, void *out, cudaStream_t st);
 cudaError_t launch_gather_sidecars(const aif_ctx *ctx, const int32_t *ids, int64_t n, void *bea_w_out, uint8_t *sig_out, cudaStream_t st);
 cudaError_t launch_transpose(const void *in, void *out, int rows, int cols, size_t el, cudaStream_t st);

@@ -91,15 +91,14 @@ __global__ void __launch_bounds__(256) k_refresh_rows(uint4 *__restrict__ table,
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5, n_warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     int best = 0;
     for (int64_t r0 = warp * RPS; r0 < n; r0 += n_warps * RPS) {
-        int my = -1;
-        if (lane < RPS && r0 + lane < n) {
-            const int64_t dst = ids ? (int64_t)ids[r0 + lane] : r0 + lane;
-            if (dst >= 0 && dst < M) my = (int)dst;
-            else atomicOr(status, AIF_STATUS_BAD_ID);
-        }
+        // the ids and the first vectors of all rows are requested together: the ids are needed only for the stores
+        int64_t dst_row = -1;
+        const bool has_id = lane < RPS && r0 + lane < n;
+        if (has_id) dst_row = ids ? (int64_t)ids[r0 + lane] : r0 + lane;
         float ss[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u) ss[u] = 0.f;
+        int my = -1;
         for (int c0 = c; c0 - c < vpr; c0 += G) {
             uint4 v[8];
 #pragma unroll
@@ -107,6 +106,7 @@ __global__ void __launch_bounds__(256) k_refresh_rows(uint4 *__restrict__ table,
                 const int64_t r = r0 + u * RPI + sub;
                 v[u] = r < n && c0 < vpr ? __ldcs(rows + r * vpr + c0) : make_uint4(0, 0, 0, 0);
             }
+            my = dst_row >= 0 && dst_row < M ? (int)dst_row : -1;
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
                 const int dst = __shfl_sync(0xffffffffu, my, u * RPI + sub);
@@ -116,6 +116,7 @@ __global__ void __launch_bounds__(256) k_refresh_rows(uint4 *__restrict__ table,
                 }
             }
         }
+        if (has_id && my < 0) atomicOr(status, AIF_STATUS_BAD_ID);
         if (norm_max) {
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
@@ -165,17 +166,19 @@ __global__ void __launch_bounds__(256) k_gather_rows(const uint4 *__restrict__ t
 }
 
 // Copies candidate ids from page-locked host memory that is mapped into the device's address space.
-__global__ void __launch_bounds__(256) k_stage_ids(const int32_t *__restrict__ src, int32_t *__restrict__ dst, int n)
+__global__ void __launch_bounds__(256) k_stage_ids(const int32_t *__restrict__ src, int32_t *__restrict__ dst, int64_t n)
 {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) dst[i] = src[i];
+    grid_dep_launch();
+    grid_dep_wait();
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) dst[i] = src[i];
 }
 
-cudaError_t launch_stage_ids(const int32_t *mapped_src, int32_t *dst, int n, cudaStream_t st)
+cudaError_t launch_stage_ids(const int32_t *mapped_src, int32_t *dst, int64_t n, cudaStream_t st)
 {
-    const int grid = (n + 255) / 256 < 148 ? (n + 255) / 256 : 148;
-    k_stage_ids<<<grid, 256, 0, st>>>(mapped_src, dst, n);
+    const int grid = (int)((n + 255) / 256 < 592 ? (n + 255) / 256 : 592);
+    const cudaError_t e = launch_pdl(k_stage_ids, dim3(grid), dim3(256), 0, st, mapped_src, dst, n);
     count_launch();
-    return cudaGetLastError();
+    return e;
 }
 
 static int grid_for(int64_t items, int per_block, int cap)
@@ -243,7 +246,7 @@ __global__ void __launch_bounds__(256) k_gather_rows_w(const uint4 *__restrict__
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
             const int64_t r = r0 + u * RPI + sub;
-            if (r < n) out[r * VPR + c] = v[u];
+            if (r < n) __stcs(out + r * VPR + c, v[u]);
         }
     }
 }

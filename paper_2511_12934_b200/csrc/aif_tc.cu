@@ -123,30 +123,45 @@ __device__ __forceinline__ TileInfo decode_tile(const LayerParams &p, int tile, 
 
 // Cross-feature index generation for a whole launch (Section 3.3, "real-time generation" from the candidate's
 // attribute): xb[pos][f] = bucket of candidate pos in field f, or kNoBucket for an id outside the item table.  Done
-// once per call so that the layer kernel's gather threads only look the bucket up.
+// once per call so that the layer kernel's gather threads only look the bucket up.  Ids in mapped host memory are copied
+// to ids_copy on the way, for the kernels that follow.
 constexpr uint32_t kNoBucket = 0xFFFFu;
 __global__ void __launch_bounds__(256) k_cross_buckets(const int32_t *__restrict__ ids, int64_t total, int64_t M, int F, int B,
-                                                        int b_mask, int mode, uint16_t *__restrict__ xb)
+                                                        int b_mask, int mode, uint16_t *__restrict__ xb, int32_t *__restrict__ ids_copy)
 {
     grid_dep_launch();
     grid_dep_wait();
-    // eight threads per candidate, each taking every eighth field: the id is read once per thread, nothing is divided,
-    // and a warp's stores cover four candidates' rows of F entries
-    const int sub = threadIdx.x & 7;
-    for (int64_t pos = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 3; pos < total; pos += ((int64_t)gridDim.x * blockDim.x) >> 3) {
-        const int id = ids[pos];
-        const bool good = id >= 0 && (int64_t)id < M;
-        uint16_t *row = xb + pos * F;
-        for (int f = sub; f < F; f += 8) {
-            uint32_t bk = kNoBucket;
-            if (good) {
-                if (mode == AIF_BUCKET_MOD) bk = (uint32_t)(id % B);
-                else {
-                    const uint64_t h = mix64((uint64_t)id, (uint64_t)f);
-                    bk = b_mask >= 0 ? (uint32_t)(h & (uint64_t)b_mask) : (uint32_t)(h % (uint64_t)B);
+    // A warp takes 32 consecutive candidates: one coalesced read of their ids (128 bytes, also the right size for a read
+    // across the bus), then 32 F hashes that depend on nothing else, two per thread and round, leaving as one 4-byte store
+    // per thread (an odd number of fields, possible only with embeddings of 64 columns and more, takes one hash per round).
+    const int lane = threadIdx.x & 31, step = F & 1 ? 1 : 2;
+    const int64_t n_warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t base = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; base < total; base += n_warps * 32) {
+        int my = -1;
+        if (base + lane < total) {
+            my = ids[base + lane];
+            if (ids_copy && blockIdx.y == 0) ids_copy[base + lane] = my;
+        }
+        const int n = (int)min((int64_t)32, total - base) * F;
+        uint16_t *out = xb + base * F;
+        // small launches spread a warp's hashes over gridDim.y warps (the ids are then read that many times)
+        for (int i0 = 32 * step * (int)blockIdx.y; i0 < 32 * F; i0 += 32 * step * (int)gridDim.y) {
+            const int i = i0 + lane * step, c = i / F, f = i - c * F;
+            const int id = __shfl_sync(0xffffffffu, my, c & 31);
+            const bool good = id >= 0 && (int64_t)id < M;
+            uint32_t bk[2] = {kNoBucket, kNoBucket};
+#pragma unroll
+            for (int q = 0; q < 2; ++q)
+                if (good && q < step) {
+                    if (mode == AIF_BUCKET_MOD) bk[q] = (uint32_t)(id % B);
+                    else {
+                        const uint64_t h = mix64((uint64_t)id, (uint64_t)(f + q));
+                        bk[q] = b_mask >= 0 ? (uint32_t)(h & (uint64_t)b_mask) : (uint32_t)(h % (uint64_t)B);
+                    }
                 }
-            }
-            row[f] = (uint16_t)bk;
+            if (i >= n) continue;
+            if (step == 2) *reinterpret_cast<uint32_t *>(out + i) = bk[0] | (bk[1] << 16);
+            else out[i] = (uint16_t)bk[0];
         }
     }
 }
@@ -1093,6 +1108,12 @@ cudaError_t launch_score_tc_scratch(const aif_ctx *ctx, const ScoreLaunch &sl_in
         timing_mark(ctx, "score_fused", st);
         return e;
     }
+    // ids across the bus: on the way through the bucket kernel where that one comes first, else by a copy of their own
+    if (sl.ids_copy && (c.n_categories > 0 || !(c.blocks & AIF_BLK_CROSS))) {
+        cudaError_t e = launch_stage_ids(sl.ids, sl.ids_copy, sl.total, st);
+        if (e != cudaSuccess) return e;
+        sl.ids = sl.ids_copy, sl.ids_copy = nullptr;
+    }
     if (c.n_categories > 0) {
         // candidates grouped by (request, category): tiles, grouped ids and the way back to the caller's order
         if (sc.rows < (size_t)sl.total + kTcTile || !ctx->sim_plan) return cudaErrorInvalidValue;
@@ -1108,10 +1129,15 @@ cudaError_t launch_score_tc_scratch(const aif_ctx *ctx, const ScoreLaunch &sl_in
     }
     if (c.blocks & AIF_BLK_CROSS) {
         StageRange range("aif buckets");
-        const int64_t n = sl.total * 8;   // eight threads per candidate
+        const int64_t n = sl.total;   // a warp per 32 candidates
         const int grid = (int)((n + 255) / 256 < 148 * 16 ? (n + 255) / 256 : 148 * 16);
-        cudaError_t e = launch_pdl(k_cross_buckets, dim3(grid), dim3(256), 0, st, sl.ids, sl.total, c.M, c.F, c.B,
-                                   (c.B & (c.B - 1)) == 0 ? c.B - 1 : -1, c.bucket_mode, (uint16_t *)sc.xb);
+        // launches that leave SMs without a block split the fields of a candidate over up to eight warps, except where a read
+        // of the ids crosses the bus
+        const int rounds = c.F & 1 ? c.F : c.F / 2, want_y = sl.ids_copy ? 1 : 296 / grid;
+        const int grid_y = want_y < 1 ? 1 : want_y > 8 ? (rounds < 8 ? rounds : 8) : want_y > rounds ? rounds : want_y;
+        cudaError_t e = launch_pdl(k_cross_buckets, dim3(grid, grid_y), dim3(256), 0, st, sl.ids, sl.total, c.M, c.F, c.B,
+                                   (c.B & (c.B - 1)) == 0 ? c.B - 1 : -1, c.bucket_mode, (uint16_t *)sc.xb, sl.ids_copy);
+        if (sl.ids_copy) sl.ids = sl.ids_copy;
         count_launch();
         timing_mark(ctx, "buckets", st);
         if (e != cudaSuccess) return e;

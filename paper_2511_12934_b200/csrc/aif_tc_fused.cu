@@ -119,9 +119,12 @@ __global__ void __launch_bounds__(kFThreads, 1) k_request_fused(const __grid_con
         const ReqDev rq0 = find_request(p.sl, blockIdx.x);
         int start0, cnt0;
         tile_range(blockIdx.x - rq0.tile_begin, rq0.n, kTcTile, p.mini_batch, start0, cnt0);
-        const int r0 = (tid - kFProdWarp0 * 32) >> 3;
+        // every id is read once per tile (they may lie in host memory across the bus): lane l takes row 4 w + l % 4 + 16 (l / 4)
+        // of warp w's rows, the threads that copy a row get it by shuffle
+        const int w = warp - kFProdWarp0, r = 4 * w + (lane & 3) + 16 * (lane >> 2);
+        const int mine = r < cnt0 ? p.sl.ids[rq0.off + start0 + r] : -1;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) id[i] = r0 + 16 * i < cnt0 ? p.sl.ids[rq0.off + start0 + r0 + 16 * i] : -1;
+        for (int i = 0; i < 8; ++i) id[i] = __shfl_sync(0xffffffffu, mine, (lane >> 3) + 4 * i);
     }
     if (warp == kFMmaWarp) tmem_alloc(smem_u32(tmem_slot), 512);
     tc_fence_before();
