@@ -1,23 +1,21 @@
 // Tensor-core scoring path for sm_100a (bf16 storage): the scoring MLP as tcgen05 GEMMs with a fused gather
 // prologue and fused epilogues.
 //
-// One layer = one persistent kernel (k_layer_tc<MODE>).  A work item is one or two 128-candidate tiles times one or two
-// 256-wide slices of the layer's outputs (LayerCfg below).  Roles inside a CTA (one accumulator: 320 threads, two: 576):
-//   epilogue   4 warps per accumulator: read the fp32 accumulator from TMEM (tcgen05.ld), add the bias (for the first
-//              layer the request's cached user partial p_u), ReLU, then either store bf16 activations for the next
-//              layer (through a staging slab and a TMA tile store), reduce against w_out and write the logit, or (item
-//              side of the nearline pipeline) store without ReLU / pack the sign bits of the outputs
-//   MMA        one warp allocates TMEM; one lane issues tcgen05.mma (M=128, N<=256, K=16, bf16 in, fp32 accumulate)
-//   A producer 4 warps per tile: gather the tile's input rows chunk by chunk (64 columns = 128 bytes per row) with
-//              16-byte cp.async into the 128B-swizzled K-major layout the MMA reads: item-table rows by candidate
-//              id, cross-feature rows by (field, bucket) from the request's pre-cache with the bucket looked up in
-//              the table k_cross_buckets wrote; dense rows (attention output, previous activations, raw item
-//              features) come by position as one TMA tile per chunk.
-//              Ids of the next item and the sources of the next chunk are fetched ahead of their use.
-//   B producer one lane streams the weight slice with TMA (cp.async.bulk.tensor, 128B swizzle)
-// Shared-memory rings (mbarriers) decouple producers from the MMA.  Two TMEM accumulators of 256 columns: with one
-// accumulator per item they alternate so that the epilogue of one item overlaps the main loop of the next; with two,
-// each tile (or output slice) of the item owns one.  Every wait is bounded: on expiry the CTA raises
+// One layer = one persistent kernel (k_layer_pair).  A work item is a pair of 128-candidate tiles, one per CTA of a cluster of
+// two, times a slice of up to 256 of the layer's outputs.  Roles inside a CTA:
+//   epilogue   8 warps: read the fp32 accumulator from TMEM (tcgen05.ld), add the bias (for the first layer the request's
+//              cached user partial p_u), ReLU, then either store bf16 activations for the next layer (through a staging slab
+//              and a TMA tile store), reduce against w_out and write the logit, or (item side of the nearline pipeline)
+//              store without ReLU / pack the sign bits of the outputs
+//   MMA        one warp allocates TMEM; one lane of the even CTA issues tcgen05.mma.cta_group::2 (M=256, N<=256, K=16, bf16
+//              in, fp32 accumulate)
+//   A producer 6 warps: bring the tile's input rows chunk by chunk (64 columns = 128 bytes per row) into the 128B-swizzled
+//              K-major layout the MMA reads: with 16-byte cp.async item-table rows by candidate id and cross-feature rows by
+//              (field, bucket) from the request's pre-cache, the bucket looked up in the table k_cross_buckets wrote; dense
+//              rows (attention output, previous activations, raw item features) by position as one TMA tile per chunk
+//   B producer one lane streams the CTA's half of the weight slice with TMA (cp.async.bulk.tensor, 128B swizzle)
+// A shared-memory ring (mbarriers) decouples producers from the MMA; two TMEM accumulators of 256 columns alternate so that the
+// epilogue of one item overlaps the main loop of the next.  Every wait is bounded: on expiry the CTA raises
 // AIF_STATUS_TIMEOUT, all roles leave their loops, TMEM is freed and the kernel returns.
 #include <cuda.h>
 
@@ -44,6 +42,7 @@ struct ChunkSrc {
 struct LayerParams {
     ScoreLaunch sl;
     int32_t n_nchunks, n_cols, n_k, mini_batch;
+    int32_t n_out;                // outputs of the layer (the last slice may be narrower than n_cols)
     // A sources
     const uint8_t *E;
     int64_t M;
@@ -51,6 +50,8 @@ struct LayerParams {
     int32_t x_row_bytes;
     const uint8_t *X;             // dense rows, indexed by candidate position in the launch
     const uint16_t *xb;           // cross-feature buckets [positions x F], written by k_cross_buckets
+    const uint8_t *T0;            // cross pre-cache of slot 0; slot i's lies i * slot_bytes further
+    int64_t slot_bytes;
     int32_t F, B, dc;
     int32_t check_ids;            // first layer: flag ids outside the table
     // epilogue
@@ -62,36 +63,6 @@ struct LayerParams {
     const __nv_bfloat16 *w_out;
     const float *b_out;
     ChunkSrc src[kMaxChunks];
-};
-
-// Geometry of the layer kernel.  A work item fills one or two 256-column TMEM accumulators:
-//   MODE 0  one tile, one 256-wide output slice; the two accumulators alternate between consecutive items so that the
-//           epilogue of one overlaps the main loop of the next (small launches, every item on its own SM)
-//   MODE 1  two tiles, one slice: one weight chunk in shared memory feeds both tiles, which halves the weight traffic
-//           per candidate (large launches)
-//   MODE 2  one tile, two slices: one gathered A chunk feeds both slices, so the tile's rows are gathered once instead
-//           of once per slice (launches that would otherwise need a second round of items)
-//   MODE 3  as MODE 1 with a deeper A ring and a shallower B ring, for the first layer: its cross-feature rows come
-//           from per-request tables that may live in HBM, the weights from L2
-// A and B have rings of their own: gathered rows have the longer latency and the smaller chunks.
-template <int MODE>
-struct LayerCfg {
-    static constexpr int G = (MODE == 1 || MODE == 3) ? 2 : 1;   // tiles per work item
-    static constexpr int NB = MODE == 2 ? 2 : 1;         // output slices per work item
-    static constexpr int kAcc = G * NB;                  // accumulators a work item fills
-    static constexpr int kStagesA = MODE == 1 ? 3 : 4;
-    static constexpr int kStagesB = MODE == 0 ? 4 : (MODE == 1 ? 3 : 2);
-    static constexpr int kAStage = G * kABytes, kBStage = NB * kBBytes;
-    static constexpr int kEpiWarps = 4 * kAcc;
-    static constexpr int kMmaWarp = kEpiWarps;
-    static constexpr int kProdWarp0 = kEpiWarps + 1;
-    static constexpr int kProdThreads = 128 * G;    // 128 producer threads per tile of the group, 8 rows each
-    static constexpr int kBWarp = kProdWarp0 + 4 * G;
-    static constexpr int kThreads = (kBWarp + 1) * 32;
-    static constexpr int kSlabs = MODE == 0 ? 2 : 1;    // output staging slabs (2 KB) per epilogue warp
-    static_assert(1024 + kStagesA * kAStage + kStagesB * kBStage + kEpiWarps * kSlabs * 2048 + 8192 <= 227 * 1024, "shared memory");
-    static constexpr size_t kSmem = 1024 + (size_t)kStagesA * kAStage + (size_t)kStagesB * kBStage + (2 * kStagesA + 2 * kStagesB + 4) * 8 +
-                                    32 + 2 * kAcc * 256 * 4 + kEpiWarps * kSlabs * 2048 + 2 * G * 128 * 4;
 };
 
 struct TileInfo {
@@ -184,115 +155,127 @@ __global__ void __launch_bounds__(256) k_tile_table(ScoreLaunch sl, int mini_bat
     out[tile] = t;
 }
 
-// ---- the layer kernel -----------------------------------------------------------------------------------------
-template <int MODE>
-__global__ void __launch_bounds__(LayerCfg<MODE>::kThreads, 1) k_layer_tc(const __grid_constant__ CUtensorMap tmapB,
-                                                                          const __grid_constant__ CUtensorMap tmapOut,
-                                                                          const __grid_constant__ CUtensorMap tmapA, const LayerParams p)
+// ---- the layer kernel ---------------------------------------------------------------------------------------------
+// Every product spans two SMs (cta_group::2).  What bounds a layer is the rate at which an SM takes in operands (59 bytes per
+// clock).  With both tiles of an item in one SM, which that rate asks for, their accumulators filled tensor memory and the
+// epilogue was exposed, 6 k of 22 k cycles per item (64 requests of 10^4 candidates, first layer).  Here a CTA holds its tile's
+// rows and half of the weight slice, 32 KB per 64-column chunk for 512 cycles of products, the same intake per flop, and one
+// 256-column accumulator: two fit, and the epilogue of an item runs under the products of the next.
+// First layer of 64 x 10^4 candidates (K = 768, 512 outputs): 471 -> 386 us; of 256 x 4000 candidates at d = 256 (K = 2560,
+// 1024 outputs): 5.17 -> 4.11 ms; second layers 176 -> 140 and 1125 -> 800 us.
+// Slices narrower than 256 are rounded up to a multiple of 64 (each CTA brings half of the weight rows, its epilogue warps
+// take whole 32-column pieces); weight rows beyond the last output arrive as zeros.
+// Roles per CTA (512 threads): 8 epilogue warps (two per quarter of the rows, half of the columns each), the MMA warp (the
+// even CTA's lane issues), 6 gather warps and one weight warp.  One ring of six stages, rows and weights of a chunk together,
+// and one arrival per CTA that both have landed: the issuing lane has one wait per chunk, which is shorter than the product it
+// leaves in the queue.
+struct PairCfg {
+    static constexpr int kStages = 6, kStage = 2 * kABytes;
+    // one gather warp per stage: a warp meets every phase of its own stage in turn, so that a wait on the phase's parity can
+    // never be answered by an older phase
+    static constexpr int kEpiWarps = 8, kMmaWarp = 8, kProdWarp0 = 9, kProdWarps = kStages, kBWarp = kProdWarp0 + kProdWarps;
+    static constexpr int kThreads = (kBWarp + 1) * 32;
+    static constexpr int kOffSlab = kStages * kStage, kOffMisc = kOffSlab + kEpiWarps * 2048;
+    // barriers and the tensor-memory slot | bias, output weights [256] | dot products of the upper halves [128]
+    static constexpr size_t kSmem = 1024 + kOffMisc + 256 + 2 * 256 * 4 + 128 * 4;
+    static_assert(kSmem <= 227 * 1024, "shared memory");
+};
+
+__global__ void __launch_bounds__(PairCfg::kThreads, 1) k_layer_pair(const __grid_constant__ CUtensorMap tmapB,
+                                                                     const __grid_constant__ CUtensorMap tmapOut,
+                                                                     const __grid_constant__ CUtensorMap tmapA, const LayerParams p)
 {
-    using C = LayerCfg<MODE>;
-    constexpr int G = C::G, NB = C::NB, kAcc = C::kAcc, kSA = C::kStagesA, kSB = C::kStagesB;
+    using C = PairCfg;
+    constexpr int kS = C::kStages;
     extern __shared__ unsigned char smem_dyn[];
     unsigned char *base = reinterpret_cast<unsigned char *>(((uintptr_t)smem_dyn + 1023) & ~(uintptr_t)1023);
-    // A ring (per stage: one chunk per tile of the group), B ring (per stage: one chunk per output slice), the output
-    // staging slabs (2 KB each) of the epilogue warps, then barriers and small arrays
-    unsigned char *smA = base, *smB = base + kSA * C::kAStage;
-    unsigned char *out_stage = smB + kSB * C::kBStage;
-    uint64_t *bars = reinterpret_cast<uint64_t *>(out_stage + C::kEpiWarps * C::kSlabs * 2048);
-    uint64_t *full_a = bars, *empty_a = full_a + kSA, *full_b = empty_a + kSA, *empty_b = full_b + kSB;
-    uint64_t *acc_full = empty_b + kSB, *acc_empty = acc_full + 2;
+    unsigned char *out_stage = base + C::kOffSlab;
+    uint64_t *bars = reinterpret_cast<uint64_t *>(base + C::kOffMisc);
+    uint64_t *full = bars, *empty = full + kS, *landed = empty + kS, *acc_full = landed + kS, *acc_empty = acc_full + 2;
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(acc_empty + 2);
     volatile uint32_t *abort_flag = tmem_slot + 1;
-    float *bias_s = reinterpret_cast<float *>(((uintptr_t)(tmem_slot + 4) + 15) & ~(uintptr_t)15);   // [kAcc][256]
-    float *wout_s = bias_s + kAcc * 256;                         // [kAcc][256]
-    int *ids_s = reinterpret_cast<int *>(wout_s + kAcc * 256);   // [2][G][128] validated ids of the current / next item
+    float *bias_s = reinterpret_cast<float *>(base + C::kOffMisc + 256), *wout_s = bias_s + 256, *dot_s = wout_s + 256;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int rank = (int)cluster_rank();   // 0: issues the products
 
     if (tid == 0) {
-        for (int s = 0; s < kSA; ++s) {
-            mbar_init(smem_u32(full_a + s), C::kProdThreads);
-            mbar_init(smem_u32(empty_a + s), 1);
-        }
-        for (int s = 0; s < kSB; ++s) {
-            mbar_init(smem_u32(full_b + s), 1);
-            mbar_init(smem_u32(empty_b + s), 1);
+        for (int s = 0; s < kS; ++s) {
+            mbar_init(smem_u32(full + s), 2);      // a gather warp of each CTA (used in the even one)
+            mbar_init(smem_u32(landed + s), 2);    // TMA copies of this CTA: announced by the weight lane and by the gather warp
+            mbar_init(smem_u32(empty + s), 1);
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(smem_u32(acc_full + b), 1);
-            mbar_init(smem_u32(acc_empty + b), 4);
+            mbar_init(smem_u32(acc_empty + b), 2 * C::kEpiWarps);   // the epilogue warps of both CTAs (used in the even one)
         }
         *abort_flag = 0u;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == C::kMmaWarp) tmem_alloc(smem_u32(tmem_slot), 512);
+    if (warp == C::kMmaWarp) tmem_alloc_pair(smem_u32(tmem_slot), 512);
     tc_fence_before();
     __syncthreads();
+    cluster_sync();   // the other CTA's barriers exist
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
     grid_dep_launch();
-    grid_dep_wait();   // everything above overlapped the tail of the previous kernel; from here on its results are read
-    // tiles formed on the device (candidates grouped by category): their number is read here
+    // The weights are older than any launch this one may overlap: where the number of tiles is known to the host, their lane
+    // starts at once.
+    const bool early = warp == C::kBWarp && !p.sl.n_tiles_dev;
+    if (!early) grid_dep_wait();
     const int n_tiles = p.sl.n_tiles_dev ? *p.sl.n_tiles_dev : p.sl.n_tiles;
-    const int n_groups = (n_tiles + G - 1) / G;
-    const int n_ncg = p.n_nchunks / NB;             // groups of output slices
-    const int n_items = n_groups * n_ncg;
+    const int n_items = ((n_tiles + 1) / 2) * p.n_nchunks;
+    const int item0 = (int)(blockIdx.x >> 1), item_step = (int)(gridDim.x >> 1);
 
     if (warp < C::kEpiWarps) {
         // ===================== epilogue =====================
-        const int a = warp >> 2;                     // accumulator this warp quartet serves
-        const int g = G == 2 ? a : 0;                // its tile of the group
-        const int row = (warp & 3) * 32 + lane;      // TMEM lane = candidate row of the tile
-        float *bs = bias_s + a * 256, *ws = wout_s + a * 256;
-        // staging slabs of 32 rows x 64 bytes, 64-byte swizzle (the layout tmapOut expects)
-        unsigned char *stg = out_stage + warp * (C::kSlabs * 2048);
-        uint32_t slab = 0;
-        int it = 0;
+        const int wq = warp & 3, half = warp >> 2;
+        const int row = wq * 32 + lane;              // TMEM lane = candidate row of the tile
+        const int hc = p.n_cols >> 1, col_lo = half * hc;
+        unsigned char *sb = out_stage + warp * 2048;   // staging slab of 32 rows x 64 bytes, 64-byte swizzle (the layout tmapOut expects)
+        const int l4 = lane & 3, r8 = lane >> 2, wrow0 = wq * 32;
+        uint32_t empty_addr[2];
+#pragma unroll
+        for (int b = 0; b < 2; ++b) empty_addr[b] = cluster_addr(smem_u32(acc_empty + b), 0u);
         // a wait that ran out in an earlier kernel of this call left its outputs unwritten: logits computed from them are
         // replaced by NaN
         const bool poisoned = p.epi == EPI_DOT && (*reinterpret_cast<volatile const uint32_t *>(p.sl.status) & AIF_STATUS_TIMEOUT) != 0u;
-        for (int item = blockIdx.x; item < n_items; item += gridDim.x, ++it) {
-            const int grp = item / n_ncg, nc = (item - grp * n_ncg) * NB + (NB == 2 ? a : 0), n0 = nc * p.n_cols;
-            const int buf = kAcc == 1 ? (it & 1) : a;
-            const uint32_t ph = kAcc == 1 ? (uint32_t)((it >> 1) & 1) : (uint32_t)(it & 1);
-            const TileInfo t = decode_tile(p, grp * G + g, n_tiles);
+        int it = 0;
+        for (int item = item0; item < n_items; item += item_step, ++it) {
+            const int grp = item / p.n_nchunks, n0 = (item - grp * p.n_nchunks) * p.n_cols;
+            const int buf = it & 1;
+            const TileInfo t = decode_tile(p, grp * 2 + rank, n_tiles);
+            const bool valid = row < t.cnt;
+            int id = -1;
+            if (p.epi == EPI_DOT && half == 0 && valid) id = p.sl.ids[t.pos0 + row];
             if (t.cnt > 0) {
                 const float *bias = p.bias_from_slot ? p.sl.slots[t.rq.slot].p_u : p.bias;
-                for (int j = row; j < p.n_cols; j += 128) {
-                    bs[j] = bias[n0 + j];
-                    if (p.epi == EPI_DOT) ws[j] = __bfloat162float(p.w_out[n0 + j]);
+                if (tid < p.n_cols) {
+                    const bool is_out = n0 + tid < p.n_out;
+                    bias_s[tid] = is_out ? bias[n0 + tid] : 0.f;
+                    if (p.epi == EPI_DOT) wout_s[tid] = is_out ? __bfloat162float(p.w_out[n0 + tid]) : 0.f;
                 }
             }
-            named_bar_sync(1 + a, 128);
-            // a wait that ran out is carried to the barrier at the end of the item, so that the four warps of an
-            // accumulator leave together and none is left waiting there
-            const bool got = __all_sync(0xffffffffu, mbar_wait(smem_u32(acc_full + buf), ph, abort_flag));
+            named_bar_sync(1, 256);
+            // a wait that ran out is carried to the barrier at the end of the item, so that the warps leave together
+            const bool got = __all_sync(0xffffffffu, mbar_wait(smem_u32(acc_full + buf), (uint32_t)((it >> 1) & 1), abort_flag));
             tc_fence_after();
-            const bool valid = row < t.cnt;
-            const uint32_t taddr = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(buf * 256);
+            const uint32_t taddr = tmem_base + ((uint32_t)wrow0 << 16) + (uint32_t)(buf * 256 + col_lo);
             float dot = 0.f;
-            const float floor_v = p.linear_out ? -INFINITY : 0.f;
             if (got && t.cnt > 0 && p.epi == EPI_STORE) {
-                // Activations of a hidden layer.  The accumulator is read in the 16x256b shape: a thread then owns two
-                // columns (per group of eight) over four rows, needs eight bias values per 32 columns instead of all 32,
-                // and the bias reads, which every row thread used to repeat, no longer fill the shared memory's return
-                // path.  Three instructions per pair of outputs: bias added to both (f32x2), rounded to bf16, ReLU on
-                // the rounded pair (rounding is monotonic and keeps zero: the same result in either order).
-                const int l4 = lane & 3, r8 = lane >> 2;
-                const __nv_bfloat162 floor2 = __float2bfloat162_rn(floor_v);
-                const int wrow0 = (warp & 3) * 32;
-                for (int c0 = 0; c0 < p.n_cols; c0 += 32) {
+                // The accumulator is read in the 16x256b shape: a thread owns two columns (per group of eight) over four rows
+                // and needs eight bias values per 32 columns.  Three instructions per pair of outputs: bias added to both
+                // (f32x2), rounded to bf16, ReLU on the rounded pair (rounding is monotonic and keeps zero).
+                const __nv_bfloat162 floor2 = __float2bfloat162_rn(p.linear_out ? -INFINITY : 0.f);
+                for (int c0 = 0; c0 < hc && n0 + col_lo + c0 < p.n_out; c0 += 32) {   // stored widths are multiples of 32
                     uint32_t ra[16], rb[16];
                     tmem_ld16x256(taddr + (uint32_t)c0, ra);                    // rows 0..15 of this warp's 32
                     tmem_ld16x256(taddr + (16u << 16) + (uint32_t)c0, rb);      // rows 16..31
                     uint64_t bias2[4];
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) bias2[j] = *reinterpret_cast<const uint64_t *>(bs + c0 + 8 * j + 2 * l4);
+                    for (int j = 0; j < 4; ++j) bias2[j] = *reinterpret_cast<const uint64_t *>(bias_s + col_lo + c0 + 8 * j + 2 * l4);
+                    if (lane == 0) bulk_wait_read<0>();   // the store that last read the slab is done with it
                     tmem_ld_wait();
-                    // through a staging slab (32 rows x 64 bytes, 64-byte swizzle): the rows of a full slab leave with one
-                    // asynchronous tile store, a ragged slab (last tile of a request or mini-batch) with guarded stores
-                    unsigned char *sb = stg + slab * 2048;
-                    if (lane == 0) bulk_wait_read<C::kSlabs - 1>();   // the store that last read this slab is done with it
                     __syncwarp();
                     auto emit = [&](const uint32_t (&r)[16], int row_h) {
 #pragma unroll
@@ -312,47 +295,41 @@ __global__ void __launch_bounds__(LayerCfg<MODE>::kThreads, 1) k_layer_tc(const 
                         fence_proxy_async();
                         __syncwarp();
                         if (lane == 0) {
-                            tma_store_2d(&tmapOut, smem_u32(sb), n0 + c0, (int)(t.pos0 + wrow0));
+                            tma_store_2d(&tmapOut, smem_u32(sb), n0 + col_lo + c0, (int)(t.pos0 + wrow0));
                             bulk_commit();
                         }
-                    } else {
+                    } else {   // ragged last tile of a request or mini-batch: guarded stores
                         __syncwarp();
 #pragma unroll
                         for (int j = 0; j < 4; ++j) {
                             const int rr = 8 * j + (lane >> 2), q = lane & 3;
                             const uint4 v = *reinterpret_cast<const uint4 *>(sb + rr * 64 + ((q ^ ((rr >> 1) & 3)) << 4));
                             if (wrow0 + rr < t.cnt)
-                                *reinterpret_cast<uint4 *>(p.out + (size_t)(t.pos0 + wrow0 + rr) * p.out_stride + n0 + c0 + q * 8) = v;
+                                *reinterpret_cast<uint4 *>(p.out + (size_t)(t.pos0 + wrow0 + rr) * p.out_stride + n0 + col_lo + c0 + q * 8) = v;
                         }
                         __syncwarp();
                     }
-                    slab = (slab + 1u) % (uint32_t)C::kSlabs;
                 }
             } else if (got && t.cnt > 0 && p.epi == EPI_DOT) {
-                // Last hidden layer: ReLU(x + b) . w_out per row, in the same 16x256b shape (eight bias and eight output
-                // weights per thread and 32 columns).  A thread sums its column pairs for its four rows; the four
-                // threads of a row are joined by shuffles at the end, and the row's own thread takes the result.
-                const int l4 = lane & 3;
-                uint64_t acc[4] = {0ull, 0ull, 0ull, 0ull};   // rows r8, r8 + 8, r8 + 16, r8 + 24 (r8 = lane / 4), two columns each
-                for (int c0 = 0; c0 < p.n_cols; c0 += 32) {
+                // Last hidden layer: ReLU(x + b) . w_out per row over this warp's columns, in the same shape; the four threads
+                // of a row are joined by shuffles, the two halves of the columns through shared memory.
+                uint64_t acc[4] = {0ull, 0ull, 0ull, 0ull};   // rows r8 + 8 i, two columns each
+                for (int c0 = 0; c0 < hc; c0 += 32) {
                     uint32_t ra[16], rb[16];
                     tmem_ld16x256(taddr + (uint32_t)c0, ra);
                     tmem_ld16x256(taddr + (16u << 16) + (uint32_t)c0, rb);
-                    // the last width may end in the middle of these 32 columns (a multiple of 16): the rest is skipped
-                    const int n_j = (p.n_cols - c0) >> 3;
                     uint64_t bias2[4], w2[4];
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
-                        const int col = c0 + 8 * (j < n_j ? j : 0) + 2 * l4;
-                        bias2[j] = *reinterpret_cast<const uint64_t *>(bs + col);
-                        w2[j] = *reinterpret_cast<const uint64_t *>(ws + col);
+                        const int col = col_lo + c0 + 8 * j + 2 * l4;
+                        bias2[j] = *reinterpret_cast<const uint64_t *>(bias_s + col);
+                        w2[j] = *reinterpret_cast<const uint64_t *>(wout_s + col);
                     }
                     tmem_ld_wait();
 #pragma unroll
                     for (int j = 0; j < 4; ++j)
 #pragma unroll
                         for (int q = 0; q < 2; ++q) {
-                            if (j >= n_j) continue;   // columns no product wrote
                             float x0, x1, y0, y1;
                             unpack_f32x2(add_f32x2(pack_f32x2(__uint_as_float(ra[4 * j + 2 * q]), __uint_as_float(ra[4 * j + 2 * q + 1])), bias2[j]), x0, x1);
                             unpack_f32x2(add_f32x2(pack_f32x2(__uint_as_float(rb[4 * j + 2 * q]), __uint_as_float(rb[4 * j + 2 * q + 1])), bias2[j]), y0, y1);
@@ -371,273 +348,233 @@ __global__ void __launch_bounds__(LayerCfg<MODE>::kThreads, 1) k_layer_tc(const 
                     v = __shfl_sync(0xffffffffu, v, 4 * (lane & 7));
                     if ((lane >> 3) == i) dot = v;
                 }
-            } else if (got && t.cnt > 0) {
-                for (int c0 = 0; c0 < p.n_cols; c0 += 32) {
+                if (half == 1) dot_s[row] = dot;
+            } else if (got && t.cnt > 0) {   // EPI_SIGN
+                for (int c0 = 0; c0 < hc && n0 + col_lo + c0 < p.n_out; c0 += 32) {
                     uint32_t r[32];
                     tmem_ld32(taddr + (uint32_t)c0, r);
                     tmem_ld_wait();
-                    if (p.epi == EPI_SIGN) {
-                        // eq. 5: one bit per output, set where the projection is positive; eight bits per byte, first bit
-                        // most significant
-                        uint32_t word = 0u;
+                    // eq. 5: one bit per output, set where the projection is positive; eight bits per byte, first bit most
+                    // significant
+                    uint32_t word = 0u;
 #pragma unroll
-                        for (int i = 0; i < 32; ++i)
-                            word |= (__uint_as_float(r[i]) > 0.f ? 1u : 0u) << (8 * (i >> 3) + 7 - (i & 7));
-                        if (valid) *reinterpret_cast<uint32_t *>(p.sig_out + (size_t)(t.pos0 + row) * (p.out_stride >> 3) + ((n0 + c0) >> 3)) = word;
-                    }
+                    for (int i = 0; i < 32; ++i) word |= (__uint_as_float(r[i]) > 0.f ? 1u : 0u) << (8 * (i >> 3) + 7 - (i & 7));
+                    if (valid) *reinterpret_cast<uint32_t *>(p.sig_out + (size_t)(t.pos0 + row) * (p.out_stride >> 3) + ((n0 + col_lo + c0) >> 3)) = word;
                 }
             }
             tc_fence_before();
             __syncwarp();
-            if (got && lane == 0) mbar_arrive(smem_u32(acc_empty + buf));
-            if (p.epi == EPI_DOT && valid) {
-                float logit = dot + p.b_out[0];
+            if (got && lane == 0) mbar_arrive_cluster(empty_addr[buf]);
+            const bool out = named_bar_or(1, 256, !got);   // also orders dot_s
+            if (p.epi == EPI_DOT && half == 0 && valid) {
+                float logit = dot + dot_s[row] + p.b_out[0];
                 if (p.emit_sigmoid) logit = 1.0f / (1.0f + expf(-logit));
-                const int id = p.sl.ids[t.pos0 + row];
-                // no number for an id outside the table, nor for a tile whose inputs never arrived (here or in an
-                // earlier kernel of the call: the status word says so)
-                if (id < 0 || (int64_t)id >= p.M || !got || poisoned) logit = __int_as_float(0x7fc00000);
+                // no number for an id outside the table, nor for a tile whose inputs never arrived (here or in an earlier
+                // kernel of the call: the status word says so)
+                if (id < 0 || (int64_t)id >= p.M || out || poisoned) logit = __int_as_float(0x7fc00000);
                 p.sl.logits[p.sl.out_index ? (int64_t)p.sl.out_index[t.pos0 + row] : t.pos0 + row] = logit;
             }
-            if (named_bar_or(1 + a, 128, !got)) break;
+            if (out) break;
         }
         if (lane == 0) bulk_wait<0>();   // all tile stores of this warp have reached global memory
     } else if (warp == C::kMmaWarp) {
-        // ===================== MMA issuer =====================
-        if (lane == 0) {
-            const uint32_t idesc = umma_idesc_bf16(kTcTile, p.n_cols);
-            const int n_k = p.n_k;
-            // descriptors of stage 0 of each ring; stage s lies s stage sizes further (the address field counts 16 bytes)
-            const uint64_t bdesc0 = umma_desc_sw128(smem_u32(smB));
-            uint64_t adesc0[G];
-#pragma unroll
-            for (int g = 0; g < G; ++g) adesc0[g] = umma_desc_sw128(smem_u32(smA + g * kABytes));
-            int it = 0, sa = 0, sb = 0;
-            uint32_t pha = 0, phb = 0;
+        if (lane == 0 && rank == 0) {
+            // ===================== MMA issuer =====================
+            const uint32_t idesc = umma_idesc_bf16(2 * kTcTile, p.n_cols);
+            const uint64_t adesc0 = umma_desc_sw128(smem_u32(base)), bdesc0 = umma_desc_sw128(smem_u32(base + kABytes));
+            int it = 0, s = 0;
+            uint32_t ph = 0;
             bool ok = true;
-            for (int item = blockIdx.x; ok && item < n_items; item += gridDim.x, ++it) {
-                for (int kc = 0; kc < n_k; ++kc) {
-                    if (!mbar_wait(smem_u32(full_a + sa), pha, abort_flag) || !mbar_wait(smem_u32(full_b + sb), phb, abort_flag)) {
+            for (int item = item0; ok && item < n_items; item += item_step, ++it) {
+                const int buf = it & 1;
+                // the accumulator must have been drained by both CTAs' epilogues of its previous use
+                if (!mbar_wait(smem_u32(acc_empty + buf), (uint32_t)((it >> 1) & 1) ^ 1u, abort_flag)) break;
+                const uint32_t d_tmem = tmem_base + (uint32_t)(buf * 256);
+                for (int kc = 0; kc < p.n_k; ++kc) {
+                    if (!mbar_wait(smem_u32(full + s), ph, abort_flag)) {
                         ok = false;
                         break;
                     }
-                    // the A chunk was written by cp.async (generic proxy) and is read by the MMA (async proxy)
-                    fence_proxy_async();
+                    fence_proxy_async();   // gathered rows were written by cp.async (generic proxy)
                     tc_fence_after();
-                    const uint64_t aoff = (uint64_t)(uint32_t)(sa * (C::kAStage >> 4)), boff = (uint64_t)(uint32_t)(sb * (C::kBStage >> 4));
+                    const uint64_t off = (uint64_t)(uint32_t)(s * (C::kStage >> 4));
 #pragma unroll
-                    for (int a = 0; a < kAcc; ++a) {
-                        const int buf = kAcc == 1 ? (it & 1) : a;
-                        if (kc == 0) {   // the accumulator must have been drained by the epilogue of its previous use
-                            const uint32_t eph = (kAcc == 1 ? (uint32_t)((it >> 1) & 1) : (uint32_t)(it & 1)) ^ 1u;
-                            if (!mbar_wait(smem_u32(acc_empty + buf), eph, abort_flag)) {
-                                ok = false;
-                                break;
-                            }
-                            tc_fence_after();
-                        }
-                        const uint32_t d_tmem = tmem_base + (uint32_t)(buf * 256);
-                        const uint64_t adesc = adesc0[G == 2 ? a : 0] + aoff;
-                        const uint64_t bdesc = bdesc0 + boff + (uint64_t)(NB == 2 ? a * (kBBytes >> 4) : 0);
-                        // 4 x K=16 inside the 64-column chunk: +32 bytes (2 units) per step
-                        umma_bf16(d_tmem, adesc, bdesc, idesc, kc != 0 ? 1u : 0u);
-                        umma_bf16_acc(d_tmem, adesc + 2, bdesc + 2, idesc);
-                        umma_bf16_acc(d_tmem, adesc + 4, bdesc + 4, idesc);
-                        umma_bf16_acc(d_tmem, adesc + 6, bdesc + 6, idesc);
-                        if (kc == n_k - 1) umma_commit(smem_u32(acc_full + buf));
-                    }
-                    if (!ok) break;
-                    umma_commit(smem_u32(empty_a + sa));
-                    umma_commit(smem_u32(empty_b + sb));
-                    if (++sa == kSA) sa = 0, pha ^= 1u;
-                    if (++sb == kSB) sb = 0, phb ^= 1u;
+                    for (int kk = 0; kk < 4; ++kk)   // 4 x K=16 inside the 64-column chunk: +32 bytes (2 units) per step
+                        umma_bf16_pair(d_tmem, adesc0 + off + 2 * kk, bdesc0 + off + 2 * kk, idesc, (kc | kk) != 0 ? 1u : 0u);
+                    umma_commit_pair(smem_u32(empty + s));
+                    if (kc == p.n_k - 1) umma_commit_pair(smem_u32(acc_full + buf));
+                    if (++s == kS) s = 0, ph ^= 1u;
                 }
             }
         }
         __syncwarp();
     } else if (warp < C::kBWarp) {
-        // ===================== A producer (128 threads per tile of the group) =====================
-        const int pt = tid - C::kProdWarp0 * 32;
-        const int gt = pt >> 7, lp = pt & 127;   // tile of the group this thread serves; its index among that tile's threads
-        const int sub = lp & 7;                  // 16-byte slot inside the 128-byte row chunk
-        const int r0 = lp >> 3;                  // rows r0, r0+16, ...
-        const uint32_t a_off = (uint32_t)(gt * kABytes + r0 * 128) + (uint32_t)((sub ^ (r0 & 7)) << 4);
-        const bool deep = p.n_k >= 2;            // bucket look-ups run two chunks ahead (needs the next item at most)
-
-        // The tile of the current / next item: registers hold where it lies, shared memory its validated ids
-        // (ids_s[buffer][tile][row], -1 for rows beyond the tile and for ids outside the table).
-        struct Rows {
-            uint32_t rowmask;        // bit i: row r0 + 16 i lies inside the tile
-            uint32_t pos0;
-            const uint8_t *Tt;
-            const uint16_t *xb;      // bucket row of this thread's first row
+        // ===================== A producers: every warp fills the stage of its number, all 128 rows of a chunk =====================
+        // Lane l: 16-byte slot l % 8 of the 128-byte rows l / 8 + 4 i.  The sources of a chunk are one number per row, the item
+        // id or the bucket(s) of the chunk's field(s): lane l fetches those of rows l + 32 j with coalesced loads while the
+        // previous chunk of this warp is landing, the copying lanes get them by shuffle.  What the fetch itself needs, the
+        // tile's place, is requested one chunk earlier still: a fetch that had to wait for it took 1250 to 3000 of a chunk's
+        // 3300 cycles.  A warp waits for its own copies (five others have theirs in flight meanwhile) and tells the issuer
+        // with one arrival: an arrival per gathering thread (256 serial operations on the stage's barrier) cost more than the
+        // 512 cycles of products a chunk is.
+        const int sub = lane & 7, r0 = lane >> 3;
+        const uint32_t swz[2] = {(uint32_t)((sub ^ r0) << 4), (uint32_t)((sub ^ (r0 + 4)) << 4)};   // row & 7 alternates between r0 and r0 + 4
+        const int n_k = p.n_k;
+        const bool two = p.dc == 32;      // two fields per chunk; wider embeddings: one field spans one or more chunks
+        const bool narrow = p.dc < 32;    // four and more fields per chunk: the copying lanes look their buckets up themselves
+        const int s = warp - C::kProdWarp0;
+        const uint32_t dst0 = smem_u32(base + s * C::kStage) + (uint32_t)(r0 * 128);
+        struct Place {
+            int item, kc;
         };
-        const uint32_t xb_step = (uint32_t)(16 * p.F);   // elements between the bucket rows of rows r0 + 16 i and r0 + 16 (i + 1)
-        auto load_rows = [&](int item, Rows &R, int &pend) {
-            const TileInfo t = decode_tile(p, (item / n_ncg) * G + gt, n_tiles);
-            const int nrows = t.cnt > r0 ? (t.cnt - r0 + 15) >> 4 : 0;
-            R.rowmask = (1u << nrows) - 1u, R.pos0 = (uint32_t)t.pos0;
-            R.Tt = t.cnt > 0 ? reinterpret_cast<const uint8_t *>(p.sl.slots[t.rq.slot].T) : p.E;
-            R.xb = p.xb + (size_t)(t.pos0 + r0) * p.F;
-            int id = -1;
-            if (lp < t.cnt) {   // this thread fetches the id of row lp; the others read it from shared memory
-                id = p.sl.ids ? p.sl.ids[t.pos0 + lp] : 0;   // no id array: a launch over dense rows only
-                if (id < 0 || (int64_t)id >= p.M) {
-                    id = -1;
-                    if (p.check_ids) atomicOr(p.sl.status, AIF_STATUS_BAD_ID);
-                }
-            }
-            pend = id;
+        auto step = [&](Place &q, int by) {
+            q.kc += by;
+            while (q.kc >= n_k) q.kc -= n_k, q.item += item_step;
         };
-        // returns true if some producer thread's wait ran out: they all learn it here and leave together, so that none
-        // is left waiting at this barrier
-        auto publish = [&](int buf, int pend, bool failed) {
-            const bool any = named_bar_or(9, C::kProdThreads, failed);   // every producer thread is done reading what this buffer held
-            ids_s[(buf * G + gt) * 128 + lp] = pend;
-            named_bar_sync(9, C::kProdThreads);
-            return any;
+        auto tile_of = [&](const Place &q) { return decode_tile(p, q.item < n_items ? (q.item / p.n_nchunks) * 2 + rank : n_tiles, n_tiles); };
+        struct Chunk {
+            int kind;
+            int32_t v[4];           // per row lane + 32 j: id as read, or bucket (both fields' buckets); -1: zero row
+            const uint8_t *bp;      // this lane's 16 bytes of row 0 of the table the rows come from
+            const uint16_t *xb;     // narrow fields: this lane's field of the tile's first row of buckets
+            uint32_t row_bytes;     // of that table
+            int cnt;                // rows of the tile
+            int tma_x, tma_y;       // dense chunk; tma_x < 0: the tile does not exist
         };
-        // bucket of this thread's rows in the field its slot of chunk kc belongs to (cross chunks only); rows outside
-        // the tile read other candidates' entries or stale scratch, which rowmask discards
-        auto fetch = [&](int kc, const Rows &R, uint32_t (&raw)[8]) {
-            const ChunkSrc src = p.src[kc];
-            if (src.kind != SRC_CROSS) return;
-            const uint16_t *xb = R.xb + (src.off + sub * 8) / p.dc;
-#pragma unroll
-            for (int i = 0; i < 8; ++i) raw[i] = (uint32_t)__ldg(xb + i * xb_step);
-        };
-        // global sources of chunk kc: a base pointer and, per row, an offset in 16-byte units; rows whose bit in `mask`
-        // is clear are zero-filled
-        // (dense chunks: consecutive rows of X / the previous activations, fetched as one TMA tile by the tile's first
-        // producer thread; tma_x < 0 marks every other kind)
-        auto resolve = [&](int kc, const Rows &R, const int *ids, uint32_t (&raw)[8], bool have_raw, const uint8_t *&bp,
-                           uint32_t (&off)[8], uint32_t &mask, int &tma_x, int &tma_y) {
-            const ChunkSrc src = p.src[kc];
-            tma_x = -1;
+        auto fetch = [&](Chunk &c, const Place &q, const TileInfo &t) {
+            const ChunkSrc src = p.src[q.kc];
+            c.kind = src.kind, c.cnt = t.cnt;
             if (src.kind == SRC_DENSE) {
                 // rows beyond the tile bring other candidates' values along; their results are never stored
-                tma_x = R.rowmask != 0u || lp != 0 ? src.off >> 1 : -2;   // -2: the tile does not exist, nothing to fetch
-                tma_y = (int)R.pos0;
-                mask = 0;
+                c.tma_x = t.cnt > 0 ? src.off >> 1 : -1, c.tma_y = (int)t.pos0;
             } else if (src.kind == SRC_ITEM) {
-                const uint32_t row16 = (uint32_t)(p.e_row_bytes >> 4), c16 = (uint32_t)(src.off >> 4) + sub;
-                bp = p.E;
-                mask = 0;
+                c.bp = p.E + src.off + sub * 16, c.row_bytes = (uint32_t)p.e_row_bytes;
 #pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const int id = ids[r0 + 16 * i];
-                    off[i] = (uint32_t)(id >= 0 ? id : 0) * row16 + c16;
-                    if (id >= 0) mask |= 1u << i;
-                }
+                for (int j = 0; j < 4; ++j) c.v[j] = lane + 32 * j < t.cnt ? p.sl.ids[t.pos0 + lane + 32 * j] : -1;
+            } else if (narrow) {
+                const int col = src.off + sub * 8, f = col / p.dc;
+                c.row_bytes = (uint32_t)p.dc * 2;
+                c.bp = p.T0 + (size_t)t.rq.slot * p.slot_bytes + ((size_t)f * p.B * p.dc + (col - f * p.dc)) * 2;
+                c.xb = p.xb + (size_t)t.pos0 * p.F + f;
             } else {
-                const int col = src.off + sub * 8;
-                const int f = col / p.dc, kin = col - f * p.dc;
-                const uint32_t row16 = (uint32_t)(p.dc >> 3), base16 = (uint32_t)(f * p.B) * row16 + (uint32_t)(kin >> 3);
-                bp = R.Tt;
-                if (!have_raw) {
-                    const uint16_t *xb = R.xb + f;
+                const int f = src.off / p.dc, col = two ? (sub & 3) * 8 : src.off - f * p.dc + sub * 8;
+                c.row_bytes = (uint32_t)p.dc * 2;
+                c.bp = p.T0 + (size_t)t.rq.slot * p.slot_bytes + ((size_t)(f + (two ? sub >> 2 : 0)) * p.B * p.dc + col) * 2;
+                const uint16_t *xb = p.xb + (size_t)t.pos0 * p.F + f;
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) raw[i] = (uint32_t)__ldg(xb + i * xb_step);
+                for (int j = 0; j < 4; ++j) {
+                    c.v[j] = -1;
+                    if (lane + 32 * j < t.cnt) {
+                        const uint16_t *w = xb + (size_t)(lane + 32 * j) * p.F;
+                        // F is even where dc = 32; a bucket that does not exist is 0xFFFF, both of a pair at once
+                        c.v[j] = two ? __ldg(reinterpret_cast<const int32_t *>(w)) : (int32_t)((uint32_t)__ldg(w) | 0xFFFF0000u);
+                    }
                 }
-                mask = 0;
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    if (raw[i] != kNoBucket) mask |= 1u << i;
-                    off[i] = raw[i] * row16 + base16;
-                }
-                mask &= R.rowmask;
             }
         };
-
-        int s = 0, buf = 0;
         uint32_t ph = 0;
-        bool ok = true;
-        Rows cur, nxt;
-        int pend = -1;
-        const uint8_t *bp = p.E;
-        uint32_t off[8], raw[8], mask = 0;
-        int tma_x = -1, tma_y = 0;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) off[i] = 0, raw[i] = 0;
-        if ((int)blockIdx.x < n_items) {
-            load_rows(blockIdx.x, cur, pend);
-            publish(0, pend, false);
-            resolve(0, cur, ids_s + gt * 128, raw, false, bp, off, mask, tma_x, tma_y);
-            if (deep) fetch(1, cur, raw);
-        }
-        nxt = cur;
-        for (int item = blockIdx.x; item < n_items; item += gridDim.x, buf ^= 1) {
-            const int next_item = item + gridDim.x;
-            const bool has_next = next_item < n_items;
-            const int *ids_cur = ids_s + (buf * G + gt) * 128, *ids_nxt = ids_s + ((buf ^ 1) * G + gt) * 128;
-            if (has_next) load_rows(next_item, nxt, pend);   // the id load lands while chunk 0 is copied
-            bool all_out = false;
-            for (int kc = 0; kc < p.n_k; ++kc) {
-                // a thread whose wait ran out keeps walking (no copies, no arrivals) until the next publish barrier
-                if (ok && !mbar_wait(smem_u32(empty_a + s), ph ^ 1u, abort_flag)) ok = false;
-                if (!ok) {
-                    if (kc == 0 && has_next) all_out = publish(buf ^ 1, pend, true);
-                    if (all_out) break;
-                    continue;
+        Place cur{item0, 0}, nxt;
+        step(cur, s);
+        nxt = cur, step(nxt, C::kProdWarps);
+        Chunk c;
+        if (cur.item < n_items) fetch(c, cur, tile_of(cur));
+        TileInfo tn = tile_of(nxt);
+        while (cur.item < n_items) {
+            if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(empty + s), ph ^ 1u, abort_flag))) break;
+            const bool gathered = c.kind != SRC_DENSE;
+            if (!gathered) {
+                if (lane == 0) {
+                    if (c.tma_x >= 0) {
+                        mbar_expect_tx(smem_u32(landed + s), (uint32_t)kABytes);
+                        tma_load_2d(smem_u32(base + s * C::kStage), &tmapA, smem_u32(landed + s), c.tma_x, c.tma_y);
+                    } else
+                        mbar_arrive(smem_u32(landed + s));
                 }
-                if (tma_x == -1) {
-                    const uint32_t dst0 = smem_u32(smA + s * C::kAStage) + a_off;
+            } else {
+                if (lane == 0) mbar_arrive(smem_u32(landed + s));
+                // row r0 + 4 i: register i / 8 of lane r0 + 4 (i % 8)
+                if (c.kind == SRC_ITEM) {
+                    bool bad = false;
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        const bool on = (mask >> i) & 1u;
-                        cp_async16(dst0 + (uint32_t)(i * 16 * 128), on ? bp + ((size_t)off[i] << 4) : p.E, on ? 16u : 0u);
+                    for (int j = 0; j < 4; ++j)
+                        if (c.v[j] < 0 || (int64_t)c.v[j] >= p.M) {
+                            bad |= lane + 32 * j < c.cnt;
+                            c.v[j] = -1;
+                        }
+                    if (bad && p.check_ids && cur.kc == 0) atomicOr(p.sl.status, AIF_STATUS_BAD_ID);
+#pragma unroll
+                    for (int i = 0; i < 32; ++i) {
+                        const int v = __shfl_sync(0xffffffffu, c.v[i >> 3], r0 + 4 * (i & 7));
+                        cp_async16(dst0 + (uint32_t)(i * 512) + swz[i & 1], c.bp + (size_t)(uint32_t)max(v, 0) * c.row_bytes, v >= 0 ? 16u : 0u);
                     }
-                } else if (lp == 0 && tma_x >= 0) {
-                    mbar_expect_tx_only(smem_u32(full_a + s), (uint32_t)kABytes);
-                    tma_load_2d(smem_u32(smA + s * C::kAStage + gt * kABytes), &tmapA, smem_u32(full_a + s), tma_x, tma_y);
+                } else if (narrow) {
+#pragma unroll 1
+                    for (int i0 = 0; i0 < 32; i0 += 8) {
+                        uint32_t v[8];
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) {
+                            const int row = r0 + 4 * (i0 + i);
+                            v[i] = row < c.cnt ? (uint32_t)__ldg(c.xb + (size_t)row * p.F) : kNoBucket;
+                        }
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) {
+                            const bool on = v[i] != kNoBucket;
+                            cp_async16(dst0 + (uint32_t)((i0 + i) * 512) + swz[i & 1], c.bp + (size_t)(on ? v[i] : 0u) * c.row_bytes, on ? 16u : 0u);
+                        }
+                    }
+                } else {
+                    const uint32_t pick = two && sub >= 4 ? 0x4432u : 0x4410u;   // byte permute: the pair's upper or lower half
+#pragma unroll
+                    for (int i = 0; i < 32; ++i) {
+                        const uint32_t v = __byte_perm((uint32_t)__shfl_sync(0xffffffffu, c.v[i >> 3], r0 + 4 * (i & 7)), 0u, pick);
+                        const bool on = v != kNoBucket;
+                        cp_async16(dst0 + (uint32_t)(i * 512) + swz[i & 1], c.bp + (size_t)(on ? v : 0u) * c.row_bytes, on ? 16u : 0u);
+                    }
                 }
-                // the stage's barrier receives this thread's arrival when its copies have landed: no thread waits for them
-                cp_async_arrive_noinc(smem_u32(full_a + s));
-                if (++s == kSA) s = 0, ph ^= 1u;
-                if (kc == 0 && has_next && publish(buf ^ 1, pend, false)) {
-                    all_out = true;
-                    break;
-                }
-                // sources of the next chunk from the buckets fetched one iteration ago; then start the fetch for the
-                // chunk after it, so that its latency is covered by a whole iteration
-                if (kc + 1 < p.n_k) resolve(kc + 1, cur, ids_cur, raw, deep, bp, off, mask, tma_x, tma_y);
-                else if (has_next) resolve(0, nxt, ids_nxt, raw, deep, bp, off, mask, tma_x, tma_y);
-                if (deep) {
-                    if (kc + 2 < p.n_k) fetch(kc + 2, cur, raw);
-                    else if (has_next) fetch(kc + 2 - p.n_k, nxt, raw);
-                }
+                cp_async_commit();
             }
-            if (all_out) break;
             cur = nxt;
+            step(nxt, C::kProdWarps);
+            if (cur.item < n_items) fetch(c, cur, tn);   // these loads are in flight while the copies land
+            tn = tile_of(nxt);
+            if (gathered) {
+                cp_async_wait<0>();
+                fence_proxy_async();   // written by cp.async (generic proxy), read by the products through the async proxy
+            }
+            __syncwarp();
+            bool ok = true;
+            if (lane == 0) {
+                ok = mbar_wait(smem_u32(landed + s), ph, abort_flag);   // the stage's weights, and a dense chunk's rows
+                if (ok) mbar_arrive_cluster(cluster_addr(smem_u32(full + s), 0u));
+            }
+            if (!__all_sync(0xffffffffu, ok)) break;
+            ph ^= 1u;
         }
         cp_async_wait_all();
     } else {
-        // ===================== B producer (TMA) =====================
+        // ===================== B producer (TMA): this CTA's half of the slice's weight rows =====================
         if (lane == 0) {
             int s = 0;
             uint32_t ph = 0;
             bool ok = true;
-            const uint32_t bytes = (uint32_t)p.n_cols * 128u;
-            for (int item = blockIdx.x; ok && item < n_items; item += gridDim.x) {
-                const int grp = item / n_ncg, nc0 = (item - grp * n_ncg) * NB;
+            const int rows = p.n_cols >> 1;
+            for (int item = item0; ok && item < n_items; item += item_step) {
+                const int n0 = (item % p.n_nchunks) * p.n_cols + rank * rows;
                 for (int kc = 0; kc < p.n_k; ++kc) {
-                    if (!mbar_wait(smem_u32(empty_b + s), ph ^ 1u, abort_flag)) {
+                    if (!mbar_wait(smem_u32(empty + s), ph ^ 1u, abort_flag)) {
                         ok = false;
                         break;
                     }
-                    mbar_expect_tx(smem_u32(full_b + s), NB * bytes);
-#pragma unroll
-                    for (int nb = 0; nb < NB; ++nb)
-                        tma_load_2d(smem_u32(smB + s * C::kBStage + nb * kBBytes), &tmapB, smem_u32(full_b + s), kc * 64,
-                                    (nc0 + nb) * p.n_cols);
-                    if (++s == kSB) s = 0, ph ^= 1u;
+                    mbar_expect_tx(smem_u32(landed + s), (uint32_t)rows * 128u);
+                    tma_load_2d(smem_u32(base + s * C::kStage + kABytes), &tmapB, smem_u32(landed + s), kc * 64, n0);
+                    if (++s == kS) s = 0, ph ^= 1u;
                 }
             }
         }
         __syncwarp();
     }
 
-    // ---- teardown: everybody arrives here, also after an abort
+    // ---- teardown: everybody arrives here, also after an abort; neither CTA leaves while the other may still reach it
     if (*abort_flag) {
         if (tid == 0) atomicOr(p.sl.status, AIF_STATUS_TIMEOUT);
         // let copies and MMAs that are still in flight land before shared memory and TMEM go away
@@ -646,7 +583,8 @@ __global__ void __launch_bounds__(LayerCfg<MODE>::kThreads, 1) k_layer_tc(const 
     }
     tc_fence_before();
     __syncthreads();
-    if (warp == C::kMmaWarp) tmem_dealloc(tmem_base, 512);
+    cluster_sync();
+    if (warp == C::kMmaWarp) tmem_dealloc_pair(tmem_base, 512);
 }
 
 // The tile of a block in the kernels below: from the launch's tile table when it was formed on the device, else from the
@@ -818,6 +756,7 @@ struct TcPlan {
     int n_k[kMaxHidden] = {}, n_cols[kMaxHidden] = {}, n_nchunks[kMaxHidden] = {};
     ChunkSrc src0[kMaxChunks] = {};
     CUtensorMap tmap[kMaxHidden];
+    CUtensorMap tmap_half[kMaxHidden];   // the same weights, boxes of half a slice's rows (layer kernel)
     size_t cap_rows = 0;                 // rows of the context's own scratch arrays
     __nv_bfloat16 *W[kMaxHidden] = {};
     __nv_bfloat16 *H[kMaxHidden] = {};   // activations after layer k (k < last)
@@ -827,6 +766,18 @@ struct TcPlan {
     size_t tiles_cap = 0;                // its entries
     bool maps_ready = false;
 };
+
+// Slices of a layer's outputs: 256 wide, a narrower layer rounded up to a multiple of 64.
+int slice_cols(int H) { return H <= 256 ? (H + 63) / 64 * 64 : 256; }
+
+// Launches the layer kernel over a launch's tiles: persistent, one pair of CTAs per two SMs.
+cudaError_t launch_layer(const LayerParams &p, int n_tiles, const CUtensorMap &tb, const CUtensorMap &to, const CUtensorMap &ta, cudaStream_t st)
+{
+    const int items = (n_tiles + 1) / 2 * p.n_nchunks;
+    const cudaError_t e = launch_pdl_pair(k_layer_pair, dim3(2 * (items < 74 ? items : 74)), dim3(PairCfg::kThreads), PairCfg::kSmem, st, tb, to, ta, p);
+    count_launch();
+    return e;
+}
 
 int dense_cols(const aif_config &c)
 {
@@ -911,8 +862,8 @@ cudaError_t tc_prepare_context(aif_ctx *ctx)
     for (int k = 0; k < c.n_hidden; ++k) {
         const int H = c.hidden[k];
         pl->n_k[k] = in_w / 64;
-        pl->n_cols[k] = H <= 256 ? H : 256;
-        pl->n_nchunks[k] = H / pl->n_cols[k];
+        pl->n_cols[k] = slice_cols(H);
+        pl->n_nchunks[k] = (H + pl->n_cols[k] - 1) / pl->n_cols[k];
         if ((e = alloc((void **)&pl->W[k], (size_t)H * in_w * 2)) != cudaSuccess) return e;
         if (k + 1 < c.n_hidden && (e = alloc((void **)&pl->H[k], cap * H * 2)) != cudaSuccess) return e;
         in_w = H;
@@ -928,13 +879,7 @@ cudaError_t tc_prepare_context(aif_ctx *ctx)
         pl->tiles_cap = body + (size_t)c.max_user_states * (mb ? tpm : 1) + 64;
         if ((e = alloc((void **)&pl->tiles, pl->tiles_cap * sizeof(TileDev))) != cudaSuccess) return e;
     }
-    e = cudaFuncSetAttribute(k_layer_tc<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LayerCfg<0>::kSmem);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_layer_tc<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LayerCfg<1>::kSmem);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_layer_tc<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LayerCfg<2>::kSmem);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_layer_tc<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LayerCfg<3>::kSmem);
+    e = cudaFuncSetAttribute(k_layer_pair, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PairCfg::kSmem);
     if (e != cudaSuccess) return e;
     // tensor maps over the packed weights: [H x in_w] bf16, box = 64 columns x n_cols rows, 128-byte swizzle
     EncodeFn enc = encode_fn();
@@ -943,12 +888,14 @@ cudaError_t tc_prepare_context(aif_ctx *ctx)
     for (int k = 0; k < c.n_hidden; ++k) {
         const cuuint64_t dims[2] = {(cuuint64_t)in_w, (cuuint64_t)c.hidden[k]};
         const cuuint64_t strides[1] = {(cuuint64_t)in_w * 2};
-        const cuuint32_t box[2] = {64, (cuuint32_t)pl->n_cols[k]};
         const cuuint32_t estr[2] = {1, 1};
-        CUresult r = enc(&pl->tmap[k], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, pl->W[k], dims, strides, box, estr,
-                         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-        if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
+        for (int half = 0; half < 2; ++half) {   // whole slices (single-launch kernel) and halves (layer kernel)
+            const cuuint32_t box[2] = {64, (cuuint32_t)pl->n_cols[k] >> half};
+            CUresult r = enc(half ? &pl->tmap_half[k] : &pl->tmap[k], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, pl->W[k], dims, strides, box, estr,
+                             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+            if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
+        }
         in_w = c.hidden[k];
     }
     pl->maps_ready = true;
@@ -1031,7 +978,7 @@ cudaError_t tc_dense_layer(const aif_ctx *ctx, const DenseLayer &L, int64_t rows
     p.sl.single = ReqDev{0, (int32_t)rows, 0, 0, 0};
     p.sl.n_tiles = (int32_t)((rows + kTcTile - 1) / kTcTile), p.sl.total = rows, p.sl.max_L = 0;
     p.sl.ids = nullptr, p.sl.logits = nullptr, p.sl.status = ctx->status;
-    p.n_cols = L.H <= 256 ? L.H : 256, p.n_nchunks = L.H / p.n_cols, p.n_k = L.in_w / 64, p.mini_batch = 0;
+    p.n_cols = slice_cols(L.H), p.n_nchunks = (L.H + p.n_cols - 1) / p.n_cols, p.n_out = L.H, p.n_k = L.in_w / 64, p.mini_batch = 0;
     p.E = (const uint8_t *)ctx->E, p.M = ctx->cfg.M, p.e_row_bytes = ctx->cfg.d * 2;
     p.X = (const uint8_t *)L.A, p.x_row_bytes = L.in_w * 2;
     p.B = 1, p.dc = 8, p.F = 0, p.xb = nullptr, p.check_ids = 0;
@@ -1045,7 +992,7 @@ cudaError_t tc_dense_layer(const aif_ctx *ctx, const DenseLayer &L, int64_t rows
     {
         const cuuint64_t dims[2] = {(cuuint64_t)L.in_w, (cuuint64_t)L.H};
         const cuuint64_t strides[1] = {(cuuint64_t)L.in_w * 2};
-        const cuuint32_t box[2] = {64, (cuuint32_t)p.n_cols};
+        const cuuint32_t box[2] = {64, (cuuint32_t)p.n_cols / 2};
         if (enc(&tmap_b, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(L.W), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                 CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return cudaErrorInvalidValue;
@@ -1067,17 +1014,7 @@ cudaError_t tc_dense_layer(const aif_ctx *ctx, const DenseLayer &L, int64_t rows
                 CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return cudaErrorInvalidValue;
     }
-    const int single = p.sl.n_tiles * p.n_nchunks;
-    const bool pair = ((p.sl.n_tiles + 1) / 2) * p.n_nchunks >= 2 * 148;
-    const bool wide = !pair && p.n_nchunks % 2 == 0 && single > 148;
-    const int items = pair ? ((p.sl.n_tiles + 1) / 2) * p.n_nchunks : wide ? single / 2 : single;
-    const int grid = items < 148 ? items : 148;
-    cudaError_t e;
-    if (pair) e = launch_pdl(k_layer_tc<1>, dim3(grid), dim3(LayerCfg<1>::kThreads), LayerCfg<1>::kSmem, st, tmap_b, tmap_out, tmap_a, p);
-    else if (wide) e = launch_pdl(k_layer_tc<2>, dim3(grid), dim3(LayerCfg<2>::kThreads), LayerCfg<2>::kSmem, st, tmap_b, tmap_out, tmap_a, p);
-    else e = launch_pdl(k_layer_tc<0>, dim3(grid), dim3(LayerCfg<0>::kThreads), LayerCfg<0>::kSmem, st, tmap_b, tmap_out, tmap_a, p);
-    count_launch();
-    return e;
+    return launch_layer(p, p.sl.n_tiles, tmap_b, tmap_out, tmap_a, st);
 }
 
 cudaError_t launch_score_tc(const aif_ctx *ctx, const ScoreLaunch &sl, int64_t, cudaStream_t st)
@@ -1189,9 +1126,10 @@ cudaError_t launch_score_tc_scratch(const aif_ctx *ctx, const ScoreLaunch &sl_in
         StageRange range(range_names[k]);
         LayerParams p{};
         p.sl = sl;
-        p.n_nchunks = pl->n_nchunks[k], p.n_cols = pl->n_cols[k], p.n_k = pl->n_k[k], p.mini_batch = c.mini_batch;
+        p.n_nchunks = pl->n_nchunks[k], p.n_cols = pl->n_cols[k], p.n_out = c.hidden[k], p.n_k = pl->n_k[k], p.mini_batch = c.mini_batch;
         p.E = (const uint8_t *)ctx->E, p.M = c.M, p.e_row_bytes = c.d * 2;
         p.B = c.B > 0 ? c.B : 1, p.dc = c.dc > 0 ? c.dc : 8, p.F = c.F, p.xb = (const uint16_t *)sc.xb;
+        p.T0 = (const uint8_t *)ctx->slots[0].dev.T, p.slot_bytes = (int64_t)ctx->slot_bytes;
         p.check_ids = k == 0;
         if (k == 0) {
             p.X = (const uint8_t *)sc.X, p.x_row_bytes = pl->x_cols * 2;
@@ -1217,13 +1155,6 @@ cudaError_t launch_score_tc_scratch(const aif_ctx *ctx, const ScoreLaunch &sl_in
         p.bias_from_slot = k == 0, p.bias = ctx->b[k], p.emit_sigmoid = c.emit_sigmoid;
         p.out = (__nv_bfloat16 *)sc.H[k], p.out_stride = c.hidden[k];
         p.w_out = (const __nv_bfloat16 *)ctx->w_out, p.b_out = ctx->b_out;
-        // two tiles per item once that still leaves every SM at least two items; else, if single items would need a
-        // second round on some SMs, one tile with two output slices per item
-        const int single = sl.n_tiles * p.n_nchunks;
-        const bool pair = ((sl.n_tiles + 1) / 2) * p.n_nchunks >= 2 * 148;
-        const bool wide = !pair && p.n_nchunks % 2 == 0 && single > 148;
-        const int items = pair ? ((sl.n_tiles + 1) / 2) * p.n_nchunks : wide ? single / 2 : single;
-        const int grid = items < 148 ? items : 148;
         // load source of the dense chunks: X (layer 1) or the previous activations, 64-column x 128-row tiles
         CUtensorMap tmap_a = pl->tmap[k];
         const int dense_w = k == 0 ? pl->x_cols : c.hidden[k - 1];
@@ -1237,13 +1168,7 @@ cudaError_t launch_score_tc_scratch(const aif_ctx *ctx, const ScoreLaunch &sl_in
                                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
             if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
         }
-        cudaError_t e;
-        if (pair && k == 0 && (c.blocks & AIF_BLK_CROSS))
-            e = launch_pdl(k_layer_tc<3>, dim3(grid), dim3(LayerCfg<3>::kThreads), LayerCfg<3>::kSmem, st, pl->tmap[k], tmap_out, tmap_a, p);
-        else if (pair) e = launch_pdl(k_layer_tc<1>, dim3(grid), dim3(LayerCfg<1>::kThreads), LayerCfg<1>::kSmem, st, pl->tmap[k], tmap_out, tmap_a, p);
-        else if (wide) e = launch_pdl(k_layer_tc<2>, dim3(grid), dim3(LayerCfg<2>::kThreads), LayerCfg<2>::kSmem, st, pl->tmap[k], tmap_out, tmap_a, p);
-        else e = launch_pdl(k_layer_tc<0>, dim3(grid), dim3(LayerCfg<0>::kThreads), LayerCfg<0>::kSmem, st, pl->tmap[k], tmap_out, tmap_a, p);
-        count_launch();
+        const cudaError_t e = launch_layer(p, sl.n_tiles, pl->tmap_half[k], tmap_out, tmap_a, st);
         timing_mark(ctx, names[k], st);
         if (e != cudaSuccess) return e;
     }

@@ -139,3 +139,47 @@ def test_bridge_embedding_columns_around_half_a_tile(base, n_bridge):
         _check(srv.score_ids(states[2], lists[2]), want[2])
     assert srv.ctx.poll_status() == B.STATUS_BAD_ID
     srv.close()
+
+
+@pytest.mark.parametrize("F,dc,hidden", [(16, 8, (256, 128)), (8, 16, (512, 80)), (2, 32, (64,)), (3, 64, (1024, 64, 16)), (1, 128, (256, 192)),
+                                         (4, 32, (768, 256, 48))])
+def test_layer_kernel_over_the_field_widths_and_slices_it_accepts(F, dc, hidden):
+    """The layer kernel on CTA pairs: one, two, four and eight fields per 64-column chunk and fields over several chunks; one to
+    four output slices, slices rounded up to 64 columns; one tile alone, an odd number of tiles, ragged tiles; ids outside the
+    table."""
+    wl = helpers.MINI["c3"].with_(name=f"layers_{F}_{dc}_{len(hidden)}", R=3, N=400, M=3000, L=260, F=F, dc=dc, B=300, hidden=hidden,
+                                  bucket_mode=synth.BUCKET_HASH)
+    weights, table = synth.make_weights(wl, zero_bias=False), synth.make_item_table(wl)
+    srv, oracle = serving.Server(wl, weights, table), helpers.make_oracle(wl, weights, M=wl.M)
+    rqs = [synth.make_request(wl, r) for r in range(3)]
+    states = [srv.precompute(r, srv.upload_request(rq, B.USER_PROJECTED)) for r, rq in enumerate(rqs)]
+    g = np.random.default_rng(4)
+    for sizes in ((1, 128, 129), (256, 31, 400)):
+        lists = [g.choice(wl.M, n, replace=False).astype(np.int32) for n in sizes]
+        lists[2][7] = -3
+        want = [oracle.score(table, helpers.projected_request(wl, rq), ids) for rq, ids in zip(rqs, lists)]
+        for got, w in zip(srv.score_many(states, lists), want):
+            _check(got, w)
+        for st, ids, w in zip(states, lists, want):
+            _check(srv.score_ids(st, ids), w)
+    assert srv.ctx.poll_status() == B.STATUS_BAD_ID
+    srv.close()
+
+
+def test_layer_kernel_with_several_items_per_pair():
+    """More pairs of tiles than the GPU has pairs of SMs, four slices each: accumulators and ring stages in every phase, checked
+    on the candidates around the tile edges of a few requests."""
+    wl = helpers.MINI["c5"].with_(name="layers_many", R=12, N=1700, M=4000, L=20, F=4, B=64)
+    weights, table = synth.make_weights(wl, zero_bias=False), synth.make_item_table(wl)
+    srv, oracle = serving.Server(wl, weights, table), helpers.make_oracle(wl, weights, M=wl.M)
+    rqs = [synth.make_request(wl, r) for r in range(wl.R)]
+    states = [srv.precompute(r, srv.upload_request(rq, B.USER_PROJECTED)) for r, rq in enumerate(rqs)]
+    g = np.random.default_rng(6)
+    lists = [g.choice(wl.M, 1700 - 13 * r, replace=False).astype(np.int32) for r in range(wl.R)]
+    got = srv.score_many(states, lists)
+    for r in (0, 5, 11):
+        n = len(lists[r])
+        at = np.unique(np.clip(np.concatenate([np.arange(0, n, 128), np.arange(127, n, 128), [n - 1], g.integers(0, n, 40)]), 0, n - 1))
+        _check(got[r][at], oracle.score(table, helpers.projected_request(wl, rqs[r]), lists[r][at]))
+    assert srv.ctx.poll_status() == 0
+    srv.close()
