@@ -196,5 +196,62 @@ __device__ inline ReqDev find_request(const ScoreLaunch &sl, int t)
     return sl.reqs[lo];
 }
 
+// One tile, or (SPLIT) one piece of a tile's keys, as every role of the attention and LSH kernels needs it.
+struct KeyTile {
+    int slot, cnt, nb, L;      // nb: key blocks to walk, at least one (an empty one is masked: the roles' hand-overs stay the same)
+    int key0;                  // first key row: 0, or where the tile's category's sub-sequence begins, plus the piece's offset
+    int part, n_parts, pslot;  // n_parts = 0: a piece of a tile that has fewer key blocks than pieces, nothing to deliver
+    int L_tile;
+    int64_t pos0;
+};
+
+template <bool SPLIT>
+__device__ __forceinline__ int key_jobs(const ScoreLaunch &sl)
+{
+    if (!SPLIT) return sl.n_tiles_dev ? *sl.n_tiles_dev : sl.n_tiles;
+    return sl.jobs ? *sl.n_jobs_dev : sl.n_tiles * sl.parts;
+}
+
+template <int BN, bool SPLIT>
+__device__ __forceinline__ KeyTile key_tile(const ScoreLaunch &sl, int job, int mini_batch)
+{
+    KeyTile t;
+    t.part = 0, t.n_parts = 1, t.pslot = 0;
+    if (SPLIT && sl.jobs) {
+        const JobDev j = sl.jobs[job];
+        t.slot = j.slot, t.cnt = j.cnt, t.pos0 = j.pos0, t.L = j.L, t.key0 = j.key0;
+        t.part = j.part, t.n_parts = j.n_parts, t.pslot = j.pslot, t.L_tile = j.L_tile;
+        t.nb = t.L > 0 ? (t.L + BN - 1) / BN : 1;
+        return t;
+    }
+    const int tile = SPLIT ? job / sl.parts : job;
+    if (sl.tiles) {   // looked up once per launch (k_tile_table)
+        const int4 v = *reinterpret_cast<const int4 *>(sl.tiles + tile);   // slot, cnt, pos0
+        t.slot = v.x, t.cnt = v.y;
+        t.pos0 = ((int64_t)(uint32_t)v.w << 32) | (int64_t)(uint32_t)v.z;
+        t.L = sl.tiles[tile].L, t.key0 = sl.tiles[tile].key0;
+        t.nb = t.L > 0 ? (t.L + BN - 1) / BN : 1;
+    } else {
+        const ReqDev rq = find_request(sl, tile);
+        int start, cnt;
+        tile_range(tile - rq.tile_begin, rq.n, kTcTile, mini_batch, start, cnt);
+        t.slot = rq.slot, t.cnt = cnt, t.pos0 = rq.off + start;
+        t.L = sl.slots[rq.slot].L, t.key0 = 0;
+        t.nb = (t.L + BN - 1) / BN;
+    }
+    t.L_tile = t.L;
+    if (SPLIT) {   // whole key blocks, as evenly as they go
+        const int nb = t.nb;
+        t.part = job - tile * sl.parts, t.n_parts = min(sl.parts, nb), t.pslot = tile * sl.parts;
+        if (t.part >= t.n_parts) t.L = 0, t.n_parts = 0;
+        else if (t.n_parts > 1) {
+            const int b0 = nb * t.part / t.n_parts, b1 = nb * (t.part + 1) / t.n_parts;
+            t.key0 += b0 * BN;
+            t.L = min(t.L - b0 * BN, (b1 - b0) * BN);
+        }
+        t.nb = t.L > 0 ? (t.L + BN - 1) / BN : 1;
+    }
+    return t;
+}
 
 }  // namespace aif

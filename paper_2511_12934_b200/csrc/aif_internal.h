@@ -74,6 +74,26 @@ struct TileDev {
     int32_t pad_[2];
 };
 
+// A piece of a tile's keys, the unit of the attention and LSH kernels where tiles with many keys are split over several CTAs.
+struct JobDev {
+    int32_t slot, cnt;
+    int64_t pos0;
+    int32_t L, key0;         // keys of this piece, first key row
+    int32_t part, n_parts;   // piece `part` of the tile's n_parts
+    int32_t pslot;           // the tile's first record of partial results (n_parts of them, in the order of the pieces)
+    int32_t L_tile;          // keys of the whole tile
+};
+
+// Results of the pieces of a tile, for k_join_pieces to put together.
+struct SplitScratch {
+    float *rows;        // [slots][d / 4][128] float4: unnormalised rows of a piece, column groups of four, row by row
+    float *stats;       // [slots][2][128]: row sum and exponent offset (attention)
+    int32_t *tiers;     // [slots][16][128] tier counts, or nullptr (no SimTier)
+    int32_t slots;      // records there is room for (0: no splitting)
+};
+constexpr int kSplitSlots = 4 * 148;       // of a scoring launch: at most two pieces per SM and launch, twice that after rounding up
+constexpr int kSplitSlotsUser = 2 * 148;   // of the user side's self-attention
+
 struct ScoreLaunch {
     const SlotDev *slots;   // device array of all slots
     const ReqDev *reqs;     // device array [n_req], or nullptr: use `single`
@@ -93,6 +113,13 @@ struct ScoreLaunch {
     const int32_t *n_tiles_dev;
     const int32_t *out_index;
     int32_t grouped;        // 1: key blocks come from the grouped sequence
+    // pieces of tiles: a table formed on the device (categories on), or `parts` equal pieces of every tile
+    const JobDev *jobs;
+    const int32_t *n_jobs_dev;   // [2] jobs, split tiles
+    const int32_t *joins;        // jobs that are the first pieces of split tiles
+    int32_t n_jobs;              // upper bound of the number of jobs
+    int32_t parts;               // 0 or 1: tiles are not split
+    SplitScratch split;
 };
 
 struct HostSlot {
@@ -199,6 +226,7 @@ struct aif_ctx {
     aif_stats stats{};
     mutable aif::KernelTiming timing;
     std::vector<void *> allocations;
+    aif::SplitScratch split{}, split_user{};   // partial results of split tiles: scoring launches, user-side self-attention
 };
 
 namespace aif {
@@ -261,8 +289,29 @@ cudaError_t sim_prepare(aif_ctx *ctx);
 void sim_destroy(aif_ctx *ctx);
 size_t sim_tile_capacity(const aif_ctx *ctx);
 cudaError_t sim_group_sequence(const aif_ctx *ctx, HostSlot &hs, const int32_t *seq_cat, int L, cudaStream_t st);
-// fills sl (ids, tiles, n_tiles upper bound, n_tiles_dev, out_index) for a launch whose original ids are sl.ids
-cudaError_t sim_group_candidates(const aif_ctx *ctx, ScoreLaunch &sl, cudaStream_t st);
+// Where the candidates of a grouped launch go: candidate pos to grouped position grp_start[where[pos].x] + where[pos].y.
+struct SimPlace {
+    const int2 *where;       // nullptr: candidates stay where they are
+    const int32_t *grp_start;
+    int32_t *ids, *out_index;   // by grouped position: id, and the candidate's position in the caller's arrays
+};
+// fills sl (tiles, jobs, their numbers, out_index) for a launch whose original ids are sl.ids; the candidates themselves are
+// placed by the bucket kernel, after which the launch's ids are place.ids
+cudaError_t sim_group_candidates(const aif_ctx *ctx, ScoreLaunch &sl, SimPlace &place, cudaStream_t st);
+// pieces per tile that even a launch of n_tiles tiles of `blocks` key blocks out over the SMs (aif_tc.cu)
+int split_parts(int n_tiles, int blocks, int slots);
+// Puts the pieces of a launch's tiles together (after the attention or LSH kernel of a split launch): rows into columns
+// [col, col + d) of X (col < 0: none), tier counts into 64 columns from x_tier on (x_tier < 0: none).
+struct JoinParams {
+    ScoreLaunch sl;
+    __nv_bfloat16 *X;
+    int64_t M;
+    int32_t x_stride, col, x_tier, n_tiers, d, mini_batch;
+    int32_t attention;          // rows are divided by their sums; else multiplied by row_scale (and divided by the keys: row_mean)
+    float row_scale;
+    int32_t row_mean, tier_mean;
+};
+cudaError_t launch_join_pieces(const JoinParams &p, cudaStream_t st);
 // whole scoring pass of a tile in one CTA (aif_tc_fused.cu); the tensor maps it shares with the other kernels
 bool tc_fused_supported(const aif_config &cfg);
 cudaError_t tc_fused_prepare(aif_ctx *ctx);
@@ -278,6 +327,7 @@ struct TcScratch {
     void *H[kMaxHidden];   // activations after hidden layer k (k < last), [rows x hidden[k]] bf16
     void *xb;              // cross-feature buckets, [rows x F] uint16
     void *tiles;           // tile table, [rows / 128 + requests] TileDev, or nullptr
+    bool split;            // the context's records of partial results are this launch's to use
     size_t rows;           // rows every array has room for
 };
 size_t tc_scratch_row_bytes(const aif_ctx *ctx);

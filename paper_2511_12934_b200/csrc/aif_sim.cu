@@ -11,6 +11,7 @@
 // order through an index.
 #include "aif_device.cuh"
 #include "aif_internal.h"
+#include "aif_tc_ptx.cuh"
 
 namespace aif {
 namespace {
@@ -139,109 +140,181 @@ __device__ __forceinline__ int group_of(const ScoreLaunch &sl, int64_t pos, int6
     return r * n_cat + c;
 }
 
-__global__ void __launch_bounds__(256) k_sim_count(ScoreLaunch sl, int64_t M, int n_cat, int mode, int32_t *__restrict__ grp_cnt)
+// where[pos] = (group of candidate pos, its rank inside the group); the group counts.  The order inside a group is arbitrary.
+__global__ void __launch_bounds__(256) k_sim_count(ScoreLaunch sl, int64_t M, int n_cat, int mode, int32_t *__restrict__ grp_cnt, int2 *__restrict__ where)
 {
+    grid_dep_launch();
+    grid_dep_wait();
     for (int64_t pos = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; pos < sl.total; pos += (int64_t)gridDim.x * blockDim.x) {
         int id;
-        atomicAdd(&grp_cnt[group_of(sl, pos, M, n_cat, mode, id)], 1);
+        const int g = group_of(sl, pos, M, n_cat, mode, id);
+        where[pos] = make_int2(g, atomicAdd(&grp_cnt[g], 1));
     }
 }
 
 // One block over the groups: first grouped position of every group (exclusive scan of the counts), the tile records, the
-// number of tiles; the counts are turned into cursors (zero) for the placement.  Tiles are laid out by the size of their
-// sub-sequence, longest first (in classes of powers of two): a tile's cost is its number of key blocks, the kernels hand
-// tile t to CTA t mod grid, and a long tile that started late would be what everything else waits for.
+// number of tiles; the counts go back to zero for the next launch (the ranks place the candidates: k_cross_buckets).
+// Beside the tiles, the jobs of the attention and LSH kernels: a tile's cost there is its number of key blocks, from none to
+// hundreds (a user's favourite category holds a fifth of the sequence), so tiles are cut into pieces of about half of what an
+// SM gets on average; a tile left whole made the launch as long as the longest sub-sequence (150 key blocks of one tile against
+// 22 per SM on average).  Jobs are laid out by size, largest first (in classes of a quarter octave), and every second row of 148
+// runs backwards: job j goes to CTA j mod 148, so the CTA with the largest job of one row gets the smallest of the next (4 x 10^4
+// candidates over 100 categories of 10^5 items: at most 29 blocks per SM for 22 on average; 38 in plain order).
+struct SimGroup {
+    int32_t cnt, start, slot, len, key0, np, t0, j0, p0;
+};
+
 __global__ void __launch_bounds__(1024) k_sim_tiles(ScoreLaunch sl, int n_groups, int n_cat, int32_t *__restrict__ grp_cnt,
                                                     int32_t *__restrict__ grp_start, TileDev *__restrict__ tiles, int tile_cap,
-                                                    int32_t *__restrict__ n_tiles_out)
+                                                    JobDev *__restrict__ jobs, int job_cap, int32_t *__restrict__ joins,
+                                                    int32_t *__restrict__ n_out)
 {
-    constexpr int kClasses = 32;
-    __shared__ int32_t part_c[1024];
-    __shared__ int32_t carry_c;
-    __shared__ int32_t cls_tiles[kClasses], cls_base[kClasses];
-    if (threadIdx.x == 0) carry_c = 0;
-    if (threadIdx.x < kClasses) cls_tiles[threadIdx.x] = 0;
+    constexpr int kClasses = 128;
+    __shared__ SimGroup grp[1024];
+    __shared__ int32_t warp_sum_s[32];
+    __shared__ long long warp_blocks_s[32];
+    __shared__ int32_t carry_c, tile_cur, pslot_cur, join_cur;
+    __shared__ int32_t cls_jobs[kClasses], cls_base[kClasses];
+    __shared__ int32_t n_jobs_s;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    grid_dep_launch();
+    grid_dep_wait();
+    if (tid == 0) carry_c = 0, tile_cur = 0, pslot_cur = 0, join_cur = 0;
+    if (tid < kClasses) cls_jobs[tid] = 0;
     __syncthreads();
-    auto group_info = [&](int g, int &slot, int &len, int &key0) {
-        const int r = g / n_cat, c = g - r * n_cat;
-        slot = sl.reqs ? sl.reqs[r].slot : sl.single.slot;
-        const SlotDev *sd = sl.slots + slot;
-        len = sd->cat_len[c], key0 = sd->cat_off[c];
+    auto key_blocks = [](int len) { return len > 0 ? (len + 127) / 128 : 1; };
+    auto class_of = [](int blocks) {   // four classes per octave (below four blocks: one per octave)
+        const int k = 31 - __clz(blocks);
+        return k < 2 ? 4 * k : 4 * k + ((blocks >> (k - 2)) & 3);
     };
-    auto class_of = [](int len) { return len > 0 ? 32 - __clz(len) : 0; };   // 0: empty sub-sequence, else floor(log2) + 1
-    // pass 1: grouped positions (scan of the counts) and tiles per size class
+    // a thread per group and batch of 1024 groups; what it looked up stays with it where one batch is all there is
+    SimGroup me{};
+    auto look_up = [&](int g) {
+        me.cnt = g < n_groups ? grp_cnt[g] : 0;
+        if (me.cnt == 0) return;
+        const int r = g / n_cat, c = g - r * n_cat;
+        me.slot = sl.reqs ? sl.reqs[r].slot : sl.single.slot;
+        const SlotDev *sd = sl.slots + me.slot;
+        me.len = sd->cat_len[c], me.key0 = sd->cat_off[c];
+    };
+    // pass 1: grouped positions (exclusive scan of the counts) and the launch's key blocks
+    long long blocks = 0;
     for (int g0 = 0; g0 < n_groups; g0 += 1024) {
-        const int g = g0 + threadIdx.x;
-        const int cnt = g < n_groups ? grp_cnt[g] : 0;
-        part_c[threadIdx.x] = cnt;
-        __syncthreads();
-        for (int o = 1; o < 1024; o <<= 1) {
-            const int ac = (int)threadIdx.x >= o ? part_c[threadIdx.x - o] : 0;
-            __syncthreads();
-            part_c[threadIdx.x] += ac;
-            __syncthreads();
+        const int g = g0 + tid;
+        look_up(g);
+        int run = me.cnt;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, run, o);
+            if (lane >= o) run += v;
         }
-        if (g < n_groups) {
-            grp_start[g] = carry_c + part_c[threadIdx.x] - cnt;
-            if (cnt > 0) {
-                int slot, len, key0;
-                group_info(g, slot, len, key0);
-                atomicAdd(&cls_tiles[class_of(len)], (cnt + kTcTile - 1) / kTcTile);
+        if (lane == 31) warp_sum_s[warp] = run;
+        __syncthreads();
+        int before = lane < warp ? warp_sum_s[lane] : 0;
+        before = __reduce_add_sync(0xffffffffu, before) + carry_c;
+        me.start = before + run - me.cnt;
+        if (g < n_groups) grp_start[g] = me.start;
+        if (me.cnt > 0) blocks += (long long)((me.cnt + kTcTile - 1) / kTcTile) * key_blocks(me.len);
+        __syncthreads();
+        if (tid == 1023) carry_c = me.start + me.cnt;
+        __syncthreads();
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) blocks += __shfl_xor_sync(0xffffffffu, blocks, o);
+    if (lane == 0) warp_blocks_s[warp] = blocks;
+    __syncthreads();
+    blocks = warp_blocks_s[lane];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) blocks += __shfl_xor_sync(0xffffffffu, blocks, o);
+    // Key blocks of a piece.  Tiles with more are cut into ceil(blocks / piece) pieces: at most 2 blocks / piece <= kSplitSlots
+    // records of partial results.  Below four blocks a piece is mostly its own start and end.
+    const int piece = sl.split.slots >= kSplitSlots ? max(4, (int)((blocks + 2 * 148 - 1) / (2 * 148))) : 0x7fffffff;
+    auto pieces_of = [&](int len) {
+        const int nb = key_blocks(len);
+        return nb > piece ? (nb + piece - 1) / piece : 1;
+    };
+    const bool one_batch = n_groups <= 1024;
+    // pass 2: jobs per size class (a piece's share of the keys)
+    for (int g0 = 0; g0 < n_groups; g0 += 1024) {
+        if (!one_batch) look_up(g0 + tid);
+        if (me.cnt > 0) {
+            me.np = pieces_of(me.len);
+            atomicAdd(&cls_jobs[class_of(key_blocks(me.len) / me.np)], (me.cnt + kTcTile - 1) / kTcTile * me.np);
+        }
+    }
+    __syncthreads();
+    if (warp == 0) {   // first job of every class, largest first
+        int n[4], run = 0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) n[i] = cls_jobs[kClasses - 1 - 4 * lane - i], run += n[i];
+        int before = run;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, before, o);
+            if (lane >= o) before += v;
+        }
+        if (lane == 31) n_out[1] = n_jobs_s = min(before, job_cap);
+        before -= run;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            cls_base[kClasses - 1 - 4 * lane - i] = before;
+            cls_jobs[kClasses - 1 - 4 * lane - i] = 0;   // from here on the class's cursor
+            before += n[i];
+        }
+    }
+    __syncthreads();
+    // row j / 148 of the jobs, whole rows in turn forwards and backwards
+    auto place_of = [&](int j) {
+        const int row = j / 148, col = j - row * 148;
+        return (row & 1) && row < n_jobs_s / 148 ? row * 148 + 147 - col : j;
+    };
+    // pass 3: the records, a warp per group of the batch; the counts go back to zero
+    for (int g0 = 0; g0 < n_groups; g0 += 1024) {
+        const int g = g0 + tid;
+        if (!one_batch) {
+            look_up(g);
+            if (g < n_groups) me.start = grp_start[g];
+        }
+        if (me.cnt > 0) {
+            grp_cnt[g] = 0;
+            me.np = pieces_of(me.len);
+            const int nt = (me.cnt + kTcTile - 1) / kTcTile, k = class_of(key_blocks(me.len) / me.np);
+            me.t0 = atomicAdd(&tile_cur, nt), me.j0 = cls_base[k] + atomicAdd(&cls_jobs[k], nt * me.np);
+            if (me.np > 1) me.p0 = atomicAdd(&pslot_cur, nt * me.np);
+        }
+        grp[tid] = me;
+        __syncthreads();
+        for (int i = warp; i < min(1024, n_groups - g0); i += 32) {
+            const SimGroup q = grp[i];
+            if (q.cnt == 0) continue;
+            const int nt = (q.cnt + kTcTile - 1) / kTcTile, nb = key_blocks(q.len);
+            for (int e = lane; e < nt * q.np; e += 32) {
+                const int t = e / q.np, part = e - t * q.np, n = min(kTcTile, q.cnt - t * kTcTile);
+                const int64_t pos0 = (int64_t)q.start + (int64_t)t * kTcTile;
+                // (within the caps for a launch within the context's limits, sim_prepare)
+                if (part == 0 && q.t0 + t < tile_cap) tiles[q.t0 + t] = TileDev{q.slot, n, pos0, q.len, q.key0, {0, 0}};
+                const int b0 = nb * part / q.np, b1 = nb * (part + 1) / q.np;
+                if (q.j0 + e < job_cap) {
+                    const int j = place_of(q.j0 + e);
+                    jobs[j] = JobDev{q.slot, n, pos0, q.np == 1 ? q.len : min(q.len - b0 * 128, (b1 - b0) * 128), q.key0 + b0 * 128, part, q.np,
+                                            q.p0 + t * q.np, q.len};
+                    if (part == 0 && q.np > 1) joins[atomicAdd(&join_cur, 1)] = j;
+                }
             }
         }
         __syncthreads();
-        if (threadIdx.x == 1023) carry_c += part_c[1023];
-        __syncthreads();
     }
-    // first tile of every class, longest sub-sequences first
-    if (threadIdx.x == 0) {
-        int run = 0;
-        for (int k = kClasses - 1; k >= 0; --k) {
-            cls_base[k] = run;
-            run += cls_tiles[k];
-            cls_tiles[k] = 0;   // from here on the class's cursor
-        }
-        *n_tiles_out = min(run, tile_cap);
-    }
-    __syncthreads();
-    // pass 2: the tile records; the counts become the placement cursors
-    for (int g = threadIdx.x; g < n_groups; g += 1024) {
-        const int cnt = grp_cnt[g];
-        grp_cnt[g] = 0;
-        if (cnt == 0) continue;
-        int slot, len, key0;
-        group_info(g, slot, len, key0);
-        const int nt = (cnt + kTcTile - 1) / kTcTile, k = class_of(len);
-        const int t0 = cls_base[k] + atomicAdd(&cls_tiles[k], nt);
-        const int start = grp_start[g];
-        for (int i = 0; i < nt; ++i) {
-            if (t0 + i >= tile_cap) break;   // cannot happen for a launch within the context's limits (sim_prepare)
-            TileDev t;
-            t.slot = slot, t.cnt = min(kTcTile, cnt - i * kTcTile), t.pos0 = (int64_t)start + (int64_t)i * kTcTile;
-            t.L = len, t.key0 = key0, t.pad_[0] = t.pad_[1] = 0;
-            tiles[t0 + i] = t;
-        }
-    }
-}
-
-// grouped ids and, for every grouped position, where its logit belongs
-__global__ void __launch_bounds__(256) k_sim_place(ScoreLaunch sl, int64_t M, int n_cat, int mode, const int32_t *__restrict__ grp_start,
-                                                   int32_t *__restrict__ cursor, int32_t *__restrict__ ids_out, int32_t *__restrict__ out_index)
-{
-    for (int64_t pos = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; pos < sl.total; pos += (int64_t)gridDim.x * blockDim.x) {
-        int id;
-        const int g = group_of(sl, pos, M, n_cat, mode, id);
-        const int p = grp_start[g] + atomicAdd(&cursor[g], 1);
-        ids_out[p] = id;
-        out_index[p] = (int32_t)pos;
-    }
+    if (tid == 0) n_out[0] = min(tile_cur, tile_cap), n_out[2] = join_cur;
 }
 
 struct SimPlan {
     int n_groups_max = 0;
     size_t tile_cap = 0, cap = 0;
-    int32_t *grp_cnt = nullptr, *grp_start = nullptr, *ids_sorted = nullptr, *out_index = nullptr, *n_tiles_dev = nullptr;
+    int32_t *grp_cnt = nullptr, *grp_start = nullptr, *ids_sorted = nullptr, *out_index = nullptr, *n_tiles_dev = nullptr;   // [3]: tiles, jobs, split tiles
     TileDev *tiles = nullptr;
+    int2 *where = nullptr;       // [cap] group and rank of every candidate
+    JobDev *jobs = nullptr;      // [tile_cap + kSplitSlots]
+    int32_t *joins = nullptr;    // [kSplitSlots] first pieces of the split tiles
 };
 
 SimPlan *plan_of(const aif_ctx *ctx) { return reinterpret_cast<SimPlan *>(ctx->sim_plan); }
@@ -274,8 +347,11 @@ cudaError_t sim_prepare(aif_ctx *ctx)
     if ((e = alloc((void **)&pl->grp_start, (size_t)pl->n_groups_max * 4)) != cudaSuccess) return e;
     if ((e = alloc((void **)&pl->ids_sorted, (pl->cap + kTcTile) * 4)) != cudaSuccess) return e;
     if ((e = alloc((void **)&pl->out_index, (pl->cap + kTcTile) * 4)) != cudaSuccess) return e;
+    if ((e = alloc((void **)&pl->where, pl->cap * sizeof(int2))) != cudaSuccess) return e;
     if ((e = alloc((void **)&pl->n_tiles_dev, 256)) != cudaSuccess) return e;
     if ((e = alloc((void **)&pl->tiles, pl->tile_cap * sizeof(TileDev))) != cudaSuccess) return e;
+    if ((e = alloc((void **)&pl->jobs, (pl->tile_cap + kSplitSlots) * sizeof(JobDev))) != cudaSuccess) return e;
+    if ((e = alloc((void **)&pl->joins, kSplitSlots * 4)) != cudaSuccess) return e;
     return cudaSuccess;
 }
 
@@ -315,24 +391,24 @@ cudaError_t sim_group_sequence(const aif_ctx *ctx, HostSlot &hs, const int32_t *
     return cudaGetLastError();
 }
 
-cudaError_t sim_group_candidates(const aif_ctx *ctx, ScoreLaunch &sl, cudaStream_t st)
+cudaError_t sim_group_candidates(const aif_ctx *ctx, ScoreLaunch &sl, SimPlace &place, cudaStream_t st)
 {
     const aif_config &c = ctx->cfg;
     SimPlan *pl = plan_of(ctx);
     const int n_groups = sl.n_req * c.n_categories;
-    cudaError_t e = cudaMemsetAsync(pl->grp_cnt, 0, (size_t)n_groups * 4, st);
-    if (e != cudaSuccess) return e;
     const int grid = (int)((sl.total + 255) / 256 < 1184 ? (sl.total + 255) / 256 : 1184);
-    k_sim_count<<<grid, 256, 0, st>>>(sl, c.M, c.n_categories, c.bucket_mode, pl->grp_cnt);
-    k_sim_tiles<<<1, 1024, 0, st>>>(sl, n_groups, c.n_categories, pl->grp_cnt, pl->grp_start, pl->tiles, (int)pl->tile_cap, pl->n_tiles_dev);
-    k_sim_place<<<grid, 256, 0, st>>>(sl, c.M, c.n_categories, c.bucket_mode, pl->grp_start, pl->grp_cnt, pl->ids_sorted, pl->out_index);
-    count_launch(3);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    cudaError_t e = launch_pdl(k_sim_count, dim3(grid), dim3(256), 0, st, sl, c.M, c.n_categories, c.bucket_mode, pl->grp_cnt, pl->where);
+    if (e != cudaSuccess) return e;
+    e = launch_pdl(k_sim_tiles, dim3(1), dim3(1024), 0, st, sl, n_groups, c.n_categories, pl->grp_cnt, pl->grp_start, pl->tiles, (int)pl->tile_cap, pl->jobs,
+                   (int)pl->tile_cap + kSplitSlots, pl->joins, pl->n_tiles_dev);
+    if (e != cudaSuccess) return e;
+    count_launch(2);
+    place = SimPlace{pl->where, pl->grp_start, pl->ids_sorted, pl->out_index};
     const int64_t groups = (int64_t)n_groups < sl.total ? (int64_t)n_groups : sl.total;
     sl.n_tiles = (int32_t)(sl.total / kTcTile + groups + 1 < (int64_t)pl->tile_cap ? sl.total / kTcTile + groups + 1 : (int64_t)pl->tile_cap);
-    sl.ids = pl->ids_sorted;
     sl.tiles = pl->tiles;
     sl.n_tiles_dev = pl->n_tiles_dev;
+    sl.joins = pl->joins, sl.jobs = pl->jobs, sl.n_jobs_dev = pl->n_tiles_dev + 1, sl.n_jobs = sl.n_tiles + (sl.split.slots >= kSplitSlots ? kSplitSlots : 0);
     sl.out_index = pl->out_index;
     sl.grouped = 1;
     return cudaSuccess;

@@ -95,10 +95,11 @@ __device__ __forceinline__ TileInfo decode_tile(const LayerParams &p, int tile, 
 // Cross-feature index generation for a whole launch (Section 3.3, "real-time generation" from the candidate's
 // attribute): xb[pos][f] = bucket of candidate pos in field f, or kNoBucket for an id outside the item table.  Done
 // once per call so that the layer kernel's gather threads only look the bucket up.  Ids in mapped host memory are copied
-// to ids_copy on the way, for the kernels that follow.
+// to ids_copy on the way, for the kernels that follow; candidates that are grouped by category are placed on the way (pl.where:
+// pos becomes the grouped position; F = 0 does nothing else).
 constexpr uint32_t kNoBucket = 0xFFFFu;
 __global__ void __launch_bounds__(256) k_cross_buckets(const int32_t *__restrict__ ids, int64_t total, int64_t M, int F, int B,
-                                                        int b_mask, int mode, uint16_t *__restrict__ xb, int32_t *__restrict__ ids_copy)
+                                                        int b_mask, int mode, uint16_t *__restrict__ xb, int32_t *__restrict__ ids_copy, const SimPlace pl)
 {
     grid_dep_launch();
     grid_dep_wait();
@@ -108,17 +109,23 @@ __global__ void __launch_bounds__(256) k_cross_buckets(const int32_t *__restrict
     const int lane = threadIdx.x & 31, step = F & 1 ? 1 : 2;
     const int64_t n_warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t base = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; base < total; base += n_warps * 32) {
-        int my = -1;
+        int my = -1, to = lane;   // to: the candidate's row of xb, counted from base
         if (base + lane < total) {
             my = ids[base + lane];
             if (ids_copy && blockIdx.y == 0) ids_copy[base + lane] = my;
+            if (pl.where) {
+                const int2 w = pl.where[base + lane];
+                const int at = pl.grp_start[w.x] + w.y;
+                to = at - (int)base;
+                if (blockIdx.y == 0) pl.ids[at] = my, pl.out_index[at] = (int)base + lane;
+            }
         }
         const int n = (int)min((int64_t)32, total - base) * F;
         uint16_t *out = xb + base * F;
         // small launches spread a warp's hashes over gridDim.y warps (the ids are then read that many times)
         for (int i0 = 32 * step * (int)blockIdx.y; i0 < 32 * F; i0 += 32 * step * (int)gridDim.y) {
             const int i = i0 + lane * step, c = i / F, f = i - c * F;
-            const int id = __shfl_sync(0xffffffffu, my, c & 31);
+            const int id = __shfl_sync(0xffffffffu, my, c & 31), row = __shfl_sync(0xffffffffu, to, c & 31);
             const bool good = id >= 0 && (int64_t)id < M;
             uint32_t bk[2] = {kNoBucket, kNoBucket};
 #pragma unroll
@@ -131,8 +138,9 @@ __global__ void __launch_bounds__(256) k_cross_buckets(const int32_t *__restrict
                     }
                 }
             if (i >= n) continue;
-            if (step == 2) *reinterpret_cast<uint32_t *>(out + i) = bk[0] | (bk[1] << 16);
-            else out[i] = (uint16_t)bk[0];
+            uint16_t *o = out + (int64_t)row * F + f;
+            if (step == 2) *reinterpret_cast<uint32_t *>(o) = bk[0] | (bk[1] << 16);
+            else *o = (uint16_t)bk[0];
         }
     }
 }
@@ -723,6 +731,82 @@ __global__ void __launch_bounds__(256) k_interact_x(ModelDev md, ScoreLaunch sl,
     }
 }
 
+constexpr int kJoinCols = 16;
+__device__ __forceinline__ void join_tile(const JoinParams &p, const KeyTile &t, int y)
+{
+    if (t.n_parts < 2) return;   // one key block in the whole tile: the first piece has delivered
+    const int row = threadIdx.x & 127, half = threadIdx.x >> 7;
+    if (row >= t.cnt) return;
+    const int id = p.sl.ids[t.pos0 + row];
+    const bool good = id >= 0 && (int64_t)id < p.M;   // an id outside the table: a zero row
+    const SplitScratch &sp = p.sl.split;
+    __nv_bfloat16 *x = p.X + (size_t)(t.pos0 + row) * p.x_stride;
+    const int n = t.n_parts;
+    if (p.col >= 0 && y < p.d / kJoinCols) {
+        const int g0 = y * (kJoinCols / 4) + half * 2;   // two groups of four columns per thread
+        const float4 *rows = reinterpret_cast<const float4 *>(sp.rows) + ((size_t)t.pslot * (p.d / 4) + g0) * 128 + row;
+        const size_t piece = (size_t)(p.d / 4) * 128;
+        const float *st = sp.stats + (size_t)t.pslot * 256 + row;
+        float m = 0.f, l = 0.f, acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        if (p.attention) {
+            m = -INFINITY;
+            for (int q = 0; q < n; ++q) m = fmaxf(m, st[q * 256 + 128]);
+        }
+#pragma unroll 4
+        for (int q = 0; q < n; ++q) {
+            const float4 a = rows[q * piece], b = rows[q * piece + 128];
+            float w = 1.f;
+            if (p.attention) {
+                w = fast_exp2(st[q * 256 + 128] - m);   // 1 where no piece needed a running maximum
+                l = fmaf(st[q * 256], w, l);
+            }
+            acc[0] = fmaf(w, a.x, acc[0]), acc[1] = fmaf(w, a.y, acc[1]), acc[2] = fmaf(w, a.z, acc[2]), acc[3] = fmaf(w, a.w, acc[3]);
+            acc[4] = fmaf(w, b.x, acc[4]), acc[5] = fmaf(w, b.y, acc[5]), acc[6] = fmaf(w, b.z, acc[6]), acc[7] = fmaf(w, b.w, acc[7]);
+        }
+        const float scale = p.attention ? (l > 0.f ? 1.0f / l : 0.f) : p.row_scale * (p.row_mean ? 1.0f / (float)t.L_tile : 1.0f);
+        uint4 o;
+        __nv_bfloat162 *h = reinterpret_cast<__nv_bfloat162 *>(&o);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) h[i] = __floats2bfloat162_rn(good ? acc[2 * i] * scale : 0.f, good ? acc[2 * i + 1] * scale : 0.f);
+        *reinterpret_cast<uint4 *>(x + p.col + g0 * 4) = o;
+    } else {
+        // 64 columns of tier counts, the first n_tiers used: half 0 the first 32, half 1 the rest (zero)
+        const float nrm = p.tier_mean ? 1.0f / (float)t.L_tile : 1.0f;
+        const int32_t *c = sp.tiers + (size_t)t.pslot * 16 * 128 + row;
+        uint4 o[4];
+        __nv_bfloat162 *h = reinterpret_cast<__nv_bfloat162 *>(o);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) h[i] = __floats2bfloat162_rn(0.f, 0.f);
+        if (half == 0 && good) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                int a = 0, b = 0;
+                if (2 * i < p.n_tiers)
+                    for (int q = 0; q < n; ++q) a += c[(q * 16 + 2 * i) * 128], b += c[(q * 16 + 2 * i + 1) * 128];
+                h[i] = __floats2bfloat162_rn((float)a * nrm, 2 * i + 1 < p.n_tiers ? (float)b * nrm : 0.f);
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) *reinterpret_cast<uint4 *>(x + p.x_tier + half * 32 + i * 8) = o[i];
+    }
+}
+
+// Puts the pieces of split tiles together, in their order: an item is sixteen columns of a tile's rows or (SimTier on) its tier
+// counts.  The pieces' sums are joined by a launch of their own and not by whichever piece comes last: a tile's records are
+// 64 KB per piece, and one SM takes in 59 bytes per clock (8 pieces: 9 k cycles at the end of the launch, eq. 2's attention over
+// 1000 items 13.7 -> 23 us); here a tile is read by as many SMs as there are columns to share out.
+__global__ void __launch_bounds__(256) k_join_pieces(const JoinParams p)
+{
+    grid_dep_launch();
+    grid_dep_wait();
+    const int n_y = (p.col >= 0 ? p.d / kJoinCols : 0) + (p.x_tier >= 0 ? 1 : 0);
+    const int n_items = (p.sl.jobs ? p.sl.n_jobs_dev[1] : p.sl.n_tiles) * n_y;
+    for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
+        const int tile = item / n_y, y = item - tile * n_y, job = p.sl.jobs ? p.sl.joins[tile] : tile * p.sl.parts;
+        join_tile(p, p.d == 128 ? key_tile<128, true>(p.sl, job, p.mini_batch) : key_tile<64, true>(p.sl, job, p.mini_batch), y);
+    }
+}
+
 // Self-test of the bounded wait: one thread waits, with a short limit, on an mbarrier that nobody arrives on.  The wait
 // gives up, raises the status bit and the kernel returns normally: this is the path a scoring kernel takes when a
 // producer never delivers, exercised without any fault.
@@ -899,11 +983,44 @@ cudaError_t tc_prepare_context(aif_ctx *ctx)
         in_w = c.hidden[k];
     }
     pl->maps_ready = true;
+    const bool key_kernels = tc_att_supported(c) || tc_lsh_supported(c);
+    auto take_split = [&](SplitScratch &sp, int slots, bool tiers) -> cudaError_t {
+        cudaError_t err;
+        if ((err = alloc((void **)&sp.rows, (size_t)slots * 128 * c.d * 4)) != cudaSuccess) return err;
+        if ((err = alloc((void **)&sp.stats, (size_t)slots * 256 * 4)) != cudaSuccess) return err;
+        if (tiers && (err = alloc((void **)&sp.tiers, (size_t)slots * 16 * 128 * 4)) != cudaSuccess) return err;
+        sp.slots = slots;
+        return cudaSuccess;
+    };
+    if (key_kernels && (e = take_split(ctx->split, kSplitSlots, (c.blocks & AIF_BLK_SIMTIER) != 0)) != cudaSuccess) return e;
+    if (tc_att_supported(c) && (e = take_split(ctx->split_user, kSplitSlotsUser, false)) != cudaSuccess) return e;
     if (tc_att_supported(c) && (e = tc_att_prepare(ctx)) != cudaSuccess) return e;
     if (tc_fused_supported(c) && (e = tc_fused_prepare(ctx)) != cudaSuccess) return e;
     if (tc_lsh_supported(c) && (e = tc_lsh_prepare(ctx)) != cudaSuccess) return e;
     if (c.n_categories > 0 && (e = sim_prepare(ctx)) != cudaSuccess) return e;
     return cudaSuccess;
+}
+
+// A launch takes ceil(jobs / 148) rounds of (key blocks of a job + what a job costs besides: the query gather before its first
+// scores, its output), in units of a key block (0.9 us), and a split one the joining launch on top (about 5 us).  Splitting pays
+// where the tiles leave SMs without work or fill the last round badly; a gain below a tenth is not worth the traffic.  Eq. 2 over
+// 1000 items (8 tiles of 8 blocks) takes as long either way, which is where this line lies.
+int split_parts(int n_tiles, int blocks, int slots)
+{
+    auto cost = [&](int parts) { return ((int64_t)n_tiles * parts + 147) / 148 * ((blocks + parts - 1) / parts + (parts > 1 ? 3 : 2)) + (parts > 1 ? 5 : 0); };
+    int best = 1;
+    for (int parts = 2; parts <= blocks && parts <= 32 && (int64_t)n_tiles * parts <= slots; ++parts)
+        if (cost(parts) < cost(best)) best = parts;
+    return best > 1 && 10 * cost(best) < 9 * cost(1) ? best : 1;
+}
+
+cudaError_t launch_join_pieces(const JoinParams &p, cudaStream_t st)
+{
+    const int n_y = (p.col >= 0 ? p.d / kJoinCols : 0) + (p.x_tier >= 0 ? 1 : 0);
+    const int items = (p.sl.jobs ? kSplitSlots / 2 : p.sl.n_tiles) * n_y, grid = items < 148 * 6 ? items : 148 * 6;
+    const cudaError_t e = launch_pdl(k_join_pieces, dim3(grid), dim3(256), 0, st, p);
+    count_launch();
+    return e;
 }
 
 const void *tc_weight_tmap(const aif_ctx *ctx, int k) { return &plan_of(ctx)->tmap[k]; }
@@ -963,6 +1080,7 @@ void tc_scratch_layout(const aif_ctx *ctx, void *base, size_t rows, TcScratch *o
     }
     out->xb = (c.blocks & AIF_BLK_CROSS) ? p : nullptr;
     out->tiles = nullptr;
+    out->split = false;
     out->rows = rows;
 }
 
@@ -1024,6 +1142,7 @@ cudaError_t launch_score_tc(const aif_ctx *ctx, const ScoreLaunch &sl, int64_t, 
     sc.X = pl->X;
     sc.xb = pl->xb;
     sc.tiles = pl->tiles;
+    sc.split = true;
     sc.rows = pl->cap_rows;
     for (int k = 0; k < kMaxHidden; ++k) sc.H[k] = pl->H[k];
     return launch_score_tc_scratch(ctx, sl, st, sc);
@@ -1034,6 +1153,7 @@ cudaError_t launch_score_tc_scratch(const aif_ctx *ctx, const ScoreLaunch &sl_in
     if (sl_in.n_tiles <= 0) return cudaSuccess;
     ScoreLaunch sl = sl_in;
     sl.tiles = nullptr;
+    if (sc.split) sl.split = ctx->split;
     const aif_config &c = ctx->cfg;
     TcPlan *pl = plan_of(ctx);
     const ModelDev md = make_model(ctx);
@@ -1051,11 +1171,12 @@ cudaError_t launch_score_tc_scratch(const aif_ctx *ctx, const ScoreLaunch &sl_in
         if (e != cudaSuccess) return e;
         sl.ids = sl.ids_copy, sl.ids_copy = nullptr;
     }
+    SimPlace place{};
     if (c.n_categories > 0) {
         // candidates grouped by (request, category): tiles, grouped ids and the way back to the caller's order
         if (sc.rows < (size_t)sl.total + kTcTile || !ctx->sim_plan) return cudaErrorInvalidValue;
         StageRange range("aif group");
-        cudaError_t e = sim_group_candidates(ctx, sl, st);
+        cudaError_t e = sim_group_candidates(ctx, sl, place, st);
         timing_mark(ctx, "group", st);
         if (e != cudaSuccess) return e;
     } else if (sl.reqs && sc.tiles) {   // several requests: look every tile up once
@@ -1064,22 +1185,26 @@ cudaError_t launch_score_tc_scratch(const aif_ctx *ctx, const ScoreLaunch &sl_in
         if (e != cudaSuccess) return e;
         sl.tiles = (const TileDev *)sc.tiles;
     }
-    if (c.blocks & AIF_BLK_CROSS) {
+    const int F = (c.blocks & AIF_BLK_CROSS) ? c.F : 0;
+    if (F > 0 || place.where) {
         StageRange range("aif buckets");
         const int64_t n = sl.total;   // a warp per 32 candidates
         const int grid = (int)((n + 255) / 256 < 148 * 16 ? (n + 255) / 256 : 148 * 16);
         // launches that leave SMs without a block split the fields of a candidate over up to eight warps, except where a read
         // of the ids crosses the bus
-        const int rounds = c.F & 1 ? c.F : c.F / 2, want_y = sl.ids_copy ? 1 : 296 / grid;
+        const int rounds = F == 0 ? 1 : F & 1 ? F : F / 2, want_y = sl.ids_copy ? 1 : 296 / grid;
         const int grid_y = want_y < 1 ? 1 : want_y > 8 ? (rounds < 8 ? rounds : 8) : want_y > rounds ? rounds : want_y;
-        cudaError_t e = launch_pdl(k_cross_buckets, dim3(grid, grid_y), dim3(256), 0, st, sl.ids, sl.total, c.M, c.F, c.B,
-                                   (c.B & (c.B - 1)) == 0 ? c.B - 1 : -1, c.bucket_mode, (uint16_t *)sc.xb, sl.ids_copy);
+        cudaError_t e = launch_pdl(k_cross_buckets, dim3(grid, grid_y), dim3(256), 0, st, sl.ids, sl.total, c.M, F, c.B,
+                                   (c.B & (c.B - 1)) == 0 ? c.B - 1 : -1, c.bucket_mode, (uint16_t *)sc.xb, sl.ids_copy, place);
         if (sl.ids_copy) sl.ids = sl.ids_copy;
+        if (place.where) sl.ids = place.ids;
         count_launch();
         timing_mark(ctx, "buckets", st);
         if (e != cudaSuccess) return e;
     }
     const bool att_tc = ctx->tc_att_plan != nullptr;
+    // few tiles with many keys: their keys over several CTAs each (the table of jobs does it where categories are on)
+    if (!sl.jobs) sl.parts = split_parts(sl.n_tiles, (sl.max_L + (c.d == 128 ? 127 : 63)) / (c.d == 128 ? 128 : 64), sl.split.slots);
     if (att_tc) {
         StageRange range("aif attention");
         cudaError_t e = launch_att_tc(ctx, sl, st, sc.X, pl->x_cols, sc.rows);

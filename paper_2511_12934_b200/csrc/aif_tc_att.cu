@@ -73,41 +73,15 @@ struct AttCfg {
     static constexpr int kPvWarp = kSoftWarps + 3;     // issues the P V products (kMmaWarp: Q K^T, and owns tensor memory)
     static constexpr int kEpiWarp0 = kSoftWarps + 4;   // first of the four output warps (kSplitEpi)
     static constexpr int kThreads = (kSoftWarps + 4 + (kSplitEpi ? 4 : 0)) * 32;
-    // barriers and the tensor-memory slot; row sums [2 tiles][kHalves][128]; block maxima [2 blocks][2][128]
-    static constexpr int kMisc = 512 + (kSplitEpi ? 2 * kHalves * 512 : 0) + (kHalves == 2 ? 2048 : 0);
+    // barriers and the tensor-memory slot; row sums [2 tiles][kHalves][128] and exponent offsets [2 tiles][128]; block maxima
+    // [2 blocks][2][128]
+    static constexpr int kMisc = 512 + (kSplitEpi ? 2 * kHalves * 512 + 1024 : 0) + (kHalves == 2 ? 2048 : 0);
     static constexpr size_t kSmem = 1024 + kQBufs * kQBytes + kKvStages * kKvBytes + kMisc;
 };
 
-// One tile of the launch as every role needs it.
-struct AttTile {
-    int slot, cnt, nb, L;
-    int key0;   // first key row: 0, or where the tile's category's sub-sequence begins in the grouped sequence
-    int64_t pos0;
-};
-
-template <int BN>
-__device__ __forceinline__ AttTile att_tile(const AttParams &p, int tile)
-{
-    AttTile t;
-    if (p.sl.tiles) {   // looked up once per launch (k_tile_table)
-        const int4 v = *reinterpret_cast<const int4 *>(p.sl.tiles + tile);   // slot, cnt, pos0
-        t.slot = v.x, t.cnt = v.y;
-        t.pos0 = ((int64_t)(uint32_t)v.w << 32) | (int64_t)(uint32_t)v.z;
-        t.L = p.sl.tiles[tile].L, t.key0 = p.sl.tiles[tile].key0;
-        // an empty sub-sequence still walks one key block, every column of it masked: the roles' hand-overs stay the same
-        t.nb = t.L > 0 ? (t.L + BN - 1) / BN : 1;
-        return t;
-    }
-    const ReqDev rq = find_request(p.sl, tile);
-    int start, cnt;
-    tile_range(tile - rq.tile_begin, rq.n, kTcTile, p.mini_batch, start, cnt);
-    t.slot = rq.slot, t.cnt = cnt, t.pos0 = rq.off + start;
-    t.L = p.sl.slots[rq.slot].L, t.key0 = 0;
-    t.nb = (t.L + BN - 1) / BN;
-    return t;
-}
-
-template <int D, int BN>
+// SPLIT: the launch's tiles are cut into pieces of their keys; a copy of its own, because the form that long sequences run uses
+// every register.
+template <int D, int BN, bool SPLIT>
 __global__ void __launch_bounds__((AttCfg<D, BN>::kThreads), 1) k_att_tc(const __grid_constant__ CUtensorMap tmapS,
                                                            const __grid_constant__ CUtensorMap tmapX, const AttParams p)
 {
@@ -127,6 +101,7 @@ __global__ void __launch_bounds__((AttCfg<D, BN>::kThreads), 1) k_att_tc(const _
     volatile uint32_t *abort_flag = tmem_slot + 1;
     float *l_s = reinterpret_cast<float *>(tmem_slot + 4);   // [2][kHalves][128] row sums handed to the output warps
     float *mx_s = l_s + (kSplit ? 2 * C::kHalves * 128 : 0);    // [2][2][128] block maxima exchanged between partner warps
+    float *m_s = mx_s + (C::kHalves == 2 ? 512 : 0);            // [2][128] exponent offsets handed to the output warps
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
@@ -160,11 +135,11 @@ __global__ void __launch_bounds__((AttCfg<D, BN>::kThreads), 1) k_att_tc(const _
     grid_dep_launch();
     grid_dep_wait();   // the set-up above overlapped the previous kernel; the request table and slots are read from here on
 
-    const int n_tiles = p.sl.n_tiles_dev ? *p.sl.n_tiles_dev : p.sl.n_tiles;
+    const int n_tiles = key_jobs<SPLIT>(p.sl);   // tiles, or pieces of tiles
 
     // Normalises a finished tile's O accumulator and stores the attention rows.  Run by the softmax warps themselves
     // (d = 256) or by the epilogue warps (d = 128); wq = the warp's quarter of the TMEM lanes.
-    auto tile_epilogue = [&](int k, const AttTile &t, float l_sum, int wq, int lane) {
+    auto tile_epilogue = [&](int k, const KeyTile &t, float l_sum, float m_sum, int wq, int lane) {
         const int row = wq * 32 + lane;
         const uint32_t lane_base = tmem_base + ((uint32_t)(wq * 32) << 16);
         const uint32_t o_col = (uint32_t)C::kTmemO;
@@ -214,21 +189,33 @@ __global__ void __launch_bounds__((AttCfg<D, BN>::kThreads), 1) k_att_tc(const _
                     dst[q] = make_uint4(packed[4 * q], packed[4 * q + 1], packed[4 * q + 2], packed[4 * q + 3]);
             }
         };
-        // two chunks of 32 columns per round; the load of the next chunk is in flight while one is converted and staged
-        uint32_t ra[32], rb[32];
-        tmem_ld32(lane_base + o_col, ra);
-#pragma unroll 1
-        for (int c0 = 0; c0 < D; c0 += 64) {
-            tmem_ld_wait();
-            tmem_ld32(lane_base + o_col + (uint32_t)(c0 + 32), rb);
-            emit(ra, c0);
-            tmem_ld_wait();
-            if (c0 + 64 < D) tmem_ld32(lane_base + o_col + (uint32_t)(c0 + 64), ra);
-            else {   // O is in registers: the next tile's first P V may overwrite the accumulator
-                tc_fence_before();
-                mbar_arrive(smem_u32(o_free_k));
+        if (SPLIT && t.n_parts != 1) {
+            // a piece of the tile's keys: its unnormalised rows, sums and exponent offsets go to the tile's records, four columns
+            // of 32 rows per store, for k_join_pieces
+            if (t.n_parts > 0) {
+                tmem_rows_out(lane_base + o_col, D, reinterpret_cast<float4 *>(p.sl.split.rows) + (size_t)(t.pslot + t.part) * (D / 4) * 128 + row);
+                float *st = p.sl.split.stats + (size_t)(t.pslot + t.part) * 256 + row;
+                __stcg(st, l_sum), __stcg(st + 128, m_sum);
             }
-            emit(rb, c0 + 32);
+            tc_fence_before();
+            mbar_arrive(smem_u32(o_free_k));
+        } else {
+            // two chunks of 32 columns per round; the load of the next chunk is in flight while one is converted and staged
+            uint32_t ra[32], rb[32];
+            tmem_ld32(lane_base + o_col, ra);
+#pragma unroll 1
+            for (int c0 = 0; c0 < D; c0 += 64) {
+                tmem_ld_wait();
+                tmem_ld32(lane_base + o_col + (uint32_t)(c0 + 32), rb);
+                emit(ra, c0);
+                tmem_ld_wait();
+                if (c0 + 64 < D) tmem_ld32(lane_base + o_col + (uint32_t)(c0 + 64), ra);
+                else {   // O is in registers: the next tile's first P V may overwrite the accumulator
+                    tc_fence_before();
+                    mbar_arrive(smem_u32(o_free_k));
+                }
+                emit(rb, c0 + 32);
+            }
         }
         if (lane == 0) {
             bulk_wait_read<0>();   // the staging is no longer read: the query buffer may take its next tenant
@@ -251,7 +238,7 @@ __global__ void __launch_bounds__((AttCfg<D, BN>::kThreads), 1) k_att_tc(const _
         if ((int)blockIdx.x < n_tiles) {
             // The CTA's first tile has nobody to prefetch it: these warps, idle until the first scores arrive, gather
             // its queries (8 threads per row, 16 bytes each per 128-byte chunk); later tiles come from the gather warp.
-            const AttTile t = att_tile<BN>(p, blockIdx.x);
+            const KeyTile t = key_tile<BN, SPLIT>(p.sl, blockIdx.x, p.mini_batch);
             const int sub = tid & 7, r0 = tid >> 3;
 #pragma unroll
             for (int i = 0; i < 8 / kH; ++i) {
@@ -269,7 +256,7 @@ __global__ void __launch_bounds__((AttCfg<D, BN>::kThreads), 1) k_att_tc(const _
             cp_async_arrive_noinc(smem_u32(q_first));
         }
         for (int tile = blockIdx.x; ok && tile < n_tiles; tile += gridDim.x, ++k) {
-            const AttTile t = att_tile<BN>(p, tile);
+            const KeyTile t = key_tile<BN, SPLIT>(p.sl, tile, p.mini_batch);
             const int L = t.L;
             // Decided once per tile and agreed on by the warps that meet at a barrier in the other mode: two warps
             // reading a bound that a refresh is raising meanwhile must not come to different answers.
@@ -432,6 +419,7 @@ __global__ void __launch_bounds__((AttCfg<D, BN>::kThreads), 1) k_att_tc(const _
                     break;
                 }
                 l_s[((k & 1) * kH + half) * 128 + row] = l_sum;
+                if (SPLIT && half == 0) m_s[(k & 1) * 128 + row] = m_used;   // the two warps of a row quarter agree on it
                 mbar_arrive(smem_u32(l_ready + (k & 1)));
             } else {
                 if (!mbar_wait(smem_u32(o_final), (uint32_t)(k & 1), abort_flag)) {
@@ -439,7 +427,7 @@ __global__ void __launch_bounds__((AttCfg<D, BN>::kThreads), 1) k_att_tc(const _
                     break;
                 }
                 tc_fence_after();
-                tile_epilogue(k, t, l_sum, warp, lane);
+                tile_epilogue(k, t, l_sum, m_used, warp, lane);
             }
         }
         if (lane == 0) bulk_wait<0>();   // all tile stores of this warp have reached global memory
@@ -456,7 +444,7 @@ __global__ void __launch_bounds__((AttCfg<D, BN>::kThreads), 1) k_att_tc(const _
                 uint32_t gb;
                 int nb_next;   // key blocks of the tile after this one, fetched a whole tile ahead of its use
             };
-            auto blocks_of = [&](int tile) { return tile < n_tiles ? att_tile<BN>(p, tile).nb : 0; };
+            auto blocks_of = [&](int tile) { return tile < n_tiles ? key_tile<BN, SPLIT>(p.sl, tile, p.mini_batch).nb : 0; };
             auto open_tile = [&](Cursor &c) {
                 c.nb = c.nb_next;
                 c.nb_next = blocks_of(c.tile + (int)gridDim.x);
@@ -534,7 +522,7 @@ __global__ void __launch_bounds__((AttCfg<D, BN>::kThreads), 1) k_att_tc(const _
             uint32_t gb = 0;
             bool ok = true;
             for (int tile = blockIdx.x; ok && tile < n_tiles; tile += gridDim.x) {
-                const AttTile t = att_tile<BN>(p, tile);
+                const KeyTile t = key_tile<BN, SPLIT>(p.sl, tile, p.mini_batch);
                 for (int j = 0; j < t.nb; ++j, ++gb) {
                     const int s = (int)(gb % kS);
                     if (!mbar_wait(smem_u32(kv_empty + s), ((gb / kS) & 1u) ^ 1u, abort_flag)) {
@@ -555,7 +543,7 @@ __global__ void __launch_bounds__((AttCfg<D, BN>::kThreads), 1) k_att_tc(const _
         const int wq = warp & 3;   // the quarter of the tensor-memory lanes this warp may read
         int k = 0;
         for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, ++k) {
-            const AttTile t = att_tile<BN>(p, tile);
+            const KeyTile t = key_tile<BN, SPLIT>(p.sl, tile, p.mini_batch);
             const int b = k & 1;
             const uint32_t parity = (uint32_t)((k >> 1) & 1);
             if (!mbar_wait(smem_u32(l_ready + b), parity, abort_flag)) break;
@@ -564,7 +552,7 @@ __global__ void __launch_bounds__((AttCfg<D, BN>::kThreads), 1) k_att_tc(const _
             for (int h = 0; h < C::kHalves; ++h) l_sum += l_s[(b * C::kHalves + h) * 128 + wq * 32 + lane];
             if (!mbar_wait(smem_u32(o_final + b), parity, abort_flag)) break;
             tc_fence_after();
-            tile_epilogue(k, t, l_sum, wq, lane);
+            tile_epilogue(k, t, l_sum, SPLIT ? m_s[b * 128 + wq * 32 + lane] : 0.f, wq, lane);
         }
         if (lane == 0) bulk_wait<0>();   // all tile stores of this warp have reached global memory
     } else if (warp == C::kGatherWarp) {
@@ -576,7 +564,7 @@ __global__ void __launch_bounds__((AttCfg<D, BN>::kThreads), 1) k_att_tc(const _
             const int qb = k % kQB;
             // the buffer's previous tenant is tile k - kQB (the first tile, tenant of buffer 0, included)
             if (k >= kQB && !mbar_wait(smem_u32(q_empty + qb), (uint32_t)(((k - kQB) / kQB) & 1), abort_flag)) break;
-            const AttTile t = att_tile<BN>(p, tile);
+            const KeyTile t = key_tile<BN, SPLIT>(p.sl, tile, p.mini_batch);
             unsigned char *q = smQ + qb * C::kQBytes;
             // the tile's 128 ids with four coalesced loads per lane (rows lane, lane + 32, ...); -1 = zero row
             int idv[4];
@@ -672,10 +660,14 @@ cudaError_t tc_att_prepare(aif_ctx *ctx)
         count_launch();
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
-    if (c.d == 128)
-        e = cudaFuncSetAttribute(k_att_tc<128, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)AttCfg<128, 128>::kSmem);
-    else
-        e = cudaFuncSetAttribute(k_att_tc<256, 64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)AttCfg<256, 64>::kSmem);
+    auto allow = [](auto kernel, size_t smem) { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); };
+    if (c.d == 128) {
+        e = allow(k_att_tc<128, 128, false>, AttCfg<128, 128>::kSmem);
+        if (e == cudaSuccess) e = allow(k_att_tc<128, 128, true>, AttCfg<128, 128>::kSmem);
+    } else {
+        e = allow(k_att_tc<256, 64, false>, AttCfg<256, 64>::kSmem);
+        if (e == cudaSuccess) e = allow(k_att_tc<256, 64, true>, AttCfg<256, 64>::kSmem);
+    }
     return e;
 }
 
@@ -706,6 +698,28 @@ static cudaError_t encode_x_map(CUtensorMap *m, void *X, int x_stride, size_t ro
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
+// The kernel over a launch's tiles or pieces, and for pieces the launch that puts them together.
+// One CTA per SM walking over its tiles hides a tile's query gather and output behind its neighbours' key blocks: 22 k against
+// 31 k cycles per 8-block tile, which outweighs the static assignment's rounding (8.5 tiles per SM cost 9 tile times) as soon as
+// some SM has two tiles.
+static cudaError_t run_att(int d, const AttParams &p, const CUtensorMap &ts, const CUtensorMap &tx, cudaStream_t st)
+{
+    const ScoreLaunch &sl = p.sl;
+    const bool split = sl.jobs || sl.parts > 1;
+    const int jobs = sl.jobs ? sl.n_jobs : sl.n_tiles * (split ? sl.parts : 1), grid = jobs > 148 ? 148 : jobs;
+    auto go = [&](auto kernel, int threads, size_t smem) { return launch_pdl(kernel, dim3(grid), dim3(threads), smem, st, ts, tx, p); };
+    using C1 = AttCfg<128, 128>;
+    using C2 = AttCfg<256, 64>;
+    cudaError_t e;
+    if (d == 128) e = split ? go(k_att_tc<128, 128, true>, C1::kThreads, C1::kSmem) : go(k_att_tc<128, 128, false>, C1::kThreads, C1::kSmem);
+    else e = split ? go(k_att_tc<256, 64, true>, C2::kThreads, C2::kSmem) : go(k_att_tc<256, 64, false>, C2::kThreads, C2::kSmem);
+    count_launch();
+    if (e != cudaSuccess || !split) return e;
+    JoinParams j{};
+    j.sl = sl, j.X = p.X, j.M = p.M, j.x_stride = p.x_stride, j.col = 0, j.x_tier = -1, j.d = d, j.mini_batch = p.mini_batch, j.attention = 1;
+    return launch_join_pieces(j, st);
+}
+
 cudaError_t launch_att_tc(const aif_ctx *ctx, const ScoreLaunch &sl, cudaStream_t st, void *X, int x_stride, size_t x_rows)
 {
     const aif_config &c = ctx->cfg;
@@ -718,18 +732,7 @@ cudaError_t launch_att_tc(const aif_ctx *ctx, const ScoreLaunch &sl, cudaStream_
     p.x_stride = x_stride, p.X = (__nv_bfloat16 *)X;
     p.scale_log2 = 1.4426950408889634f / sqrtf((float)c.d);
     p.q_norm = ctx->e_norm;
-    // One CTA per SM walking over its tiles hides a tile's query gather and output behind its neighbours' key blocks:
-    // 22 k against 31 k cycles per 8-block tile, which outweighs the static assignment's rounding (8.5 tiles per SM cost
-    // 9 tile times) as soon as some SM has two tiles.
-    const int grid = sl.n_tiles > 148 ? 148 : sl.n_tiles;
-    cudaError_t e;
-    const CUtensorMap &tm = sl.grouped ? pl->tmap_g : pl->tmap;
-    if (c.d == 128)
-        e = launch_pdl(k_att_tc<128, 128>, dim3(grid), dim3(AttCfg<128, 128>::kThreads), AttCfg<128, 128>::kSmem, st, tm, tmap_x, p);
-    else
-        e = launch_pdl(k_att_tc<256, 64>, dim3(grid), dim3(AttCfg<256, 64>::kThreads), AttCfg<256, 64>::kSmem, st, tm, tmap_x, p);
-    count_launch();
-    return e;
+    return run_att(c.d, p, sl.grouped ? pl->tmap_g : pl->tmap, tmap_x, st);
 }
 
 cudaError_t launch_self_att_tc(const aif_ctx *ctx, int slot_index, int L, cudaStream_t st, const void **rows_out)
@@ -741,6 +744,8 @@ cudaError_t launch_self_att_tc(const aif_ctx *ctx, int slot_index, int L, cudaSt
     sl.single = ReqDev{slot_index, L, 0, 0, 0};
     sl.n_tiles = (L + kTcTile - 1) / kTcTile, sl.total = L, sl.max_L = L;
     sl.ids = pl->iota, sl.logits = nullptr, sl.status = ctx->status;
+    // a user is a few tiles: their keys over several CTAs each
+    sl.split = ctx->split_user, sl.parts = split_parts(sl.n_tiles, (L + pl->bn - 1) / pl->bn, ctx->split_user.slots);
     AttParams p{};
     p.sl = sl, p.E = reinterpret_cast<const uint8_t *>(ctx->slots[(size_t)slot_index].dev.S), p.M = L, p.mini_batch = 0;
     p.x_stride = c.d, p.X = pl->self_rows;
@@ -749,15 +754,8 @@ cudaError_t launch_self_att_tc(const aif_ctx *ctx, int slot_index, int L, cudaSt
     CUtensorMap tmap_x;
     cudaError_t ex = encode_x_map(&tmap_x, pl->self_rows, c.d, (size_t)c.L_max + kTcTile);
     if (ex != cudaSuccess) return ex;
-    const int grid = sl.n_tiles > 148 ? 148 : sl.n_tiles;
-    cudaError_t e;
-    if (c.d == 128)
-        e = launch_pdl(k_att_tc<128, 128>, dim3(grid), dim3(AttCfg<128, 128>::kThreads), AttCfg<128, 128>::kSmem, st, pl->tmap, tmap_x, p);
-    else
-        e = launch_pdl(k_att_tc<256, 64>, dim3(grid), dim3(AttCfg<256, 64>::kThreads), AttCfg<256, 64>::kSmem, st, pl->tmap, tmap_x, p);
-    count_launch();
     *rows_out = pl->self_rows;
-    return e;
+    return run_att(c.d, p, pl->tmap, tmap_x, st);
 }
 
 }  // namespace aif

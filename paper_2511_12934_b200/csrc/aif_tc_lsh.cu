@@ -30,6 +30,8 @@
 // with P written over the scores, a block's period was the sum of both products, both conversions' latencies and four
 // barrier round trips, divided by two buffers (1470 cycles per 128-key block at d = 128 with next to no conversion work).
 // Every wait is bounded.
+#include <type_traits>
+
 #include "aif_device.cuh"
 #include "aif_internal.h"
 #include "aif_tc_ptx.cuh"
@@ -83,34 +85,6 @@ struct LshCfg {
     static_assert(kSmem <= 227 * 1024, "shared memory");
     static_assert(kQBytes >= 16384, "output staging lives in the signature buffer");
 };
-
-struct LshTile {
-    int slot, cnt, nb, L;
-    int key0;   // first key row: 0, or where the tile's category's sub-sequence begins in the grouped sequence
-    int64_t pos0;
-};
-
-template <int BN>
-__device__ __forceinline__ LshTile lsh_tile(const LshParams &p, int tile)
-{
-    LshTile t;
-    if (p.sl.tiles) {
-        const int4 v = *reinterpret_cast<const int4 *>(p.sl.tiles + tile);
-        t.slot = v.x, t.cnt = v.y;
-        t.pos0 = ((int64_t)(uint32_t)v.w << 32) | (int64_t)(uint32_t)v.z;
-        t.L = p.sl.tiles[tile].L, t.key0 = p.sl.tiles[tile].key0;
-        // an empty sub-sequence still walks one key block (its outputs are forced to zero): the hand-overs stay the same
-        t.nb = t.L > 0 ? (t.L + BN - 1) / BN : 1;
-        return t;
-    }
-    const ReqDev rq = find_request(p.sl, tile);
-    int start, cnt;
-    tile_range(tile - rq.tile_begin, rq.n, kTcTile, p.mini_batch, start, cnt);
-    t.slot = rq.slot, t.cnt = cnt, t.pos0 = rq.off + start;
-    t.L = p.sl.slots[rq.slot].L, t.key0 = 0;
-    t.nb = (t.L + BN - 1) / BN;
-    return t;
-}
 
 __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel)
 {
@@ -191,7 +165,8 @@ __device__ __forceinline__ void lsh_block(uint32_t s_col, uint32_t p_col, float 
     }
 }
 
-template <int D, int BN>
+// SPLIT: the launch's tiles are cut into pieces of their keys.
+template <int D, int BN, bool SPLIT>
 __global__ void __launch_bounds__((LshCfg<D, BN>::kThreads), 1) k_lsh_tc(const __grid_constant__ CUtensorMap tmapS,
                                                                          const __grid_constant__ CUtensorMap tmapG,
                                                                          const __grid_constant__ CUtensorMap tmapX, const LshParams p)
@@ -248,31 +223,45 @@ __global__ void __launch_bounds__((LshCfg<D, BN>::kThreads), 1) k_lsh_tc(const _
     grid_dep_launch();
     grid_dep_wait();
 
-    const int n_tiles = p.sl.n_tiles_dev ? *p.sl.n_tiles_dev : p.sl.n_tiles;
+    const int n_tiles = key_jobs<SPLIT>(p.sl);   // tiles, or pieces of tiles
 
-    // A row's item signature as +-1 bytes in the operand layout (128-byte swizzled K-major chunks): 8 threads per row,
-    // 16 bits (two signature bytes) each per 128-bit chunk.
-    auto expand_row = [&](unsigned char *q, int r, int sub, int id) {
+    // Item signatures of N rows (r0, r0 + step, ...) as +-1 bytes in the operand layout (128-byte swizzled K-major chunks): 8
+    // threads per row, 16 bits (two signature bytes) each per 128-bit chunk.  All of a thread's signature bytes are requested
+    // before the first is expanded: one after the other (the stores in between keep the compiler from moving the loads) the
+    // gather warp's 32 rows took 32 memory latencies, 25 k cycles a tile, which tiles of few key blocks do not hide.
+    auto expand_rows = [&](unsigned char *q, int r0, int step, int sub, auto n_const, auto id_of) {
+        constexpr int N = decltype(n_const)::value;
+        uint16_t two[N][C::kQChunks];
+        uint32_t good = 0u;
 #pragma unroll
-        for (int c = 0; c < C::kQChunks; ++c) {
-            uint4 v = make_uint4(0u, 0u, 0u, 0u);   // rows beyond the tile and ids outside the table: zeros
-            if (id >= 0) {
-                const uint32_t two = *reinterpret_cast<const uint16_t *>(p.sig + (size_t)id * (D / 8) + c * 16 + sub * 2);
-                v = expand_sig16(two & 0xFFu, two >> 8);
+        for (int i = 0; i < N; ++i) {
+            const int id = id_of(i);
+            if (id >= 0) good |= 1u << i;
+#pragma unroll
+            for (int c = 0; c < C::kQChunks; ++c)
+                two[i][c] = __ldg(reinterpret_cast<const uint16_t *>(p.sig + (size_t)max(id, 0) * (D / 8) + c * 16 + sub * 2));
+        }
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            const int r = r0 + step * i;
+#pragma unroll
+            for (int c = 0; c < C::kQChunks; ++c) {
+                // rows beyond the tile and ids outside the table: zeros
+                const uint4 v = (good >> i) & 1u ? expand_sig16(two[i][c] & 0xFFu, two[i][c] >> 8) : make_uint4(0u, 0u, 0u, 0u);
+                *reinterpret_cast<uint4 *>(q + c * 16384 + r * 128 + ((sub ^ (r & 7)) << 4)) = v;
             }
-            *reinterpret_cast<uint4 *>(q + c * 16384 + r * 128 + ((sub ^ (r & 7)) << 4)) = v;
         }
     };
 
     // Scales a finished tile's O accumulator and stores the LSH-DIN rows.  wq = the warp's quarter of the TMEM lanes.
-    auto tile_epilogue = [&](int k, const LshTile &t, int wq, int lane) {
+    auto tile_epilogue = [&](int k, const KeyTile &t, int wq, int lane) {
         const int row = wq * 32 + lane;
         const uint32_t lane_base = tmem_base + ((uint32_t)(wq * 32) << 16);
         const uint32_t o_col = (uint32_t)C::kTmemO;
         uint64_t *o_free_k = o_free;
-        const float scale = (0.5f / (float)D) * (p.din_mean ? 1.0f / (float)t.L : 1.0f);
+        const float scale = (0.5f / (float)D) * (p.din_mean ? 1.0f / (float)t.L_tile : 1.0f);
         bool good = false;
-        if (row < t.cnt && t.L > 0) {   // an empty sub-sequence gives zero rows
+        if (row < t.cnt && t.L_tile > 0) {   // an empty sub-sequence gives zero rows
             const int id = p.sl.ids[t.pos0 + row];
             good = id >= 0 && (int64_t)id < p.M;
         }
@@ -314,20 +303,29 @@ __global__ void __launch_bounds__((LshCfg<D, BN>::kThreads), 1) k_lsh_tc(const _
                         dst[q] = make_uint4(packed[4 * q], packed[4 * q + 1], packed[4 * q + 2], packed[4 * q + 3]);
                 }
             };
-            uint32_t ra[32], rb[32];
-            tmem_ld32(lane_base + o_col, ra);
+            if (SPLIT && t.n_parts != 1) {
+                // a piece of the tile's keys: its sums go to the tile's records, four columns of 32 rows per store, for
+                // k_join_pieces
+                if (t.n_parts > 0)
+                    tmem_rows_out(lane_base + o_col, D, reinterpret_cast<float4 *>(p.sl.split.rows) + (size_t)(t.pslot + t.part) * (D / 4) * 128 + row);
+                tc_fence_before();
+                mbar_arrive(smem_u32(o_free_k));
+            } else {
+                uint32_t ra[32], rb[32];
+                tmem_ld32(lane_base + o_col, ra);
 #pragma unroll 1
-            for (int c0 = 0; c0 < D; c0 += 64) {
-                tmem_ld_wait();
-                tmem_ld32(lane_base + o_col + (uint32_t)(c0 + 32), rb);
-                emit(ra, c0);
-                tmem_ld_wait();
-                if (c0 + 64 < D) tmem_ld32(lane_base + o_col + (uint32_t)(c0 + 64), ra);
-                else {   // O is in registers: the next tile's first product may overwrite the accumulator
-                    tc_fence_before();
-                    mbar_arrive(smem_u32(o_free_k));
+                for (int c0 = 0; c0 < D; c0 += 64) {
+                    tmem_ld_wait();
+                    tmem_ld32(lane_base + o_col + (uint32_t)(c0 + 32), rb);
+                    emit(ra, c0);
+                    tmem_ld_wait();
+                    if (c0 + 64 < D) tmem_ld32(lane_base + o_col + (uint32_t)(c0 + 64), ra);
+                    else {   // O is in registers: the next tile's first product may overwrite the accumulator
+                        tc_fence_before();
+                        mbar_arrive(smem_u32(o_free_k));
+                    }
+                    emit(rb, c0 + 32);
                 }
-                emit(rb, c0 + 32);
             }
         } else {
             tc_fence_before();
@@ -352,23 +350,21 @@ __global__ void __launch_bounds__((LshCfg<D, BN>::kThreads), 1) k_lsh_tc(const _
         int k = 0;
         if ((int)blockIdx.x < n_tiles) {
             // the CTA's first tile has nobody to prefetch it: these warps build its signature operand
-            const LshTile t = lsh_tile<BN>(p, blockIdx.x);
+            const KeyTile t = key_tile<BN, SPLIT>(p.sl, blockIdx.x, p.mini_batch);
             const int sub = tid & 7, r0 = tid >> 3;
+            int idv[8 / kH];
 #pragma unroll
             for (int i = 0; i < 8 / kH; ++i) {
                 const int r = r0 + 16 * kH * i;
-                int id = -1;
-                if (r < t.cnt) {
-                    id = p.sl.ids[t.pos0 + r];
-                    if (id < 0 || (int64_t)id >= p.M) id = -1;
-                }
-                expand_row(smQ, r, sub, id);
+                idv[i] = r < t.cnt ? p.sl.ids[t.pos0 + r] : -1;
+                if ((int64_t)idv[i] >= p.M) idv[i] = -1;
             }
+            expand_rows(smQ, r0, 16 * kH, sub, std::integral_constant<int, 8 / kH>{}, [&](int i) { return idv[i]; });
             fence_proxy_async();   // read by the MMA through the async proxy
             mbar_arrive(smem_u32(q_first));
         }
         for (int tile = blockIdx.x; ok && tile < n_tiles; tile += gridDim.x, ++k) {
-            const LshTile t = lsh_tile<BN>(p, tile);
+            const KeyTile t = key_tile<BN, SPLIT>(p.sl, tile, p.mini_batch);
             const int L = t.L;
             uint32_t *tc = tier_s + (((kH == 2 ? (k & 1) * kH : 0) + half) * kTierSlots) * 128 + row;   // this thread's counters, stride 128
             int n_valid = 0, n_pad = 0;   // keys this thread has counted, and columns beyond the sequence it has converted
@@ -432,11 +428,13 @@ __global__ void __launch_bounds__((LshCfg<D, BN>::kThreads), 1) k_lsh_tc(const _
                     int total = n_valid, pads = n_pad;
                     if (kH == 2) total += (int)(tc1[15 * 128] & 0xFFFFFFu), pads += (int)(tc1[15 * 128] >> 24);
                     bool good = false;
-                    if (row < t.cnt && L > 0) {
+                    if (row < t.cnt && t.L_tile > 0) {
                         const int id = p.sl.ids[t.pos0 + row];
                         good = id >= 0 && (int64_t)id < p.M;
                     }
-                    const float nrm = p.tier_mean ? 1.0f / (float)L : 1.0f;
+                    const float nrm = p.tier_mean ? 1.0f / (float)t.L_tile : 1.0f;
+                    // a piece of the tile's keys leaves its counts with the tile's records
+                    const bool whole = !SPLIT || t.n_parts == 1;
                     uint32_t outw[32];
                     int below = 0;
                     float prev = 0.f;
@@ -448,6 +446,7 @@ __global__ void __launch_bounds__((LshCfg<D, BN>::kThreads), 1) k_lsh_tc(const _
                         if (tt == (p.n_tiers >> 1)) cnt_t -= pads;        // columns beyond the sequence scored 0: matches = d' / 2
                         if (tt == p.n_tiers - 1) cnt_t = total - below;   // the closed last tier takes matches = d' as well
                         below += cnt_t;
+                        if (!whole && t.n_parts > 0) __stcg(p.sl.split.tiers + ((size_t)(t.pslot + t.part) * kTierSlots + tt) * 128 + row, cnt_t);
                         const float v = (good && tt < p.n_tiers) ? (float)cnt_t * nrm : 0.f;
                         if (tt & 1) {
                             const __nv_bfloat162 h = __floats2bfloat162_rn(prev, v);
@@ -457,7 +456,7 @@ __global__ void __launch_bounds__((LshCfg<D, BN>::kThreads), 1) k_lsh_tc(const _
                     }
 #pragma unroll
                     for (int i = 8; i < 32; ++i) outw[i] = 0u;
-                    if (row < t.cnt) {
+                    if (whole && row < t.cnt) {
                         uint4 *dst = reinterpret_cast<uint4 *>(p.X + (size_t)(t.pos0 + row) * p.x_stride + p.x_tier);
 #pragma unroll
                         for (int q = 0; q < 8; ++q) dst[q] = make_uint4(outw[4 * q], outw[4 * q + 1], outw[4 * q + 2], outw[4 * q + 3]);
@@ -485,7 +484,7 @@ __global__ void __launch_bounds__((LshCfg<D, BN>::kThreads), 1) k_lsh_tc(const _
                 uint32_t gb;
                 int nb_next;
             };
-            auto blocks_of = [&](int tile) { return tile < n_tiles ? lsh_tile<BN>(p, tile).nb : 0; };
+            auto blocks_of = [&](int tile) { return tile < n_tiles ? key_tile<BN, SPLIT>(p.sl, tile, p.mini_batch).nb : 0; };
             auto open_tile = [&](Cursor &c) {
                 c.nb = c.nb_next;
                 c.nb_next = blocks_of(c.tile + (int)gridDim.x);
@@ -564,7 +563,7 @@ __global__ void __launch_bounds__((LshCfg<D, BN>::kThreads), 1) k_lsh_tc(const _
             };
             auto open = [&](Stream &c) {
                 if (c.tile < n_tiles) {
-                    const LshTile t = lsh_tile<BN>(p, c.tile);
+                    const KeyTile t = key_tile<BN, SPLIT>(p.sl, c.tile, p.mini_batch);
                     c.nb = t.nb, c.slot = t.slot, c.key0 = t.key0;
                 }
             };
@@ -609,7 +608,7 @@ __global__ void __launch_bounds__((LshCfg<D, BN>::kThreads), 1) k_lsh_tc(const _
         const int wq = warp & 3;
         int k = 0;
         for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, ++k) {
-            const LshTile t = lsh_tile<BN>(p, tile);
+            const KeyTile t = key_tile<BN, SPLIT>(p.sl, tile, p.mini_batch);
             if (!mbar_wait(smem_u32(o_final), (uint32_t)(k & 1), abort_flag)) break;
             tc_fence_after();
             tile_epilogue(k, t, wq, lane);
@@ -622,7 +621,7 @@ __global__ void __launch_bounds__((LshCfg<D, BN>::kThreads), 1) k_lsh_tc(const _
         for (int tile = blockIdx.x + gridDim.x; tile < n_tiles; tile += gridDim.x, ++k) {
             const int qb = k % kQB;
             if (k >= kQB && !mbar_wait(smem_u32(q_empty + qb), (uint32_t)(((k - kQB) / kQB) & 1), abort_flag)) break;
-            const LshTile t = lsh_tile<BN>(p, tile);
+            const KeyTile t = key_tile<BN, SPLIT>(p.sl, tile, p.mini_batch);
             unsigned char *q = smQ + qb * C::kQBytes;
             int idv[4];
 #pragma unroll
@@ -635,12 +634,7 @@ __global__ void __launch_bounds__((LshCfg<D, BN>::kThreads), 1) k_lsh_tc(const _
                 }
                 idv[u] = id;
             }
-#pragma unroll
-            for (int i = 0; i < 32; ++i) {
-                const int r = r0 + 4 * i;
-                const int id = __shfl_sync(0xffffffffu, idv[i >> 3], r0 + 4 * (i & 7));
-                expand_row(q, r, sub, id);
-            }
+            expand_rows(q, r0, 4, sub, std::integral_constant<int, 32>{}, [&](int i) { return __shfl_sync(0xffffffffu, idv[i >> 3], r0 + 4 * (i & 7)); });
             fence_proxy_async();
             mbar_arrive(smem_u32(q_full + qb));
         }
@@ -714,8 +708,16 @@ cudaError_t tc_lsh_prepare(aif_ctx *ctx)
                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return cudaErrorInvalidValue;
     }
-    if (c.d == 128) return cudaFuncSetAttribute(k_lsh_tc<128, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LshCfg<128, 128>::kSmem);
-    return cudaFuncSetAttribute(k_lsh_tc<256, 64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LshCfg<256, 64>::kSmem);
+    auto allow = [](auto kernel, size_t smem) { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); };
+    cudaError_t e;
+    if (c.d == 128) {
+        e = allow(k_lsh_tc<128, 128, false>, LshCfg<128, 128>::kSmem);
+        if (e == cudaSuccess) e = allow(k_lsh_tc<128, 128, true>, LshCfg<128, 128>::kSmem);
+    } else {
+        e = allow(k_lsh_tc<256, 64, false>, LshCfg<256, 64>::kSmem);
+        if (e == cudaSuccess) e = allow(k_lsh_tc<256, 64, true>, LshCfg<256, 64>::kSmem);
+    }
+    return e;
 }
 
 void tc_lsh_destroy(aif_ctx *ctx)
@@ -746,15 +748,21 @@ cudaError_t launch_lsh_tc(const aif_ctx *ctx, const ScoreLaunch &sl, cudaStream_
     p.x_stride = x_stride, p.x_din = x_din, p.x_tier = x_tier, p.X = (__nv_bfloat16 *)X;
     p.n_tiers = (c.blocks & AIF_BLK_SIMTIER) ? c.n_tiers : 1;
     p.din_mean = c.lsh_din_norm == AIF_NORM_MEAN, p.tier_mean = c.simtier_norm == AIF_NORM_MEAN;
-    const int grid = sl.n_tiles > 148 ? 148 : sl.n_tiles;
-    cudaError_t e;
+    const bool split = sl.jobs || sl.parts > 1;
+    const int jobs = sl.jobs ? sl.n_jobs : sl.n_tiles * (split ? sl.parts : 1), grid = jobs > 148 ? 148 : jobs;
     const CUtensorMap &ts = sl.grouped ? pl->tmap_sg : pl->tmap_s, &tg = sl.grouped ? pl->tmap_gg : pl->tmap_g;
-    if (c.d == 128)
-        e = launch_pdl(k_lsh_tc<128, 128>, dim3(grid), dim3(LshCfg<128, 128>::kThreads), LshCfg<128, 128>::kSmem, st, ts, tg, tmap_x, p);
-    else
-        e = launch_pdl(k_lsh_tc<256, 64>, dim3(grid), dim3(LshCfg<256, 64>::kThreads), LshCfg<256, 64>::kSmem, st, ts, tg, tmap_x, p);
+    auto go = [&](auto kernel, int threads, size_t smem) { return launch_pdl(kernel, dim3(grid), dim3(threads), smem, st, ts, tg, tmap_x, p); };
+    using C1 = LshCfg<128, 128>;
+    using C2 = LshCfg<256, 64>;
+    cudaError_t e;
+    if (c.d == 128) e = split ? go(k_lsh_tc<128, 128, true>, C1::kThreads, C1::kSmem) : go(k_lsh_tc<128, 128, false>, C1::kThreads, C1::kSmem);
+    else e = split ? go(k_lsh_tc<256, 64, true>, C2::kThreads, C2::kSmem) : go(k_lsh_tc<256, 64, false>, C2::kThreads, C2::kSmem);
     count_launch();
-    return e;
+    if (e != cudaSuccess || !split) return e;
+    JoinParams j{};
+    j.sl = sl, j.X = (__nv_bfloat16 *)X, j.M = c.M, j.x_stride = x_stride, j.col = x_din, j.x_tier = x_tier, j.n_tiers = p.n_tiers, j.d = c.d;
+    j.mini_batch = c.mini_batch, j.row_scale = 0.5f / (float)c.d, j.row_mean = p.din_mean, j.tier_mean = p.tier_mean;
+    return launch_join_pieces(j, st);
 }
 
 }  // namespace aif

@@ -294,6 +294,22 @@ __device__ __forceinline__ void tmem_ld16x256(uint32_t taddr, uint32_t (&r)[16])
 }
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
+// 32 lanes x n_cols fp32 columns (a multiple of 32) to global memory, column groups of four, 128 rows apart: out[c / 4][row] =
+// columns c .. c + 3 of this lane's row.
+__device__ __forceinline__ void tmem_rows_out(uint32_t taddr, int n_cols, float4 *out)
+{
+#pragma unroll 1
+    for (int c0 = 0; c0 < n_cols; c0 += 32) {
+        uint32_t r[32];
+        tmem_ld32(taddr + (uint32_t)c0, r);
+        tmem_ld_wait();
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+            __stcg(out + (c0 / 4 + q) * 128, make_float4(__uint_as_float(r[4 * q]), __uint_as_float(r[4 * q + 1]), __uint_as_float(r[4 * q + 2]),
+                                                         __uint_as_float(r[4 * q + 3])));
+    }
+}
+
 __device__ __forceinline__ void named_bar_sync(int id, int threads)
 {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");

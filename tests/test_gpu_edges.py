@@ -183,3 +183,66 @@ def test_layer_kernel_with_several_items_per_pair():
         _check(got[r][at], oracle.score(table, helpers.projected_request(wl, rqs[r]), lists[r][at]))
     assert srv.ctx.poll_status() == 0
     srv.close()
+
+
+@pytest.mark.parametrize("base", ["c2", "c5"])
+@pytest.mark.parametrize("blocks", [synth.BLK_ATT | synth.BLK_CROSS, synth.BLK_CROSS | synth.BLK_LSH_DIN | synth.BLK_SIMTIER, helpers.ALL_BLOCKS])
+def test_key_ranges_split_over_ctas(base, blocks):
+    """Few tiles with many keys: every tile's keys in pieces on CTAs of their own, joined by a launch that follows.  Requests of 1
+    to 3000 items in one launch (tiles with fewer key blocks than pieces among them), ragged tiles, bad ids, twice in a row,
+    and each request by itself."""
+    wl = helpers.MINI[base].with_(name=f"split_{base}_{blocks}", R=4, N=130, M=2000, L=3000, F=2, B=64, mini_batch=0, blocks=blocks, n_tiers=9)
+    weights, table = synth.make_weights(wl, zero_bias=False), synth.make_item_table(wl)
+    srv, oracle = serving.Server(wl, weights, table), helpers.make_oracle(wl, weights, M=wl.M)
+    rqs = [synth.make_request(wl, r, L=L) for r, L in enumerate((3000, 1, 129, 1500))]
+    states = [srv.precompute(r, srv.upload_request(rq, B.USER_PROJECTED)) for r, rq in enumerate(rqs)]
+    g = np.random.default_rng(8)
+    lists = [g.choice(wl.M, n, replace=False).astype(np.int32) for n in (130, 5, 128, 1)]
+    lists[0][11] = wl.M
+    want = [oracle.score(table, helpers.projected_request(wl, rq), ids) for rq, ids in zip(rqs, lists)]
+    first = srv.score_many(states, lists)
+    again = srv.score_many(states, lists)
+    for got, rep, w, st, ids in zip(first, again, want, states, lists):
+        _check(got, w)
+        assert np.array_equal(got, rep, equal_nan=True)
+        _check(srv.score_ids(st, ids), w)
+    assert srv.ctx.poll_status() == B.STATUS_BAD_ID
+    srv.close()
+
+
+@pytest.mark.parametrize("s_scale", [1.0, 1024.0])
+def test_split_pieces_with_and_without_a_running_maximum(s_scale):
+    """Sequence rows so large that every piece keeps a maximum of its own: the pieces are joined at different exponent offsets.
+    Inputs 1024 times off the workload's distribution leave attention rows of that magnitude, rounded to bf16 (2^-9 relative):
+    1e-2 of the largest logit, as for the unsplit kernel."""
+    wl = helpers.MINI["c2"].with_(name="split_sharp", R=1, N=200, M=2000, L=2500, F=2, B=64, mini_batch=0)
+    weights, table = synth.make_weights(wl, zero_bias=False), synth.make_item_table(wl)
+    rq = synth.make_request(wl, 0)
+    rq["S"] = synth.store(synth.as_f32(rq["S"], wl.dtype) * np.float32(s_scale), wl.dtype)
+    srv, oracle = serving.Server(wl, weights, table), helpers.make_oracle(wl, weights, M=wl.M)
+    st = srv.precompute(0, srv.upload_request(rq, B.USER_PROJECTED))
+    ids = np.random.default_rng(3).choice(wl.M, 200, replace=False).astype(np.int32)
+    want = oracle.score(table, helpers.projected_request(wl, rq), ids)
+    _check(srv.score_ids(st, ids), want, TOL if s_scale == 1.0 else 1e-2 * max(1.0, np.abs(want).max()))
+    assert srv.ctx.poll_status() == 0
+    srv.close()
+
+
+@pytest.mark.parametrize("n_cat", [3, 1500])
+def test_category_jobs_over_one_and_several_batches_of_groups(n_cat):
+    """Sub-sequences cut into pieces, among them long, short and empty ones: few categories (every tile split) and more groups than
+    the placing block has threads (two requests x 1500 categories)."""
+    wl = helpers.MINI["c2"].with_(name=f"sim_jobs_{n_cat}", R=2, N=600, M=4000, L=6000, F=2, B=64, mini_batch=0, n_categories=n_cat,
+                                  blocks=synth.BLK_ATT | synth.BLK_CROSS | synth.BLK_LSH_DIN | synth.BLK_SIMTIER)
+    weights, table = synth.make_weights(wl, zero_bias=False), synth.make_item_table(wl)
+    srv, oracle = serving.Server(wl, weights, table), helpers.make_oracle(wl, weights, M=wl.M)
+    rqs = [synth.make_request(wl, r) for r in range(2)]
+    states = [srv.precompute(r, srv.upload_request(rq, B.USER_PROJECTED)) for r, rq in enumerate(rqs)]
+    g = np.random.default_rng(2)
+    lists = [g.choice(wl.M, n, replace=False).astype(np.int32) for n in (600, 333)]
+    want = [oracle.score(table, helpers.projected_request(wl, rq), ids) for rq, ids in zip(rqs, lists)]
+    for got, w in zip(srv.score_many(states, lists), want):
+        _check(got, w)
+    _check(srv.score_ids(states[1], lists[1]), want[1])
+    assert srv.ctx.poll_status() == 0
+    srv.close()
