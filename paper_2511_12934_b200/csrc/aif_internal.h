@@ -14,7 +14,6 @@ namespace aif {
 
 constexpr int kMaxHidden = 4;
 constexpr int kSimtTile = 8;        // candidates per block in the CUDA-core scoring kernel
-constexpr int kSimtThreads = 256;
 constexpr int kTcTile = 128;        // candidates per tile in the tensor-core kernels (UMMA M)
 
 // One user-state slot as the kernels see it.  Pointers are fixed when the arena is laid out; only L changes.

@@ -1,5 +1,7 @@
 // CUDA-core kernels of libaif: table refresh / gather and the general scoring kernel (any storage type, all
 // interaction blocks, fp32 arithmetic).  The user-side network lives in aif_user.cu, the tensor-core kernels in aif_tc*.cu.
+#include <type_traits>
+
 #include "aif_internal.h"
 #include "aif_device.cuh"
 #include "aif_tc_ptx.cuh"
@@ -335,205 +337,515 @@ cudaError_t launch_transpose(const void *in, void *out, int rows, int cols, size
 int simt_tiles_for(const aif_ctx *ctx, int n) { return tiles_of(n, kSimtTile, ctx->cfg.mini_batch); }
 
 // ------------------------------------------------------------------------------------------------
-// general scoring kernel: one block = one tile of kSimtTile candidates, one warp per candidate for the
-// interaction blocks, then all threads for the MLP with the decomposed first layer.
+// General scoring kernel (fp32, and bf16 shapes the tensor-core kernels do not take): one block = one tile of kSimtTile
+// candidates, a warp per candidate for the interaction blocks, then all of them for the MLP with the decomposed first layer.
+// A request of 1000 candidates is 125 blocks, so what counts is the length of one block's dependent chain.  A block has
+// 8 x (k1 H1 + H1 H2 + ..) multiply-adds to issue (6.1 k cycles for 256 -> 256 -> 128) and as many weight bytes to take in
+// (393 KB at 59 bytes per clock: 6.7 k); everything else is kept short of that:
+//   * key rows go through shared memory, 32 at a time, once per block; a lane scores one key from padded rows (conflict-free
+//     16-byte reads).  Read from global memory by every warp, a whole row per lane and then once more key by key, 50 keys cost
+//     more than the MLP.
+//   * the weights come through a ring of 32 KB stages (bulk copies, requested by a warp of their own) from the kernel's first
+//     moment on, across the layers; loaded by the threads that multiply, at most 32 KB were in flight and a layer waited for
+//     every batch.
+//   * shared memory returns 128 bytes per clock, broadcasts at full width: a lane's tile is 8 outputs x 8 candidates, 64 bytes per
+//     64 multiply-adds and row (one output x 8 candidates, 36 bytes per 8: four times the multiply-adds' own time).  A warp takes
+//     64 outputs, its lanes every fourth row of a stage, the next row's reads under this one's products; the four partial sums
+//     meet in 48 shuffles, those of the warps that share 64 outputs in shared memory.
+// Measured, 1000 candidates, 50 keys, d 64, fp32, from the call to the logits: 29.3 -> 16.8 us (the weight ring alone 22.9; 16 warps,
+// two per candidate, at half the registers: 21.4, bound by instructions that were not products).  Now 17 of 31 k cycles are the
+// MLP (10 in the products), 6 the attention, 5 the ids and rows.
 // ------------------------------------------------------------------------------------------------
+template <int DQ>
+__device__ __forceinline__ float dot_shared(const float *row, const float *q)
+{
+    float acc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int k = 0; k < 32 * DQ; k += 4) {
+        const float4 r = *reinterpret_cast<const float4 *>(row + k), w = *reinterpret_cast<const float4 *>(q + k);
+        acc[0] = fmaf(r.x, w.x, acc[0]), acc[1] = fmaf(r.y, w.y, acc[1]), acc[2] = fmaf(r.z, w.z, acc[2]), acc[3] = fmaf(r.w, w.w, acc[3]);
+    }
+    return (acc[0] + acc[1]) + (acc[2] + acc[3]);
+}
+template <int DQ>
+__device__ __forceinline__ float dot_shared(const __nv_bfloat16 *row, const float *q)
+{
+    float acc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int k = 0; k < 32 * DQ; k += 8) {
+        const uint4 r = *reinterpret_cast<const uint4 *>(row + k);
+        const float4 a = *reinterpret_cast<const float4 *>(q + k), b = *reinterpret_cast<const float4 *>(q + k + 4);
+        const __nv_bfloat162 *h = reinterpret_cast<const __nv_bfloat162 *>(&r);
+        const float2 f0 = __bfloat1622float2(h[0]), f1 = __bfloat1622float2(h[1]), f2 = __bfloat1622float2(h[2]), f3 = __bfloat1622float2(h[3]);
+        acc[0] = fmaf(f0.x, a.x, acc[0]), acc[1] = fmaf(f0.y, a.y, acc[1]), acc[2] = fmaf(f1.x, a.z, acc[2]), acc[3] = fmaf(f1.y, a.w, acc[3]);
+        acc[0] = fmaf(f2.x, b.x, acc[0]), acc[1] = fmaf(f2.y, b.y, acc[1]), acc[2] = fmaf(f3.x, b.z, acc[2]), acc[3] = fmaf(f3.y, b.w, acc[3]);
+    }
+    return (acc[0] + acc[1]) + (acc[2] + acc[3]);
+}
+__device__ __forceinline__ float4 load4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
+__device__ __forceinline__ float4 load4(const __nv_bfloat16 *p)
+{
+    const uint2 v = *reinterpret_cast<const uint2 *>(p);
+    const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&v.x)), b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&v.y));
+    return make_float4(a.x, a.y, b.x, b.y);
+}
+
+constexpr int kSimtKeys = 32;            // keys of a chunk
+constexpr int kSimtWarps = kSimtTile, kSimtThreads = 32 * kSimtWarps;   // a warp per candidate; one warp more requests the weights
+constexpr int kSimtMaxStages = 4, kSimtStageBytes = 32768;
+constexpr int kSimtRed = kSimtWarps * 64 * kSimtTile;   // floats: partial sums of the warps
+
+// Shared memory of the kernel, in floats; the key chunks lie where the activations come later.
+struct SimtLayout {
+    int32_t max_h;
+    int32_t region;      // of activations / key chunks
+    int32_t key_bufs;    // chunk buffers, 2 or 1; 0: no room, keys are read from global memory
+    int32_t stages;      // of the weight ring; 0: no room, weights are read from global memory
+    int32_t red, ps;     // partial sums, kSimtRed or 0 (one warp per 64 outputs then); probabilities and similarities of the key chunks
+};
+
+// Outputs of a layer go in blocks of up to 256 columns, the weights of a block in stages of `rows` rows.
+struct SimtBlock {
+    int cols, rows;
+};
 template <typename T>
-__global__ void __launch_bounds__(kSimtThreads) k_score_simt(ModelDev md, ScoreLaunch sl, int max_h)
+__device__ __forceinline__ SimtBlock simt_block(int H, int c0)
+{
+    SimtBlock b;
+    b.cols = min(256, H - c0);
+    b.rows = min(128, kSimtStageBytes / (b.cols * (int)sizeof(T)));
+    return b;
+}
+
+// The weights of all layers, stage by stage, by one thread.
+template <typename T>
+__device__ __forceinline__ bool simt_weights(const ModelDev &md, unsigned char *ring, uint64_t *full, uint64_t *empty, int stages, volatile uint32_t *abort_flag)
+{
+    int s = 0, filled = 0;
+    uint32_t ph = 1;
+    for (int layer = 0; layer < md.n_hidden; ++layer) {
+        const int H = md.hidden[layer], in_w = layer ? md.hidden[layer - 1] : md.k1;
+        const T *W0 = reinterpret_cast<const T *>(md.Wt[layer]) + (layer == 0 ? (size_t)md.d * H : 0);
+        for (int c0 = 0; c0 < H; c0 += 256) {
+            const SimtBlock b = simt_block<T>(H, c0);
+            for (int k0 = 0; k0 < in_w; k0 += b.rows) {
+                const int rows = min(b.rows, in_w - k0);
+                const T *W = W0 + (size_t)k0 * H + c0;
+                const uint32_t dst = smem_u32(ring + s * kSimtStageBytes), bar = smem_u32(full + s), bytes = (uint32_t)(b.cols * sizeof(T));
+                if (filled >= stages && !mbar_wait(smem_u32(empty + s), ph, abort_flag)) return false;
+                mbar_expect_tx(bar, rows * bytes);
+                if (b.cols == H) bulk_load(dst, W, rows * bytes, bar);
+                else
+                    for (int r = 0; r < rows; ++r) bulk_load(dst + r * bytes, W + (size_t)r * H, bytes, bar);
+                ++filled;
+                if (++s == stages) s = 0, ph ^= 1u;
+            }
+        }
+    }
+    return true;
+}
+
+// The sequence blocks of one candidate by one warp (all warps in step: the chunks of keys are shared).
+template <typename T, int DQ, typename Fetch>
+__device__ __forceinline__ void simt_keys(const ModelDev &md, const uint8_t *sigS, int L, bool live, const float *q, const uint32_t *sigq,
+                                          int *tiers, float *pp, float *pm, const unsigned char *keys, int n_bufs, float *xs_att,
+                                          float *xs_din, Fetch fetch)
+{
+    constexpr int D = 32 * DQ, stride = D * (int)sizeof(T) + 16, TM = kSimtTile;
+    const int lane = threadIdx.x & 31, n_chunks = (L + kSimtKeys - 1) / kSimtKeys, words = md.lsh_bits >> 5;
+    const bool do_att = md.blocks & AIF_BLK_ATT, do_din = md.blocks & AIF_BLK_LSH_DIN, do_tier = md.blocks & AIF_BLK_SIMTIER;
+    const float scale = rsqrtf((float)D), inv_bits = 1.0f / (float)md.lsh_bits;
+    float att[DQ], din[DQ], m = -INFINITY, l = 0.f;
+#pragma unroll
+    for (int c = 0; c < DQ; ++c) att[c] = din[c] = 0.f;
+    for (int ch = 0; ch < n_chunks; ++ch) {
+        if (n_bufs == 2 && ch + 1 < n_chunks) cp_async_wait<1>();
+        else cp_async_wait<0>();
+        named_bar_sync(1, kSimtThreads);
+        const unsigned char *buf = keys + (ch % n_bufs) * kSimtKeys * stride;
+        if (live) {
+            const int j = ch * kSimtKeys + lane;
+            const bool valid = j < L;
+            if (do_din || do_tier) {
+                float simv = 0.f;
+                if (valid) {
+                    const uint32_t *sj = reinterpret_cast<const uint32_t *>(sigS + (size_t)j * (md.lsh_bits >> 3));
+                    int diff = 0;
+                    for (int w = 0; w < words; ++w) diff += __popc(sigq[w] ^ __ldg(sj + w));
+                    const int matches = md.lsh_bits - diff;
+                    simv = (float)matches * inv_bits;
+                    if (do_tier) {
+                        const int t = (matches * md.n_tiers) / md.lsh_bits;
+                        atomicAdd(&tiers[t < md.n_tiers - 1 ? t : md.n_tiers - 1], 1);
+                    }
+                }
+                pm[lane] = simv;
+            }
+            if (do_att) {
+                const float s = valid ? dot_shared<DQ>(reinterpret_cast<const T *>(buf + lane * stride), q) * scale : -INFINITY;
+                const float m_new = fmaxf(m, warp_max(s)), sc = expf(m - m_new), p = valid ? expf(s - m_new) : 0.f;
+                pp[lane] = p;
+                l = l * sc + warp_sum(p);
+                m = m_new;
+#pragma unroll
+                for (int c = 0; c < DQ; ++c) att[c] *= sc;
+            }
+            __syncwarp();
+            const int n = min(kSimtKeys, L - ch * kSimtKeys);   // up to three keys more: weight 0 times rows of zeros
+            auto weigh = [&](const float *w, float (&acc)[DQ]) {
+#pragma unroll 2
+                for (int j0 = 0; j0 < n; j0 += 4) {
+                    const float4 p4 = *reinterpret_cast<const float4 *>(w + j0);
+                    const float pj[4] = {p4.x, p4.y, p4.z, p4.w};
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const T *row = reinterpret_cast<const T *>(buf + (j0 + u) * stride) + lane;
+#pragma unroll
+                        for (int c = 0; c < DQ; ++c) acc[c] = fmaf(pj[u], to_f(row[32 * c]), acc[c]);
+                    }
+                }
+            };
+            if (do_att) weigh(pp, att);
+            if (do_din) weigh(pm, din);
+        }
+        if (ch + n_bufs < n_chunks) {
+            named_bar_sync(1, kSimtThreads);
+            fetch(ch + n_bufs);
+        }
+    }
+    if (!live) return;
+    const float inv = 1.0f / l, nrm = md.lsh_din_norm == AIF_NORM_MEAN ? 1.0f / (float)L : 1.0f;
+#pragma unroll
+    for (int c = 0; c < DQ; ++c) {
+        if (do_att) xs_att[(lane + 32 * c) * TM] = att[c] * inv;
+        if (do_din) xs_din[(lane + 32 * c) * TM] = din[c] * nrm;
+    }
+}
+
+// RING: weights through the ring; else (inputs so wide that there is no room for it) straight from global memory.
+template <typename T, bool RING>
+__global__ void __launch_bounds__(kSimtThreads + 32, 1) k_score_simt(const __grid_constant__ ModelDev md, const __grid_constant__ ScoreLaunch sl, const SimtLayout lay)
 {
     constexpr int TM = kSimtTile;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    float *xs = reinterpret_cast<float *>(smem_raw);        // [k1][TM]   candidate-dependent input, transposed
+    unsigned char *ring = smem_raw;
+    float *xs = reinterpret_cast<float *>(smem_raw + (RING ? lay.stages * kSimtStageBytes : 0));   // [k1][TM] candidate-dependent input, transposed
     float *ha = xs + (size_t)md.k1 * TM;                     // [max_h][TM]
-    float *hb = ha + (size_t)max_h * TM;                     // [max_h][TM]
-    float *qv = hb + (size_t)max_h * TM;                     // [TM][d]    item vectors as fp32 rows (queries)
-    uint32_t *sigq = reinterpret_cast<uint32_t *>(qv + (size_t)TM * md.d);   // [TM][8]
+    float *hb = ha + (size_t)lay.max_h * TM;                 // [max_h][TM]
+    unsigned char *keys = reinterpret_cast<unsigned char *>(ha);   // [key_bufs][kSimtKeys] rows of d elements and 16 bytes
+    float *red = ha + lay.region;                            // [kSimtRed] partial sums of the layers
+    float *qv = red + lay.red;                               // [TM][d]    item vectors as fp32 rows (queries)
+    float *ps = qv + (size_t)TM * md.d;                      // [2][warp][kSimtKeys] probabilities, similarities
+    uint32_t *sigq = reinterpret_cast<uint32_t *>(ps + lay.ps);   // [TM][8]
     int *tiers = reinterpret_cast<int *>(sigq + TM * 8);     // [TM][16]
-    int *bkt = tiers + TM * 16;                              // [TM][F]
-    int *id_s = bkt + TM * md.F;                             // [TM]
+    uint64_t *full = reinterpret_cast<uint64_t *>(tiers + TM * 16);
+    uint64_t *empty = full + kSimtMaxStages;
+    volatile uint32_t *abort_flag = reinterpret_cast<volatile uint32_t *>(empty + kSimtMaxStages);
 
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x, lane = tid & 31, c = tid >> 5;   // candidate of this warp
+    const int d = md.d;
+    if (tid == kSimtThreads) {
+        for (int s = 0; s < kSimtMaxStages; ++s) mbar_init(smem_u32(full + s), 1), mbar_init(smem_u32(empty + s), kSimtWarps);
+        *abort_flag = 0u;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    grid_dep_launch();
+    for (int i = tid; i < md.k1 * TM; i += kSimtThreads + 32) xs[i] = 0.f;
+    for (int i = tid; i < TM * 16; i += kSimtThreads + 32) tiers[i] = 0;
+    __syncthreads();   // xs is zero, the barriers exist
+    if (tid >= kSimtThreads) {
+        // the weights are older than any launch this one may overlap: no wait for the previous kernel
+        if (RING && lane == 0 && !simt_weights<T>(md, ring, full, empty, lay.stages, abort_flag)) *abort_flag = 1u;
+        return;
+    }
+    grid_dep_wait();
     const ReqDev rq = find_request(sl, blockIdx.x);
     int start, cnt;
     tile_range(blockIdx.x - rq.tile_begin, rq.n, TM, md.mini_batch, start, cnt);
-    const SlotDev slot = sl.slots[rq.slot];
-    const int32_t *ids = sl.ids + rq.off + start;
-    float *logits = sl.logits + rq.off + start;
-    const int d = md.d, dq = d >> 5;
-
-    if (tid < TM) {
-        int id = -1;
-        if (tid < cnt) {
-            id = ids[tid];
-            if (id < 0 || (int64_t)id >= md.M) {
-                id = -1;
-                atomicOr(sl.status, AIF_STATUS_BAD_ID);
-            }
+    const SlotDev &slot = sl.slots[rq.slot];
+    const int L = slot.L;
+    const T *S = reinterpret_cast<const T *>(slot.S);
+    int id = c < cnt ? sl.ids[rq.off + start + c] : -1;
+    const float b_out = md.b_out[0];
+    const bool do_att = md.blocks & AIF_BLK_ATT, do_din = md.blocks & AIF_BLK_LSH_DIN, do_tier = md.blocks & AIF_BLK_SIMTIER;
+    const bool do_lsh = do_din || do_tier, chunked = lay.key_bufs && (do_att || do_lsh);
+    const int row_bytes = d * (int)sizeof(T), stride = row_bytes + 16, vpr = row_bytes >> 4;
+    auto fetch = [&](int ch) {   // keys beyond the sequence as zeros
+        const uint32_t buf = smem_u32(keys + (ch % lay.key_bufs) * kSimtKeys * stride);
+        for (int i = tid; i < kSimtKeys * vpr; i += kSimtThreads) {
+            const int r = i / vpr, v = i - r * vpr, j = ch * kSimtKeys + r;
+            cp_async16(buf + r * stride + v * 16, reinterpret_cast<const unsigned char *>(S) + (size_t)(j < L ? j : 0) * row_bytes + v * 16, j < L ? 16u : 0u);
         }
-        id_s[tid] = id;
+        cp_async_commit();
+    };
+    if (chunked) {
+        fetch(0);
+        if (lay.key_bufs == 2 && L > kSimtKeys) fetch(1);
     }
-    for (int i = tid; i < md.k1 * TM; i += kSimtThreads) xs[i] = 0.f;
-    for (int i = tid; i < TM * 16; i += kSimtThreads) tiers[i] = 0;
-    __syncthreads();
+    if (id < 0 || (int64_t)id >= md.M) {
+        id = -1;
+        if (c < cnt && lane == 0) atomicOr(sl.status, AIF_STATUS_BAD_ID);
+    }
 
-    // ---- stage A: interaction blocks, warp c <-> candidate c
+    // ---- stage A: interaction blocks (a bad id keeps its zero columns but takes part in the barriers)
     {
-        const int c = warp;
-        const int id = id_s[c];
+        const int col_cross = d + (do_att ? d : 0), col_bea = col_cross + ((md.blocks & AIF_BLK_CROSS) ? md.F * md.dc : 0);
+        const int col_din = col_bea + ((md.blocks & AIF_BLK_BEA) ? d : 0), col_tier = col_din + (do_din ? d : 0);
         if (id >= 0) {
             const T *e = reinterpret_cast<const T *>(md.E) + (size_t)id * d;
-            int col = 0;
-            for (int k = lane; k < d; k += 32) {
-                const float v = to_f(e[k]);
-                qv[c * d + k] = v;
-                xs[(col + k) * TM + c] = v;
+            for (int k0 = lane; k0 < d; k0 += 128) {
+                float v[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) v[u] = k0 + 32 * u < d ? to_f(e[k0 + 32 * u]) : 0.f;
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (k0 + 32 * u < d) qv[c * d + k0 + 32 * u] = v[u], xs[(k0 + 32 * u) * TM + c] = v[u];
             }
-            col += d;
-            const bool do_att = md.blocks & AIF_BLK_ATT, do_din = md.blocks & AIF_BLK_LSH_DIN,
-                       do_tier = md.blocks & AIF_BLK_SIMTIER, do_lsh = do_din || do_tier;
             if (do_lsh && lane < (md.lsh_bits >> 5))
                 sigq[c * 8 + lane] = reinterpret_cast<const uint32_t *>(md.sig + (size_t)id * (md.lsh_bits >> 3))[lane];
-            if (md.blocks & AIF_BLK_CROSS)
-                for (int f = lane; f < md.F; f += 32) bkt[c * md.F + f] = bucket_of(id, f, md.B, md.bucket_mode);
-            __syncwarp();
-            float att[8], din[8];
-            if (do_att || do_lsh)
-                warp_interact<T>(qv + c * d, reinterpret_cast<const T *>(slot.S), slot.L, d, rsqrtf((float)d), do_att,
-                                 do_lsh, do_tier, sigq + c * 8, slot.sigS, md.lsh_bits, md.n_tiers, tiers + c * 16, att,
-                                 din);
-            if (do_att) {
-#pragma unroll
-                for (int q = 0; q < 8; ++q)
-                    if (q < dq) xs[(col + lane + 32 * q) * TM + c] = att[q];
-                col += d;
-            }
-            if (md.blocks & AIF_BLK_CROSS) {
-                const T *Tt = reinterpret_cast<const T *>(slot.T);
-                const int fdc = md.F * md.dc;
-                for (int i = lane; i < fdc; i += 32) {
-                    const int f = i / md.dc, k = i - f * md.dc;
-                    xs[(col + i) * TM + c] = to_f(Tt[((size_t)f * md.B + bkt[c * md.F + f]) * md.dc + k]);
-                }
-                col += fdc;
-            }
             if (md.blocks & AIF_BLK_BEA) {
                 const T *wh = reinterpret_cast<const T *>(md.bea_w) + (size_t)id * md.n_bridge;
                 const T *V = reinterpret_cast<const T *>(slot.V);
                 for (int k = lane; k < d; k += 32) {
                     float acc = 0.f;
                     for (int b = 0; b < md.n_bridge; ++b) acc = fmaf(to_f(wh[b]), to_f(V[(size_t)b * d + k]), acc);
-                    xs[(col + k) * TM + c] = acc;
+                    xs[(col_bea + k) * TM + c] = acc;
                 }
-                col += d;
             }
-            if (do_din) {
-                const float nrm = md.lsh_din_norm == AIF_NORM_MEAN ? 1.0f / (float)slot.L : 1.0f;
+            if (md.blocks & AIF_BLK_CROSS) {
+                const T *Tt = reinterpret_cast<const T *>(slot.T);
+                const int fdc = md.F * md.dc;
+                auto cell = [&](int i) {
+                    const int f = i / md.dc;
+                    return Tt + ((size_t)f * md.B + bucket_of(id, f, md.B, md.bucket_mode)) * md.dc + (i - f * md.dc);
+                };
+                if (sizeof(T) == 4) {   // element by element straight to its place; the first layer waits for them
+                    for (int i = lane; i < fdc; i += 32) cp_async4(smem_u32(xs + (col_cross + i) * TM + c), cell(i));
+                } else
+                    for (int i0 = lane; i0 < fdc; i0 += 128) {   // four independent reads per round
+                        float v[4];
 #pragma unroll
-                for (int q = 0; q < 8; ++q)
-                    if (q < dq) xs[(col + lane + 32 * q) * TM + c] = din[q] * nrm;
-                col += d;
+                        for (int u = 0; u < 4; ++u) v[u] = to_f(*cell(min(i0 + 32 * u, fdc - 1)));
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+                            if (i0 + 32 * u < fdc) xs[(col_cross + i0 + 32 * u) * TM + c] = v[u];
+                    }
             }
-            if (do_tier) {
-                __syncwarp();
-                const float nrm = md.simtier_norm == AIF_NORM_MEAN ? 1.0f / (float)slot.L : 1.0f;
-                if (lane < md.n_tiers) xs[(col + lane) * TM + c] = (float)tiers[c * 16 + lane] * nrm;
+        }
+        cp_async_commit();
+        float *x_att = xs + d * TM + c, *x_din = xs + col_din * TM + c;
+        if (chunked) {
+            auto run = [&](auto dq) {
+                simt_keys<T, decltype(dq)::value>(md, slot.sigS, L, id >= 0, qv + c * d, sigq + c * 8, tiers + c * 16, ps + c * kSimtKeys,
+                                                  ps + (kSimtWarps + c) * kSimtKeys, keys, lay.key_bufs, x_att, x_din, fetch);
+            };
+            switch (d >> 5) {
+                case 1: run(std::integral_constant<int, 1>{}); break;
+                case 2: run(std::integral_constant<int, 2>{}); break;
+                case 3: run(std::integral_constant<int, 3>{}); break;
+                case 4: run(std::integral_constant<int, 4>{}); break;
+                case 5: run(std::integral_constant<int, 5>{}); break;
+                case 6: run(std::integral_constant<int, 6>{}); break;
+                case 7: run(std::integral_constant<int, 7>{}); break;
+                default: run(std::integral_constant<int, 8>{}); break;
             }
+        } else if (id >= 0 && (do_att || do_lsh)) {
+            __syncwarp();
+            float att[8], din[8];
+            warp_interact<T>(qv + c * d, S, L, d, rsqrtf((float)d), do_att, do_lsh, do_tier, sigq + c * 8, slot.sigS, md.lsh_bits, md.n_tiers,
+                             tiers + c * 16, att, din);
+            const float nrm = md.lsh_din_norm == AIF_NORM_MEAN ? 1.0f / (float)L : 1.0f;
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+                if (q < (d >> 5)) {
+                    if (do_att) x_att[(lane + 32 * q) * TM] = att[q];
+                    if (do_din) x_din[(lane + 32 * q) * TM] = din[q] * nrm;
+                }
+        }
+        if (do_tier && id >= 0) {
+            __syncwarp();
+            const float nrm = md.simtier_norm == AIF_NORM_MEAN ? 1.0f / (float)L : 1.0f;
+            if (lane < md.n_tiers) xs[(col_tier + lane) * TM + c] = (float)tiers[c * 16 + lane] * nrm;
         }
     }
-    __syncthreads();
 
     // ---- stage B: MLP.  First layer = cached user partial + candidate-dependent columns.
+    cp_async_wait_all();
     const float *in_act = xs;
     float *out_act = ha;
-    int in_w = md.k1;
+    int in_w = md.k1, s = 0;
+    uint32_t ph = 0;
+    bool ok = true, next = false;   // next: the stage after this one has been seen to be there
+    const int ql = lane & 7, kp = lane >> 3;   // outputs 4 ql .. + 3 and 32 + 4 ql .. + 3 of the warp's 64; rows kp, kp + 4, ... of a stage
     for (int layer = 0; layer < md.n_hidden; ++layer) {
         const int H = md.hidden[layer];
-        const T *W = reinterpret_cast<const T *>(md.Wt[layer]) + (layer == 0 ? (size_t)d * H : 0);
         const float *bias = layer == 0 ? slot.p_u : md.b[layer];
-        for (int j = tid; j < H; j += kSimtThreads) {
-            float acc[TM];
-            const float b0 = bias[j];
+        named_bar_sync(1, kSimtThreads);   // the layer's inputs are written
+        for (int c0 = 0; c0 < H; c0 += 256) {
+            const SimtBlock b = simt_block<T>(H, c0);
+            const int groups = (b.cols + 63) >> 6, splits = lay.red ? kSimtWarps / groups : 1;   // groups of 64 outputs; warps per group
+            const int grp = c % groups, part = c / groups;
+            const bool busy = part < splits;
+            uint64_t acc2[8][TM / 2];   // two candidates per register pair: half the instructions (f32x2)
 #pragma unroll
-            for (int c = 0; c < TM; ++c) acc[c] = b0;
-            // weights in batches of 32 independent loads (the accumulation order over k stays sequential): after an L2
-            // flush every weight comes from HBM, and one load per iteration would expose that latency 32 times as often
-            auto step = [&](int k, float w) {
-                const float4 a = *reinterpret_cast<const float4 *>(in_act + k * TM);
-                const float4 b = *reinterpret_cast<const float4 *>(in_act + k * TM + 4);
-                acc[0] = fmaf(w, a.x, acc[0]);
-                acc[1] = fmaf(w, a.y, acc[1]);
-                acc[2] = fmaf(w, a.z, acc[2]);
-                acc[3] = fmaf(w, a.w, acc[3]);
-                acc[4] = fmaf(w, b.x, acc[4]);
-                acc[5] = fmaf(w, b.y, acc[5]);
-                acc[6] = fmaf(w, b.z, acc[6]);
-                acc[7] = fmaf(w, b.w, acc[7]);
-            };
-            int k = 0;
-            for (; k + 32 <= in_w; k += 32) {
-                float w[32];
+            for (int o = 0; o < 8; ++o)
 #pragma unroll
-                for (int u = 0; u < 32; ++u) w[u] = to_f(W[(size_t)(k + u) * H + j]);
+                for (int cc = 0; cc < TM / 2; ++cc) acc2[o][cc] = 0ull;
+            // (lanes beyond the block's last column read its last outputs again)
+            const int col_a = min(64 * grp + 4 * ql, b.cols - 4), col_b = min(64 * grp + 32 + 4 * ql, b.cols - 4);
+            for (int k0 = 0; k0 < in_w; k0 += b.rows) {
+                const int rows = min(b.rows, in_w - k0);
+                if (RING) ok = __all_sync(0xffffffffu, ok && (next || mbar_wait(smem_u32(full + s), ph, abort_flag)));
+                if (RING) next = mbar_test(smem_u32(full + (s + 1 == lay.stages ? 0 : s + 1)), s + 1 == lay.stages ? ph ^ 1u : ph);
+                const T *w0 = RING ? reinterpret_cast<const T *>(ring + s * kSimtStageBytes)
+                                   : reinterpret_cast<const T *>(md.Wt[layer]) + (layer == 0 ? (size_t)d * H : 0) + (size_t)k0 * H + c0;
+                const int ws = RING ? b.cols : H;
+                if (ok && busy) {
+                    const float *x0 = in_act + k0 * TM;
+                    // two rows in registers: the reads of one travel while the other is multiplied
+                    struct Row {
+                        float4 wa, wb;
+                        ulonglong2 xa, xb;
+                    } a, bb;
+                    const int step = 4 * splits, last = rows - 1;   // reads beyond the stage repeat its last row and are not multiplied
+                    auto read = [&](Row &q, int rr) {
+                        q.wa = load4(w0 + (size_t)rr * ws + col_a), q.wb = load4(w0 + (size_t)rr * ws + col_b);
+                        q.xa = *reinterpret_cast<const ulonglong2 *>(x0 + rr * TM), q.xb = *reinterpret_cast<const ulonglong2 *>(x0 + rr * TM + 4);
+                    };
+                    auto multiply = [&](const Row &q) {
+                        const uint64_t x[4] = {q.xa.x, q.xa.y, q.xb.x, q.xb.y};
+                        const float w[8] = {q.wa.x, q.wa.y, q.wa.z, q.wa.w, q.wb.x, q.wb.y, q.wb.z, q.wb.w};
 #pragma unroll
-                for (int u = 0; u < 32; ++u) step(k + u, w[u]);
+                        for (int o = 0; o < 8; ++o)
+#pragma unroll
+                            for (int cc = 0; cc < TM / 2; ++cc) acc2[o][cc] = fma_f32x2(pack_f32x2(w[o], w[o]), x[cc], acc2[o][cc]);
+                    };
+                    int r = kp + 4 * part;
+                    read(a, min(r, last));
+#pragma unroll 1
+                    for (; r + step < rows; r += 2 * step) {
+                        read(bb, r + step);
+                        multiply(a);
+                        read(a, min(r + 2 * step, last));
+                        multiply(bb);
+                    }
+                    if (r < rows) multiply(a);
+                }
+                if (RING) {
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(smem_u32(empty + s));
+                    if (++s == lay.stages) s = 0, ph ^= 1u;
+                }
             }
-            for (; k < in_w; ++k) step(k, to_f(W[(size_t)k * H + j]));
+            // the four row slices meet: lane (kp, ql) ends with outputs 4 ql + kp and 32 + 4 ql + kp of the warp's 64
+            float4 *r = reinterpret_cast<float4 *>(red) + (part * groups + grp) * 128 + 8 * ql;   // unit 2 * output + half, its low bits mixed with ql: no bank conflicts
+            const bool hi = kp & 2, odd = kp & 1;
 #pragma unroll
-            for (int c = 0; c < TM; ++c) out_act[j * TM + c] = fmaxf(acc[c], 0.f);
+            for (int g = 0; g < 2; ++g) {
+                float v[TM];
+#pragma unroll
+                for (int cc = 0; cc < TM / 2; ++cc) {
+                    float a[4][2], h[2][2];
+#pragma unroll
+                    for (int o = 0; o < 4; ++o) unpack_f32x2(acc2[4 * g + o][cc], a[o][0], a[o][1]);
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+#pragma unroll
+                        for (int o = 0; o < 2; ++o) h[o][e] = (hi ? a[2 + o][e] : a[o][e]) + __shfl_xor_sync(0xffffffffu, hi ? a[o][e] : a[2 + o][e], 16);
+                        v[2 * cc + e] = (odd ? h[1][e] : h[0][e]) + __shfl_xor_sync(0xffffffffu, odd ? h[0][e] : h[1][e], 8);
+                    }
+                }
+                if (busy && !lay.red) {
+                    const int o = 64 * grp + 32 * g + 4 * ql + kp;
+                    if (o < b.cols)
+#pragma unroll
+                        for (int cc = 0; cc < TM; ++cc) out_act[(size_t)(c0 + o) * TM + cc] = fmaxf(v[cc] + bias[c0 + o], 0.f);
+                } else if (busy) {
+                    r[64 * g + ((2 * kp) ^ ql)] = make_float4(v[0], v[1], v[2], v[3]);
+                    r[64 * g + ((2 * kp + 1) ^ ql)] = make_float4(v[4], v[5], v[6], v[7]);
+                }
+            }
+            if (!lay.red) continue;
+            // ... and those of the warps: [part][group][64 outputs][TM], every thread sums outputs of its own
+            const int first = tid >> 1;
+            const float b_first = first < b.cols ? bias[c0 + first] : 0.f;
+            named_bar_sync(1, kSimtThreads);
+            for (int i = tid; i < 2 * b.cols; i += kSimtThreads) {
+                const int o = i >> 1, h = i & 1;
+                const float b0 = o == first ? b_first : bias[c0 + o];
+                float4 v = make_float4(b0, b0, b0, b0);
+#pragma unroll 4
+                for (int q = 0; q < splits; ++q) {
+                    const float4 t = reinterpret_cast<const float4 *>(red)[q * groups * 128 + (i ^ (i >> 3 & 7))];
+                    v.x += t.x, v.y += t.y, v.z += t.z, v.w += t.w;
+                }
+                *reinterpret_cast<float4 *>(out_act + (size_t)(c0 + o) * TM + 4 * h) =
+                    make_float4(fmaxf(v.x, 0.f), fmaxf(v.y, 0.f), fmaxf(v.z, 0.f), fmaxf(v.w, 0.f));
+            }
+            if (c0 + 256 < H) named_bar_sync(1, kSimtThreads);   // the partial sums are read before the next block's are written
         }
-        __syncthreads();
         in_act = out_act;
         out_act = (out_act == ha) ? hb : ha;
         in_w = H;
     }
+    const T *wo = reinterpret_cast<const T *>(md.w_out);
+    float w_first[4];   // requested before the barrier
+#pragma unroll
+    for (int u = 0; u < 4; ++u) w_first[u] = lane + 32 * u < in_w ? to_f(wo[lane + 32 * u]) : 0.f;
+    const bool bad = named_bar_or(1, kSimtThreads, !ok);
     // ---- output layer: warp c reduces candidate c in a fixed order
-    {
-        const int c = warp;
-        if (c < cnt) {
-            const T *wo = reinterpret_cast<const T *>(md.w_out);
-            float acc = 0.f;
-            for (int j = lane; j < in_w; j += 32) acc = fmaf(to_f(wo[j]), in_act[j * TM + c], acc);
-            acc = warp_sum(acc);
-            if (lane == 0) {
-                float logit = acc + md.b_out[0];
-                if (md.emit_sigmoid) logit = 1.0f / (1.0f + expf(-logit));
-                logits[c] = id_s[c] >= 0 ? logit : __int_as_float(0x7fc00000);
-            }
+    if (c < cnt) {
+        float acc = 0.f;
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (lane + 32 * u < in_w) acc = fmaf(w_first[u], in_act[(lane + 32 * u) * TM + c], acc);
+        for (int j = lane + 128; j < in_w; j += 32) acc = fmaf(to_f(wo[j]), in_act[j * TM + c], acc);
+        acc = warp_sum(acc);
+        if (lane == 0) {
+            float logit = acc + b_out;
+            if (md.emit_sigmoid) logit = 1.0f / (1.0f + expf(-logit));
+            sl.logits[rq.off + start + c] = id >= 0 && !bad ? logit : __int_as_float(0x7fc00000);
         }
     }
-}
-
-static size_t simt_smem_bytes(const aif_ctx *ctx, int &max_h)
-{
-    const aif_config &c = ctx->cfg;
-    max_h = 0;
-    for (int k = 0; k < c.n_hidden; ++k) max_h = c.hidden[k] > max_h ? c.hidden[k] : max_h;
-    const int k1 = ctx->input_width - c.d;
-    size_t fl = (size_t)(k1 + 2 * max_h + c.d) * kSimtTile;
-    size_t ints = (size_t)kSimtTile * (8 + 16 + c.F + 1);
-    return (fl + ints) * 4 + 16;
+    if (bad) {   // a wait that ran out: copies in flight land before shared memory goes away
+        if (tid == 0) atomicOr(sl.status, AIF_STATUS_TIMEOUT);
+        const long long t0 = clock64();
+        while (clock64() - t0 < 2000000ll) __nanosleep(1000);
+    }
 }
 
 cudaError_t launch_score_simt(const aif_ctx *ctx, const ScoreLaunch &sl, cudaStream_t st)
 {
     if (sl.n_tiles <= 0) return cudaSuccess;
-    int max_h;
-    const size_t smem = simt_smem_bytes(ctx, max_h);
+    const aif_config &c = ctx->cfg;
+    SimtLayout lay{};
+    for (int k = 0; k < c.n_hidden; ++k) lay.max_h = c.hidden[k] > lay.max_h ? c.hidden[k] : lay.max_h;
+    const int k1 = ctx->input_width - c.d, act = 2 * lay.max_h * kSimtTile;
+    const int chunk = kSimtKeys * (int)(c.d * ctx->el + 16) / 4;
+    auto bytes = [&](int stages, int bufs, bool red) {
+        lay.stages = stages, lay.key_bufs = bufs, lay.region = act > bufs * chunk ? act : bufs * chunk;
+        lay.red = red ? kSimtRed : 0, lay.ps = bufs ? 2 * kSimtWarps * kSimtKeys : 0;
+        return ((size_t)(k1 + c.d) * kSimtTile + lay.region + lay.red + lay.ps + (size_t)kSimtTile * (8 + 16) + 16) * 4 + (size_t)kSimtMaxStages * 16 +
+               (size_t)stages * kSimtStageBytes;
+    };
+    // wide inputs leave less room: for key buffers and stages first, then for none of the ring, then for no key chunks, at last for no
+    // partial sums
+    size_t smem = 0;
+    static const int tries[][3] = {{4, 2, 1}, {4, 1, 1}, {3, 1, 1}, {2, 1, 1}, {0, 1, 1}, {0, 0, 1}, {0, 0, 0}};
+    for (const auto &t : tries)
+        if ((smem = bytes(t[0], t[1], t[2] != 0)) <= 227 * 1024) break;
     const ModelDev md = make_model(ctx);
-    cudaError_t e;
     timing_begin(ctx, st);
-    if (ctx->cfg.dtype == AIF_F32) {
-        e = cudaFuncSetAttribute(k_score_simt<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        k_score_simt<float><<<sl.n_tiles, kSimtThreads, smem, st>>>(md, sl, max_h);
-    } else {
-        e = cudaFuncSetAttribute(k_score_simt<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        k_score_simt<__nv_bfloat16><<<sl.n_tiles, kSimtThreads, smem, st>>>(md, sl, max_h);
-    }
+    auto go = [&](auto kernel) {
+        const cudaError_t e = smem <= 48 * 1024 ? cudaSuccess : cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        return e != cudaSuccess ? e : launch_pdl(kernel, dim3(sl.n_tiles), dim3(kSimtThreads + 32), smem, st, md, sl, lay);
+    };
+    const bool f32 = c.dtype == AIF_F32;
+    const cudaError_t e = lay.stages ? (f32 ? go(k_score_simt<float, true>) : go(k_score_simt<__nv_bfloat16, true>))
+                                     : (f32 ? go(k_score_simt<float, false>) : go(k_score_simt<__nv_bfloat16, false>));
     count_launch();
     timing_mark(ctx, "score_simt", st);
-    return cudaGetLastError();
+    return e;
 }
 
 // ------------------------------------------------------------------------------------------------

@@ -246,3 +246,28 @@ def test_category_jobs_over_one_and_several_batches_of_groups(n_cat):
     _check(srv.score_ids(states[1], lists[1]), want[1])
     assert srv.ctx.poll_status() == 0
     srv.close()
+
+
+@pytest.mark.parametrize("dtype,d,hidden,F,dc,blocks", [
+    ("f32", 64, (256, 128), 8, 16, helpers.ALL_BLOCKS), ("f32", 32, (264, 8), 3, 8, synth.BLK_ATT | synth.BLK_CROSS),
+    ("f32", 96, (1024, 40, 520), 5, 24, helpers.ALL_BLOCKS), ("f32", 256, (8,), 2, 8, synth.BLK_CROSS | synth.BLK_LSH_DIN | synth.BLK_SIMTIER),
+    ("bf16", 160, (72, 264), 4, 8, helpers.ALL_BLOCKS), ("bf16", 224, (1000,), 1, 8, synth.BLK_ATT),
+    ("f32", 32, (64, 32), 256, 16, synth.BLK_ATT | synth.BLK_CROSS), ("f32", 32, (32, 16), 256, 24, synth.BLK_ATT | synth.BLK_CROSS | synth.BLK_LSH_DIN)])
+def test_cuda_core_scoring_over_widths_and_sequence_lengths(dtype, d, hidden, F, dc, blocks):
+    """The CUDA-core kernel: sequence lengths around its 32-key chunks, layers narrower than a warp's outputs, of whole and of partial
+    column blocks, inputs too wide for the weight ring and for the key chunks (the last two rows); every d it accepts a step of."""
+    wl = synth.C1.with_(name=f"simt_{dtype}_{d}_{len(hidden)}_{F}", dtype=dtype, d=d, hidden=hidden, F=F, dc=dc, B=16, R=1, N=75, M=800, L=160, blocks=blocks,
+                        emit_sigmoid=0, lsh_din_norm=synth.NORM_MEAN, simtier_norm=synth.NORM_MEAN, mini_batch=30, bucket_mode=synth.BUCKET_HASH)
+    weights, table = synth.make_weights(wl, zero_bias=False), synth.make_item_table(wl)
+    srv, oracle = serving.Server(wl, weights, table, path=B.PATH_SIMT), helpers.make_oracle(wl, weights, M=wl.M)
+    ids = np.random.default_rng(1).choice(wl.M, 75, replace=False).astype(np.int32)
+    ids[9] = -1
+    for L in (1, 31, 32, 33, 64, 65, 101, 160):
+        rq = synth.make_request(wl, L, L=L)
+        st = srv.precompute(L, srv.upload_request(rq, B.USER_PROJECTED))
+        want = oracle.score(table, helpers.projected_request(wl, rq), ids)
+        # fp32 arithmetic throughout (sums of up to 6500 terms: 1e-5 of the largest logit where that exceeds 1); bf16 storage as elsewhere
+        _check(srv.score_ids(st, ids), want, 1e-5 * max(1.0, np.nanmax(np.abs(want))) if dtype == "f32" else TOL)
+        st.release()
+    assert srv.ctx.poll_status() == B.STATUS_BAD_ID
+    srv.close()
