@@ -70,6 +70,7 @@ struct LshCfg {
     // tensor memory: two score buffers, two P buffers of their own (BN / 2 columns of packed bf16 pairs each: the next
     // signature product only waits until the scores are in registers, not for the product that reads P), one O accumulator
     static constexpr int kTmemP = 2 * BN;
+    static constexpr int kParts = BN / 64;               // a block's counts are handed over, and multiplied, 64 keys at a time
     static constexpr int kTmemO = D <= 128 ? 384 : 256;
     static_assert(kTmemP + BN <= kTmemO && kTmemO + D <= 512, "tensor memory");
     static constexpr bool kSplitEpi = D <= 128;
@@ -94,75 +95,107 @@ __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel)
 }
 
 // A chunk of a candidate row's scores against a key block: 32 scores (2 matches - d', exact integers in fp32) -> P = 2 matches as packed
-// bf16 pairs, and the tier counts in 8-bit counters (tier t in byte t & 3 of cnt[t >> 2]), 32 keys at a time.
+// bf16 pairs, and the tier counts.
 //
 // Tier of a pair (eq. 9, equal-width tiers, the last one closed): n = floor(matches N / d').  d' is a power of two here, so
 // 2 matches * (N / 2 d') is exact in fp32 and a fused multiply-add that rounds towards minus infinity onto 1.5 * 2^23 leaves
-// n in the low mantissa bits (fp32 counts in ones between 2^23 and 2^24).  An integer multiply by 0x1111 copies n into the
-// four low nibbles.  Up to eight tiers: adding 0x0123 makes nibble p equal to n + 3 - p, which is 3 exactly where p = n and 7
-// where p + 4 = n, never carries (n <= 8) and has bit 3 set (the byte permute's sign-replicating mode: zero for these
-// pools) when it is 8 or more; byte permutes with that selector over a pool whose byte 3, or byte 7, is 0x01 yield the
-// increments 1 << 8 n of the two packed counters.  More than eight tiers: the nibbles are xor-ed with their positions
-// instead (p ^ n is zero only where p = n) and n is capped at 15.  matches = d' gives n = N, one past the last tier: those
-// pairs land in no counted slot and the last tier is derived from the total.  The per-thread work here is what bounds
-// the kernel (about seven instructions per pair with SimTier on), so every instruction counts.
+// n in the low mantissa bits (fp32 counts in ones between 2^23 and 2^24).  matches = d' gives n = N, one past the last tier: those
+// pairs land in no counted slot and the last tier is derived from the total.
+// Up to eight tiers: integer multiply-adds put the tiers of four pairs into the four nibbles of a byte permute's selector, and
+// the permute looks all four up at once, in a table of eight bytes that counts two tiers in the halves of a byte (four tables;
+// a nibble of 8 picks the sign of byte 0, which is clear).  After 32 pairs, when no half can exceed 8, the bytes are summed into
+// the thread's own 32-bit counters, cnt[2 k] += lower halves of table k and cnt[2 k + 1] += whole bytes (lower + 16 upper,
+// taken apart at the end of the tile).  More than eight tiers: an integer multiply by 0x1111 copies n, capped at 15, into
+// four nibbles which are xor-ed with their positions, and the permutes yield the increments 1 << 8 n of packed 8-bit counters
+// (tier t in byte t & 3 of cnt[t >> 2]).
+// The work per pair is what bounds the kernel, above all on the half-rate integer pipe: 2.3 instead of 3.8 of its instructions
+// per pair, 5.0 instead of 7.3 in all, with the tables in place of a permute per pair and packed counter.
 template <int D, bool TIERS, bool WIDE>
-__device__ __forceinline__ void lsh_convert(const uint32_t (&sc)[32], float c1, float n_cap, uint32_t p_col, uint32_t (&cnt)[4])
+__device__ __forceinline__ void lsh_convert(const uint32_t (&sc)[32], float c1, float n_cap, uint32_t p_col, uint32_t (&cnt)[8])
 {
-    uint32_t packed[16];
+    uint32_t packed[16], sum[4] = {0u, 0u, 0u, 0u};
     // the offset and the rounding multiply-add take two scores per instruction (f32x2)
     const uint64_t d2 = pack_f32x2((float)D, (float)D), c2 = pack_f32x2(c1, c1), magic2 = pack_f32x2(12582912.0f, 12582912.0f);
 #pragma unroll
-    for (int i = 0; i < 32; i += 2) {
-        const uint64_t pp = add_f32x2(pack_f32x2(__uint_as_float(sc[i]), __uint_as_float(sc[i + 1])), d2);   // 2 matches
-        float p0, p1;
-        unpack_f32x2(pp, p0, p1);
-        if (TIERS) {
-            float w0, w1;
-            unpack_f32x2(fma_rm_f32x2(pp, c2, magic2), w0, w1);
-            if (WIDE) {
-                w0 = fminf(w0, n_cap), w1 = fminf(w1, n_cap);
-                const uint32_t r0 = __float_as_uint(w0) * 0x1111u, r1 = __float_as_uint(w1) * 0x1111u;
-                cnt[0] += prmt(1u, 0u, r0 ^ 0x3210u) + prmt(1u, 0u, r1 ^ 0x3210u);
-                cnt[1] += prmt(0u, 1u, r0 ^ 0x3210u) + prmt(0u, 1u, r1 ^ 0x3210u);
-                cnt[2] += prmt(1u, 0u, r0 ^ 0xBA98u) + prmt(1u, 0u, r1 ^ 0xBA98u);
-                cnt[3] += prmt(0u, 1u, r0 ^ 0xBA98u) + prmt(0u, 1u, r1 ^ 0xBA98u);
-            } else {
-                const uint32_t s0 = __float_as_uint(w0) * 0x1111u + 0x0123u, s1 = __float_as_uint(w1) * 0x1111u + 0x0123u;
-                cnt[0] += prmt(0x01000000u, 0u, s0) + prmt(0x01000000u, 0u, s1);
-                cnt[1] += prmt(0u, 0x01000000u, s0) + prmt(0u, 0x01000000u, s1);
+    for (int i0 = 0; i0 < 32; i0 += 8) {
+        uint32_t sel[2];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            float w[4];
+#pragma unroll
+            for (int u = 0; u < 4; u += 2) {
+                const int i = i0 + 4 * q + u;
+                const uint64_t pp = add_f32x2(pack_f32x2(__uint_as_float(sc[i]), __uint_as_float(sc[i + 1])), d2);   // 2 matches
+                float p0, p1;
+                unpack_f32x2(pp, p0, p1);
+                if (TIERS) unpack_f32x2(fma_rm_f32x2(pp, c2, magic2), w[u], w[u + 1]);
+                const __nv_bfloat162 h = __floats2bfloat162_rn(p0, p1);
+                packed[i >> 1] = *reinterpret_cast<const uint32_t *>(&h);
             }
+            if (TIERS && WIDE) {
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const uint32_t r = __float_as_uint(fminf(w[u], n_cap)) * 0x1111u;
+                    cnt[0] += prmt(1u, 0u, r ^ 0x3210u), cnt[1] += prmt(0u, 1u, r ^ 0x3210u);
+                    cnt[2] += prmt(1u, 0u, r ^ 0xBA98u), cnt[3] += prmt(0u, 1u, r ^ 0xBA98u);
+                }
+            } else if (TIERS)   // (the permute reads the low 16 bits: what the multiples of 1.5 * 2^23 add lies above)
+                sel[q] = (__float_as_uint(w[3]) * 16u + __float_as_uint(w[2])) * 256u + (__float_as_uint(w[1]) * 16u + __float_as_uint(w[0]));
         }
-        const __nv_bfloat162 h = __floats2bfloat162_rn(p0, p1);
-        packed[i >> 1] = *reinterpret_cast<const uint32_t *>(&h);
+        if (TIERS && !WIDE) {
+            sum[0] += prmt(0x00001001u, 0u, sel[0]) + prmt(0x00001001u, 0u, sel[1]);
+            sum[1] += prmt(0x10010000u, 0u, sel[0]) + prmt(0x10010000u, 0u, sel[1]);
+            sum[2] += prmt(0u, 0x00001001u, sel[0]) + prmt(0u, 0x00001001u, sel[1]);
+            sum[3] += prmt(0u, 0x10010000u, sel[0]) + prmt(0u, 0x10010000u, sel[1]);
+        }
     }
     tmem_st16(p_col, packed);
+    if (TIERS && !WIDE) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            cnt[2 * k] = __dp4a(sum[k] & 0x0F0F0F0Fu, 0x01010101u, cnt[2 * k]);
+            cnt[2 * k + 1] = __dp4a(sum[k], 0x01010101u, cnt[2 * k + 1]);
+        }
+    }
 }
 
 // One key block of a candidate row: BN scores from the score buffer at s_col -> P at p_col and the packed tier counts,
-// 32 columns at a time with the load of the next chunk in flight while one is converted.  Returns after the last load
-// has landed and `s_free` has been told so; the stores may still be in flight.
+// 32 columns at a time with the load of the next chunk in flight while one is converted.  Every 64 columns are a part of their
+// own: its columns of P must have been multiplied for block gb - 2 (`wait`), and are handed over as soon as they are written.
+// Waiting for the block's whole previous product instead tied a warp's next block to the end of its last one's, conversion,
+// hand-over, product and commit in one chain: 2040 cycles per block of 128 keys (16 requests of 10^4 candidates, 10^4 keys, d
+// 128), for 768 cycles of products.
 // Columns beyond the sequence need no special case: their signatures and their rows of S are zero (the user side pads
 // both to the key block), so they add nothing to O, and their score of 0 (matches = d' / 2) lands in tier floor(N / 2),
 // from which the caller takes them out again.
-template <int D, int BN, bool TIERS, bool WIDE>
-__device__ __forceinline__ void lsh_block(uint32_t s_col, uint32_t p_col, float c1, float n_cap, uint32_t s_free_bar, uint32_t (&cnt)[4])
+template <int D, int BN, bool TIERS, bool WIDE, typename Wait>
+__device__ __forceinline__ bool lsh_block(uint32_t s_col, uint32_t p_col, float c1, float n_cap, uint32_t s_free_bar, uint32_t p_full_bar, Wait wait,
+                                          uint32_t (&cnt)[8])
 {
+    const int lane = threadIdx.x & 31;
     uint32_t ra[32], rb[32];
     tmem_ld32(s_col, ra);
 #pragma unroll 1
     for (int c0 = 0; c0 < BN; c0 += 64) {
+        const bool got = wait(c0 >> 6);
         tmem_ld_wait();
+        if (!got) return false;
         tmem_ld32(s_col + (uint32_t)(c0 + 32), rb);
         lsh_convert<D, TIERS, WIDE>(ra, c1, n_cap, p_col + (uint32_t)(c0 >> 1), cnt);
         tmem_ld_wait();
         if (c0 + 64 < BN) tmem_ld32(s_col + (uint32_t)(c0 + 64), ra);
         else {   // all scores are in registers: the signature product of block gb + 2 may overwrite the buffer
             tc_fence_before();
-            mbar_arrive(s_free_bar);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(s_free_bar);
         }
         lsh_convert<D, TIERS, WIDE>(rb, c1, n_cap, p_col + (uint32_t)((c0 + 32) >> 1), cnt);
+        tmem_st_wait();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(p_full_bar + (uint32_t)(c0 >> 6) * 8u);
     }
+    return true;
 }
 
 // SPLIT: the launch's tiles are cut into pieces of their keys.
@@ -174,7 +207,7 @@ __global__ void __launch_bounds__((LshCfg<D, BN>::kThreads), 1) k_lsh_tc(const _
     using C = LshCfg<D, BN>;
     constexpr int kSG = C::kStagesG, kSV = C::kStagesV, kQB = C::kQBufs;
     constexpr bool kSplit = C::kSplitEpi;
-    constexpr int kH = C::kHalves;
+    constexpr int kH = C::kHalves, kPt = C::kParts;
     extern __shared__ unsigned char smem_dyn[];
     unsigned char *base = reinterpret_cast<unsigned char *>(((uintptr_t)smem_dyn + 1023) & ~(uintptr_t)1023);
     unsigned char *smQ = base;
@@ -182,7 +215,7 @@ __global__ void __launch_bounds__((LshCfg<D, BN>::kThreads), 1) k_lsh_tc(const _
     unsigned char *smG = smV + kSV * C::kVBytes;
     uint64_t *bars = reinterpret_cast<uint64_t *>(smG + kSG * C::kGBytes);
     uint64_t *v_full = bars, *v_empty = bars + kSV, *g_full = v_empty + kSV, *g_empty = g_full + kSG;
-    uint64_t *s_full = g_empty + kSG, *p_full = s_full + 2, *pv_done = p_full + 2, *s_free = pv_done + 2;
+    uint64_t *s_full = g_empty + kSG, *p_full = s_full + 2, *pv_done = p_full + 2 * kPt, *s_free = pv_done + 2 * kPt;   // p_full, pv_done: [buffer][part]
     uint64_t *q_full = s_free + 2, *q_empty = q_full + 2, *o_final = q_empty + 2, *o_free = o_final + 2;
     uint64_t *q_first = o_free + 2;
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(q_first + 1);
@@ -202,10 +235,9 @@ __global__ void __launch_bounds__((LshCfg<D, BN>::kThreads), 1) k_lsh_tc(const _
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(smem_u32(s_full + b), 1);
-            mbar_init(smem_u32(p_full + b), 128);
-            mbar_init(smem_u32(pv_done + b), 1);
-            mbar_init(smem_u32(s_free + b), 128);
-            mbar_init(smem_u32(q_full + b), 32);
+            for (int h = 0; h < kPt; ++h) mbar_init(smem_u32(p_full + b * kPt + h), 4), mbar_init(smem_u32(pv_done + b * kPt + h), 1);
+            mbar_init(smem_u32(s_free + b), 4);   // the four warps that convert the buffer's block
+            mbar_init(smem_u32(q_full + b), 1);
             mbar_init(smem_u32(q_empty + b), 5);   // the tenant's last signature product, and the four output warps' staging
             mbar_init(smem_u32(o_final + b), 1);
             mbar_init(smem_u32(o_free + b), 128);
@@ -367,6 +399,7 @@ __global__ void __launch_bounds__((LshCfg<D, BN>::kThreads), 1) k_lsh_tc(const _
             const KeyTile t = key_tile<BN, SPLIT>(p.sl, tile, p.mini_batch);
             const int L = t.L;
             uint32_t *tc = tier_s + (((kH == 2 ? (k & 1) * kH : 0) + half) * kTierSlots) * 128 + row;   // this thread's counters, stride 128
+            uint32_t cnt[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};   // up to eight tiers: of the tile so far; else of the block
             int n_valid = 0, n_pad = 0;   // keys this thread has counted, and columns beyond the sequence it has converted
             for (int j = 0; j < t.nb; ++j, ++gb) {
                 // d = 128: the two warps of a row quarter take alternate key blocks (block gb, and with it score and P buffer
@@ -379,36 +412,31 @@ __global__ void __launch_bounds__((LshCfg<D, BN>::kThreads), 1) k_lsh_tc(const _
                     break;
                 }
                 tc_fence_after();
-                // P buffer b was last read by the product of block gb - 2
-                if (gb >= 2 && !__all_sync(0xffffffffu, mbar_wait(smem_u32(pv_done + b), ((gb - 2) >> 1) & 1u, abort_flag))) {
-                    ok = false;
-                    break;
-                }
-                tc_fence_after();
+                // P buffer b was last read by the products of block gb - 2
+                auto p_free = [&](int h) {
+                    if (gb < 2) return true;
+                    const bool got = __all_sync(0xffffffffu, mbar_wait(smem_u32(pv_done + b * kPt + h), ((gb - 2) >> 1) & 1u, abort_flag));
+                    tc_fence_after();
+                    return got;
+                };
                 const uint32_t s_col = lane_base + (uint32_t)(b * BN), p_col = lane_base + (uint32_t)(C::kTmemP + b * (BN / 2));
-                uint32_t cnt[4] = {0u, 0u, 0u, 0u};
-                if (!tiers) lsh_block<D, BN, false, false>(s_col, p_col, tc1, n_cap, smem_u32(s_free + b), cnt);
-                else if (!wide) lsh_block<D, BN, true, false>(s_col, p_col, tc1, n_cap, smem_u32(s_free + b), cnt);
-                else lsh_block<D, BN, true, true>(s_col, p_col, tc1, n_cap, smem_u32(s_free + b), cnt);
-                tmem_st_wait();
-                tc_fence_before();
-                mbar_arrive(smem_u32(p_full + b));
+                const uint32_t s_bar = smem_u32(s_free + b), p_bar = smem_u32(p_full + b * kPt);
+                if (wide) cnt[0] = cnt[1] = cnt[2] = cnt[3] = 0u;
+                ok = !tiers  ? lsh_block<D, BN, false, false>(s_col, p_col, tc1, n_cap, s_bar, p_bar, p_free, cnt)
+                     : !wide ? lsh_block<D, BN, true, false>(s_col, p_col, tc1, n_cap, s_bar, p_bar, p_free, cnt)
+                             : lsh_block<D, BN, true, true>(s_col, p_col, tc1, n_cap, s_bar, p_bar, p_free, cnt);
+                if (!ok) break;
                 n_valid += vc, n_pad += BN - vc;
-                // the block's packed counts (at most 128 per slot) into the tile's 32-bit counters
-                if (tiers) {
+                if (tiers && wide) {   // the block's packed counts (at most 128 per slot) into the tile's 32-bit counters
 #pragma unroll
-                    for (int t4 = 0; t4 < 4; ++t4) {
-                        tc[t4 * 128] += (cnt[0] >> (8 * t4)) & 0xFFu;
-                        tc[(4 + t4) * 128] += (cnt[1] >> (8 * t4)) & 0xFFu;
-                    }
-                    if (wide) {
+                    for (int t4 = 0; t4 < 4; ++t4)
 #pragma unroll
-                        for (int t4 = 0; t4 < 4; ++t4) {
-                            tc[(8 + t4) * 128] += (cnt[2] >> (8 * t4)) & 0xFFu;
-                            tc[(12 + t4) * 128] += (cnt[3] >> (8 * t4)) & 0xFFu;
-                        }
-                    }
+                        for (int q = 0; q < 4; ++q) tc[(4 * q + t4) * 128] += (cnt[q] >> (8 * t4)) & 0xFFu;
                 }
+            }
+            if (tiers && !wide && ok) {
+#pragma unroll
+                for (int q = 0; q < 4; ++q) tc[2 * q * 128] = cnt[2 * q], tc[(2 * q + 1) * 128] = (cnt[2 * q + 1] - cnt[2 * q]) >> 4;
             }
             // ---- SimTier columns of the tile (eq. 9): 64 bf16 per row, the first n_tiers used
             if (p.x_tier >= 0) {
@@ -533,18 +561,23 @@ __global__ void __launch_bounds__((LshCfg<D, BN>::kThreads), 1) k_lsh_tc(const _
                 while (ok && c.tile < n_tiles) {
                     const int s = (int)(c.gb % kSV);
                     if (!mbar_wait(smem_u32(v_full + s), (c.gb / kSV) & 1u, abort_flag)) break;
-                    if (!mbar_wait(smem_u32(p_full + (c.gb & 1u)), (c.gb >> 1) & 1u, abort_flag)) break;
                     // the first product of a tile overwrites O: the previous tile's rows must have been read
                     if (c.j == 0 && c.k > 0 && !mbar_wait(smem_u32(o_free), (uint32_t)((c.k - 1) & 1), abort_flag)) break;
-                    tc_fence_after();
                     const uint32_t o_tmem = tmem_base + (uint32_t)C::kTmemO;
                     const uint32_t p_tmem = tmem_base + (uint32_t)(C::kTmemP + (c.gb & 1u) * (BN / 2));
                     const uint64_t vd = vdesc0 + (uint64_t)(uint32_t)(s * (C::kVBytes >> 4));
 #pragma unroll
-                    for (int kk = 0; kk < BN / 16; ++kk)
-                        umma_bf16_ts(o_tmem, p_tmem + (uint32_t)(kk * 8), vd + (uint64_t)(kk * (2048 >> 4)), idesc_pv,
-                                     (c.j > 0 || kk > 0) ? 1u : 0u);
-                    umma_commit(smem_u32(pv_done + (c.gb & 1u)));
+                    for (int h = 0; h < kPt; ++h) {
+                        ok = ok && mbar_wait(smem_u32(p_full + (c.gb & 1u) * kPt + h), (c.gb >> 1) & 1u, abort_flag);
+                        if (!ok) break;
+                        tc_fence_after();
+#pragma unroll
+                        for (int kk = 4 * h; kk < 4 * h + 4; ++kk)
+                            umma_bf16_ts(o_tmem, p_tmem + (uint32_t)(kk * 8), vd + (uint64_t)(kk * (2048 >> 4)), idesc_pv,
+                                         (c.j > 0 || kk > 0) ? 1u : 0u);
+                        umma_commit(smem_u32(pv_done + (c.gb & 1u) * kPt + h));
+                    }
+                    if (!ok) break;
                     umma_commit(smem_u32(v_empty + s));
                     if (c.j == c.nb - 1) umma_commit(smem_u32(o_final));
                     advance(c);
@@ -636,7 +669,8 @@ __global__ void __launch_bounds__((LshCfg<D, BN>::kThreads), 1) k_lsh_tc(const _
             }
             expand_rows(q, r0, 4, sub, std::integral_constant<int, 32>{}, [&](int i) { return __shfl_sync(0xffffffffu, idv[i >> 3], r0 + 4 * (i & 7)); });
             fence_proxy_async();
-            mbar_arrive(smem_u32(q_full + qb));
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(q_full + qb));
         }
     }
 
