@@ -228,7 +228,10 @@ __global__ void __launch_bounds__(1024) k_sim_tiles(ScoreLaunch sl, int n_groups
     for (int o = 16; o > 0; o >>= 1) blocks += __shfl_xor_sync(0xffffffffu, blocks, o);
     // Key blocks of a piece.  Tiles with more are cut into ceil(blocks / piece) pieces: at most 2 blocks / piece <= kSplitSlots
     // records of partial results.  Below four blocks a piece is mostly its own start and end.
-    const int piece = sl.split.slots >= kSplitSlots ? max(4, (int)((blocks + 2 * 148 - 1) / (2 * 148))) : 0x7fffffff;
+    // An SM's share of the launch is one piece: every record is 64 KB written and read again.  With pieces of half a share the two
+    // joins took 26 of 212 us (4 x 10^4 candidates, 10^5 keys in 100 categories), with shares 203 us in all; with two shares to a
+    // piece the longest tiles are alone at the end (215 us).
+    const int piece = sl.split.slots >= kSplitSlots ? max(4, (int)((blocks + 148 - 1) / 148)) : 0x7fffffff;
     auto pieces_of = [&](int len) {
         const int nb = key_blocks(len);
         return nb > piece ? (nb + piece - 1) / piece : 1;
