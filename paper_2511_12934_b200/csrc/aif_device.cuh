@@ -196,6 +196,15 @@ __device__ inline ReqDev find_request(const ScoreLaunch &sl, int t)
     return sl.reqs[lo];
 }
 
+// Record of tile `tile` of the launch's requests.
+__device__ inline TileDev tile_entry(const ScoreLaunch &sl, int tile, int mini_batch)
+{
+    const ReqDev rq = find_request(sl, tile);
+    int start, cnt;
+    tile_range(tile - rq.tile_begin, rq.n, kTcTile, mini_batch, start, cnt);
+    return TileDev{rq.slot, cnt, rq.off + start, sl.slots[rq.slot].L, 0, {0, 0}};
+}
+
 // One tile, or (SPLIT) one piece of a tile's keys, as every role of the attention and LSH kernels needs it.
 struct KeyTile {
     int slot, cnt, nb, L;      // nb: key blocks to walk, at least one (an empty one is masked: the roles' hand-overs stay the same)

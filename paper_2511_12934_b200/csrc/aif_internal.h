@@ -296,7 +296,7 @@ struct SimPlace {
 };
 // fills sl (tiles, jobs, their numbers, out_index) for a launch whose original ids are sl.ids; the candidates themselves are
 // placed by the bucket kernel, after which the launch's ids are place.ids
-cudaError_t sim_group_candidates(const aif_ctx *ctx, ScoreLaunch &sl, SimPlace &place, cudaStream_t st);
+cudaError_t sim_group_candidates(const aif_ctx *ctx, ScoreLaunch &sl, SimPlace &place, TileDev *row_tiles, cudaStream_t st);
 // pieces per tile that even a launch of n_tiles tiles of `blocks` key blocks out over the SMs (aif_tc.cu)
 int split_parts(int n_tiles, int blocks, int slots);
 // Puts the pieces of a launch's tiles together (after the attention or LSH kernel of a split launch): rows into columns

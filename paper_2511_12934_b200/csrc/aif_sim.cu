@@ -141,10 +141,15 @@ __device__ __forceinline__ int group_of(const ScoreLaunch &sl, int64_t pos, int6
 }
 
 // where[pos] = (group of candidate pos, its rank inside the group); the group counts.  The order inside a group is arbitrary.
-__global__ void __launch_bounds__(256) k_sim_count(ScoreLaunch sl, int64_t M, int n_cat, int mode, int32_t *__restrict__ grp_cnt, int2 *__restrict__ where)
+// On the way, the tiles of the launch's requests as they would be without categories, for the kernels that take them so.
+__global__ void __launch_bounds__(256) k_sim_count(ScoreLaunch sl, int64_t M, int n_cat, int mode, int32_t *__restrict__ grp_cnt, int2 *__restrict__ where,
+                                                   int mini_batch, TileDev *__restrict__ row_tiles)
 {
     grid_dep_launch();
     grid_dep_wait();
+    if (row_tiles)
+        for (int tile = (int)(blockIdx.x * blockDim.x + threadIdx.x); tile < sl.n_tiles; tile += (int)(gridDim.x * blockDim.x))
+            row_tiles[tile] = tile_entry(sl, tile, mini_batch);
     for (int64_t pos = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; pos < sl.total; pos += (int64_t)gridDim.x * blockDim.x) {
         int id;
         const int g = group_of(sl, pos, M, n_cat, mode, id);
@@ -394,13 +399,14 @@ cudaError_t sim_group_sequence(const aif_ctx *ctx, HostSlot &hs, const int32_t *
     return cudaGetLastError();
 }
 
-cudaError_t sim_group_candidates(const aif_ctx *ctx, ScoreLaunch &sl, SimPlace &place, cudaStream_t st)
+cudaError_t sim_group_candidates(const aif_ctx *ctx, ScoreLaunch &sl, SimPlace &place, TileDev *row_tiles, cudaStream_t st)
 {
     const aif_config &c = ctx->cfg;
     SimPlan *pl = plan_of(ctx);
     const int n_groups = sl.n_req * c.n_categories;
     const int grid = (int)((sl.total + 255) / 256 < 1184 ? (sl.total + 255) / 256 : 1184);
-    cudaError_t e = launch_pdl(k_sim_count, dim3(grid), dim3(256), 0, st, sl, c.M, c.n_categories, c.bucket_mode, pl->grp_cnt, pl->where);
+    cudaError_t e = launch_pdl(k_sim_count, dim3(grid), dim3(256), 0, st, sl, c.M, c.n_categories, c.bucket_mode, pl->grp_cnt, pl->where,
+                               c.mini_batch, row_tiles);
     if (e != cudaSuccess) return e;
     e = launch_pdl(k_sim_tiles, dim3(1), dim3(1024), 0, st, sl, n_groups, c.n_categories, pl->grp_cnt, pl->grp_start, pl->tiles, (int)pl->tile_cap, pl->jobs,
                    (int)pl->tile_cap + kSplitSlots, pl->joins, pl->n_tiles_dev);

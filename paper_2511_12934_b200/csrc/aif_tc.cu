@@ -154,13 +154,7 @@ __global__ void __launch_bounds__(256) k_tile_table(ScoreLaunch sl, int mini_bat
     grid_dep_wait();
     const int tile = blockIdx.x * blockDim.x + threadIdx.x;
     if (tile >= sl.n_tiles) return;
-    const ReqDev rq = find_request(sl, tile);
-    int start, cnt;
-    tile_range(tile - rq.tile_begin, rq.n, kTcTile, mini_batch, start, cnt);
-    TileDev t;
-    t.slot = rq.slot, t.cnt = cnt, t.pos0 = rq.off + start, t.L = sl.slots[rq.slot].L;
-    t.pad_[0] = t.pad_[1] = t.pad_[2] = 0;
-    out[tile] = t;
+    out[tile] = tile_entry(sl, tile, mini_batch);
 }
 
 // ---- the layer kernel ---------------------------------------------------------------------------------------------
@@ -1176,7 +1170,7 @@ cudaError_t launch_score_tc_scratch(const aif_ctx *ctx, const ScoreLaunch &sl_in
         // candidates grouped by (request, category): tiles, grouped ids and the way back to the caller's order
         if (sc.rows < (size_t)sl.total + kTcTile || !ctx->sim_plan) return cudaErrorInvalidValue;
         StageRange range("aif group");
-        cudaError_t e = sim_group_candidates(ctx, sl, place, st);
+        cudaError_t e = sim_group_candidates(ctx, sl, place, sl.reqs ? (TileDev *)sc.tiles : nullptr, st);
         timing_mark(ctx, "group", st);
         if (e != cudaSuccess) return e;
     } else if (sl.reqs && sc.tiles) {   // several requests: look every tile up once
@@ -1202,6 +1196,11 @@ cudaError_t launch_score_tc_scratch(const aif_ctx *ctx, const ScoreLaunch &sl_in
         timing_mark(ctx, "buckets", st);
         if (e != cudaSuccess) return e;
     }
+    // What does not depend on the category takes the grouped candidates request by request, in whole tiles: the groups of a request
+    // are its positions, in another order.  By the groups' tiles the layers ran on rows that were mostly padding (20 candidates per
+    // category: 800 tiles instead of 130).
+    ScoreLaunch sl_rows = sl;
+    if (c.n_categories > 0) sl_rows.n_tiles = sl_in.n_tiles, sl_rows.n_tiles_dev = nullptr, sl_rows.tiles = sl.reqs ? (const TileDev *)sc.tiles : nullptr;
     const bool att_tc = ctx->tc_att_plan != nullptr;
     // few tiles with many keys: their keys over several CTAs each (the table of jobs does it where categories are on)
     if (!sl.jobs) sl.parts = split_parts(sl.n_tiles, (sl.max_L + (c.d == 128 ? 127 : 63)) / (c.d == 128 ? 128 : 64), sl.split.slots);
@@ -1230,7 +1229,7 @@ cudaError_t launch_score_tc_scratch(const aif_ctx *ctx, const ScoreLaunch &sl_in
     if (c.blocks & AIF_BLK_BEA) {
         StageRange range("aif bea");
         const size_t smem = (size_t)c.n_bridge * c.d * 2 + (size_t)kBeaRows * c.n_bridge * 4;
-        cudaError_t e = launch_pdl(k_bea_x, dim3(sl.n_tiles, kTcTile / kBeaRows), dim3(256), smem, st, md, sl, (__nv_bfloat16 *)sc.X, pl->x_cols,
+        cudaError_t e = launch_pdl(k_bea_x, dim3(sl_rows.n_tiles, kTcTile / kBeaRows), dim3(256), smem, st, md, sl_rows, (__nv_bfloat16 *)sc.X, pl->x_cols,
                                    (c.blocks & AIF_BLK_ATT) ? c.d : 0);
         count_launch();
         timing_mark(ctx, "bea", st);
@@ -1250,7 +1249,7 @@ cudaError_t launch_score_tc_scratch(const aif_ctx *ctx, const ScoreLaunch &sl_in
     for (int k = 0; k < c.n_hidden; ++k) {
         StageRange range(range_names[k]);
         LayerParams p{};
-        p.sl = sl;
+        p.sl = sl_rows;
         p.n_nchunks = pl->n_nchunks[k], p.n_cols = pl->n_cols[k], p.n_out = c.hidden[k], p.n_k = pl->n_k[k], p.mini_batch = c.mini_batch;
         p.E = (const uint8_t *)ctx->E, p.M = c.M, p.e_row_bytes = c.d * 2;
         p.B = c.B > 0 ? c.B : 1, p.dc = c.dc > 0 ? c.dc : 8, p.F = c.F, p.xb = (const uint16_t *)sc.xb;
@@ -1293,7 +1292,7 @@ cudaError_t launch_score_tc_scratch(const aif_ctx *ctx, const ScoreLaunch &sl_in
                                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
             if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
         }
-        const cudaError_t e = launch_layer(p, sl.n_tiles, pl->tmap_half[k], tmap_out, tmap_a, st);
+        const cudaError_t e = launch_layer(p, sl_rows.n_tiles, pl->tmap_half[k], tmap_out, tmap_a, st);
         timing_mark(ctx, names[k], st);
         if (e != cudaSuccess) return e;
     }

@@ -271,3 +271,25 @@ def test_cuda_core_scoring_over_widths_and_sequence_lengths(dtype, d, hidden, F,
         st.release()
     assert srv.ctx.poll_status() == B.STATUS_BAD_ID
     srv.close()
+
+
+@pytest.mark.parametrize("mini_batch", [0, 50, 128])
+def test_category_rows_in_whole_tiles_of_their_requests(mini_batch):
+    """Categories of a few candidates each, every block on: the kernels that do not depend on the category take the grouped
+    candidates of a request in whole tiles, whatever the mini-batch; requests of one and of several tiles, ids outside the table."""
+    wl = helpers.MINI["c2"].with_(name=f"sim_rows_{mini_batch}", R=3, N=600, M=4000, L=900, F=2, B=64, mini_batch=mini_batch, n_categories=40,
+                                  blocks=helpers.ALL_BLOCKS)
+    weights, table = synth.make_weights(wl, zero_bias=False), synth.make_item_table(wl)
+    srv, oracle = serving.Server(wl, weights, table), helpers.make_oracle(wl, weights, M=wl.M)
+    rqs = [synth.make_request(wl, r) for r in range(3)]
+    states = [srv.precompute(r, srv.upload_request(rq, B.USER_PROJECTED)) for r, rq in enumerate(rqs)]
+    g = np.random.default_rng(4)
+    lists = [g.choice(wl.M, n, replace=False).astype(np.int32) for n in (600, 1, 333)]
+    lists[2][7], lists[2][300] = -1, wl.M
+    want = [oracle.score(table, helpers.projected_request(wl, rq), ids) for rq, ids in zip(rqs, lists)]
+    for got, w in zip(srv.score_many(states, lists), want):
+        _check(got, w)
+    for i in (0, 2):
+        _check(srv.score_ids(states[i], lists[i]), want[i])
+    assert srv.ctx.poll_status() == B.STATUS_BAD_ID
+    srv.close()
