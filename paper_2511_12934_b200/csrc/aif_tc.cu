@@ -157,6 +157,104 @@ __global__ void __launch_bounds__(256) k_tile_table(ScoreLaunch sl, int mini_bat
     out[tile] = tile_entry(sl, tile, mini_batch);
 }
 
+// Rows of a chunk of the first layer's input, brought into a stage by one warp.  Lane l: 16-byte slot l % 8 of the 128-byte rows
+// l / 8 + 4 i.  The sources of a chunk are one number per row, the item id or the bucket(s) of the chunk's field(s): lane l
+// fetches those of rows l + 32 j with coalesced loads (fetch), the copying lanes get them by shuffle (copy).
+struct ChunkRows {
+    int kind;
+    int32_t v[4];           // per row lane + 32 j: id as read, or bucket (both fields' buckets); -1: zero row
+    const uint8_t *bp;      // this lane's 16 bytes of row 0 of the table the rows come from
+    const uint16_t *xb;     // narrow fields: this lane's field of the tile's first row of buckets
+    uint32_t row_bytes;     // of that table
+    int cnt;                // rows of the tile
+    int tma_x, tma_y;       // dense chunk; tma_x < 0: the tile does not exist
+};
+struct RowGather {
+    int lane, sub, r0;
+    uint32_t swz0, swz1;   // row & 7 alternates between r0 and r0 + 4
+    bool two;          // two fields per chunk; wider embeddings: one field spans one or more chunks
+    bool narrow;       // four and more fields per chunk: the copying lanes look their buckets up themselves
+    __device__ __forceinline__ RowGather(const LayerParams &p, int l)
+        : lane(l), sub(l & 7), r0(l >> 3), swz0((uint32_t)((sub ^ r0) << 4)), swz1((uint32_t)((sub ^ (r0 + 4)) << 4)), two(p.dc == 32), narrow(p.dc < 32)
+    {
+    }
+    __device__ __forceinline__ void fetch(ChunkRows &c, const LayerParams &p, int kc, const TileInfo &t) const
+    {
+        const ChunkSrc src = p.src[kc];
+        c.kind = src.kind, c.cnt = t.cnt;
+        if (src.kind == SRC_DENSE) {
+            // rows beyond the tile bring other candidates' values along; their results are never stored
+            c.tma_x = t.cnt > 0 ? src.off >> 1 : -1, c.tma_y = (int)t.pos0;
+        } else if (src.kind == SRC_ITEM) {
+            c.bp = p.E + src.off + sub * 16, c.row_bytes = (uint32_t)p.e_row_bytes;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) c.v[j] = lane + 32 * j < t.cnt ? p.sl.ids[t.pos0 + lane + 32 * j] : -1;
+        } else if (narrow) {
+            const int col = src.off + sub * 8, f = col / p.dc;
+            c.row_bytes = (uint32_t)p.dc * 2;
+            c.bp = p.T0 + (size_t)t.rq.slot * p.slot_bytes + ((size_t)f * p.B * p.dc + (col - f * p.dc)) * 2;
+            c.xb = p.xb + (size_t)t.pos0 * p.F + f;
+        } else {
+            const int f = src.off / p.dc, col = two ? (sub & 3) * 8 : src.off - f * p.dc + sub * 8;
+            c.row_bytes = (uint32_t)p.dc * 2;
+            c.bp = p.T0 + (size_t)t.rq.slot * p.slot_bytes + ((size_t)(f + (two ? sub >> 2 : 0)) * p.B * p.dc + col) * 2;
+            const uint16_t *xb = p.xb + (size_t)t.pos0 * p.F + f;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                c.v[j] = -1;
+                if (lane + 32 * j < t.cnt) {
+                    const uint16_t *w = xb + (size_t)(lane + 32 * j) * p.F;
+                    // F is even where dc = 32; a bucket that does not exist is 0xFFFF, both of a pair at once
+                    c.v[j] = two ? __ldg(reinterpret_cast<const int32_t *>(w)) : (int32_t)((uint32_t)__ldg(w) | 0xFFFF0000u);
+                }
+            }
+        }
+    }
+    // a gathered chunk (not SRC_DENSE); c is used up
+    __device__ __forceinline__ void copy(ChunkRows &c, const LayerParams &p, uint32_t dst0, bool first) const
+    {
+        // row r0 + 4 i: register i / 8 of lane r0 + 4 (i % 8)
+        if (c.kind == SRC_ITEM) {
+            bool bad = false;
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (c.v[j] < 0 || (int64_t)c.v[j] >= p.M) {
+                    bad |= lane + 32 * j < c.cnt;
+                    c.v[j] = -1;
+                }
+            if (bad && p.check_ids && first) atomicOr(p.sl.status, AIF_STATUS_BAD_ID);
+#pragma unroll
+            for (int i = 0; i < 32; ++i) {
+                const int v = __shfl_sync(0xffffffffu, c.v[i >> 3], r0 + 4 * (i & 7));
+                cp_async16(dst0 + (uint32_t)(i * 512) + (i & 1 ? swz1 : swz0), c.bp + (size_t)(uint32_t)max(v, 0) * c.row_bytes, v >= 0 ? 16u : 0u);
+            }
+        } else if (narrow) {
+#pragma unroll 1
+            for (int i0 = 0; i0 < 32; i0 += 8) {
+                uint32_t v[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int row = r0 + 4 * (i0 + i);
+                    v[i] = row < c.cnt ? (uint32_t)__ldg(c.xb + (size_t)row * p.F) : kNoBucket;
+                }
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const bool on = v[i] != kNoBucket;
+                    cp_async16(dst0 + (uint32_t)((i0 + i) * 512) + (i & 1 ? swz1 : swz0), c.bp + (size_t)(on ? v[i] : 0u) * c.row_bytes, on ? 16u : 0u);
+                }
+            }
+        } else {
+            const uint32_t pick = two && sub >= 4 ? 0x4432u : 0x4410u;   // byte permute: the pair's upper or lower half
+#pragma unroll
+            for (int i = 0; i < 32; ++i) {
+                const uint32_t v = __byte_perm((uint32_t)__shfl_sync(0xffffffffu, c.v[i >> 3], r0 + 4 * (i & 7)), 0u, pick);
+                const bool on = v != kNoBucket;
+                cp_async16(dst0 + (uint32_t)(i * 512) + (i & 1 ? swz1 : swz0), c.bp + (size_t)(on ? v : 0u) * c.row_bytes, on ? 16u : 0u);
+            }
+        }
+    }
+};
+
 // ---- the layer kernel ---------------------------------------------------------------------------------------------
 // Every product spans two SMs (cta_group::2).  What bounds a layer is the rate at which an SM takes in operands (59 bytes per
 // clock).  With both tiles of an item in one SM, which that rate asks for, their accumulators filled tensor memory and the
@@ -419,13 +517,10 @@ __global__ void __launch_bounds__(PairCfg::kThreads, 1) k_layer_pair(const __gri
         // 3300 cycles.  A warp waits for its own copies (five others have theirs in flight meanwhile) and tells the issuer
         // with one arrival: an arrival per gathering thread (256 serial operations on the stage's barrier) cost more than the
         // 512 cycles of products a chunk is.
-        const int sub = lane & 7, r0 = lane >> 3;
-        const uint32_t swz[2] = {(uint32_t)((sub ^ r0) << 4), (uint32_t)((sub ^ (r0 + 4)) << 4)};   // row & 7 alternates between r0 and r0 + 4
+        const RowGather g(p, lane);
         const int n_k = p.n_k;
-        const bool two = p.dc == 32;      // two fields per chunk; wider embeddings: one field spans one or more chunks
-        const bool narrow = p.dc < 32;    // four and more fields per chunk: the copying lanes look their buckets up themselves
         const int s = warp - C::kProdWarp0;
-        const uint32_t dst0 = smem_u32(base + s * C::kStage) + (uint32_t)(r0 * 128);
+        const uint32_t dst0 = smem_u32(base + s * C::kStage) + (uint32_t)(g.r0 * 128);
         struct Place {
             int item, kc;
         };
@@ -434,52 +529,12 @@ __global__ void __launch_bounds__(PairCfg::kThreads, 1) k_layer_pair(const __gri
             while (q.kc >= n_k) q.kc -= n_k, q.item += item_step;
         };
         auto tile_of = [&](const Place &q) { return decode_tile(p, q.item < n_items ? (q.item / p.n_nchunks) * 2 + rank : n_tiles, n_tiles); };
-        struct Chunk {
-            int kind;
-            int32_t v[4];           // per row lane + 32 j: id as read, or bucket (both fields' buckets); -1: zero row
-            const uint8_t *bp;      // this lane's 16 bytes of row 0 of the table the rows come from
-            const uint16_t *xb;     // narrow fields: this lane's field of the tile's first row of buckets
-            uint32_t row_bytes;     // of that table
-            int cnt;                // rows of the tile
-            int tma_x, tma_y;       // dense chunk; tma_x < 0: the tile does not exist
-        };
-        auto fetch = [&](Chunk &c, const Place &q, const TileInfo &t) {
-            const ChunkSrc src = p.src[q.kc];
-            c.kind = src.kind, c.cnt = t.cnt;
-            if (src.kind == SRC_DENSE) {
-                // rows beyond the tile bring other candidates' values along; their results are never stored
-                c.tma_x = t.cnt > 0 ? src.off >> 1 : -1, c.tma_y = (int)t.pos0;
-            } else if (src.kind == SRC_ITEM) {
-                c.bp = p.E + src.off + sub * 16, c.row_bytes = (uint32_t)p.e_row_bytes;
-#pragma unroll
-                for (int j = 0; j < 4; ++j) c.v[j] = lane + 32 * j < t.cnt ? p.sl.ids[t.pos0 + lane + 32 * j] : -1;
-            } else if (narrow) {
-                const int col = src.off + sub * 8, f = col / p.dc;
-                c.row_bytes = (uint32_t)p.dc * 2;
-                c.bp = p.T0 + (size_t)t.rq.slot * p.slot_bytes + ((size_t)f * p.B * p.dc + (col - f * p.dc)) * 2;
-                c.xb = p.xb + (size_t)t.pos0 * p.F + f;
-            } else {
-                const int f = src.off / p.dc, col = two ? (sub & 3) * 8 : src.off - f * p.dc + sub * 8;
-                c.row_bytes = (uint32_t)p.dc * 2;
-                c.bp = p.T0 + (size_t)t.rq.slot * p.slot_bytes + ((size_t)(f + (two ? sub >> 2 : 0)) * p.B * p.dc + col) * 2;
-                const uint16_t *xb = p.xb + (size_t)t.pos0 * p.F + f;
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    c.v[j] = -1;
-                    if (lane + 32 * j < t.cnt) {
-                        const uint16_t *w = xb + (size_t)(lane + 32 * j) * p.F;
-                        // F is even where dc = 32; a bucket that does not exist is 0xFFFF, both of a pair at once
-                        c.v[j] = two ? __ldg(reinterpret_cast<const int32_t *>(w)) : (int32_t)((uint32_t)__ldg(w) | 0xFFFF0000u);
-                    }
-                }
-            }
-        };
         uint32_t ph = 0;
         Place cur{item0, 0}, nxt;
         step(cur, s);
         nxt = cur, step(nxt, C::kProdWarps);
-        Chunk c;
-        if (cur.item < n_items) fetch(c, cur, tile_of(cur));
+        ChunkRows c;
+        if (cur.item < n_items) g.fetch(c, p, cur.kc, tile_of(cur));
         TileInfo tn = tile_of(nxt);
         while (cur.item < n_items) {
             if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(empty + s), ph ^ 1u, abort_flag))) break;
@@ -494,50 +549,12 @@ __global__ void __launch_bounds__(PairCfg::kThreads, 1) k_layer_pair(const __gri
                 }
             } else {
                 if (lane == 0) mbar_arrive(smem_u32(landed + s));
-                // row r0 + 4 i: register i / 8 of lane r0 + 4 (i % 8)
-                if (c.kind == SRC_ITEM) {
-                    bool bad = false;
-#pragma unroll
-                    for (int j = 0; j < 4; ++j)
-                        if (c.v[j] < 0 || (int64_t)c.v[j] >= p.M) {
-                            bad |= lane + 32 * j < c.cnt;
-                            c.v[j] = -1;
-                        }
-                    if (bad && p.check_ids && cur.kc == 0) atomicOr(p.sl.status, AIF_STATUS_BAD_ID);
-#pragma unroll
-                    for (int i = 0; i < 32; ++i) {
-                        const int v = __shfl_sync(0xffffffffu, c.v[i >> 3], r0 + 4 * (i & 7));
-                        cp_async16(dst0 + (uint32_t)(i * 512) + swz[i & 1], c.bp + (size_t)(uint32_t)max(v, 0) * c.row_bytes, v >= 0 ? 16u : 0u);
-                    }
-                } else if (narrow) {
-#pragma unroll 1
-                    for (int i0 = 0; i0 < 32; i0 += 8) {
-                        uint32_t v[8];
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) {
-                            const int row = r0 + 4 * (i0 + i);
-                            v[i] = row < c.cnt ? (uint32_t)__ldg(c.xb + (size_t)row * p.F) : kNoBucket;
-                        }
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) {
-                            const bool on = v[i] != kNoBucket;
-                            cp_async16(dst0 + (uint32_t)((i0 + i) * 512) + swz[i & 1], c.bp + (size_t)(on ? v[i] : 0u) * c.row_bytes, on ? 16u : 0u);
-                        }
-                    }
-                } else {
-                    const uint32_t pick = two && sub >= 4 ? 0x4432u : 0x4410u;   // byte permute: the pair's upper or lower half
-#pragma unroll
-                    for (int i = 0; i < 32; ++i) {
-                        const uint32_t v = __byte_perm((uint32_t)__shfl_sync(0xffffffffu, c.v[i >> 3], r0 + 4 * (i & 7)), 0u, pick);
-                        const bool on = v != kNoBucket;
-                        cp_async16(dst0 + (uint32_t)(i * 512) + swz[i & 1], c.bp + (size_t)(on ? v : 0u) * c.row_bytes, on ? 16u : 0u);
-                    }
-                }
+                g.copy(c, p, dst0, cur.kc == 0);
                 cp_async_commit();
             }
             cur = nxt;
             step(nxt, C::kProdWarps);
-            if (cur.item < n_items) fetch(c, cur, tn);   // these loads are in flight while the copies land
+            if (cur.item < n_items) g.fetch(c, p, cur.kc, tn);   // these loads are in flight while the copies land
             tn = tile_of(nxt);
             if (gathered) {
                 cp_async_wait<0>();
@@ -571,6 +588,297 @@ __global__ void __launch_bounds__(PairCfg::kThreads, 1) k_layer_pair(const __gri
                     tma_load_2d(smem_u32(base + s * C::kStage + kABytes), &tmapB, smem_u32(landed + s), kc * 64, n0);
                     if (++s == kS) s = 0, ph ^= 1u;
                 }
+            }
+        }
+        __syncwarp();
+    }
+
+    // ---- teardown: everybody arrives here, also after an abort; neither CTA leaves while the other may still reach it
+    if (*abort_flag) {
+        if (tid == 0) atomicOr(p.sl.status, AIF_STATUS_TIMEOUT);
+        // let copies and MMAs that are still in flight land before shared memory and TMEM go away
+        const long long t0 = clock64();
+        while (clock64() - t0 < 2000000ll) __nanosleep(1000);
+    }
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync();
+    if (warp == C::kMmaWarp) tmem_dealloc_pair(tmem_base, 512);
+}
+
+// ---- both layers of a two-layer MLP -------------------------------------------------------------------------------
+// Launches of at most one tile per SM, 512 and at most 256 units: the whole MLP of a tile in one kernel.  In the layer kernel
+// 10^4 candidates are 80 items of the first layer on 74 pairs of SMs, two rounds for little more than one, and either
+// layer's start and end (tile look-up, first rows, last accumulators, stores) is as long as its products.  Here a CTA keeps its tile:
+// both 256-column accumulators of the first layer fill its tensor memory, the activations go back there as bf16 (A operand of
+// the second layer) over accumulator columns already read, and nothing but the logits is written.  Products span a pair of CTAs
+// as in the layer kernel (the two tiles may belong to different requests): with whole weight slices per CTA, operand intake
+// (1360 cycles per 64-column chunk at 59 bytes per clock) would bound it, not the products (1024).
+// Roles per CTA (448 threads): 8 epilogue warps (group g: output slice g, later half g of the second layer's units), the MMA warp,
+// 4 gather warps, one per stage, one weight warp.  A stage is a 64-column chunk of the rows and of both slices' weights, later
+// two chunks of the second layer's weights.  The first layer's accumulators start from the bias instead of zero.
+// Tensor memory: accumulators [0, 256) and [256, 512), packed activations [0, 128) and [384, 512), second layer [128, 128 + H2).
+struct MlpCfg {
+    static constexpr int kH1 = 512;
+    static constexpr int kStages = 4, kStage = 3 * kABytes;
+    static constexpr int kMmaWarp = 8, kProdWarp0 = 9, kBWarp = kProdWarp0 + kStages, kThreads = (kBWarp + 1) * 32;
+    static constexpr int kOffMisc = kStages * kStage;
+    // barriers and the tensor-memory slot | bias, output weights [256] | dot products of the upper halves [128]
+    static constexpr size_t kSmem = 1024 + kOffMisc + 256 + (2 * 256 + 128) * 4;
+    static_assert(kSmem <= 227 * 1024, "shared memory");
+};
+struct MlpParams {
+    LayerParams l;   // the first layer's
+    int32_t H2;
+    const float *b2;
+};
+
+__global__ void __launch_bounds__(MlpCfg::kThreads, 1) k_mlp_pair(const __grid_constant__ CUtensorMap tmapA, const __grid_constant__ CUtensorMap tmapW1,
+                                                                  const __grid_constant__ CUtensorMap tmapW2, const __grid_constant__ MlpParams mp)
+{
+    using C = MlpCfg;
+    constexpr int kS = C::kStages;
+    const LayerParams &p = mp.l;
+    extern __shared__ unsigned char smem_dyn[];
+    unsigned char *base = reinterpret_cast<unsigned char *>(((uintptr_t)smem_dyn + 1023) & ~(uintptr_t)1023);
+    uint64_t *bars = reinterpret_cast<uint64_t *>(base + C::kOffMisc);
+    uint64_t *full = bars, *empty = full + kS, *landed = empty + kS, *preset = landed + kS, *acc1 = preset + 1, *h1 = acc1 + 1, *acc2 = h1 + 1;
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(acc2 + 1);
+    volatile uint32_t *abort_flag = tmem_slot + 1;
+    float *bias_s = reinterpret_cast<float *>(base + C::kOffMisc + 256), *wout_s = bias_s + 256, *dot_s = wout_s + 256;
+
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int rank = (int)cluster_rank();   // 0: issues the products
+
+    if (tid == 0) {
+        for (int s = 0; s < kS; ++s) {
+            mbar_init(smem_u32(full + s), 2);      // a gather warp of each CTA (used in the even one)
+            mbar_init(smem_u32(landed + s), 2);    // TMA copies of this CTA: announced by the weight lane and by the gather warp
+            mbar_init(smem_u32(empty + s), 1);
+        }
+        mbar_init(smem_u32(preset), 16);           // the epilogue warps of both CTAs (used in the even one)
+        mbar_init(smem_u32(h1), 16);
+        mbar_init(smem_u32(acc1), 1);
+        mbar_init(smem_u32(acc2), 1);
+        *abort_flag = 0u;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == C::kMmaWarp) tmem_alloc_pair(smem_u32(tmem_slot), 512);
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync();   // the other CTA's barriers exist
+    tc_fence_after();
+    const uint32_t tmem_base = *tmem_slot;
+    grid_dep_launch();
+    const int n_stages = p.n_k + C::kH1 / 128;   // uses of the ring
+    if (warp != C::kBWarp) grid_dep_wait();      // the weights are older than any launch this one may overlap
+
+    if (warp < 8) {
+        // ===================== epilogues: one thread per row in each group =====================
+        const int g = warp >> 2, wq = warp & 3, row = wq * 32 + lane;
+        const uint32_t lane_base = tmem_base + ((uint32_t)(wq * 32) << 16);
+        bool ok = true;
+        auto wait = [&](uint64_t *b) {
+            const bool got = mbar_wait(smem_u32(b), 0u, abort_flag);
+            ok = __all_sync(0xffffffffu, ok && got);
+        };
+        auto arrive_even = [&](uint64_t *b) {
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive_cluster(cluster_addr(smem_u32(b), 0u));
+        };
+        const TileInfo t = decode_tile(p, (int)blockIdx.x, p.sl.n_tiles);
+        {
+            const float4 *pu = reinterpret_cast<const float4 *>(p.sl.slots[t.rq.slot].p_u + 256 * g);
+#pragma unroll 1
+            for (int c = 0; c < 256; c += 32) {
+                uint32_t r[32];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const float4 v = pu[c / 4 + j];
+                    r[4 * j] = __float_as_uint(v.x), r[4 * j + 1] = __float_as_uint(v.y), r[4 * j + 2] = __float_as_uint(v.z), r[4 * j + 3] = __float_as_uint(v.w);
+                }
+                tmem_st32(lane_base + (uint32_t)(256 * g + c), r);
+            }
+            tmem_st_wait();
+            arrive_even(preset);
+        }
+        // a wait that ran out in an earlier kernel of this call left its outputs unwritten: logits computed from them are
+        // replaced by NaN
+        const bool poisoned = (*reinterpret_cast<volatile const uint32_t *>(p.sl.status) & AIF_STATUS_TIMEOUT) != 0u;
+        const bool valid = row < t.cnt;
+        int id = -1;
+        if (g == 0 && valid) id = p.sl.ids[t.pos0 + row];
+        if (tid < mp.H2) bias_s[tid] = mp.b2[tid], wout_s[tid] = __bfloat162float(p.w_out[tid]);
+        named_bar_sync(1, 256);
+        // ---- first layer: slice g, ReLU, 32 accumulator columns -> 16 columns of packed bf16, over accumulator columns already
+        // read (slice 0 upwards, slice 1 downwards: the 256 columns in between become free)
+        wait(acc1);
+        tc_fence_after();
+        if (ok) {
+            uint32_t ra[32], rb[32];
+            const uint32_t col0 = lane_base + (uint32_t)(g * 256);
+            auto finish = [&](const uint32_t (&r)[32], int c) {
+                uint32_t packed[16];
+#pragma unroll
+                for (int q = 0; q < 16; ++q) {
+                    const __nv_bfloat162 h = __hmax2(__floats2bfloat162_rn(__uint_as_float(r[2 * q]), __uint_as_float(r[2 * q + 1])), __float2bfloat162_rn(0.f));
+                    packed[q] = *reinterpret_cast<const uint32_t *>(&h);
+                }
+                tmem_st16(lane_base + (uint32_t)((g ? 384 : 0) + 16 * c), packed);
+            };
+            auto chunk_of = [&](int i) { return g ? 7 - i : i; };
+            tmem_ld32(col0 + (uint32_t)(32 * chunk_of(0)), ra);
+#pragma unroll 1
+            for (int i = 0; i < 8; i += 2) {
+                tmem_ld_wait();
+                tmem_ld32(col0 + (uint32_t)(32 * chunk_of(i + 1)), rb);
+                finish(ra, chunk_of(i));
+                tmem_ld_wait();
+                if (i + 2 < 8) tmem_ld32(col0 + (uint32_t)(32 * chunk_of(i + 2)), ra);
+                finish(rb, chunk_of(i + 1));
+            }
+            tmem_st_wait();
+        }
+        arrive_even(h1);
+        // ---- second layer: half g of the units, bias, ReLU, reduced against w_out
+        wait(acc2);
+        tc_fence_after();
+        float dot = 0.f;
+        if (ok) {
+            const int hn = mp.H2 >> 1;   // a multiple of 32
+            const uint32_t col0 = lane_base + 128u + (uint32_t)(g * hn);
+            float d4[4] = {0.f, 0.f, 0.f, 0.f};
+            uint32_t ra[32], rb[32];
+            auto reduce = [&](const uint32_t (&r)[32], int c0) {
+                const float4 *b4 = reinterpret_cast<const float4 *>(bias_s + g * hn + c0), *w4 = reinterpret_cast<const float4 *>(wout_s + g * hn + c0);
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    const float4 b = b4[q], w = w4[q];
+                    d4[0] = fmaf(fmaxf(__uint_as_float(r[4 * q]) + b.x, 0.f), w.x, d4[0]);
+                    d4[1] = fmaf(fmaxf(__uint_as_float(r[4 * q + 1]) + b.y, 0.f), w.y, d4[1]);
+                    d4[2] = fmaf(fmaxf(__uint_as_float(r[4 * q + 2]) + b.z, 0.f), w.z, d4[2]);
+                    d4[3] = fmaf(fmaxf(__uint_as_float(r[4 * q + 3]) + b.w, 0.f), w.w, d4[3]);
+                }
+            };
+            tmem_ld32(col0, ra);
+#pragma unroll 1
+            for (int c0 = 0; c0 < hn; c0 += 64) {
+                tmem_ld_wait();
+                if (c0 + 32 < hn) tmem_ld32(col0 + (uint32_t)(c0 + 32), rb);
+                reduce(ra, c0);
+                if (c0 + 32 < hn) {
+                    tmem_ld_wait();
+                    if (c0 + 64 < hn) tmem_ld32(col0 + (uint32_t)(c0 + 64), ra);
+                    reduce(rb, c0 + 32);
+                }
+            }
+            dot = (d4[0] + d4[1]) + (d4[2] + d4[3]);
+        }
+        if (g == 1) dot_s[row] = dot;
+        const bool out = named_bar_or(1, 256, !ok);   // also orders dot_s
+        if (g == 0 && valid) {
+            float logit = dot + dot_s[row] + p.b_out[0];
+            if (p.emit_sigmoid) logit = 1.0f / (1.0f + expf(-logit));
+            // no number for an id outside the table, nor for a tile whose inputs never arrived (here or in an earlier kernel of
+            // the call: the status word says so)
+            if (id < 0 || (int64_t)id >= p.M || out || poisoned) logit = __int_as_float(0x7fc00000);
+            p.sl.logits[p.sl.out_index ? (int64_t)p.sl.out_index[t.pos0 + row] : t.pos0 + row] = logit;
+        }
+    } else if (warp == C::kMmaWarp) {
+        if (lane == 0 && rank == 0) {
+            // ===================== MMA issuer =====================
+            constexpr uint32_t idesc1 = umma_idesc_bf16(2 * kTcTile, 256);
+            const uint32_t idesc2 = umma_idesc_bf16(2 * kTcTile, mp.H2);
+            const uint64_t desc0 = umma_desc_sw128(smem_u32(base));
+            bool ok = mbar_wait(smem_u32(preset), 0u, abort_flag);
+#pragma unroll 1
+            for (int i = 0; ok && i < n_stages; ++i) {
+                const int s = i % kS;
+                if (i == p.n_k) {
+                    umma_commit_pair(smem_u32(acc1));
+                    if (!mbar_wait(smem_u32(h1), 0u, abort_flag)) ok = false;
+                }
+                if (!ok || !mbar_wait(smem_u32(full + s), (uint32_t)((i / kS) & 1), abort_flag)) {
+                    ok = false;
+                    break;
+                }
+                fence_proxy_async();   // gathered rows were written by cp.async (generic proxy)
+                tc_fence_after();
+                const uint64_t d = desc0 + (uint64_t)(uint32_t)(s * (C::kStage >> 4));
+                if (i < p.n_k) {
+#pragma unroll
+                    for (int sl = 0; sl < 2; ++sl)
+#pragma unroll
+                        for (int kk = 0; kk < 4; ++kk)
+                            umma_bf16_pair(tmem_base + 256u * sl, d + 2 * kk, d + (uint64_t)((1 + sl) * (kABytes >> 4) + 2 * kk), idesc1, 1u);
+                } else {
+                    const int k0 = 8 * (i - p.n_k);   // sixteens of activations: 8 packed columns each
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) {
+                        const int k16 = k0 + q;
+                        umma_bf16_ts_pair(tmem_base + 128u, tmem_base + (uint32_t)(k16 < 16 ? 8 * k16 : 384 + 8 * (k16 - 16)),
+                                          d + (uint64_t)((1 + (q >> 2)) * (kABytes >> 4) + 2 * (q & 3)), idesc2, k16 > 0 ? 1u : 0u);
+                    }
+                }
+                umma_commit_pair(smem_u32(empty + s));
+            }
+            if (ok) umma_commit_pair(smem_u32(acc2));
+        }
+        __syncwarp();
+    } else if (warp < C::kBWarp) {
+        // ===================== rows: every warp fills the stage of its number (see the layer kernel) =====================
+        const RowGather g(p, lane);
+        const int s = warp - C::kProdWarp0;
+        const uint32_t dst0 = smem_u32(base + s * C::kStage) + (uint32_t)(g.r0 * 128);
+        const TileInfo t = decode_tile(p, (int)blockIdx.x, p.sl.n_tiles);
+        ChunkRows c;
+        if (s < p.n_k) g.fetch(c, p, s, t);
+        uint32_t ph = 0;
+#pragma unroll 1
+        for (int i = s; i < n_stages; i += kS) {
+            if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(empty + s), ph ^ 1u, abort_flag))) break;
+            const bool rows = i < p.n_k, gathered = rows && c.kind != SRC_DENSE;
+            if (lane == 0) {
+                if (rows && !gathered && c.tma_x >= 0) {
+                    mbar_expect_tx(smem_u32(landed + s), (uint32_t)kABytes);
+                    tma_load_2d(smem_u32(base + s * C::kStage), &tmapA, smem_u32(landed + s), c.tma_x, c.tma_y);
+                } else
+                    mbar_arrive(smem_u32(landed + s));
+            }
+            if (gathered) {
+                g.copy(c, p, dst0, i == 0);
+                cp_async_commit();
+            }
+            if (i + kS < p.n_k) g.fetch(c, p, i + kS, t);   // these loads are in flight while the copies land
+            if (gathered) {
+                cp_async_wait<0>();
+                fence_proxy_async();   // written by cp.async (generic proxy), read by the products through the async proxy
+            }
+            __syncwarp();
+            bool ok = true;
+            if (lane == 0) {
+                ok = mbar_wait(smem_u32(landed + s), ph, abort_flag);   // the stage's weights, and a dense chunk's rows
+                if (ok) mbar_arrive_cluster(cluster_addr(smem_u32(full + s), 0u));
+            }
+            if (!__all_sync(0xffffffffu, ok)) break;
+            ph ^= 1u;
+        }
+        cp_async_wait_all();
+    } else {
+        // ===================== weights (TMA): this CTA's half of every slice's rows =====================
+        if (lane == 0) {
+            const int half2 = mp.H2 >> 1;
+#pragma unroll 1
+            for (int i = 0; i < n_stages; ++i) {
+                const int s = i % kS;
+                if (!mbar_wait(smem_u32(empty + s), (uint32_t)((i / kS) & 1) ^ 1u, abort_flag)) break;
+                const bool first = i < p.n_k;
+                mbar_expect_tx(smem_u32(landed + s), first ? 2u * kABytes : 2u * (uint32_t)half2 * 128u);
+#pragma unroll
+                for (int q = 0; q < 2; ++q)
+                    tma_load_2d(smem_u32(base + s * C::kStage + (1 + q) * kABytes), first ? &tmapW1 : &tmapW2, smem_u32(landed + s),
+                                first ? 64 * i : 64 * (2 * (i - p.n_k) + q), first ? 256 * q + 128 * rank : half2 * rank);
             }
         }
         __syncwarp();
@@ -958,6 +1266,7 @@ cudaError_t tc_prepare_context(aif_ctx *ctx)
         if ((e = alloc((void **)&pl->tiles, pl->tiles_cap * sizeof(TileDev))) != cudaSuccess) return e;
     }
     e = cudaFuncSetAttribute(k_layer_pair, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PairCfg::kSmem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_mlp_pair, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MlpCfg::kSmem);
     if (e != cudaSuccess) return e;
     // tensor maps over the packed weights: [H x in_w] bf16, box = 64 columns x n_cols rows, 128-byte swizzle
     EncodeFn enc = encode_fn();
@@ -1244,6 +1553,8 @@ cudaError_t launch_score_tc_scratch(const aif_ctx *ctx, const ScoreLaunch &sl_in
         timing_mark(ctx, "interact", st);
         if (e != cudaSuccess) return e;
     }
+    // two layers of 512 and at most 256 units, all tiles at once on the machine: one kernel
+    const bool whole_mlp = c.n_hidden == 2 && c.hidden[0] == MlpCfg::kH1 && c.hidden[1] <= 256 && c.hidden[1] % 64 == 0 && sl_rows.n_tiles <= 148;
     static const char *names[kMaxHidden] = {"layer1", "layer2", "layer3", "layer4"};
     static const char *range_names[kMaxHidden] = {"aif layer1", "aif layer2", "aif layer3", "aif layer4"};
     for (int k = 0; k < c.n_hidden; ++k) {
@@ -1291,6 +1602,14 @@ cudaError_t launch_score_tc_scratch(const aif_ctx *ctx, const ScoreLaunch &sl_in
                                      CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
             if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
+        }
+        if (whole_mlp) {
+            MlpParams mp{p, c.hidden[1], ctx->b[1]};
+            const cudaError_t e = launch_pdl_pair(k_mlp_pair, dim3((sl_rows.n_tiles + 1) / 2 * 2), dim3(MlpCfg::kThreads), MlpCfg::kSmem, st, tmap_a, pl->tmap_half[0],
+                                                  pl->tmap_half[1], mp);
+            count_launch();
+            timing_mark(ctx, "mlp", st);
+            return e;
         }
         const cudaError_t e = launch_layer(p, sl_rows.n_tiles, pl->tmap_half[k], tmap_out, tmap_a, st);
         timing_mark(ctx, names[k], st);
