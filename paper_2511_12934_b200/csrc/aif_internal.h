@@ -118,6 +118,10 @@ struct ScoreLaunch {
     const int32_t *joins;        // jobs that are the first pieces of split tiles
     int32_t n_jobs;              // upper bound of the number of jobs
     int32_t parts;               // 0 or 1: tiles are not split
+    // 1: the kernel needs nothing of the kernels of its call before it and runs beside them; its first block waits for them before it ends, so
+    // that whoever waits for it has waited for all.  Kernels with such successors let them start only after their own wait: the
+    // earlier calls of the stream are then complete.
+    int32_t late;
     SplitScratch split;
 };
 

@@ -99,10 +99,10 @@ __device__ __forceinline__ TileInfo decode_tile(const LayerParams &p, int tile, 
 // pos becomes the grouped position; F = 0 does nothing else).
 constexpr uint32_t kNoBucket = 0xFFFFu;
 __global__ void __launch_bounds__(256) k_cross_buckets(const int32_t *__restrict__ ids, int64_t total, int64_t M, int F, int B,
-                                                        int b_mask, int mode, uint16_t *__restrict__ xb, int32_t *__restrict__ ids_copy, const SimPlace pl)
+                                                        int b_mask, int mode, uint16_t *__restrict__ xb, int32_t *__restrict__ ids_copy, const SimPlace pl, int late)
 {
+    if (!late) grid_dep_wait();
     grid_dep_launch();
-    grid_dep_wait();
     // A warp takes 32 consecutive candidates: one coalesced read of their ids (128 bytes, also the right size for a read
     // across the bus), then 32 F hashes that depend on nothing else, two per thread and round, leaving as one 4-byte store
     // per thread (an odd number of fields, possible only with embeddings of 64 columns and more, takes one hash per round).
@@ -143,6 +143,7 @@ __global__ void __launch_bounds__(256) k_cross_buckets(const int32_t *__restrict
             else *o = (uint16_t)bk[0];
         }
     }
+    if (late && (blockIdx.x | blockIdx.y) == 0) grid_dep_wait();
 }
 
 // Tile table of a launch over several requests: one thread per tile does the search of the request table that every
@@ -928,11 +929,14 @@ __global__ void __launch_bounds__(256) k_bea_x(ModelDev md, ScoreLaunch sl, __nv
     const int d = md.d, nb = md.n_bridge, tid = threadIdx.x;
     __nv_bfloat16 *V = reinterpret_cast<__nv_bfloat16 *>(smem_raw);          // [nb][d]
     float *w = reinterpret_cast<float *>(smem_raw + (size_t)nb * d * 2);     // [kBeaRows][nb]
+    if (!sl.late) grid_dep_wait();
     grid_dep_launch();
-    grid_dep_wait();
     const BlockTile t = block_tile(sl, blockIdx.x, md.mini_batch);
     const int first = blockIdx.y * kBeaRows, cnt = min(kBeaRows, t.cnt - first);
-    if (cnt <= 0) return;
+    if (cnt <= 0) {
+        if (sl.late && (blockIdx.x | blockIdx.y) == 0) grid_dep_wait();
+        return;
+    }
     const int64_t pos0 = t.pos0 + first;
     const uint4 *Vg = reinterpret_cast<const uint4 *>(sl.slots[t.slot].V);
     for (int i = tid; i < nb * d / 8; i += 256) reinterpret_cast<uint4 *>(V)[i] = Vg[i];
@@ -962,6 +966,7 @@ __global__ void __launch_bounds__(256) k_bea_x(ModelDev md, ScoreLaunch sl, __nv
         for (int q = 0; q < 4; ++q) oh[q] = __floats2bfloat162_rn(acc[2 * q], acc[2 * q + 1]);
         *reinterpret_cast<uint4 *>(X + (size_t)(pos0 + c) * x_stride + col + k) = o;
     }
+    if (sl.late && (blockIdx.x | blockIdx.y) == 0) grid_dep_wait();
 }
 
 // ---- interaction blocks that feed dense columns (CUDA cores; one warp per candidate) ---------------------------
@@ -1489,7 +1494,8 @@ cudaError_t launch_score_tc_scratch(const aif_ctx *ctx, const ScoreLaunch &sl_in
         sl.tiles = (const TileDev *)sc.tiles;
     }
     const int F = (c.blocks & AIF_BLK_CROSS) ? c.F : 0;
-    if (F > 0 || place.where) {
+    auto buckets = [&](int late) -> cudaError_t {
+        if (F == 0 && !place.where) return cudaSuccess;
         StageRange range("aif buckets");
         const int64_t n = sl.total;   // a warp per 32 candidates
         const int grid = (int)((n + 255) / 256 < 148 * 16 ? (n + 255) / 256 : 148 * 16);
@@ -1498,19 +1504,27 @@ cudaError_t launch_score_tc_scratch(const aif_ctx *ctx, const ScoreLaunch &sl_in
         const int rounds = F == 0 ? 1 : F & 1 ? F : F / 2, want_y = sl.ids_copy ? 1 : 296 / grid;
         const int grid_y = want_y < 1 ? 1 : want_y > 8 ? (rounds < 8 ? rounds : 8) : want_y > rounds ? rounds : want_y;
         cudaError_t e = launch_pdl(k_cross_buckets, dim3(grid, grid_y), dim3(256), 0, st, sl.ids, sl.total, c.M, F, c.B,
-                                   (c.B & (c.B - 1)) == 0 ? c.B - 1 : -1, c.bucket_mode, (uint16_t *)sc.xb, sl.ids_copy, place);
+                                   (c.B & (c.B - 1)) == 0 ? c.B - 1 : -1, c.bucket_mode, (uint16_t *)sc.xb, sl.ids_copy, place, late);
         if (sl.ids_copy) sl.ids = sl.ids_copy;
         if (place.where) sl.ids = place.ids;
         count_launch();
         timing_mark(ctx, "buckets", st);
-        if (e != cudaSuccess) return e;
-    }
+        return e;
+    };
+    const bool att_tc = ctx->tc_att_plan != nullptr;
+    const int lsh_blocks = c.blocks & (AIF_BLK_LSH_DIN | AIF_BLK_SIMTIER);
+    const bool lsh_tc = lsh_blocks && ctx->tc_lsh_plan != nullptr;
+    // Attention, bridge columns, LSH and buckets need nothing of each other: behind the first one the others run beside it, on the SMs
+    // it leaves idle (78 tiles are 78 CTAs of an attention kernel that fills an SM with one) and in its tail.  The buckets come
+    // first where they bring the ids.
+    const bool buckets_first = place.where || sl.ids_copy || !(att_tc || lsh_tc);
+    cudaError_t eb = buckets_first ? buckets(0) : cudaSuccess;
+    if (eb != cudaSuccess) return eb;
     // What does not depend on the category takes the grouped candidates request by request, in whole tiles: the groups of a request
     // are its positions, in another order.  By the groups' tiles the layers ran on rows that were mostly padding (20 candidates per
     // category: 800 tiles instead of 130).
     ScoreLaunch sl_rows = sl;
     if (c.n_categories > 0) sl_rows.n_tiles = sl_in.n_tiles, sl_rows.n_tiles_dev = nullptr, sl_rows.tiles = sl.reqs ? (const TileDev *)sc.tiles : nullptr;
-    const bool att_tc = ctx->tc_att_plan != nullptr;
     // few tiles with many keys: their keys over several CTAs each (the table of jobs does it where categories are on)
     if (!sl.jobs) sl.parts = split_parts(sl.n_tiles, (sl.max_L + (c.d == 128 ? 127 : 63)) / (c.d == 128 ? 128 : 64), sl.split.slots);
     if (att_tc) {
@@ -1519,8 +1533,20 @@ cudaError_t launch_score_tc_scratch(const aif_ctx *ctx, const ScoreLaunch &sl_in
         timing_mark(ctx, "attention", st);
         if (e != cudaSuccess) return e;
     }
-    const int lsh_blocks = c.blocks & (AIF_BLK_LSH_DIN | AIF_BLK_SIMTIER);
-    const bool lsh_tc = lsh_blocks && ctx->tc_lsh_plan != nullptr;
+    int late = att_tc;
+    auto bea = [&]() -> cudaError_t {
+        if (!(c.blocks & AIF_BLK_BEA)) return cudaSuccess;
+        StageRange range("aif bea");
+        ScoreLaunch sl_bea = sl_rows;
+        sl_bea.late = late;
+        const size_t smem = (size_t)c.n_bridge * c.d * 2 + (size_t)kBeaRows * c.n_bridge * 4;
+        cudaError_t e = launch_pdl(k_bea_x, dim3(sl_rows.n_tiles, kTcTile / kBeaRows), dim3(256), smem, st, md, sl_bea, (__nv_bfloat16 *)sc.X, pl->x_cols,
+                                   (c.blocks & AIF_BLK_ATT) ? c.d : 0);
+        count_launch();
+        timing_mark(ctx, "bea", st);
+        return e;
+    };
+    if (att_tc && (eb = bea()) != cudaSuccess) return eb;
     if (lsh_tc) {
         // columns of X: [ att | v_bea | lsh_din | simtier (64) ], enabled blocks only
         int col = 0;
@@ -1530,20 +1556,16 @@ cudaError_t launch_score_tc_scratch(const aif_ctx *ctx, const ScoreLaunch &sl_in
         if (c.blocks & AIF_BLK_LSH_DIN) col += c.d;
         const int x_tier = (c.blocks & AIF_BLK_SIMTIER) ? col : -1;
         StageRange range("aif lsh");
-        cudaError_t e = launch_lsh_tc(ctx, sl, st, sc.X, pl->x_cols, sc.rows, x_din, x_tier);
+        ScoreLaunch sl_lsh = sl;
+        sl_lsh.late = late && !sl.jobs && sl.parts <= 1;   // (pieces of keys share the records that the attention's join reads)
+        cudaError_t e = launch_lsh_tc(ctx, sl_lsh, st, sc.X, pl->x_cols, sc.rows, x_din, x_tier);
         timing_mark(ctx, "lsh", st);
         if (e != cudaSuccess) return e;
+        late = 1;
     }
     const bool need_att = (c.blocks & AIF_BLK_ATT) && !att_tc, need_lsh = lsh_blocks && !lsh_tc;
-    if (c.blocks & AIF_BLK_BEA) {
-        StageRange range("aif bea");
-        const size_t smem = (size_t)c.n_bridge * c.d * 2 + (size_t)kBeaRows * c.n_bridge * 4;
-        cudaError_t e = launch_pdl(k_bea_x, dim3(sl_rows.n_tiles, kTcTile / kBeaRows), dim3(256), smem, st, md, sl_rows, (__nv_bfloat16 *)sc.X, pl->x_cols,
-                                   (c.blocks & AIF_BLK_ATT) ? c.d : 0);
-        count_launch();
-        timing_mark(ctx, "bea", st);
-        if (e != cudaSuccess) return e;
-    }
+    if (!att_tc && (eb = bea()) != cudaSuccess) return eb;
+    if (!buckets_first && (eb = buckets(late)) != cudaSuccess) return eb;
     if (need_att || need_lsh) {
         StageRange range("aif interact");
         const size_t smem = (size_t)8 * c.d * 4 + 64 * 4 + 128 * 4;
