@@ -229,7 +229,7 @@ struct aif_ctx {
     aif_stats stats{};
     mutable aif::KernelTiming timing;
     std::vector<void *> allocations;
-    aif::SplitScratch split{}, split_user{};   // partial results of split tiles: scoring launches, user-side self-attention
+    aif::SplitScratch split{}, split_lsh{}, split_user{};   // partial results of split tiles: scoring launches (LSH beside an attention), user-side self-attention
 };
 
 namespace aif {
@@ -267,6 +267,19 @@ int simt_tiles_for(const aif_ctx *ctx, int n);
 // user side (aif_user.cu)
 cudaError_t launch_user_network(const aif_ctx *ctx, HostSlot &hs, int slot_index, const aif_user_inputs *in, int L, cudaStream_t st);
 
+// Puts the pieces of a launch's tiles together (after the attention or LSH kernel of a split launch): rows into columns
+// [col, col + d) of X (col < 0: none), tier counts into 64 columns from x_tier on (x_tier < 0: none).
+// d == 0: nothing to join.
+struct JoinParams {
+    ScoreLaunch sl;
+    __nv_bfloat16 *X;
+    int64_t M;
+    int32_t x_stride, col, x_tier, n_tiers, d, mini_batch;
+    int32_t attention;          // rows are divided by their sums; else multiplied by row_scale (and divided by the keys: row_mean)
+    float row_scale;
+    int32_t row_mean, tier_mean;
+};
+
 // tensor-core path (aif_tc.cu)
 bool tc_supported(const aif_config &cfg);
 cudaError_t tc_prepare_context(aif_ctx *ctx);
@@ -278,13 +291,14 @@ void tc_att_destroy(aif_ctx *ctx);
 // eq. 2's attention rows softmax(S S^T / sqrt(d)) S of one user state with the same kernel (queries = the sequence rows);
 // *rows_out: [L x d] bf16 in scratch of the attention plan, valid until the next call
 cudaError_t launch_self_att_tc(const aif_ctx *ctx, int slot_index, int L, cudaStream_t st, const void **rows_out);
-cudaError_t launch_att_tc(const aif_ctx *ctx, const ScoreLaunch &sl, cudaStream_t st, void *X, int x_stride, size_t x_rows);
+// (a split launch leaves its join to the caller)
+cudaError_t launch_att_tc(const aif_ctx *ctx, const ScoreLaunch &sl, cudaStream_t st, void *X, int x_stride, size_t x_rows, JoinParams &join);
 // LSH similarity, LSH-DIN and SimTier on the tensor cores (aif_tc_lsh.cu)
 bool tc_lsh_supported(const aif_config &cfg);
 cudaError_t tc_lsh_prepare(aif_ctx *ctx);
 void tc_lsh_destroy(aif_ctx *ctx);
 cudaError_t launch_lsh_tc(const aif_ctx *ctx, const ScoreLaunch &sl, cudaStream_t st, void *X, int x_stride, size_t x_rows, int x_din,
-                          int x_tier);
+                          int x_tier, JoinParams &join);
 // category sub-sequences (aif_sim.cu): the user-side grouping of a sequence, and the grouping of a launch's candidates by
 // (request, category) into tiles
 size_t sim_grouped_rows(int L_max, int n_categories);
@@ -303,17 +317,6 @@ struct SimPlace {
 cudaError_t sim_group_candidates(const aif_ctx *ctx, ScoreLaunch &sl, SimPlace &place, TileDev *row_tiles, cudaStream_t st);
 // pieces per tile that even a launch of n_tiles tiles of `blocks` key blocks out over the SMs (aif_tc.cu)
 int split_parts(int n_tiles, int blocks, int slots);
-// Puts the pieces of a launch's tiles together (after the attention or LSH kernel of a split launch): rows into columns
-// [col, col + d) of X (col < 0: none), tier counts into 64 columns from x_tier on (x_tier < 0: none).
-struct JoinParams {
-    ScoreLaunch sl;
-    __nv_bfloat16 *X;
-    int64_t M;
-    int32_t x_stride, col, x_tier, n_tiers, d, mini_batch;
-    int32_t attention;          // rows are divided by their sums; else multiplied by row_scale (and divided by the keys: row_mean)
-    float row_scale;
-    int32_t row_mean, tier_mean;
-};
 cudaError_t launch_join_pieces(const JoinParams &p, cudaStream_t st);
 // whole scoring pass of a tile in one CTA (aif_tc_fused.cu); the tensor maps it shares with the other kernels
 bool tc_fused_supported(const aif_config &cfg);

@@ -1104,14 +1104,15 @@ __device__ __forceinline__ void join_tile(const JoinParams &p, const KeyTile &t,
 // 1000 items 13.7 -> 23 us); here a tile is read by as many SMs as there are columns to share out.
 __global__ void __launch_bounds__(256) k_join_pieces(const JoinParams p)
 {
+    if (!p.sl.late) grid_dep_wait();
     grid_dep_launch();
-    grid_dep_wait();
     const int n_y = (p.col >= 0 ? p.d / kJoinCols : 0) + (p.x_tier >= 0 ? 1 : 0);
     const int n_items = (p.sl.jobs ? p.sl.n_jobs_dev[1] : p.sl.n_tiles) * n_y;
     for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
         const int tile = item / n_y, y = item - tile * n_y, job = p.sl.jobs ? p.sl.joins[tile] : tile * p.sl.parts;
         join_tile(p, p.d == 128 ? key_tile<128, true>(p.sl, job, p.mini_batch) : key_tile<64, true>(p.sl, job, p.mini_batch), y);
     }
+    if (p.sl.late && blockIdx.x == 0) grid_dep_wait();
 }
 
 // Self-test of the bounded wait: one thread waits, with a short limit, on an mbarrier that nobody arrives on.  The wait
@@ -1301,6 +1302,7 @@ cudaError_t tc_prepare_context(aif_ctx *ctx)
         return cudaSuccess;
     };
     if (key_kernels && (e = take_split(ctx->split, kSplitSlots, (c.blocks & AIF_BLK_SIMTIER) != 0)) != cudaSuccess) return e;
+    if (tc_att_supported(c) && tc_lsh_supported(c) && (e = take_split(ctx->split_lsh, kSplitSlots, (c.blocks & AIF_BLK_SIMTIER) != 0)) != cudaSuccess) return e;
     if (tc_att_supported(c) && (e = take_split(ctx->split_user, kSplitSlotsUser, false)) != cudaSuccess) return e;
     if (tc_att_supported(c) && (e = tc_att_prepare(ctx)) != cudaSuccess) return e;
     if (tc_fused_supported(c) && (e = tc_fused_prepare(ctx)) != cudaSuccess) return e;
@@ -1527,9 +1529,10 @@ cudaError_t launch_score_tc_scratch(const aif_ctx *ctx, const ScoreLaunch &sl_in
     if (c.n_categories > 0) sl_rows.n_tiles = sl_in.n_tiles, sl_rows.n_tiles_dev = nullptr, sl_rows.tiles = sl.reqs ? (const TileDev *)sc.tiles : nullptr;
     // few tiles with many keys: their keys over several CTAs each (the table of jobs does it where categories are on)
     if (!sl.jobs) sl.parts = split_parts(sl.n_tiles, (sl.max_L + (c.d == 128 ? 127 : 63)) / (c.d == 128 ? 128 : 64), sl.split.slots);
+    JoinParams join_att{}, join_lsh{};
     if (att_tc) {
         StageRange range("aif attention");
-        cudaError_t e = launch_att_tc(ctx, sl, st, sc.X, pl->x_cols, sc.rows);
+        cudaError_t e = launch_att_tc(ctx, sl, st, sc.X, pl->x_cols, sc.rows, join_att);
         timing_mark(ctx, "attention", st);
         if (e != cudaSuccess) return e;
     }
@@ -1557,11 +1560,18 @@ cudaError_t launch_score_tc_scratch(const aif_ctx *ctx, const ScoreLaunch &sl_in
         const int x_tier = (c.blocks & AIF_BLK_SIMTIER) ? col : -1;
         StageRange range("aif lsh");
         ScoreLaunch sl_lsh = sl;
-        sl_lsh.late = late && !sl.jobs && sl.parts <= 1;   // (pieces of keys share the records that the attention's join reads)
-        cudaError_t e = launch_lsh_tc(ctx, sl_lsh, st, sc.X, pl->x_cols, sc.rows, x_din, x_tier);
+        sl_lsh.late = late;
+        if (att_tc && sc.split) sl_lsh.split = ctx->split_lsh;   // records of its own: the attention's are not joined yet
+        cudaError_t e = launch_lsh_tc(ctx, sl_lsh, st, sc.X, pl->x_cols, sc.rows, x_din, x_tier, join_lsh);
         timing_mark(ctx, "lsh", st);
         if (e != cudaSuccess) return e;
         late = 1;
+    }
+    // the pieces of keys: the first join waits for both kernels, the second one runs beside it
+    if (join_att.d && (eb = launch_join_pieces(join_att, st)) != cudaSuccess) return eb;
+    if (join_lsh.d) {
+        join_lsh.sl.late = join_att.d != 0;
+        if ((eb = launch_join_pieces(join_lsh, st)) != cudaSuccess) return eb;
     }
     const bool need_att = (c.blocks & AIF_BLK_ATT) && !att_tc, need_lsh = lsh_blocks && !lsh_tc;
     if (!att_tc && (eb = bea()) != cudaSuccess) return eb;

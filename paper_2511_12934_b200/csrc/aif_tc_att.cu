@@ -702,7 +702,7 @@ static cudaError_t encode_x_map(CUtensorMap *m, void *X, int x_stride, size_t ro
 // One CTA per SM walking over its tiles hides a tile's query gather and output behind its neighbours' key blocks: 22 k against
 // 31 k cycles per 8-block tile, which outweighs the static assignment's rounding (8.5 tiles per SM cost 9 tile times) as soon as
 // some SM has two tiles.
-static cudaError_t run_att(int d, const AttParams &p, const CUtensorMap &ts, const CUtensorMap &tx, cudaStream_t st)
+static cudaError_t run_att(int d, const AttParams &p, const CUtensorMap &ts, const CUtensorMap &tx, JoinParams &j, cudaStream_t st)
 {
     const ScoreLaunch &sl = p.sl;
     const bool split = sl.jobs || sl.parts > 1;
@@ -714,13 +714,13 @@ static cudaError_t run_att(int d, const AttParams &p, const CUtensorMap &ts, con
     if (d == 128) e = split ? go(k_att_tc<128, 128, true>, C1::kThreads, C1::kSmem) : go(k_att_tc<128, 128, false>, C1::kThreads, C1::kSmem);
     else e = split ? go(k_att_tc<256, 64, true>, C2::kThreads, C2::kSmem) : go(k_att_tc<256, 64, false>, C2::kThreads, C2::kSmem);
     count_launch();
+    j = JoinParams{};
     if (e != cudaSuccess || !split) return e;
-    JoinParams j{};
     j.sl = sl, j.X = p.X, j.M = p.M, j.x_stride = p.x_stride, j.col = 0, j.x_tier = -1, j.d = d, j.mini_batch = p.mini_batch, j.attention = 1;
-    return launch_join_pieces(j, st);
+    return cudaSuccess;
 }
 
-cudaError_t launch_att_tc(const aif_ctx *ctx, const ScoreLaunch &sl, cudaStream_t st, void *X, int x_stride, size_t x_rows)
+cudaError_t launch_att_tc(const aif_ctx *ctx, const ScoreLaunch &sl, cudaStream_t st, void *X, int x_stride, size_t x_rows, JoinParams &join)
 {
     const aif_config &c = ctx->cfg;
     const AttPlan *pl = reinterpret_cast<const AttPlan *>(ctx->tc_att_plan);
@@ -732,7 +732,7 @@ cudaError_t launch_att_tc(const aif_ctx *ctx, const ScoreLaunch &sl, cudaStream_
     p.x_stride = x_stride, p.X = (__nv_bfloat16 *)X;
     p.scale_log2 = 1.4426950408889634f / sqrtf((float)c.d);
     p.q_norm = ctx->e_norm;
-    return run_att(c.d, p, sl.grouped ? pl->tmap_g : pl->tmap, tmap_x, st);
+    return run_att(c.d, p, sl.grouped ? pl->tmap_g : pl->tmap, tmap_x, join, st);
 }
 
 cudaError_t launch_self_att_tc(const aif_ctx *ctx, int slot_index, int L, cudaStream_t st, const void **rows_out)
@@ -755,7 +755,9 @@ cudaError_t launch_self_att_tc(const aif_ctx *ctx, int slot_index, int L, cudaSt
     cudaError_t ex = encode_x_map(&tmap_x, pl->self_rows, c.d, (size_t)c.L_max + kTcTile);
     if (ex != cudaSuccess) return ex;
     *rows_out = pl->self_rows;
-    return run_att(c.d, p, pl->tmap, tmap_x, st);
+    JoinParams join;
+    ex = run_att(c.d, p, pl->tmap, tmap_x, join, st);
+    return ex != cudaSuccess || join.d == 0 ? ex : launch_join_pieces(join, st);
 }
 
 }  // namespace aif

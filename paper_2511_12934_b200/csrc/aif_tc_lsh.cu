@@ -764,7 +764,7 @@ void tc_lsh_destroy(aif_ctx *ctx)
 // LSH-DIN rows into columns [x_din, x_din + d) and SimTier rows into [x_tier, x_tier + 64) of X; a negative column turns
 // that output off.
 cudaError_t launch_lsh_tc(const aif_ctx *ctx, const ScoreLaunch &sl, cudaStream_t st, void *X, int x_stride, size_t x_rows, int x_din,
-                          int x_tier)
+                          int x_tier, JoinParams &j)
 {
     const aif_config &c = ctx->cfg;
     const LshPlan *pl = reinterpret_cast<const LshPlan *>(ctx->tc_lsh_plan);
@@ -793,11 +793,11 @@ cudaError_t launch_lsh_tc(const aif_ctx *ctx, const ScoreLaunch &sl, cudaStream_
     if (c.d == 128) e = split ? go(k_lsh_tc<128, 128, true>, C1::kThreads, C1::kSmem) : go(k_lsh_tc<128, 128, false>, C1::kThreads, C1::kSmem);
     else e = split ? go(k_lsh_tc<256, 64, true>, C2::kThreads, C2::kSmem) : go(k_lsh_tc<256, 64, false>, C2::kThreads, C2::kSmem);
     count_launch();
+    j = JoinParams{};
     if (e != cudaSuccess || !split) return e;
-    JoinParams j{};
     j.sl = sl, j.X = (__nv_bfloat16 *)X, j.M = c.M, j.x_stride = x_stride, j.col = x_din, j.x_tier = x_tier, j.n_tiers = p.n_tiers, j.d = c.d;
     j.mini_batch = c.mini_batch, j.row_scale = 0.5f / (float)c.d, j.row_mean = p.din_mean, j.tier_mean = p.tier_mean;
-    return launch_join_pieces(j, st);
+    return cudaSuccess;
 }
 
 }  // namespace aif
