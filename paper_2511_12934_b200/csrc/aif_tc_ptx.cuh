@@ -304,6 +304,15 @@ __device__ __forceinline__ void umma_commit_pair(uint32_t bar)
                  : "memory");
 }
 
+// Tile copy of a pair of CTAs: into this CTA's shared memory, completion counted by a barrier of either one (cluster address).
+__device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap *tm, uint32_t cluster_bar, int c0, int c1)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];" ::"r"(dst),
+        "l"(tm), "r"(cluster_bar), "r"(c0), "r"(c1)
+        : "memory");
+}
+
 // 32 lanes x 32 consecutive fp32 columns: thread = lane (row), register j = column j.
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32])
 {

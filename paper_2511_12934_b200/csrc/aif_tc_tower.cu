@@ -3,14 +3,17 @@
 // of the layer kernel the call is bound by the hidden activations' trip through HBM (512 B written and read per item
 // against 1.25 KB of input and output); here they never leave the SM.
 //
-// Persistent: a CTA walks over pairs of 128-row tiles; both tiles of a pair are fed from the same weight chunks, which
-// halves the weight bytes an SM takes in per item.  320 threads:
-//   warps 0-7  two groups of four warps, group g = tile g of the pair, one thread per row.  After layer 1: bias, ReLU,
+// Persistent, on CTA pairs (cta_group::2): an item is a pair of 128-row tiles, one per CTA, and every product spans both, so that a
+// CTA takes in half of the weights (288 KB per item and CTA at dI = 512, hI = 256, d = 128: 4.9 k cycles at 59 bytes per
+// clock, for 5.1 k cycles of products).  A tile needs half of tensor memory, so items alternate between two buffers and the
+// epilogues of one run under the products of the next; with two tiles per CTA, which the weights' intake asked for without the
+// pair, tensor memory was full and both epilogues were exposed (19 k cycles per two tiles).  262143 rows: 93 -> XX us.  320 threads:
+//   warps 0-7  two groups of four warps, group g = the items of buffer g, one thread per row.  After layer 1: bias, ReLU,
 //              bf16, packed back into tensor memory over accumulator columns already read (A operand of layer 2).
 //              After layer 2: bias, bf16, through a staging slab and a TMA tile store into the output rows.
-//   warp 8     allocates tensor memory; one lane issues tcgen05.mma
-//   warp 9     one lane streams the raw rows (two 128 x 64 boxes per K chunk) and the weights with TMA
-// Tensor memory per tile g: layer-1 accumulator [256 g, 256 g + hI), packed activations [256 g, 256 g + hI / 2), layer-2
+//   warp 8     allocates tensor memory; the even CTA's lane issues tcgen05.mma: layer 1 of an item, in the middle of it layer 2 of the one before
+//   warp 9     one lane streams the raw rows and this CTA's half of the weights with TMA, a 64-column chunk of both per stage
+// Tensor memory of buffer g: layer-1 accumulator [256 g, 256 g + hI), packed activations [256 g, 256 g + hI / 2), layer-2
 // accumulator [256 g + 128, 256 g + 128 + d).  Shapes: dI a multiple of 64; hI in {64, 128, 192, 256}; d <= 128, a
 // multiple of 32.  Every wait is bounded (AIF_STATUS_TIMEOUT on expiry, tensor memory freed, normal return).
 #include <cuda.h>
@@ -23,12 +26,12 @@ namespace aif {
 namespace {
 
 constexpr int kTThreads = 320, kTMmaWarp = 8;   // warp 9 streams rows and weights
-constexpr int kTStagesA = 3, kTStagesB = 3, kTAStage = 32768, kTBStage = 32768;
-constexpr int kTOffB = kTStagesA * kTAStage, kTOffSlab = kTOffB + kTStagesB * kTBStage, kTOffMisc = kTOffSlab + 8 * 2048;
+constexpr int kTStages = 6, kTStage = 32768;    // 128 rows | up to 128 weight rows, 64 columns
+constexpr int kTOffSlab = kTStages * kTStage, kTOffMisc = kTOffSlab + 8 * 2048;
 constexpr size_t kTSmem = 1024 + kTOffMisc + 2048;
 
-enum { TB_FULL_A = 0, TB_EMPTY_A = TB_FULL_A + kTStagesA, TB_FULL_B = TB_EMPTY_A + kTStagesA, TB_EMPTY_B = TB_FULL_B + kTStagesB,
-       TB_ACC1 = TB_EMPTY_B + kTStagesB, TB_H_FULL, TB_ACC2, TB_TM_FREE, TB_COUNT };
+enum { TB_FULL = 0, TB_EMPTY = TB_FULL + kTStages, TB_ACC1 = TB_EMPTY + kTStages, TB_H_FULL = TB_ACC1 + 2, TB_ACC2 = TB_H_FULL + 2, TB_TM_FREE = TB_ACC2 + 2,
+       TB_COUNT = TB_TM_FREE + 2 };
 
 struct TowerParams {
     int64_t n;            // rows
@@ -45,32 +48,42 @@ __global__ void __launch_bounds__(kTThreads, 1) k_item_tower_tc(const __grid_con
 {
     extern __shared__ unsigned char smem_dyn[];
     unsigned char *base = reinterpret_cast<unsigned char *>(((uintptr_t)smem_dyn + 1023) & ~(uintptr_t)1023);
-    unsigned char *smA = base, *smB = base + kTOffB, *slabs = base + kTOffSlab;
+    unsigned char *slabs = base + kTOffSlab;
     uint64_t *bars = reinterpret_cast<uint64_t *>(base + kTOffMisc);
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + TB_COUNT);
     volatile uint32_t *abort_flag = tmem_slot + 1;
     float *b0_s = reinterpret_cast<float *>(tmem_slot + 4), *b1_s = b0_s + 256;   // [256], [128]
     auto bar = [&](int i) { return smem_u32(bars + i); };
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int rank = (int)cluster_rank(), item0 = (int)(blockIdx.x >> 1), item_step = (int)(gridDim.x >> 1);
+    auto arrive_even = [&](int i) {   // one per warp
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cluster(cluster_addr(bar(i), 0u));
+    };
 
     if (tid == 0) {
-        for (int s = 0; s < kTStagesA; ++s) mbar_init(bar(TB_FULL_A + s), 1), mbar_init(bar(TB_EMPTY_A + s), 1);
-        for (int s = 0; s < kTStagesB; ++s) mbar_init(bar(TB_FULL_B + s), 1), mbar_init(bar(TB_EMPTY_B + s), 1);
-        mbar_init(bar(TB_ACC1), 1);
-        mbar_init(bar(TB_H_FULL), 256);
-        mbar_init(bar(TB_ACC2), 1);
-        mbar_init(bar(TB_TM_FREE), 256);
+        for (int s = 0; s < kTStages; ++s) mbar_init(bar(TB_FULL + s), 1), mbar_init(bar(TB_EMPTY + s), 1);   // (full: used in the even CTA)
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(bar(TB_ACC1 + b), 1);
+            mbar_init(bar(TB_H_FULL + b), 8);    // the group's warps of both CTAs (used in the even one)
+            mbar_init(bar(TB_ACC2 + b), 1);
+            mbar_init(bar(TB_TM_FREE + b), 8);
+        }
         *abort_flag = 0u;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == kTMmaWarp) tmem_alloc(smem_u32(tmem_slot), 512);
+    if (warp == kTMmaWarp) tmem_alloc_pair(smem_u32(tmem_slot), 512);
     tc_fence_before();
     __syncthreads();
+    cluster_sync();   // the other CTA's barriers exist
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
     grid_dep_launch();
     grid_dep_wait();
-    const int n_k2 = p.hI >> 6;
+    // layer 2 of an item comes in the middle of the next one's layer 1: by then its activations are packed, and its output leaves
+    // under the other half (after the whole of it: 9.0 k cycles per item, 2.3 k of them waiting for the output)
+    const int n_k2 = p.hI >> 6, mid = p.n_k1 >> 1;
 
     if (warp < 8) {
         // ===================== epilogues =====================
@@ -87,11 +100,12 @@ __global__ void __launch_bounds__(kTThreads, 1) k_item_tower_tc(const __grid_con
             ok = __all_sync(0xffffffffu, got);
         };
         int it = 0;
-        for (int pair = blockIdx.x; pair < p.n_pairs; pair += gridDim.x, ++it) {
-            const uint32_t ph = (uint32_t)(it & 1);
-            const int64_t row0 = ((int64_t)pair * 2 + g) * kTcTile;   // first row of this group's tile
+        for (int item = item0; item < p.n_pairs; item += item_step, ++it) {
+            if ((it & 1) != g) continue;
+            const uint32_t ph = (uint32_t)((it >> 1) & 1);
+            const int64_t row0 = ((int64_t)item * 2 + rank) * kTcTile;   // first row of this CTA's tile
             // ---- after layer 1: bias, ReLU, 32 columns -> 16 packed columns over columns already read
-            wait(TB_ACC1, ph);
+            wait(TB_ACC1 + g, ph);
             tc_fence_after();
             if (!ok) break;
             {
@@ -136,10 +150,9 @@ __global__ void __launch_bounds__(kTThreads, 1) k_item_tower_tc(const __grid_con
                 }
                 tmem_st_wait();
             }
-            tc_fence_before();
-            mbar_arrive(bar(TB_H_FULL));
+            arrive_even(TB_H_FULL + g);
             // ---- after layer 2: bias, bf16, out
-            wait(TB_ACC2, ph);
+            wait(TB_ACC2 + g, ph);
             tc_fence_after();
             if (!ok) break;
             const bool whole = row0 + wq * 32 + 32 <= p.n;
@@ -154,10 +167,7 @@ __global__ void __launch_bounds__(kTThreads, 1) k_item_tower_tc(const __grid_con
 #pragma unroll
                 for (int j = 0; j < 4; ++j) bias2[j] = *reinterpret_cast<const uint64_t *>(b1_s + c0 + 8 * j + 2 * l4);
                 tmem_ld_wait();
-                if (c0 + 32 >= p.d) {   // the accumulators of this pair are in registers: the next pair may overwrite them
-                    tc_fence_before();
-                    mbar_arrive(bar(TB_TM_FREE));
-                }
+                if (c0 + 32 >= p.d) arrive_even(TB_TM_FREE + g);   // the accumulators are in registers: the buffer's next item may overwrite them
                 if (lane == 0) bulk_wait_read<0>();   // the store that last read the slab is done with it
                 __syncwarp();
 #pragma unroll
@@ -207,88 +217,98 @@ __global__ void __launch_bounds__(kTThreads, 1) k_item_tower_tc(const __grid_con
         if (lane == 0) bulk_wait<0>();
     } else if (warp == kTMmaWarp) {
         // ===================== MMA issuer =====================
-        if (lane == 0) {
-            const uint32_t idesc1 = umma_idesc_bf16(kTcTile, p.hI), idesc2 = umma_idesc_bf16(kTcTile, p.d);
-            int sa = 0, sb = 0, it = 0;
-            uint32_t pha = 0, phb = 0;
+        if (lane == 0 && rank == 0) {
+            const uint32_t idesc1 = umma_idesc_bf16(2 * kTcTile, p.hI), idesc2 = umma_idesc_bf16(2 * kTcTile, p.d);
+            const uint64_t desc0 = umma_desc_sw128(smem_u32(base));
+            int s = 0;
+            uint32_t ph = 0;
+            auto stage = [&](uint64_t &d) {
+                if (!mbar_wait(bar(TB_FULL + s), ph, abort_flag)) return false;
+                tc_fence_after();
+                d = desc0 + (uint64_t)(uint32_t)(s * (kTStage >> 4));
+                return true;
+            };
+            auto release = [&] {
+                umma_commit_pair(bar(TB_EMPTY + s));
+                if (++s == kTStages) s = 0, ph ^= 1u;
+            };
+            auto second = [&](int it) {   // layer 2 of item it
+                const int b = it & 1;
+                if (!mbar_wait(bar(TB_H_FULL + b), (uint32_t)((it >> 1) & 1), abort_flag)) return false;
+                for (int kc = 0; kc < n_k2; ++kc) {
+                    uint64_t d;
+                    if (!stage(d)) return false;
+#pragma unroll
+                    for (int kk = 0; kk < 4; ++kk)   // 16 activations = 8 packed columns
+                        umma_bf16_ts_pair(tmem_base + (uint32_t)(b * 256 + 128), tmem_base + (uint32_t)(b * 256 + 8 * (kc * 4 + kk)),
+                                          d + (uint64_t)((16384 >> 4) + 2 * kk), idesc2, (kc > 0 || kk > 0) ? 1u : 0u);
+                    release();
+                }
+                umma_commit_pair(bar(TB_ACC2 + b));
+                return true;
+            };
             bool ok = true;
-            for (int pair = blockIdx.x; ok && pair < p.n_pairs; pair += gridDim.x, ++it) {
-                // tensor memory of the previous pair must have been read out
-                if (it > 0) ok = mbar_wait(bar(TB_TM_FREE), (uint32_t)((it - 1) & 1), abort_flag);
+            int it = 0;
+            for (int item = item0; ok && item < p.n_pairs; item += item_step, ++it) {
+                const int b = it & 1;
+                // the buffer's previous item must have been read out
+                if (it > 1) ok = mbar_wait(bar(TB_TM_FREE + b), (uint32_t)(((it >> 1) - 1) & 1), abort_flag);
                 tc_fence_after();
                 for (int kc = 0; ok && kc < p.n_k1; ++kc) {
-                    ok = mbar_wait(bar(TB_FULL_A + sa), pha, abort_flag) && mbar_wait(bar(TB_FULL_B + sb), phb, abort_flag);
-                    if (!ok) break;
-                    tc_fence_after();
-                    const uint64_t bd = umma_desc_sw128(smem_u32(smB + sb * kTBStage));
+                    if (kc == mid && it > 0 && !(ok = second(it - 1))) break;
+                    uint64_t d;
+                    if (!(ok = stage(d))) break;
 #pragma unroll
-                    for (int g = 0; g < 2; ++g) {
-                        const uint64_t ad = umma_desc_sw128(smem_u32(smA + sa * kTAStage + g * 16384));
-                        const uint32_t d_tmem = tmem_base + (uint32_t)(g * 256);
-                        umma_bf16(d_tmem, ad, bd, idesc1, kc != 0 ? 1u : 0u);
-                        umma_bf16_acc(d_tmem, ad + 2, bd + 2, idesc1);
-                        umma_bf16_acc(d_tmem, ad + 4, bd + 4, idesc1);
-                        umma_bf16_acc(d_tmem, ad + 6, bd + 6, idesc1);
-                    }
-                    umma_commit(bar(TB_EMPTY_A + sa));
-                    umma_commit(bar(TB_EMPTY_B + sb));
-                    if (++sa == kTStagesA) sa = 0, pha ^= 1u;
-                    if (++sb == kTStagesB) sb = 0, phb ^= 1u;
+                    for (int kk = 0; kk < 4; ++kk)
+                        umma_bf16_pair(tmem_base + (uint32_t)(b * 256), d + 2 * kk, d + (uint64_t)((16384 >> 4) + 2 * kk), idesc1, (kc | kk) != 0 ? 1u : 0u);
+                    release();
                 }
                 if (!ok) break;
-                umma_commit(bar(TB_ACC1));
-                ok = mbar_wait(bar(TB_H_FULL), (uint32_t)(it & 1), abort_flag);
-                tc_fence_after();
-                for (int kc = 0; ok && kc < n_k2; ++kc) {
-                    ok = mbar_wait(bar(TB_FULL_B + sb), phb, abort_flag);
-                    if (!ok) break;
-                    tc_fence_after();
-                    const uint64_t bd = umma_desc_sw128(smem_u32(smB + sb * kTBStage));
-#pragma unroll
-                    for (int g = 0; g < 2; ++g)
-#pragma unroll
-                        for (int kk = 0; kk < 4; ++kk)   // 16 activations = 8 packed columns
-                            umma_bf16_ts(tmem_base + (uint32_t)(g * 256 + 128), tmem_base + (uint32_t)(g * 256 + 8 * (kc * 4 + kk)),
-                                         bd + (uint64_t)(2 * kk), idesc2, (kc > 0 || kk > 0) ? 1u : 0u);
-                    umma_commit(bar(TB_EMPTY_B + sb));
-                    if (++sb == kTStagesB) sb = 0, phb ^= 1u;
-                }
-                if (ok) umma_commit(bar(TB_ACC2));
+                umma_commit_pair(bar(TB_ACC1 + b));
             }
+            if (ok && it > 0) second(it - 1);
         }
         __syncwarp();
     } else {
-        // ===================== rows and weights (TMA) =====================
+        // ===================== rows and this CTA's half of the weights (TMA) =====================
         if (lane == 0) {
-            int sa = 0, sb = 0;
-            uint32_t pha = 0, phb = 0;
-            bool ok = true;
-            for (int pair = blockIdx.x; ok && pair < p.n_pairs; pair += gridDim.x) {
-                for (int kc = 0; ok && kc < p.n_k1; ++kc) {
-                    ok = mbar_wait(bar(TB_EMPTY_A + sa), pha ^ 1u, abort_flag);
-                    if (!ok) break;
-                    mbar_expect_tx(bar(TB_FULL_A + sa), 32768u);   // rows beyond the last one arrive as zeros
-                    tma_load_2d(smem_u32(smA + sa * kTAStage), &tmapA, bar(TB_FULL_A + sa), kc * 64, pair * 256);
-                    tma_load_2d(smem_u32(smA + sa * kTAStage + 16384), &tmapA, bar(TB_FULL_A + sa), kc * 64, pair * 256 + 128);
-                    if (++sa == kTStagesA) sa = 0, pha ^= 1u;
-                    ok = mbar_wait(bar(TB_EMPTY_B + sb), phb ^ 1u, abort_flag);
-                    if (!ok) break;
-                    mbar_expect_tx(bar(TB_FULL_B + sb), (uint32_t)p.hI * 128u);
-                    tma_load_2d(smem_u32(smB + sb * kTBStage), &tmapW0, bar(TB_FULL_B + sb), kc * 64, 0);
-                    if (++sb == kTStagesB) sb = 0, phb ^= 1u;
+            int s = 0;
+            uint32_t ph = 0;
+            const int h1 = p.hI >> 1, h2 = p.d >> 1;
+            auto stage = [&](uint32_t bytes) {   // the even CTA's barrier counts both CTAs' copies
+                if (!mbar_wait(bar(TB_EMPTY + s), ph ^ 1u, abort_flag)) return false;
+                if (rank == 0) mbar_expect_tx(bar(TB_FULL + s), 2u * bytes);
+                return true;
+            };
+            auto next = [&] {
+                if (++s == kTStages) s = 0, ph ^= 1u;
+            };
+            auto second = [&] {
+                for (int kc = 0; kc < n_k2; ++kc) {
+                    if (!stage((uint32_t)h2 * 128u)) return false;
+                    tma_load_2d_pair(smem_u32(base + s * kTStage + 16384), &tmapW1, cluster_addr(bar(TB_FULL + s), 0u), kc * 64, h2 * rank);
+                    next();
                 }
-                for (int kc = 0; ok && kc < n_k2; ++kc) {
-                    ok = mbar_wait(bar(TB_EMPTY_B + sb), phb ^ 1u, abort_flag);
-                    if (!ok) break;
-                    mbar_expect_tx(bar(TB_FULL_B + sb), (uint32_t)p.d * 128u);
-                    tma_load_2d(smem_u32(smB + sb * kTBStage), &tmapW1, bar(TB_FULL_B + sb), kc * 64, 0);
-                    if (++sb == kTStagesB) sb = 0, phb ^= 1u;
+                return true;
+            };
+            bool ok = true;
+            int it = 0;
+            for (int item = item0; ok && item < p.n_pairs; item += item_step, ++it) {
+                for (int kc = 0; ok && kc < p.n_k1; ++kc) {
+                    if (kc == mid && it > 0 && !(ok = second())) break;
+                    if (!(ok = stage(16384u + (uint32_t)h1 * 128u))) break;
+                    const uint32_t full = cluster_addr(bar(TB_FULL + s), 0u);
+                    tma_load_2d_pair(smem_u32(base + s * kTStage), &tmapA, full, kc * 64, (item * 2 + rank) * 128);   // rows beyond the last one arrive as zeros
+                    tma_load_2d_pair(smem_u32(base + s * kTStage + 16384), &tmapW0, full, kc * 64, h1 * rank);
+                    next();
                 }
             }
+            if (ok && it > 0) second();
         }
         __syncwarp();
     }
 
+    // neither CTA leaves while the other may still reach it
     if (*abort_flag) {
         if (tid == 0) atomicOr(p.status, AIF_STATUS_TIMEOUT);
         const long long t0 = clock64();
@@ -296,7 +316,8 @@ __global__ void __launch_bounds__(kTThreads, 1) k_item_tower_tc(const __grid_con
     }
     tc_fence_before();
     __syncthreads();
-    if (warp == kTMmaWarp) tmem_dealloc(tmem_base, 512);
+    cluster_sync();
+    if (warp == kTMmaWarp) tmem_dealloc_pair(tmem_base, 512);
 }
 
 cudaError_t encode2d(CUtensorMap *m, const void *base, uint64_t cols, uint64_t rows, uint32_t box_c, uint32_t box_r, CUtensorMapSwizzle sw)
@@ -328,14 +349,14 @@ cudaError_t launch_item_tower_tc(const aif_ctx *ctx, const void *I_raw, const vo
     CUtensorMap ma, m0, m1, mo;
     cudaError_t e;
     if ((e = encode2d(&ma, I_raw, (uint64_t)dI, (uint64_t)n, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B)) != cudaSuccess) return e;
-    if ((e = encode2d(&m0, W0, (uint64_t)dI, (uint64_t)hI, 64, (uint32_t)hI, CU_TENSOR_MAP_SWIZZLE_128B)) != cudaSuccess) return e;
-    if ((e = encode2d(&m1, W1, (uint64_t)hI, (uint64_t)d, 64, (uint32_t)d, CU_TENSOR_MAP_SWIZZLE_128B)) != cudaSuccess) return e;
+    if ((e = encode2d(&m0, W0, (uint64_t)dI, (uint64_t)hI, 64, (uint32_t)hI / 2, CU_TENSOR_MAP_SWIZZLE_128B)) != cudaSuccess) return e;
+    if ((e = encode2d(&m1, W1, (uint64_t)hI, (uint64_t)d, 64, (uint32_t)d / 2, CU_TENSOR_MAP_SWIZZLE_128B)) != cudaSuccess) return e;
     if ((e = encode2d(&mo, out, (uint64_t)d, (uint64_t)n, 32, 32, CU_TENSOR_MAP_SWIZZLE_64B)) != cudaSuccess) return e;
     TowerParams p{};
     p.n = n, p.n_pairs = (int)((n + 2 * kTcTile - 1) / (2 * kTcTile)), p.n_k1 = dI / 64, p.hI = hI, p.d = d;
     p.b0 = b0, p.b1 = b1, p.out = (__nv_bfloat16 *)out, p.norm_max = norm_max, p.status = ctx->status;
-    const int grid = p.n_pairs < 148 ? p.n_pairs : 148;
-    e = launch_pdl(k_item_tower_tc, dim3(grid), dim3(kTThreads), kTSmem, st, ma, m0, m1, mo, p);
+    const int grid = 2 * (p.n_pairs < 74 ? p.n_pairs : 74);
+    e = launch_pdl_pair(k_item_tower_tc, dim3(grid), dim3(kTThreads), kTSmem, st, ma, m0, m1, mo, p);
     count_launch();
     return e;
 }
