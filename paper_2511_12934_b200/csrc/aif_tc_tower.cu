@@ -7,7 +7,7 @@
 // CTA takes in half of the weights (288 KB per item and CTA at dI = 512, hI = 256, d = 128: 4.9 k cycles at 59 bytes per
 // clock, for 5.1 k cycles of products).  A tile needs half of tensor memory, so items alternate between two buffers and the
 // epilogues of one run under the products of the next; with two tiles per CTA, which the weights' intake asked for without the
-// pair, tensor memory was full and both epilogues were exposed (19 k cycles per two tiles).  262143 rows: 93 -> XX us.  320 threads:
+// pair, tensor memory was full and both epilogues were exposed (19 k cycles per two tiles).  262143 rows: 85 -> 76 us.  320 threads:
 //   warps 0-7  two groups of four warps, group g = the items of buffer g, one thread per row.  After layer 1: bias, ReLU,
 //              bf16, packed back into tensor memory over accumulator columns already read (A operand of layer 2).
 //              After layer 2: bias, bf16, through a staging slab and a TMA tile store into the output rows.
