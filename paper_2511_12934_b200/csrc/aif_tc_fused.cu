@@ -113,18 +113,16 @@ __global__ void __launch_bounds__(kFThreads, 1) k_request_fused(const __grid_con
     }
     // The gather threads fetch their candidate ids while barriers and tensor memory are being set up: the ids head the
     // longest chain of dependent memory accesses of the kernel (ids -> item rows -> scores).
-    int id[8];
+    int mine = -1;
     if (warp >= kFProdWarp0 && warp < kFBWarp) {
         grid_dep_wait();
         const ReqDev rq0 = find_request(p.sl, blockIdx.x);
         int start0, cnt0;
         tile_range(blockIdx.x - rq0.tile_begin, rq0.n, kTcTile, p.mini_batch, start0, cnt0);
         // every id is read once per tile (they may lie in host memory across the bus): lane l takes row 4 w + l % 4 + 16 (l / 4)
-        // of warp w's rows, the threads that copy a row get it by shuffle
+        // of warp w's rows, the threads that copy a row get it by shuffle (after the barrier: the load is in flight across it)
         const int w = warp - kFProdWarp0, r = 4 * w + (lane & 3) + 16 * (lane >> 2);
-        const int mine = r < cnt0 ? p.sl.ids[rq0.off + start0 + r] : -1;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) id[i] = __shfl_sync(0xffffffffu, mine, (lane >> 3) + 4 * i);
+        if (r < cnt0) mine = p.sl.ids[rq0.off + start0 + r];
     }
     if (warp == kFMmaWarp) tmem_alloc(smem_u32(tmem_slot), 512);
     tc_fence_before();
@@ -485,6 +483,9 @@ __global__ void __launch_bounds__(kFThreads, 1) k_request_fused(const __grid_con
         const int pt = tid - kFProdWarp0 * 32;
         const int sub = pt & 7, r0 = pt >> 3;   // 16-byte slot of the 128-byte chunk row; rows r0, r0 + 16, ...
         const uint32_t row_off = (uint32_t)(r0 * 128) + (uint32_t)((sub ^ (r0 & 7)) << 4);
+        int id[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) id[i] = __shfl_sync(0xffffffffu, mine, (lane >> 3) + 4 * i);
 #pragma unroll
         for (int i = 0; i < 8; ++i)
             if (r0 + 16 * i < cnt && (id[i] < 0 || (int64_t)id[i] >= p.M)) {
