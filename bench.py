@@ -540,7 +540,7 @@ def measure(args, wl, steps, warmup, dist, world, rank, full):
     if top == "lsh":
         roof["lsh_note"] = (f"eqs. 6-7 need {wl.lsh_bits // 32} xor + popc on 32-bit words per (candidate, key) pair by the definition; "
                             f"the kernel gets the counts from a +-1 fp8 product ({2 * wl.lsh_bits} tensor flop per pair, not counted "
-                            "in `achieved`) and spends about ten integer / fp32 instructions per pair on conversion and tiers")
+                            "in `achieved`) and spends about five integer / fp32 instructions per pair on conversion and tiers")
     if tensor:
         roof["frac_nominal"] = roof["achieved"] / NOMINAL_BF16_TFLOPS
         roof["peak_nominal"] = NOMINAL_BF16_TFLOPS
