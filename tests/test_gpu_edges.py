@@ -293,3 +293,59 @@ def test_category_rows_in_whole_tiles_of_their_requests(mini_batch):
         _check(srv.score_ids(states[i], lists[i]), want[i])
     assert srv.ctx.poll_status() == B.STATUS_BAD_ID
     srv.close()
+
+
+@pytest.mark.parametrize("dI,hI,d", [(64, 64, 64), (128, 192, 128), (512, 256, 128)])
+def test_item_tower_over_its_pairs_of_tiles_and_both_buffers(dI, hI, d):
+    """The one-kernel tower: rows that fill no tile, one tile of a pair, a pair, one item per pair of SMs and one or two more (both
+    buffers, first use and re-use), one and eight K chunks.  bf16 has eight significant bits, so rounding a hidden activation, and the
+    row, moves it by up to 2^-8 of itself (half of the last bit, 2^-7, just above a power of two): 2^-8 of the sum of the absolute
+    terms, and of the row and that sum's share of it; 1e-4 covers the fp32 sums of up to 512 terms of order 1."""
+    M = 74 * 256 * 2 + 129
+    ctx = B.Aif(B.make_config(dtype=B.BF16, M=M, d=d, L_max=8, hidden=(64,), blocks=B.BLK_BEA, n_bridge=2))
+    g = torch.Generator(device="cuda").manual_seed(dI)
+
+    def draw(*shape):
+        return torch.randn(*shape, generator=g, device="cuda").to(torch.bfloat16)
+
+    w = {"W_i0": draw(hI, dI) * 0.1, "b_i0": torch.randn(hI, generator=g, device="cuda"), "W_i1": draw(d, hI) * 0.1,
+         "b_i1": torch.randn(d, generator=g, device="cuda"), "bridges": draw(2, d)}
+    ctx.load_item_weights(w)
+    raw = draw(M, dI)
+    for n in (1, 128, 129, 256, 257, 74 * 256, 74 * 256 + 1, M):
+        ctx.item_nearline_compute(None, raw[:n], draw(n, d))
+        out = torch.empty(n, d, dtype=torch.bfloat16, device="cuda")
+        ctx.gather_rows(torch.arange(n, dtype=torch.int32, device="cuda"), out)
+        h = torch.relu(raw[:n].double() @ w["W_i0"].double().T + w["b_i0"].double())
+        want = h @ w["W_i1"].double().T + w["b_i1"].double()
+        moved = 2.0 ** -8 * (h @ w["W_i1"].double().abs().T)
+        bound = moved + 2.0 ** -8 * (want.abs() + moved) + 1e-4
+        ratio = (out.double() - want).abs() / bound
+        assert ratio.max().item() <= 1.0, f"n {n}: {int((ratio > 1).sum())} elements, worst {ratio.max().item():.2f} of the bound at {divmod(int(ratio.argmax()), d)}"
+        assert ctx.poll_status() == 0
+    ctx.close()
+
+
+@pytest.mark.parametrize("H2,F,dc", [(64, 4, 16), (192, 2, 64), (256, 16, 32)])
+def test_whole_mlp_in_one_kernel_at_the_edges_of_its_range(H2, F, dc):
+    """Two layers of 512 and at most 256 units, all tiles at once: one tile (the pair's other tile does not exist), odd and even numbers
+    of tiles, the last number it takes and the first it does not (148 and 149), two requests whose tiles share a pair."""
+    wl = helpers.MINI["c2"].with_(name=f"mlp_{H2}_{F}_{dc}", R=2, N=148 * 128 + 1, M=20000, L=300, mini_batch=0, hidden=(512, H2), F=F, dc=dc, B=64,
+                                  blocks=helpers.ALL_BLOCKS)
+    weights, table = synth.make_weights(wl, zero_bias=False), synth.make_item_table(wl)
+    srv, oracle = serving.Server(wl, weights, table), helpers.make_oracle(wl, weights, M=wl.M)
+    rqs = [synth.make_request(wl, r) for r in range(2)]
+    states = [srv.precompute(r, srv.upload_request(rq, B.USER_PROJECTED)) for r, rq in enumerate(rqs)]
+    g = np.random.default_rng(6)
+    ids = g.choice(wl.M, wl.N, replace=False).astype(np.int32)
+    ids[3] = -1
+    pick = np.unique(np.concatenate([g.choice(wl.N, 60), [0, 3, 127, 128, 255, 256, wl.N - 2, wl.N - 1]]))
+    want = oracle.score(table, helpers.projected_request(wl, rqs[0]), ids[pick])
+    for n in (1, 128, 129, 300, 147 * 128, 148 * 128, 148 * 128 + 1):
+        got = srv.score_ids(states[0], ids[:n])
+        _check(got[pick[pick < n]], want[pick < n])
+    a, b = ids[:200], ids[500:611]
+    for got, rq, i in zip(srv.score_many(states, [a, b]), rqs, (a, b)):
+        _check(got, oracle.score(table, helpers.projected_request(wl, rq), i))
+    assert srv.ctx.poll_status() == B.STATUS_BAD_ID
+    srv.close()
