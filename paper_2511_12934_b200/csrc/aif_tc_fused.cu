@@ -52,7 +52,7 @@ constexpr int kMaxCross = 8;                   // cross-feature chunks (64 colum
 constexpr int kH1 = 512;
 
 enum {
-    BAR_E_FULL = 0, BAR_KV_FULL, BAR_S_FULL = BAR_KV_FULL + 2, BAR_P_FULL, BAR_O_FINAL, BAR_ATT_FULL, BAR_E_FREE, BAR_ACC1_FULL,
+    BAR_E_FULL = 0, BAR_KV_FULL, BAR_S_FULL = BAR_KV_FULL + 2, BAR_P_FULL = BAR_S_FULL + 2, BAR_O_FINAL, BAR_ATT_FULL, BAR_E_FREE, BAR_ACC1_FULL,
     BAR_H1_FULL, BAR_ACC2_FULL, BAR_BIAS_FULL, BAR_FULL_A, BAR_EMPTY_A = BAR_FULL_A + kAStages, BAR_FULL_B = BAR_EMPTY_A + kAStages,
     BAR_EMPTY_B = BAR_FULL_B + kBStages, BAR_COUNT = BAR_EMPTY_B + kBStages
 };
@@ -92,6 +92,7 @@ __global__ void __launch_bounds__(kFThreads, 1) k_request_fused(const __grid_con
         mbar_init(bar(BAR_KV_FULL), 1);
         mbar_init(bar(BAR_KV_FULL + 1), 1);
         mbar_init(bar(BAR_S_FULL), 1);
+        mbar_init(bar(BAR_S_FULL + 1), 1);
         mbar_init(bar(BAR_P_FULL), 256);
         mbar_init(bar(BAR_O_FINAL), 1);
         mbar_init(bar(BAR_ATT_FULL), 256);
@@ -197,7 +198,7 @@ __global__ void __launch_bounds__(kFThreads, 1) k_request_fused(const __grid_con
         };
         float lsum = 0.f;
         if (act) {
-            wait(BAR_S_FULL);
+            wait(BAR_S_FULL + g);   // of its own key block: the first group's exponentials run under the second block's products
             tc_fence_after();
             if (ok) lsum = probabilities(0.f);
         }
@@ -391,8 +392,8 @@ __global__ void __launch_bounds__(kFThreads, 1) k_request_fused(const __grid_con
                     const uint64_t o = (uint64_t)((kk >> 2) * (kChunk >> 4) + 2 * (kk & 3));
                     umma_bf16_acc(d_tmem, qd + o, kd + o, idesc_qk);
                 }
+                umma_commit(bar(BAR_S_FULL + j));
             }
-            if (ok) umma_commit(bar(BAR_S_FULL));
             // O = P V: the probabilities from tensor memory, V = the key blocks read MN-major
             ok = ok && mbar_wait(bar(BAR_P_FULL), 0u, abort_flag);
             tc_fence_after();
