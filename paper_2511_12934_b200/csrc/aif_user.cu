@@ -457,10 +457,14 @@ __global__ void __launch_bounds__(256) k_user_prof(const T *__restrict__ S, int 
 // ------------------------------------------------------------------------------------------------
 // raw = 1: u = mean-pooled self-attention through the second FFN layer + profile attention; raw = 0: u is given.  Every block
 // forms u for itself (the partial sums it merges are tens of KB in L2) and then kFinishCols entries of p_u, so that the
-// chain of dependent steps is not followed by one block's walk over the whole of W1.  Each step spreads its loads over all
-// threads, a column group of 16 bytes and a slice of the rows per thread, and joins the slices in shared memory in a fixed
+// chain of dependent steps is not followed by one block's walk over the whole of W1.  Each step on the way to u spreads its loads
+// over all threads, a column group of 16 bytes and a slice of the rows per thread, and joins the slices in shared memory in a fixed
 // order.  One block over 1184 partial sums, with one column per thread and 2-byte loads, took 66 us at d = 128, H1 = 512.
-constexpr int kFinishCols = 64;
+// p_u itself is one running sum per entry, b1 and then the columns of u in their order, as the first layer defines it: a sum in
+// slices moves hidden activations across bf16 rounding edges, and the logits of a three-layer model by 1e-4 of their size.  The
+// columns of W1 are brought to shared memory by all threads, under the steps before, so that the chain of d multiply-adds waits for
+// nothing else.
+constexpr int kFinishCols = 64, kFinishTile = 32768;
 template <typename T>
 __global__ void __launch_bounds__(256) k_user_finish(int raw, int L, int d, const float *__restrict__ partial, int n_parts,
                                                      const float *__restrict__ ppart, int n_slices, const T *__restrict__ u_in,
@@ -470,10 +474,20 @@ __global__ void __launch_bounds__(256) k_user_finish(int raw, int L, int d, cons
 {
     __shared__ __align__(16) float red[2][1024];
     __shared__ float us[256], q_s[256], uprof[256], wgt[kProfParts], wred[8];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    constexpr int kRows = kFinishTile / (kFinishCols * (int)sizeof(T)), kUnits = kFinishCols * (int)sizeof(T) / 16;
+    __shared__ __align__(16) T w1_s[kRows * kFinishCols];   // rows k0 .. of this block's columns of W1
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, col0 = blockIdx.x * kFinishCols;
     static_assert(kProfParts == 256, "one thread per key slice");
+    auto fetch = [&](int k0) {   // 16 bytes at a time: H1 is a multiple of 8; columns beyond it as zeros
+        for (int i = tid; i < min(kRows, d - k0) * kUnits; i += 256) {
+            const int r = i / kUnits, col = col0 + (i % kUnits) * (16 / (int)sizeof(T));
+            cp_async16(smem_u32(w1_s) + i * 16, W1t + (size_t)(k0 + r) * H1 + (col < H1 ? col : 0), col < H1 ? 16u : 0u);
+        }
+        cp_async_commit();
+    };
     grid_dep_launch();
     grid_dep_wait();
+    fetch(0);
     if (raw) {
         // weights 2^(m_g - m) of the key slices
         const float m_g = tid < n_slices ? ppart[(size_t)tid * (d + 4) + d] : -INFINITY, l_g = tid < n_slices ? ppart[(size_t)tid * (d + 4) + d + 1] : 0.f;
@@ -544,29 +558,21 @@ __global__ void __launch_bounds__(256) k_user_finish(int raw, int L, int d, cons
         us[tid] = to_f(u_in[tid]);
         if (blockIdx.x == 0) u32[tid] = us[tid];
     }
-    __syncthreads();
-    // p_u: eight columns per thread, 32 threads per column group over interleaved rows
-    {
-        const int c8 = (tid & 7) * 8, col = blockIdx.x * kFinishCols + c8, r = tid >> 3;
-        float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        if (col < H1)   // H1 is a multiple of 8
-#pragma unroll 8
-            for (int k = r; k < d; k += 32) {
-                float f[8];
-                load8(W1t + (size_t)k * H1 + col, f);
-#pragma unroll
-                for (int i = 0; i < 8; ++i) acc[i] = fmaf(us[k], f[i], acc[i]);
-            }
-        float *o = red[0] + r * kFinishCols + c8;   // 32 x 64 floats: both halves of red
-#pragma unroll
-        for (int i = 0; i < 8; ++i) o[i] = acc[i];
+    const int j = col0 + tid;
+    const bool own = tid < kFinishCols && j < H1;
+    float acc = own ? b1[j] : 0.f;
+    for (int k0 = 0; k0 < d; k0 += kRows) {
+        if (k0) {
+            __syncthreads();
+            fetch(k0);
+        }
+        cp_async_wait<0>();
+        __syncthreads();   // (and us)
+        if (tid < kFinishCols)
+#pragma unroll 16
+            for (int k = 0; k < min(kRows, d - k0); ++k) acc = fmaf(us[k0 + k], to_f(w1_s[k * kFinishCols + tid]), acc);
     }
-    __syncthreads();
-    const int j = blockIdx.x * kFinishCols + tid;
-    if (tid < kFinishCols && j < H1) {
-        float acc = b1[j];
-#pragma unroll
-        for (int r = 0; r < 32; ++r) acc += red[0][r * kFinishCols + tid];
+    if (own) {
         p_u[j] = acc;
         // the same partial as two bf16 values (high part, remainder): the form in which the tensor cores add it
         const __nv_bfloat16 hi = __float2bfloat16_rn(acc);

@@ -349,3 +349,23 @@ def test_whole_mlp_in_one_kernel_at_the_edges_of_its_range(H2, F, dc):
         _check(got, oracle.score(table, helpers.projected_request(wl, rq), i))
     assert srv.ctx.poll_status() == B.STATUS_BAD_ID
     srv.close()
+
+
+@pytest.mark.parametrize("dtype,d,hidden", [("bf16", 256, (1024, 512, 256)), ("bf16", 128, (512, 256)), ("bf16", 64, (72,)), ("f32", 256, (264, 8)), ("f32", 32, (8,))])
+def test_the_users_share_of_the_first_layer_is_one_running_sum(dtype, d, hidden):
+    """p_u[j] = b1[j], then one multiply-add per column of u in their order: bit for bit, whatever the number of columns and units
+    (products of bf16 values are exact in fp32; fp32 ones, and their sums, are formed in 80 bits and rounded to fp32 once)."""
+    wl = synth.C2.with_(name=f"pu_{dtype}_{d}_{len(hidden)}", dtype=dtype, d=d, hidden=hidden, F=2, dc=32, B=16, R=1, N=10, M=500, L=20, mini_batch=0)
+    weights = synth.make_weights(wl, zero_bias=False)
+    srv = serving.Server(wl, weights, synth.make_item_table(wl))
+    rq = synth.make_request(wl, 0)
+    st = srv.precompute(0, srv.upload_request(rq, B.USER_PROJECTED))
+    u, _, pu = srv.ctx.user_state_export(st, wl.L)
+    u_in, W1 = synth.as_f32(rq["u"], dtype), synth.as_f32(weights["mlp"]["W"][0], dtype)
+    want = weights["mlp"]["b"][0].astype(np.float32)
+    for k in range(d):
+        want = (want.astype(np.longdouble) + u_in[k].astype(np.longdouble) * W1[:, k].astype(np.longdouble)).astype(np.float32)
+    assert np.array_equal(u.cpu().numpy(), u_in)
+    assert np.array_equal(pu.cpu().numpy(), want)
+    assert srv.ctx.poll_status() == 0
+    srv.close()
