@@ -1070,7 +1070,8 @@ __device__ __forceinline__ void join_tile(const JoinParams &p, const KeyTile &t,
             acc[0] = fmaf(w, a.x, acc[0]), acc[1] = fmaf(w, a.y, acc[1]), acc[2] = fmaf(w, a.z, acc[2]), acc[3] = fmaf(w, a.w, acc[3]);
             acc[4] = fmaf(w, b.x, acc[4]), acc[5] = fmaf(w, b.y, acc[5]), acc[6] = fmaf(w, b.z, acc[6]), acc[7] = fmaf(w, b.w, acc[7]);
         }
-        const float scale = p.attention ? (l > 0.f ? 1.0f / l : 0.f) : p.row_scale * (p.row_mean ? 1.0f / (float)t.L_tile : 1.0f);
+        // (no weight at all, every score minus infinity: no number, as in a tile that is not split)
+        const float scale = p.attention ? 1.0f / l : p.row_scale * (p.row_mean ? 1.0f / (float)t.L_tile : 1.0f);
         uint4 o;
         __nv_bfloat162 *h = reinterpret_cast<__nv_bfloat162 *>(&o);
 #pragma unroll

@@ -21,6 +21,7 @@
 // The running maximum is only raised when a row's block maximum exceeds it by more than 8 (in the log2 domain);
 // then the warp rescales its 32 rows of O in TMEM.  Until then probabilities stay below 2^8, which fp32 sums and
 // bf16 operands hold without loss of accuracy.  Every wait is bounded.
+#include <cfloat>
 #include <type_traits>
 
 #include "aif_device.cuh"
@@ -144,7 +145,8 @@ __global__ void __launch_bounds__((AttCfg<D, BN>::kThreads), 1) k_att_tc(const _
         const uint32_t lane_base = tmem_base + ((uint32_t)(wq * 32) << 16);
         const uint32_t o_col = (uint32_t)C::kTmemO;
         uint64_t *o_free_k = o_free + (kSplit ? (k & 1) : 0);
-        const float inv = l_sum > 0.f ? 1.0f / l_sum : 0.f;   // no key at all (an empty sub-sequence): a zero row
+        // no key at all (an empty sub-sequence): a zero row; keys without any weight (all scores minus infinity): no number
+        const float inv = l_sum > 0.f || (SPLIT && t.L > 0) ? 1.0f / l_sum : 0.f;
         bool good = false;
         if (row < t.cnt) {
             const int id = p.sl.ids[t.pos0 + row];
@@ -335,7 +337,8 @@ __global__ void __launch_bounds__((AttCfg<D, BN>::kThreads), 1) k_att_tc(const _
                     break;
                 }
                 if (j == 0) {
-                    m_used = mt;
+                    // (a piece of the keys may hold nothing but scores of minus infinity: a finite offset gives them no weight)
+                    m_used = SPLIT ? fmaxf(mt, -FLT_MAX) : mt;
                 } else {
                     const bool need = mt > m_used + 8.0f;
                     if (__any_sync(0xffffffffu, need)) {

@@ -369,3 +369,38 @@ def test_the_users_share_of_the_first_layer_is_one_running_sum(dtype, d, hidden)
     assert np.array_equal(pu.cpu().numpy(), want)
     assert srv.ctx.poll_status() == 0
     srv.close()
+
+
+def _overflow_request(wl, minus_inf):
+    """A projected request whose scores are minus infinity for the given keys against an item whose first column is 2^80 (the
+    product overflows fp32), and that column's share is zero for all others."""
+    rq = synth.make_request(wl, 0)
+    S = synth.as_f32(rq["S"], wl.dtype).copy()
+    S[:, 0] = 0.0
+    S[minus_inf, 0] = -(2.0 ** 80)
+    rq["S"] = synth.store(S, wl.dtype)
+    return rq
+
+
+@pytest.mark.parametrize("base,n_cat", [("c2", 0), ("c5", 0), ("c2", 1)])
+def test_split_pieces_that_hold_nothing_but_minus_infinity(base, n_cat):
+    """Keys whose scores overflow to minus infinity carry no weight, also where they are all that a piece of the keys holds: the
+    pieces' join gives what the other pieces say.  The layers do not read the column that overflows."""
+    wl = helpers.MINI[base].with_(name=f"split_inf_{base}_{n_cat}", R=1, N=100, M=300, L=2560, F=2, B=64, mini_batch=0, n_categories=n_cat,
+                                  blocks=synth.BLK_ATT | synth.BLK_CROSS)
+    weights, table = synth.make_weights(wl, zero_bias=False), synth.make_item_table(wl)
+    E = synth.as_f32(table["E"], wl.dtype).copy()
+    E[:, 0] = 2.0 ** 80
+    table["E"] = synth.store(E, wl.dtype)
+    weights["mlp"]["W"][0][:, wl.d] = 0
+    rq = _overflow_request(wl, slice(1280, 2560))
+    if n_cat:
+        rq["seq_cat"] = np.zeros(wl.L, dtype=np.int32)
+    srv, oracle = serving.Server(wl, weights, table), helpers.make_oracle(wl, weights, M=wl.M)
+    st = srv.precompute(0, srv.upload_request(rq, B.USER_PROJECTED))
+    ids = np.random.default_rng(3).choice(wl.M, 100, replace=False).astype(np.int32)
+    want = oracle.score(table, helpers.projected_request(wl, rq), ids)
+    assert np.isfinite(want).all()
+    _check(srv.score_ids(st, ids), want)
+    assert srv.ctx.poll_status() == 0
+    srv.close()
