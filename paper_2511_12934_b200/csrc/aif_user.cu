@@ -293,13 +293,14 @@ __device__ __forceinline__ void profile_slice(const T *__restrict__ S, int start
         }
 #pragma unroll
         for (int o = LPR; o < 32; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-        const float f = expf(m - mx);
+        const float off = mx == -INFINITY ? 0.f : mx;   // nothing but scores of minus infinity so far: no weight
+        const float f = expf(m - off);
         m = mx, l *= f;
 #pragma unroll
         for (int i = 0; i < 8; ++i) acc[i] *= f;
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
-            const float p = expf(s[u] - m);
+            const float p = expf(s[u] - off);
             l += p;
 #pragma unroll
             for (int i = 0; i < 8; ++i) acc[i] = fmaf(p, v[u][i], acc[i]);

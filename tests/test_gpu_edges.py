@@ -404,3 +404,29 @@ def test_split_pieces_that_hold_nothing_but_minus_infinity(base, n_cat):
     _check(srv.score_ids(st, ids), want)
     assert srv.ctx.poll_status() == 0
     srv.close()
+
+
+@pytest.mark.parametrize("dtype,d", [("bf16", 128), ("bf16", 256), ("bf16", 64), ("f32", 64), ("f32", 128)])
+def test_profile_attention_where_a_slice_holds_nothing_but_minus_infinity(dtype, d):
+    """Eq. 3 with scores that overflow to minus infinity for a whole step of keys (32, 16 or 8 by width), between keys that have the
+    weight: those keys have none.  Identity projections, so that S and the projected profile are the inputs."""
+    step = 8 * (4 if d <= 64 else 2 if d <= 128 else 1)
+    wl = synth.C2.with_(name=f"prof_inf_{dtype}_{d}", dtype=dtype, d=d, dU=d, hidden=(64,), F=2, dc=32, B=16, R=1, N=10, M=500, L=96, mini_batch=0)
+    weights = synth.make_weights(wl, zero_bias=False)
+    eye = synth.store(np.eye(d, dtype=np.float32), dtype)
+    weights["user"]["W_seq"], weights["user"]["W_profile"] = eye, eye.copy()
+    rq = synth.make_request(wl, 0)
+    seq, prof = synth.as_f32(rq["seq"], dtype).copy(), synth.as_f32(rq["profile"], dtype).copy()
+    prof[0] = 2.0 ** 122
+    seq[:, 0] = 0.0
+    seq[32:32 + step, 0] = -1024.0
+    rq["seq"], rq["profile"] = synth.store(seq, dtype), synth.store(prof, dtype)
+    srv, oracle = serving.Server(wl, weights, synth.make_item_table(wl)), helpers.make_oracle(wl, weights, M=wl.M)
+    st = srv.precompute(0, srv.upload_request(rq, B.USER_RAW))
+    u, _, _ = srv.ctx.user_state_export(st, wl.L)
+    u_ref, _ = oracle.user_state(rq["profile"], rq["seq"])
+    assert np.isfinite(u_ref).all()
+    # attention rows of size 10^3, rounded to bf16 where the storage is (2^-9), through a layer of order-1 weights
+    assert np.abs(u.cpu().numpy() - u_ref).max() <= (1e-2 if dtype == "bf16" else 1e-5) * np.abs(u_ref).max()
+    assert srv.ctx.poll_status() == 0
+    srv.close()
