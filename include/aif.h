@@ -271,7 +271,8 @@ int aif_user_state_export(aif_ctx *ctx, const aif_user_state *state, float *u_ou
 
 /* Real-time phase: scores n candidates of one request.  cand_ids: device int32 [n]; logits: device fp32 [n]
  * (sigmoid outputs when emit_sigmoid).  `stream` first waits for the state's ready event.  May be called once
- * per request or once per mini-batch; the result of a candidate does not depend on which.  n = 0 is a no-op.
+ * per request or once per mini-batch; the result of a candidate does not depend on which (but for the order of fp32 sums on the
+ * tensor-core path: where a call has few tiles, the keys of a long sequence are summed in pieces).  n = 0 is a no-op.
  * An id outside [0, M) gives NaN and sets AIF_STATUS_BAD_ID.  No host-device copy happens inside.
  * Errors: AIF_ERR_VERSION, AIF_ERR_NOT_READY, AIF_ERR_SHAPE (n > max_batch_candidates), AIF_ERR_ARG. */
 int aif_score(aif_ctx *ctx, const aif_user_state *state, const int32_t *cand_ids, int32_t n, float *logits,
@@ -285,20 +286,20 @@ int aif_score(aif_ctx *ctx, const aif_user_state *state, const int32_t *cand_ids
 int aif_score_batch(aif_ctx *ctx, int32_t n_req, const aif_user_state *const *states, const int32_t *cand_ids,
                     const int64_t *offsets, float *logits, aif_stream stream);
 
-/* aif_score for callers whose buffers live in host memory: brings host_ids (host) to the device, scores, leaves the
- * logits in host_logits (host), all on `stream`; returns after the stream has drained.  If both buffers are page-locked
- * and mapped into the device's address space (cudaHostAlloc / cudaHostRegister; pinned torch tensors are), a small
- * kernel reads the ids across the bus and the last scoring kernel writes the logits straight into host_logits;
- * otherwise both are staged with cudaMemcpyAsync through buffers of the context.  This is the end-to-end form the
- * benchmark times. */
+/* aif_score for callers whose buffers live in host memory: takes host_ids (host), scores, leaves the logits in host_logits
+ * (host), all on `stream`; returns after the stream has drained.  If both buffers are page-locked and mapped into the device's
+ * address space (cudaHostAlloc / cudaHostRegister; pinned torch tensors are), the scoring kernels read the ids across the bus and
+ * write the logits straight into host_logits while the call runs; both buffers must then be page-locked as a whole.  Otherwise
+ * both are staged with cudaMemcpyAsync through buffers of the context.  This is the end-to-end form the benchmark times. */
 int aif_score_host(aif_ctx *ctx, const aif_user_state *state, const int32_t *host_ids, int32_t n,
                    float *host_logits, aif_stream stream);
 
 /* aif_score_batch for callers whose buffers live in host memory (Section 3.1: the real-time phase is handed candidate ids
- * by the retrieval service and hands scores back to it): host_ids (host int32, all requests concatenated) are copied to the
- * device on `stream`, scored in one launch, and the logits copied back into host_logits (host fp32); returns after the
- * stream has drained.  Page-locked buffers make both copies asynchronous transfers of the copy engine; pageable ones are
- * staged by the runtime.  states, offsets: as for aif_score_batch.  Errors as for aif_score_batch. */
+ * by the retrieval service and hands scores back to it): host_ids (host int32, all requests concatenated) are brought to the
+ * device on `stream`, scored in one launch, and the logits left in host_logits (host fp32); returns after the stream has drained.
+ * A page-locked, mapped host_logits (see aif_score_host) is written across the bus while the call runs, a pageable one by a copy at
+ * the end.  Ids are copied to the device first, except that up to 65536 of them are read across the bus when both buffers are
+ * page-locked.  states, offsets: as for aif_score_batch.  Errors as for aif_score_batch. */
 int aif_score_batch_host(aif_ctx *ctx, int32_t n_req, const aif_user_state *const *states, const int32_t *host_ids,
                          const int64_t *offsets, float *host_logits, aif_stream stream);
 

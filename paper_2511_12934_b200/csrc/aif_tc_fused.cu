@@ -120,8 +120,9 @@ __global__ void __launch_bounds__(kFThreads, 1) k_request_fused(const __grid_con
         const ReqDev rq0 = find_request(p.sl, blockIdx.x);
         int start0, cnt0;
         tile_range(blockIdx.x - rq0.tile_begin, rq0.n, kTcTile, p.mini_batch, start0, cnt0);
-        // every id is read once per tile (they may lie in host memory across the bus): lane l takes row 4 w + l % 4 + 16 (l / 4)
-        // of warp w's rows, the threads that copy a row get it by shuffle (after the barrier: the load is in flight across it)
+        // the gather warps read every id of the tile once (they may lie in host memory across the bus): lane l takes row
+        // 4 w + l % 4 + 16 (l / 4) of warp w's rows, the threads that copy a row get it by shuffle (after the barrier: the load is
+        // in flight across it).  Either softmax group reads its rows' ids again, beside the first products.
         const int w = warp - kFProdWarp0, r = 4 * w + (lane & 3) + 16 * (lane >> 2);
         if (r < cnt0) mine = p.sl.ids[rq0.off + start0 + r];
     }
