@@ -29,6 +29,32 @@ def _check(got, want, tol=TOL):
     assert err <= tol, f"max |delta| = {err:.3e} > {tol}"
 
 
+def _bridge_weights_by_scoring(ctx, n):
+    """The bridge weights of items 0 .. n - 1 as the scoring kernels read them, exactly: V's rows are unit vectors, so a column of the
+    bridge embedding is one weight; the only layer passes it on, its positive and its negative part in units of their own.  (Rows of
+    an odd number of bf16 weights cannot be gathered.)"""
+    c, nb = ctx.cfg, ctx.cfg.n_bridge
+    H, width, col = c.hidden[0], ctx.input_width, 2 * c.d
+    assert H >= 32 and not c.blocks & (B.BLK_ATT | B.BLK_CROSS)
+    W1 = torch.zeros(H, width, dtype=ctx.torch_dtype, device="cuda")
+    for k in range(nb):
+        W1[k, col + k], W1[16 + k, col + k] = 1, -1
+    zeros = torch.zeros(c.d, dtype=ctx.torch_dtype, device="cuda")
+    V = torch.eye(nb, c.d, dtype=ctx.torch_dtype, device="cuda")
+    sig = torch.zeros(1, c.lsh_bits // 8, dtype=torch.uint8, device="cuda") if c.blocks & B.BLK_LSH_DIN else None
+    ids = torch.arange(n, dtype=torch.int32, device="cuda")
+    out = torch.empty(nb, n, dtype=torch.float32, device="cuda")
+    for k in range(nb):
+        w_out = torch.zeros(H, dtype=ctx.torch_dtype, device="cuda")
+        w_out[k], w_out[16 + k] = 1, -1
+        ctx.load_weights({"W": [W1], "b": [torch.zeros(H, device="cuda")], "w_out": w_out, "b_out": torch.zeros(1, device="cuda")})
+        st = ctx.user_precompute(k, mode=B.USER_PROJECTED, profile=zeros, seq=zeros.view(1, -1), bea_V=V, seq_sig=sig)
+        ctx.score(st, ids, out[k])
+        torch.cuda.synchronize()
+        st.release()
+    return out.t().cpu()
+
+
 @pytest.mark.parametrize("dtype,d,nb,bits", [("bf16", 128, 8, 128), ("bf16", 64, 3, 64), ("bf16", 96, 16, 32), ("bf16", 256, 5, 256),
                                              ("f32", 64, 8, 96), ("f32", 160, 1, 160), ("f32", 256, 16, 256)])
 def test_refresh_and_gathers_at_every_row_width_and_unit(dtype, d, nb, bits):
@@ -36,7 +62,8 @@ def test_refresh_and_gathers_at_every_row_width_and_unit(dtype, d, nb, bits):
     rows moved 16, 8, 4 and 2 bytes at a time (also because the caller's sidecar starts off a 16-byte boundary); counts
     around a warp's step; ids outside the table."""
     dt, M = (B.F32 if dtype == "f32" else B.BF16), 3000
-    ctx = B.Aif(B.make_config(dtype=dt, M=M, d=d, L_max=8, hidden=(64,), blocks=B.BLK_BEA | B.BLK_LSH_DIN, n_bridge=nb, lsh_bits=bits))
+    ctx = B.Aif(B.make_config(dtype=dt, M=M, d=d, L_max=8, hidden=(64,), blocks=B.BLK_BEA | B.BLK_LSH_DIN, n_bridge=nb, lsh_bits=bits,
+                              max_batch_candidates=M))
     g = torch.Generator().manual_seed(d + nb)
     E, W, S = torch.zeros(M, d, dtype=ctx.torch_dtype), torch.zeros(M, nb, dtype=ctx.torch_dtype), torch.zeros(M, bits // 8, dtype=torch.uint8)
     for n in (1, 15, 16, 17, 63, 65, 1000):
@@ -64,6 +91,8 @@ def test_refresh_and_gathers_at_every_row_width_and_unit(dtype, d, nb, bits):
         else:
             ctx.gather_sidecars(ids.cuda(), None, os_[1:])
         assert torch.equal(out.cpu(), E[ids.long()]) and torch.equal(os_[1:].cpu(), S[ids.long()])
+    assert torch.equal(_bridge_weights_by_scoring(ctx, M), W.float())
+    assert ctx.poll_status() == 0
     ctx.close()
 
 
@@ -73,7 +102,7 @@ def test_bridge_weights_of_the_nearline_call(d, nb):
     """Algorithm 1 step 3 on the matrix instructions: one and two slices of eight bridges, odd numbers of them, item counts
     around the 16 of a warp.  A weight is at most 1 and is rounded to bf16 once (2^-9)."""
     M = 700
-    ctx = B.Aif(B.make_config(dtype=B.BF16, M=M, d=d, L_max=8, hidden=(64,), blocks=B.BLK_BEA, n_bridge=nb))
+    ctx = B.Aif(B.make_config(dtype=B.BF16, M=M, d=d, L_max=8, hidden=(64,), blocks=B.BLK_BEA, n_bridge=nb, max_batch_candidates=M))
     g = torch.Generator(device="cuda").manual_seed(nb)
 
     def draw(*shape):
@@ -88,9 +117,12 @@ def test_bridge_weights_of_the_nearline_call(d, nb):
         if nb % 2 == 0:
             out = torch.empty(n, nb, dtype=torch.bfloat16, device="cuda")
             ctx.gather_sidecars(torch.arange(n, dtype=torch.int32, device="cuda"), out)
-            want = orc.item_nearline(orc.BF16, I_id=iid.cpu().view(torch.int16).numpy().view(np.uint16),
-                                     bridges=w["bridges"].cpu().view(torch.int16).numpy().view(np.uint16))["w_hat"]
-            assert np.abs(out.float().cpu().numpy() - want).max() <= 2.0 ** -9
+            got = out.float().cpu()
+        else:
+            got = _bridge_weights_by_scoring(ctx, n)
+        want = orc.item_nearline(orc.BF16, I_id=iid.cpu().view(torch.int16).numpy().view(np.uint16),
+                                 bridges=w["bridges"].cpu().view(torch.int16).numpy().view(np.uint16))["w_hat"]
+        assert np.abs(got.numpy() - want).max() <= 2.0 ** -9
         assert ctx.poll_status() == 0
     ctx.close()
 
@@ -428,5 +460,69 @@ def test_profile_attention_where_a_slice_holds_nothing_but_minus_infinity(dtype,
     assert np.isfinite(u_ref).all()
     # attention rows of size 10^3, rounded to bf16 where the storage is (2^-9), through a layer of order-1 weights
     assert np.abs(u.cpu().numpy() - u_ref).max() <= (1e-2 if dtype == "bf16" else 1e-5) * np.abs(u_ref).max()
+    assert srv.ctx.poll_status() == 0
+    srv.close()
+
+
+def _host_workload(kind):
+    if kind == "fused":
+        return helpers.MINI["c2"].with_(name="host_fused", R=2, N=300, M=4000, L=100, mini_batch=0)
+    if kind == "chain":
+        return helpers.MINI["c3"].with_(name="host_chain", R=2, N=300, M=4000, L=300)
+    if kind == "no_cross":
+        return helpers.MINI["c2"].with_(name="host_no_cross", R=2, N=300, M=4000, L=300, mini_batch=0, blocks=synth.BLK_ATT)
+    if kind == "categories":
+        return helpers.MINI["c2"].with_(name="host_cat", R=2, N=300, M=4000, L=900, F=2, B=64, mini_batch=0, n_categories=7, blocks=helpers.ALL_BLOCKS)
+    return helpers.MINI["c1"].with_(name="host_simt", R=2, N=300, M=4000)
+
+
+@pytest.mark.parametrize("kind", ["fused", "chain", "no_cross", "categories", "simt"])
+def test_host_buffers_page_locked_pageable_and_one_of_each(kind):
+    """Ids read across the bus by a scoring kernel, by a copy kernel, or copied; logits stored across the bus or copied back; logits
+    written over the ids they belong to: the device buffers' result, bit for bit, on every scoring path, for one request and several."""
+    wl = _host_workload(kind)
+    weights, table = synth.make_weights(wl, zero_bias=False), synth.make_item_table(wl)
+    srv = serving.Server(wl, weights, table)
+    states = [srv.precompute(r, srv.upload_request(synth.make_request(wl, r), B.USER_PROJECTED)) for r in range(2)]
+    g = np.random.default_rng(5)
+    lists = [g.choice(wl.M, n, replace=False).astype(np.int32) for n in (300, 37)]
+    lists[0][8] = -1
+    want, one = np.concatenate(srv.score_many(states, lists)), srv.score_ids(states[0], lists[0])
+    all_ids, offs = np.concatenate(lists), [0, 300, 337]
+    for ids_pinned in (True, False):
+        for out_pinned in (True, False):
+            ids, out = torch.from_numpy(all_ids.copy()), torch.full((337,), -7.0)
+            ids, out = ids.pin_memory() if ids_pinned else ids, out.pin_memory() if out_pinned else out
+            srv.ctx.score_batch_host(states, ids, offs, out)
+            assert np.array_equal(out.numpy(), want, equal_nan=True)
+            out.fill_(-7.0)
+            srv.ctx.score_host(states[0], ids[:300], out[:300])
+            assert np.array_equal(out[:300].numpy(), one, equal_nan=True) and (out[300:] == -7.0).all()
+    for pinned in (True, False):
+        for batch in (True, False):
+            buf = torch.from_numpy(all_ids.copy())
+            buf = buf.pin_memory() if pinned else buf
+            if batch:
+                srv.ctx.score_batch_host(states, buf, offs, buf.view(torch.float32))
+                assert np.array_equal(buf.view(torch.float32).numpy(), want, equal_nan=True)
+            else:
+                srv.ctx.score_host(states[0], buf[:300], buf.view(torch.float32)[:300])
+                assert np.array_equal(buf.view(torch.float32)[:300].numpy(), one, equal_nan=True) and np.array_equal(buf[300:].numpy(), lists[1])
+    assert srv.ctx.poll_status() == B.STATUS_BAD_ID
+    srv.close()
+
+
+@pytest.mark.parametrize("n", [8192, 8193])
+def test_host_batches_around_the_number_of_ids_read_across_the_bus(n):
+    """Up to 65536 page-locked ids are read by the kernels, longer lists are copied; the logits go straight to host memory either way."""
+    wl = helpers.MINI["c2"].with_(name=f"host_big_{n}", R=8, N=n, M=20000, L=20, mini_batch=0)
+    srv = serving.Server(wl, synth.make_weights(wl), synth.make_item_table(wl))
+    states = [srv.precompute(r, srv.upload_request(synth.make_request(wl, r), B.USER_PROJECTED)) for r in range(8)]
+    g = np.random.default_rng(5)
+    lists = [g.choice(wl.M, n, replace=False).astype(np.int32) for _ in range(8)]
+    want = np.concatenate(srv.score_many(states, lists))
+    ids, out = torch.from_numpy(np.concatenate(lists)).pin_memory(), torch.full((8 * n,), -7.0).pin_memory()
+    srv.ctx.score_batch_host(states, ids, [n * r for r in range(9)], out)
+    assert np.array_equal(out.numpy(), want)
     assert srv.ctx.poll_status() == 0
     srv.close()
