@@ -400,21 +400,21 @@ struct SimtLayout {
     int32_t max_h;
     int32_t region;      // of activations / key chunks
     int32_t key_bufs;    // chunk buffers, 2 or 1; 0: no room, keys are read from global memory
-    int32_t stages;      // of the weight ring; 0: no room, weights are read from global memory
-    int32_t red, ps;     // partial sums, kSimtRed or 0 (one warp per 64 outputs then); probabilities and similarities of the key chunks
+    int32_t stages;      // of the weight ring; 0: weights are read from global memory
+    int32_t red, ps;     // partial sums (with the ring); probabilities and similarities of the key chunks
 };
 
-// Outputs of a layer go in blocks of up to 256 columns, the weights of a block in stages of `rows` rows.
-struct SimtBlock {
-    int cols, rows;
-};
+// Where the weights of the layers come from (launch_score_simt chooses): the ring, a block per SM and layers of at most kSimtRingH units;
+// or global memory, a thread per output and 32 rows in flight per batch, with one block per SM and the registers for that
+// (SIMT_DIRECT) or three blocks (SIMT_MANY): the same sums in the same order.
+enum { SIMT_RING, SIMT_DIRECT, SIMT_MANY };
+constexpr int kSimtRingH = 256, kSimtRingWeights = 65536;
+
+// Rows of a layer of H units in one stage of the ring.
 template <typename T>
-__device__ __forceinline__ SimtBlock simt_block(int H, int c0)
+__device__ __forceinline__ int simt_stage_rows(int H)
 {
-    SimtBlock b;
-    b.cols = min(256, H - c0);
-    b.rows = min(128, kSimtStageBytes / (b.cols * (int)sizeof(T)));
-    return b;
+    return min(128, kSimtStageBytes / (H * (int)sizeof(T)));
 }
 
 // The weights of all layers, stage by stage, by one thread.
@@ -425,21 +425,15 @@ __device__ __forceinline__ bool simt_weights(const ModelDev &md, unsigned char *
     uint32_t ph = 1;
     for (int layer = 0; layer < md.n_hidden; ++layer) {
         const int H = md.hidden[layer], in_w = layer ? md.hidden[layer - 1] : md.k1;
-        const T *W0 = reinterpret_cast<const T *>(md.Wt[layer]) + (layer == 0 ? (size_t)md.d * H : 0);
-        for (int c0 = 0; c0 < H; c0 += 256) {
-            const SimtBlock b = simt_block<T>(H, c0);
-            for (int k0 = 0; k0 < in_w; k0 += b.rows) {
-                const int rows = min(b.rows, in_w - k0);
-                const T *W = W0 + (size_t)k0 * H + c0;
-                const uint32_t dst = smem_u32(ring + s * kSimtStageBytes), bar = smem_u32(full + s), bytes = (uint32_t)(b.cols * sizeof(T));
-                if (filled >= stages && !mbar_wait(smem_u32(empty + s), ph, abort_flag)) return false;
-                mbar_expect_tx(bar, rows * bytes);
-                if (b.cols == H) bulk_load(dst, W, rows * bytes, bar);
-                else
-                    for (int r = 0; r < rows; ++r) bulk_load(dst + r * bytes, W + (size_t)r * H, bytes, bar);
-                ++filled;
-                if (++s == stages) s = 0, ph ^= 1u;
-            }
+        const T *W = reinterpret_cast<const T *>(md.Wt[layer]) + (layer == 0 ? (size_t)md.d * H : 0);
+        const int stage_rows = simt_stage_rows<T>(H);
+        for (int k0 = 0; k0 < in_w; k0 += stage_rows) {
+            const uint32_t bar = smem_u32(full + s), bytes = (uint32_t)(min(stage_rows, in_w - k0) * H) * (uint32_t)sizeof(T);
+            if (filled >= stages && !mbar_wait(smem_u32(empty + s), ph, abort_flag)) return false;
+            mbar_expect_tx(bar, bytes);
+            bulk_load(smem_u32(ring + s * kSimtStageBytes), W + (size_t)k0 * H, bytes, bar);
+            ++filled;
+            if (++s == stages) s = 0, ph ^= 1u;
         }
     }
     return true;
@@ -522,11 +516,12 @@ __device__ __forceinline__ void simt_keys(const ModelDev &md, const uint8_t *sig
     }
 }
 
-// RING: weights through the ring; else (inputs so wide that there is no room for it) straight from global memory.
-template <typename T, bool RING>
-__global__ void __launch_bounds__(kSimtThreads + 32, 1) k_score_simt(const __grid_constant__ ModelDev md, const __grid_constant__ ScoreLaunch sl, const SimtLayout lay)
+template <typename T, int MODE>
+__global__ void __launch_bounds__(MODE == SIMT_RING ? kSimtThreads + 32 : kSimtThreads, MODE == SIMT_MANY ? 3 : 1) k_score_simt(const __grid_constant__ ModelDev md, const __grid_constant__ ScoreLaunch sl, const SimtLayout lay)
 {
     constexpr int TM = kSimtTile;
+    constexpr bool RING = MODE == SIMT_RING;
+    constexpr int kAll = RING ? kSimtThreads + 32 : kSimtThreads;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     unsigned char *ring = smem_raw;
     float *xs = reinterpret_cast<float *>(smem_raw + (RING ? lay.stages * kSimtStageBytes : 0));   // [k1][TM] candidate-dependent input, transposed
@@ -538,24 +533,24 @@ __global__ void __launch_bounds__(kSimtThreads + 32, 1) k_score_simt(const __gri
     float *ps = qv + (size_t)TM * md.d;                      // [2][warp][kSimtKeys] probabilities, similarities
     uint32_t *sigq = reinterpret_cast<uint32_t *>(ps + lay.ps);   // [TM][8]
     int *tiers = reinterpret_cast<int *>(sigq + TM * 8);     // [TM][16]
-    uint64_t *full = reinterpret_cast<uint64_t *>(tiers + TM * 16);
+    uint64_t *full = reinterpret_cast<uint64_t *>(tiers + TM * 16);   // (from here on with the ring only)
     uint64_t *empty = full + kSimtMaxStages;
     volatile uint32_t *abort_flag = reinterpret_cast<volatile uint32_t *>(empty + kSimtMaxStages);
 
     const int tid = threadIdx.x, lane = tid & 31, c = tid >> 5;   // candidate of this warp
     const int d = md.d;
-    if (tid == kSimtThreads) {
+    if (RING && tid == kSimtThreads) {
         for (int s = 0; s < kSimtMaxStages; ++s) mbar_init(smem_u32(full + s), 1), mbar_init(smem_u32(empty + s), kSimtWarps);
         *abort_flag = 0u;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     grid_dep_launch();
-    for (int i = tid; i < md.k1 * TM; i += kSimtThreads + 32) xs[i] = 0.f;
-    for (int i = tid; i < TM * 16; i += kSimtThreads + 32) tiers[i] = 0;
+    for (int i = tid; i < md.k1 * TM; i += kAll) xs[i] = 0.f;
+    for (int i = tid; i < TM * 16; i += kAll) tiers[i] = 0;
     __syncthreads();   // xs is zero, the barriers exist
-    if (tid >= kSimtThreads) {
+    if (RING && tid >= kSimtThreads) {
         // the weights are older than any launch this one may overlap: no wait for the previous kernel
-        if (RING && lane == 0 && !simt_weights<T>(md, ring, full, empty, lay.stages, abort_flag)) *abort_flag = 1u;
+        if (lane == 0 && !simt_weights<T>(md, ring, full, empty, lay.stages, abort_flag)) *abort_flag = 1u;
         return;
     }
     grid_dep_wait();
@@ -691,9 +686,35 @@ __global__ void __launch_bounds__(kSimtThreads + 32, 1) k_score_simt(const __gri
         const int H = md.hidden[layer];
         const float *bias = layer == 0 ? slot.p_u : md.b[layer];
         named_bar_sync(1, kSimtThreads);   // the layer's inputs are written
-        for (int c0 = 0; c0 < H; c0 += 256) {
-            const SimtBlock b = simt_block<T>(H, c0);
-            const int groups = (b.cols + 63) >> 6, splits = lay.red ? kSimtWarps / groups : 1;   // groups of 64 outputs; warps per group
+        if constexpr (!RING) {
+            const T *W = reinterpret_cast<const T *>(md.Wt[layer]) + (layer == 0 ? (size_t)d * H : 0);
+            for (int j = tid; j < H; j += kSimtThreads) {
+                float acc[TM];
+                const float b0 = bias[j];
+#pragma unroll
+                for (int cc = 0; cc < TM; ++cc) acc[cc] = b0;
+                auto row = [&](int k, float w) {
+                    const float4 a = *reinterpret_cast<const float4 *>(in_act + k * TM), b = *reinterpret_cast<const float4 *>(in_act + k * TM + 4);
+                    acc[0] = fmaf(w, a.x, acc[0]), acc[1] = fmaf(w, a.y, acc[1]), acc[2] = fmaf(w, a.z, acc[2]), acc[3] = fmaf(w, a.w, acc[3]);
+                    acc[4] = fmaf(w, b.x, acc[4]), acc[5] = fmaf(w, b.y, acc[5]), acc[6] = fmaf(w, b.z, acc[6]), acc[7] = fmaf(w, b.w, acc[7]);
+                };
+                int k = 0;
+                for (; k + 32 <= in_w; k += 32) {
+                    float w[32];
+#pragma unroll
+                    for (int u = 0; u < 32; ++u) w[u] = to_f(W[(size_t)(k + u) * H + j]);
+#pragma unroll
+                    for (int u = 0; u < 32; ++u) row(k + u, w[u]);
+                }
+                for (; k < in_w; ++k) row(k, to_f(W[(size_t)k * H + j]));
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+                    *reinterpret_cast<float4 *>(out_act + (size_t)j * TM + 4 * h) =
+                        make_float4(fmaxf(acc[4 * h], 0.f), fmaxf(acc[4 * h + 1], 0.f), fmaxf(acc[4 * h + 2], 0.f), fmaxf(acc[4 * h + 3], 0.f));
+            }
+        } else {
+            const int stage_rows = simt_stage_rows<T>(H);
+            const int groups = (H + 63) >> 6, splits = kSimtWarps / groups;   // groups of 64 outputs; warps per group
             const int grp = c % groups, part = c / groups;
             const bool busy = part < splits;
             uint64_t acc2[8][TM / 2];   // two candidates per register pair: half the instructions (f32x2)
@@ -701,15 +722,13 @@ __global__ void __launch_bounds__(kSimtThreads + 32, 1) k_score_simt(const __gri
             for (int o = 0; o < 8; ++o)
 #pragma unroll
                 for (int cc = 0; cc < TM / 2; ++cc) acc2[o][cc] = 0ull;
-            // (lanes beyond the block's last column read its last outputs again)
-            const int col_a = min(64 * grp + 4 * ql, b.cols - 4), col_b = min(64 * grp + 32 + 4 * ql, b.cols - 4);
-            for (int k0 = 0; k0 < in_w; k0 += b.rows) {
-                const int rows = min(b.rows, in_w - k0);
-                if (RING) ok = __all_sync(0xffffffffu, ok && (next || mbar_wait(smem_u32(full + s), ph, abort_flag)));
-                if (RING) next = mbar_test(smem_u32(full + (s + 1 == lay.stages ? 0 : s + 1)), s + 1 == lay.stages ? ph ^ 1u : ph);
-                const T *w0 = RING ? reinterpret_cast<const T *>(ring + s * kSimtStageBytes)
-                                   : reinterpret_cast<const T *>(md.Wt[layer]) + (layer == 0 ? (size_t)d * H : 0) + (size_t)k0 * H + c0;
-                const int ws = RING ? b.cols : H;
+            // (lanes beyond the last output read the last ones again)
+            const int col_a = min(64 * grp + 4 * ql, H - 4), col_b = min(64 * grp + 32 + 4 * ql, H - 4);
+            for (int k0 = 0; k0 < in_w; k0 += stage_rows) {
+                const int rows = min(stage_rows, in_w - k0);
+                ok = __all_sync(0xffffffffu, ok && (next || mbar_wait(smem_u32(full + s), ph, abort_flag)));
+                next = mbar_test(smem_u32(full + (s + 1 == lay.stages ? 0 : s + 1)), s + 1 == lay.stages ? ph ^ 1u : ph);
+                const T *w0 = reinterpret_cast<const T *>(ring + s * kSimtStageBytes);
                 if (ok && busy) {
                     const float *x0 = in_act + k0 * TM;
                     // two rows in registers: the reads of one travel while the other is multiplied
@@ -719,7 +738,7 @@ __global__ void __launch_bounds__(kSimtThreads + 32, 1) k_score_simt(const __gri
                     } a, bb;
                     const int step = 4 * splits, last = rows - 1;   // reads beyond the stage repeat its last row and are not multiplied
                     auto read = [&](Row &q, int rr) {
-                        q.wa = load4(w0 + (size_t)rr * ws + col_a), q.wb = load4(w0 + (size_t)rr * ws + col_b);
+                        q.wa = load4(w0 + (size_t)rr * H + col_a), q.wb = load4(w0 + (size_t)rr * H + col_b);
                         q.xa = *reinterpret_cast<const ulonglong2 *>(x0 + rr * TM), q.xb = *reinterpret_cast<const ulonglong2 *>(x0 + rr * TM + 4);
                     };
                     auto multiply = [&](const Row &q) {
@@ -741,11 +760,9 @@ __global__ void __launch_bounds__(kSimtThreads + 32, 1) k_score_simt(const __gri
                     }
                     if (r < rows) multiply(a);
                 }
-                if (RING) {
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(smem_u32(empty + s));
-                    if (++s == lay.stages) s = 0, ph ^= 1u;
-                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(empty + s));
+                if (++s == lay.stages) s = 0, ph ^= 1u;
             }
             // the four row slices meet: lane (kp, ql) ends with outputs 4 ql + kp and 32 + 4 ql + kp of the warp's 64
             float4 *r = reinterpret_cast<float4 *>(red) + (part * groups + grp) * 128 + 8 * ql;   // unit 2 * output + half, its low bits mixed with ql: no bank conflicts
@@ -765,34 +782,27 @@ __global__ void __launch_bounds__(kSimtThreads + 32, 1) k_score_simt(const __gri
                         v[2 * cc + e] = (odd ? h[1][e] : h[0][e]) + __shfl_xor_sync(0xffffffffu, odd ? h[0][e] : h[1][e], 8);
                     }
                 }
-                if (busy && !lay.red) {
-                    const int o = 64 * grp + 32 * g + 4 * ql + kp;
-                    if (o < b.cols)
-#pragma unroll
-                        for (int cc = 0; cc < TM; ++cc) out_act[(size_t)(c0 + o) * TM + cc] = fmaxf(v[cc] + bias[c0 + o], 0.f);
-                } else if (busy) {
+                if (busy) {
                     r[64 * g + ((2 * kp) ^ ql)] = make_float4(v[0], v[1], v[2], v[3]);
                     r[64 * g + ((2 * kp + 1) ^ ql)] = make_float4(v[4], v[5], v[6], v[7]);
                 }
             }
-            if (!lay.red) continue;
             // ... and those of the warps: [part][group][64 outputs][TM], every thread sums outputs of its own
             const int first = tid >> 1;
-            const float b_first = first < b.cols ? bias[c0 + first] : 0.f;
+            const float b_first = first < H ? bias[first] : 0.f;
             named_bar_sync(1, kSimtThreads);
-            for (int i = tid; i < 2 * b.cols; i += kSimtThreads) {
+            for (int i = tid; i < 2 * H; i += kSimtThreads) {
                 const int o = i >> 1, h = i & 1;
-                const float b0 = o == first ? b_first : bias[c0 + o];
+                const float b0 = o == first ? b_first : bias[o];
                 float4 v = make_float4(b0, b0, b0, b0);
 #pragma unroll 4
                 for (int q = 0; q < splits; ++q) {
                     const float4 t = reinterpret_cast<const float4 *>(red)[q * groups * 128 + (i ^ (i >> 3 & 7))];
                     v.x += t.x, v.y += t.y, v.z += t.z, v.w += t.w;
                 }
-                *reinterpret_cast<float4 *>(out_act + (size_t)(c0 + o) * TM + 4 * h) =
+                *reinterpret_cast<float4 *>(out_act + (size_t)o * TM + 4 * h) =
                     make_float4(fmaxf(v.x, 0.f), fmaxf(v.y, 0.f), fmaxf(v.z, 0.f), fmaxf(v.w, 0.f));
             }
-            if (c0 + 256 < H) named_bar_sync(1, kSimtThreads);   // the partial sums are read before the next block's are written
         }
         in_act = out_act;
         out_act = (out_act == ha) ? hb : ha;
@@ -832,27 +842,48 @@ cudaError_t launch_score_simt(const aif_ctx *ctx, const ScoreLaunch &sl, cudaStr
     for (int k = 0; k < c.n_hidden; ++k) lay.max_h = c.hidden[k] > lay.max_h ? c.hidden[k] : lay.max_h;
     const int k1 = ctx->input_width - c.d, act = 2 * lay.max_h * kSimtTile;
     const int chunk = kSimtKeys * (int)(c.d * ctx->el + 16) / 4;
-    auto bytes = [&](int stages, int bufs, bool red) {
+    auto bytes = [&](int stages, int bufs) {
         lay.stages = stages, lay.key_bufs = bufs, lay.region = act > bufs * chunk ? act : bufs * chunk;
-        lay.red = red ? kSimtRed : 0, lay.ps = bufs ? 2 * kSimtWarps * kSimtKeys : 0;
-        return ((size_t)(k1 + c.d) * kSimtTile + lay.region + lay.red + lay.ps + (size_t)kSimtTile * (8 + 16) + 16) * 4 + (size_t)kSimtMaxStages * 16 +
-               (size_t)stages * kSimtStageBytes;
+        lay.red = stages ? kSimtRed : 0, lay.ps = bufs ? 2 * kSimtWarps * kSimtKeys : 0;
+        return ((size_t)(k1 + c.d) * kSimtTile + lay.region + lay.red + lay.ps + (size_t)kSimtTile * (8 + 16)) * 4 +
+               (stages ? 64 + (size_t)kSimtMaxStages * 16 + (size_t)stages * kSimtStageBytes : 0);
     };
-    // wide inputs leave less room: for key buffers and stages first, then for none of the ring, then for no key chunks, at last for no
-    // partial sums
+    // The ring pays where there are weights enough to stream: below 65536 of them a thread per output is as fast in a small launch (96 ->
+    // 64 -> 32 units, 1000 candidates: 9.5 against 9.1 us), and three blocks per SM are faster in a large one, to which the ring leaves
+    // one (64000 candidates: 184 against 393 us; 256 -> 192 -> 64 units: 600 against 805).  At 98304 (256 -> 256 -> 128 units) 1000
+    // candidates take 16.8 us with it.  Layers of more than 256 units: 1000 candidates, 1024 -> 1024 -> 512 -> 256 units, 205 us without, 346
+    // with.  Not by the number of candidates: the two sum in different orders, and a logit does not depend on how many share its call.
+    int64_t n_weights = 0;
+    for (int k = 0; k < c.n_hidden; ++k) n_weights += (int64_t)(k ? c.hidden[k - 1] : k1) * c.hidden[k];
     size_t smem = 0;
-    static const int tries[][3] = {{4, 2, 1}, {4, 1, 1}, {3, 1, 1}, {2, 1, 1}, {0, 1, 1}, {0, 0, 1}, {0, 0, 0}};
-    for (const auto &t : tries)
-        if ((smem = bytes(t[0], t[1], t[2] != 0)) <= 227 * 1024) break;
+    int mode = SIMT_DIRECT;
+    if (lay.max_h <= kSimtRingH && n_weights >= kSimtRingWeights) {
+        // wide inputs leave less room: for key buffers and stages first, then for none of the ring
+        static const int tries[][2] = {{4, 2}, {4, 1}, {3, 1}, {2, 1}};
+        for (const auto &t : tries)
+            if ((smem = bytes(t[0], t[1])) <= 227 * 1024) {
+                mode = SIMT_RING;
+                break;
+            }
+    }
+    if (mode != SIMT_RING) {
+        // key chunks as there is room for them, three blocks per SM where that is possible
+        if ((smem = bytes(0, 2)) > 75 * 1024 && (smem = bytes(0, 1)) > 227 * 1024) smem = bytes(0, 0);
+        // up to two blocks per SM the loads of one are what counts (256 -> 512 -> 256 units, 1000 candidates: 71 against 174 us), beyond that
+        // the blocks beside each other (32000 candidates: 1886 against 1531), unless their inputs leave room for one only
+        // (1024 units and more use three all the same: the layers' reads wait less than they do side by side)
+        if (sl.n_tiles > 2 * 148 && (smem <= 113 * 1024 || lay.max_h > kSimtRingH)) mode = SIMT_MANY;
+    }
     const ModelDev md = make_model(ctx);
     timing_begin(ctx, st);
     auto go = [&](auto kernel) {
         const cudaError_t e = smem <= 48 * 1024 ? cudaSuccess : cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        return e != cudaSuccess ? e : launch_pdl(kernel, dim3(sl.n_tiles), dim3(kSimtThreads + 32), smem, st, md, sl, lay);
+        return e != cudaSuccess ? e : launch_pdl(kernel, dim3(sl.n_tiles), dim3(kSimtThreads + (mode == SIMT_RING ? 32 : 0)), smem, st, md, sl, lay);
     };
     const bool f32 = c.dtype == AIF_F32;
-    const cudaError_t e = lay.stages ? (f32 ? go(k_score_simt<float, true>) : go(k_score_simt<__nv_bfloat16, true>))
-                                     : (f32 ? go(k_score_simt<float, false>) : go(k_score_simt<__nv_bfloat16, false>));
+    const cudaError_t e = mode == SIMT_RING     ? (f32 ? go(k_score_simt<float, SIMT_RING>) : go(k_score_simt<__nv_bfloat16, SIMT_RING>))
+                          : mode == SIMT_DIRECT ? (f32 ? go(k_score_simt<float, SIMT_DIRECT>) : go(k_score_simt<__nv_bfloat16, SIMT_DIRECT>))
+                                                : (f32 ? go(k_score_simt<float, SIMT_MANY>) : go(k_score_simt<__nv_bfloat16, SIMT_MANY>));
     count_launch();
     timing_mark(ctx, "score_simt", st);
     return e;

@@ -526,3 +526,54 @@ def test_host_batches_around_the_number_of_ids_read_across_the_bus(n):
     assert np.array_equal(out.numpy(), want)
     assert srv.ctx.poll_status() == 0
     srv.close()
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_cuda_core_scoring_at_the_widest_input_that_fits_shared_memory(dtype):
+    """One cross field so wide that input, activations and item vectors all but fill shared memory: accepted, and right; eight columns
+    more are refused without harm."""
+    # 8 candidates of (k1 + d + 2 H) floats and 24 words per candidate: 227 KB holds 7240 columns, units and tier counts in all
+    wl = synth.C1.with_(name=f"widest_{dtype}", dtype=dtype, d=32, hidden=(8,), F=1, dc=7152, B=4, R=1, N=20, M=100, L=5, mini_batch=0, emit_sigmoid=0,
+                        blocks=synth.BLK_CROSS | synth.BLK_SIMTIER, n_tiers=5, simtier_norm=synth.NORM_MEAN, bucket_mode=synth.BUCKET_HASH)
+    for more, fits in ((0, True), (8, False)):
+        w = wl.with_(dc=wl.dc + more)
+        weights, table = synth.make_weights(w, zero_bias=False), synth.make_item_table(w)
+        srv, oracle = serving.Server(w, weights, table, path=B.PATH_SIMT), helpers.make_oracle(w, weights, M=w.M)
+        rq = synth.make_request(w, 0)
+        st = srv.precompute(0, srv.upload_request(rq, B.USER_PROJECTED))
+        ids = np.arange(20, dtype=np.int32)
+        if fits:
+            want = oracle.score(table, helpers.projected_request(w, rq), ids)
+            _check(srv.score_ids(st, ids), want, 1e-5 * max(1.0, np.abs(want).max()) if dtype == "f32" else TOL)
+        else:
+            with pytest.raises(B.AifError):
+                srv.score_ids(st, ids)
+        assert srv.ctx.poll_status() == 0
+        srv.close()
+
+
+@pytest.mark.parametrize("dtype,d,hidden,F,dc", [("f32", 32, (16,), 2, 8), ("f32", 64, (256, 128), 40, 8), ("bf16", 96, (264, 64), 33, 16), ("f32", 256, (520, 256), 3, 24), ("f32", 64, (192, 40), 9, 8)])
+def test_cuda_core_scoring_of_more_candidates_than_one_block_per_sm(dtype, d, hidden, F, dc):
+    """Launches of up to two blocks per SM and of more take different forms of the kernel: the candidates around the change, fields in
+    more than one group of 32, one and several requests; both forms agree with the oracle and, bit for bit, with each other."""
+    wl = synth.C1.with_(name=f"simt_many_{dtype}_{d}_{F}", dtype=dtype, d=d, hidden=hidden, F=F, dc=dc, B=16, R=2, N=296 * 8 + 9, M=3000, L=70, emit_sigmoid=0,
+                        blocks=helpers.ALL_BLOCKS, lsh_din_norm=synth.NORM_MEAN, simtier_norm=synth.NORM_MEAN, mini_batch=0, bucket_mode=synth.BUCKET_HASH)
+    weights, table = synth.make_weights(wl, zero_bias=False), synth.make_item_table(wl)
+    srv, oracle = serving.Server(wl, weights, table, path=B.PATH_SIMT), helpers.make_oracle(wl, weights, M=wl.M)
+    rqs = [synth.make_request(wl, r, L=L) for r, L in enumerate((70, 33))]
+    states = [srv.precompute(r, srv.upload_request(rq, B.USER_PROJECTED)) for r, rq in enumerate(rqs)]
+    ids = np.random.default_rng(1).choice(wl.M, wl.N, replace=False).astype(np.int32)
+    ids[9] = -1
+    pick = np.unique(np.concatenate([[0, 7, 8, 9, wl.N - 1, wl.N - 10], np.random.default_rng(2).choice(wl.N, 60)]))
+    wants = [oracle.score(table, helpers.projected_request(wl, rq), ids[pick]) for rq in rqs]
+    # sums of up to 1500 terms in fp32; bf16 storage as elsewhere
+    tol = 1e-5 * max(1.0, np.nanmax(np.abs(wants[0]))) if dtype == "f32" else TOL
+    for n in (296 * 8, 296 * 8 + 1, wl.N):
+        got = srv.score_ids(states[0], ids[:n])
+        _check(got[pick[pick < n]], wants[0][pick < n], tol)
+    parts = np.concatenate([srv.score_ids(states[0], ids[:1200]), srv.score_ids(states[0], ids[1200:])])
+    assert np.array_equal(got, parts, equal_nan=True)    # a candidate's logit does not depend on how many others there are
+    for got, w in zip(srv.score_many(states, [ids, ids]), wants):
+        _check(got[pick], w, tol)
+    assert srv.ctx.poll_status() == B.STATUS_BAD_ID
+    srv.close()
