@@ -99,7 +99,7 @@ __device__ __forceinline__ TileInfo decode_tile(const LayerParams &p, int tile, 
 // pos becomes the grouped position; F = 0 does nothing else).
 constexpr uint32_t kNoBucket = 0xFFFFu;
 __global__ void __launch_bounds__(256) k_cross_buckets(const int32_t *__restrict__ ids, int64_t total, int64_t M, int F, int B,
-                                                        int b_mask, int mode, uint16_t *__restrict__ xb, int32_t *__restrict__ ids_copy, const SimPlace pl, int late)
+                                                        int b_mask, uint64_t b_inv, int mode, uint16_t *__restrict__ xb, int32_t *__restrict__ ids_copy, const SimPlace pl, int late)
 {
     if (!late) grid_dep_wait();
     grid_dep_launch();
@@ -134,7 +134,13 @@ __global__ void __launch_bounds__(256) k_cross_buckets(const int32_t *__restrict
                     if (mode == AIF_BUCKET_MOD) bk[q] = (uint32_t)(id % B);
                     else {
                         const uint64_t h = mix64((uint64_t)id, (uint64_t)(f + q));
-                        bk[q] = b_mask >= 0 ? (uint32_t)(h & (uint64_t)b_mask) : (uint32_t)(h % (uint64_t)B);
+                        if (b_mask >= 0) bk[q] = (uint32_t)(h & (uint64_t)b_mask);
+                        else {
+                            // Barrett reduction with b_inv = floor(2^64 / B): the estimated quotient is the true one or one less, as
+                            // h (2^64 / B - b_inv) / 2^64 < 1.  With a 64-bit remainder each, 2 x 10^7 hashes took 130 us, so 62.
+                            const uint32_t r = (uint32_t)h - (uint32_t)__umul64hi(h, b_inv) * (uint32_t)B;   // below 2 B: 32 bits are enough
+                            bk[q] = r >= (uint32_t)B ? r - (uint32_t)B : r;
+                        }
                     }
                 }
             if (i >= n) continue;
@@ -1507,7 +1513,7 @@ cudaError_t launch_score_tc_scratch(const aif_ctx *ctx, const ScoreLaunch &sl_in
         const int rounds = F == 0 ? 1 : F & 1 ? F : F / 2, want_y = sl.ids_copy ? 1 : 296 / grid;
         const int grid_y = want_y < 1 ? 1 : want_y > 8 ? (rounds < 8 ? rounds : 8) : want_y > rounds ? rounds : want_y;
         cudaError_t e = launch_pdl(k_cross_buckets, dim3(grid, grid_y), dim3(256), 0, st, sl.ids, sl.total, c.M, F, c.B,
-                                   (c.B & (c.B - 1)) == 0 ? c.B - 1 : -1, c.bucket_mode, (uint16_t *)sc.xb, sl.ids_copy, place, late);
+                                   (c.B & (c.B - 1)) == 0 ? c.B - 1 : -1, c.B > 0 ? ~0ull / (uint64_t)c.B : 0ull, c.bucket_mode, (uint16_t *)sc.xb, sl.ids_copy, place, late);
         if (sl.ids_copy) sl.ids = sl.ids_copy;
         if (place.where) sl.ids = place.ids;
         count_launch();

@@ -577,3 +577,21 @@ def test_cuda_core_scoring_of_more_candidates_than_one_block_per_sm(dtype, d, hi
         _check(got[pick], w, tol)
     assert srv.ctx.poll_status() == B.STATUS_BAD_ID
     srv.close()
+
+
+@pytest.mark.parametrize("Bk", [1, 3, 255, 1000, 4096, 32769, 65534])
+def test_buckets_of_the_kernel_chain_for_numbers_that_are_no_power_of_two(Bk):
+    """The hash modulo the number of buckets, by a multiplication where that is no power of two: the smallest and the largest number,
+    and numbers around powers of two; a wrong bucket is another embedding, 0.1 in a logit."""
+    wl = helpers.MINI["c3"].with_(name=f"buckets_{Bk}", R=1, N=4000, M=30000, L=5, F=2, dc=32, B=Bk, hidden=(256, 64), blocks=synth.BLK_CROSS,
+                                  bucket_mode=synth.BUCKET_HASH, sigma=0.5)
+    weights, table = synth.make_weights(wl, zero_bias=False), synth.make_item_table(wl)
+    srv, oracle = serving.Server(wl, weights, table), helpers.make_oracle(wl, weights, M=wl.M)
+    rq = synth.make_request(wl, 0)
+    st = srv.precompute(0, srv.upload_request(rq, B.USER_PROJECTED))
+    ids = np.random.default_rng(3).choice(wl.M, wl.N, replace=False).astype(np.int32)
+    want = oracle.score(table, helpers.projected_request(wl, rq), ids)
+    # activations of order 1: bf16 budget of the largest logit
+    _check(srv.score_ids(st, ids), want, 1e-2 * max(1.0, np.abs(want).max()))
+    assert srv.ctx.poll_status() == 0
+    srv.close()
