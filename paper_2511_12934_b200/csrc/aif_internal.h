@@ -90,7 +90,8 @@ struct SplitScratch {
     int32_t *tiers;     // [slots][16][128] tier counts, or nullptr (no SimTier)
     int32_t slots;      // records there is room for (0: no splitting)
 };
-constexpr int kSplitSlots = 4 * 148;       // of a scoring launch: at most two pieces per SM and launch, twice that after rounding up
+constexpr int kMaxParts = 32;              // equal pieces of a tile's keys, at most
+constexpr int kSplitSlots = 4 * 148;       // of a scoring launch: four rounds of equal pieces (split_parts); by category at most 2 x 148 (k_sim_tiles)
 constexpr int kSplitSlotsUser = 2 * 148;   // of the user side's self-attention
 
 struct ScoreLaunch {

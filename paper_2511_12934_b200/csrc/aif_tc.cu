@@ -1308,18 +1308,34 @@ cudaError_t tc_prepare_context(aif_ctx *ctx)
         in_w = c.hidden[k];
     }
     pl->maps_ready = true;
-    const bool key_kernels = tc_att_supported(c) || tc_lsh_supported(c);
-    auto take_split = [&](SplitScratch &sp, int slots, bool tiers) -> cudaError_t {
-        cudaError_t err;
-        if ((err = alloc((void **)&sp.rows, (size_t)slots * 128 * c.d * 4)) != cudaSuccess) return err;
-        if ((err = alloc((void **)&sp.stats, (size_t)slots * 256 * 4)) != cudaSuccess) return err;
-        if (tiers && (err = alloc((void **)&sp.tiers, (size_t)slots * 16 * 128 * 4)) != cudaSuccess) return err;
-        sp.slots = slots;
-        return cudaSuccess;
+    // Records of partial results, as many as a launch of this context can use: none where a sequence is one key block, no more than
+    // its tiles have pieces (a context that only holds a table needs none).  64 KB each at d = 128, written before they are read, so
+    // never cleared.  Splitting is for speed only: where there is no room for the records the context does without.
+    auto take_split = [&](SplitScratch &sp, int64_t slots, bool tiers) -> bool {
+        if (slots < 2) return true;
+        const size_t bytes[3] = {(size_t)slots * 128 * c.d * 4, (size_t)slots * 256 * 4, tiers ? (size_t)slots * 16 * 128 * 4 : 0};
+        void *q[3] = {};
+        bool ok = true;
+        for (int i = 0; i < 3; ++i) ok = ok && (bytes[i] == 0 || cudaMalloc(&q[i], bytes[i]) == cudaSuccess);
+        if (!ok) {
+            for (int i = 0; i < 3; ++i)
+                if (q[i]) cudaFree(q[i]);
+            cudaGetLastError();
+            return false;
+        }
+        for (int i = 0; i < 3; ++i)
+            if (q[i]) ctx->allocations.push_back(q[i]), ctx->device_bytes += (int64_t)bytes[i];
+        sp.rows = (float *)q[0], sp.stats = (float *)q[1], sp.tiers = (int32_t *)q[2], sp.slots = (int32_t)slots;
+        return true;
     };
-    if (key_kernels && (e = take_split(ctx->split, kSplitSlots, (c.blocks & AIF_BLK_SIMTIER) != 0)) != cudaSuccess) return e;
-    if (tc_att_supported(c) && tc_lsh_supported(c) && (e = take_split(ctx->split_lsh, kSplitSlots, (c.blocks & AIF_BLK_SIMTIER) != 0)) != cudaSuccess) return e;
-    if (tc_att_supported(c) && (e = take_split(ctx->split_user, kSplitSlotsUser, false)) != cudaSuccess) return e;
+    const int bn = c.d == 128 ? 128 : 64, key_blocks = (c.L_max + bn - 1) / bn, most = key_blocks < kMaxParts ? key_blocks : kMaxParts;
+    auto records = [&](int64_t tiles, int cap) { return key_blocks < 2 ? 0 : tiles * most < cap ? tiles * most : (int64_t)cap; };
+    // (by category: pieces of four key blocks of 128 and more, k_sim_tiles)
+    const int64_t n_split = c.n_categories == 0 ? records((int64_t)pl->tiles_cap, kSplitSlots) : c.L_max > 4 * 128 ? kSplitSlots : 0;
+    const bool att = tc_att_supported(c), lsh = tc_lsh_supported(c), tiers = c.blocks & AIF_BLK_SIMTIER;
+    if (att || lsh) take_split(ctx->split, n_split, tiers && !att);
+    if (att && lsh && !take_split(ctx->split_lsh, n_split, tiers)) ctx->split.slots = 0;   // both kernels take the same pieces
+    if (att) take_split(ctx->split_user, records((c.L_max + kTcTile - 1) / kTcTile, kSplitSlotsUser), false);
     if (tc_att_supported(c) && (e = tc_att_prepare(ctx)) != cudaSuccess) return e;
     if (tc_fused_supported(c) && (e = tc_fused_prepare(ctx)) != cudaSuccess) return e;
     if (tc_lsh_supported(c) && (e = tc_lsh_prepare(ctx)) != cudaSuccess) return e;
@@ -1335,7 +1351,7 @@ int split_parts(int n_tiles, int blocks, int slots)
 {
     auto cost = [&](int parts) { return ((int64_t)n_tiles * parts + 147) / 148 * ((blocks + parts - 1) / parts + (parts > 1 ? 3 : 2)) + (parts > 1 ? 5 : 0); };
     int best = 1;
-    for (int parts = 2; parts <= blocks && parts <= 32 && (int64_t)n_tiles * parts <= slots; ++parts)
+    for (int parts = 2; parts <= blocks && parts <= kMaxParts && (int64_t)n_tiles * parts <= slots; ++parts)
         if (cost(parts) < cost(best)) best = parts;
     return best > 1 && 10 * cost(best) < 9 * cost(1) ? best : 1;
 }

@@ -595,3 +595,14 @@ def test_buckets_of_the_kernel_chain_for_numbers_that_are_no_power_of_two(Bk):
     _check(srv.score_ids(st, ids), want, 1e-2 * max(1.0, np.abs(want).max()))
     assert srv.ctx.poll_status() == 0
     srv.close()
+
+
+@pytest.mark.parametrize("d,L_max,n_cat,most", [(128, 1, 0, 16), (128, 128, 0, 16), (256, 64, 0, 24), (128, 512, 3, 40), (128, 300, 0, 60)])
+def test_contexts_take_no_more_room_for_partial_results_than_their_sequences_can_use(d, L_max, n_cat, most):
+    """A context whose sequences are one key block (one that only holds a table among them) never splits keys, and few tiles have few
+    pieces: megabytes in all for a table of 1000 items and 128 candidates, every block on."""
+    cfg = B.make_config(dtype=B.BF16, M=1000, d=d, L_max=L_max, hidden=(64,), F=2, B=16, dc=32, n_categories=n_cat, blocks=helpers.ALL_BLOCKS,
+                        max_batch_candidates=128, max_user_states=1)
+    ctx = B.Aif(cfg)
+    assert ctx.get_stats().device_bytes <= most << 20
+    ctx.close()
