@@ -202,7 +202,7 @@ __device__ inline TileDev tile_entry(const ScoreLaunch &sl, int tile, int mini_b
     const ReqDev rq = find_request(sl, tile);
     int start, cnt;
     tile_range(tile - rq.tile_begin, rq.n, kTcTile, mini_batch, start, cnt);
-    return TileDev{rq.slot, cnt, rq.off + start, sl.slots[rq.slot].L, 0, {0, 0}};
+    return TileDev{rq.slot, cnt, rq.off + start, sl.slots[rq.slot].L, {0, 0, 0}};
 }
 
 // One tile, or (SPLIT) one piece of a tile's keys, as every role of the attention and LSH kernels needs it.
@@ -217,7 +217,7 @@ struct KeyTile {
 template <bool SPLIT>
 __device__ __forceinline__ int key_jobs(const ScoreLaunch &sl)
 {
-    if (!SPLIT) return sl.n_tiles_dev ? *sl.n_tiles_dev : sl.n_tiles;
+    if (!SPLIT) return sl.n_tiles;
     return sl.jobs ? *sl.n_jobs_dev : sl.n_tiles * sl.parts;
 }
 
@@ -238,8 +238,8 @@ __device__ __forceinline__ KeyTile key_tile(const ScoreLaunch &sl, int job, int 
         const int4 v = *reinterpret_cast<const int4 *>(sl.tiles + tile);   // slot, cnt, pos0
         t.slot = v.x, t.cnt = v.y;
         t.pos0 = ((int64_t)(uint32_t)v.w << 32) | (int64_t)(uint32_t)v.z;
-        t.L = sl.tiles[tile].L, t.key0 = sl.tiles[tile].key0;
-        t.nb = t.L > 0 ? (t.L + BN - 1) / BN : 1;
+        t.L = sl.tiles[tile].L, t.key0 = 0;
+        t.nb = (t.L + BN - 1) / BN;
     } else {
         const ReqDev rq = find_request(sl, tile);
         int start, cnt;

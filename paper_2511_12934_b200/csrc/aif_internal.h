@@ -68,12 +68,12 @@ struct TileDev {
     int32_t slot;
     int32_t cnt;     // candidates in the tile
     int64_t pos0;    // position of its first candidate in ids / logits
-    int32_t L;       // keys of the tile: the request's sequence length, or the length of its category's sub-sequence
-    int32_t key0;    // first key row (0, or where the category's sub-sequence begins in the grouped sequence)
-    int32_t pad_[2];
+    int32_t L;       // keys of the tile: the request's sequence length
+    int32_t pad_[3];
 };
 
-// A piece of a tile's keys, the unit of the attention and LSH kernels where tiles with many keys are split over several CTAs.
+// A piece of a tile's keys, the unit of the attention and LSH kernels where tiles are formed by category (their keys are a part of
+// the grouped sequence), and where tiles with many keys are split over several CTAs.
 struct JobDev {
     int32_t slot, cnt;
     int64_t pos0;
@@ -107,15 +107,13 @@ struct ScoreLaunch {
     float *logits;
     uint32_t *status;
     const TileDev *tiles;   // [n_tiles] (tensor-core tiles), or nullptr: search `reqs` per tile
-    // categories on: tiles are formed on the device from the candidates grouped by (request, category).  n_tiles above is
-    // then an upper bound that sizes grids, the count is read from n_tiles_dev; ids are the grouped candidates, and
-    // out_index[p] is where the logit of grouped position p belongs in the caller's array.
-    const int32_t *n_tiles_dev;
+    // categories on: ids are the candidates grouped by (request, category), out_index[p] is where the logit of grouped position p
+    // belongs in the caller's array, and the tiles of the key kernels are the jobs below.  n_tiles is an upper bound of them.
     const int32_t *out_index;
     int32_t grouped;        // 1: key blocks come from the grouped sequence
     // pieces of tiles: a table formed on the device (categories on), or `parts` equal pieces of every tile
     const JobDev *jobs;
-    const int32_t *n_jobs_dev;   // [2] jobs, split tiles
+    const int32_t *n_jobs_dev;   // [2] jobs, split tiles, as the device found them
     const int32_t *joins;        // jobs that are the first pieces of split tiles
     int32_t n_jobs;              // upper bound of the number of jobs
     int32_t parts;               // 0 or 1: tiles are not split
@@ -196,7 +194,6 @@ struct aif_ctx {
 
     // weights
     void *Wt[aif::kMaxHidden] = {};      // [in x out]
-    void *Wk[aif::kMaxHidden] = {};      // [out x in] (K-major), first layer: candidate-dependent columns only, K padded
     float *b[aif::kMaxHidden] = {};
     void *w_out = nullptr;
     float *b_out = nullptr;
@@ -305,7 +302,6 @@ cudaError_t launch_lsh_tc(const aif_ctx *ctx, const ScoreLaunch &sl, cudaStream_
 size_t sim_grouped_rows(int L_max, int n_categories);
 cudaError_t sim_prepare(aif_ctx *ctx);
 void sim_destroy(aif_ctx *ctx);
-size_t sim_tile_capacity(const aif_ctx *ctx);
 cudaError_t sim_group_sequence(const aif_ctx *ctx, HostSlot &hs, const int32_t *seq_cat, int L, cudaStream_t st);
 // Where the candidates of a grouped launch go: candidate pos to grouped position grp_start[where[pos].x] + where[pos].y.
 struct SimPlace {
@@ -313,7 +309,7 @@ struct SimPlace {
     const int32_t *grp_start;
     int32_t *ids, *out_index;   // by grouped position: id, and the candidate's position in the caller's arrays
 };
-// fills sl (tiles, jobs, their numbers, out_index) for a launch whose original ids are sl.ids; the candidates themselves are
+// fills sl (jobs, their numbers, out_index) for a launch whose original ids are sl.ids; the candidates themselves are
 // placed by the bucket kernel, after which the launch's ids are place.ids
 cudaError_t sim_group_candidates(const aif_ctx *ctx, ScoreLaunch &sl, SimPlace &place, TileDev *row_tiles, cudaStream_t st);
 // pieces per tile that even a launch of n_tiles tiles of `blocks` key blocks out over the SMs (aif_tc.cu)

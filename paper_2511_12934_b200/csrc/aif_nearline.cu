@@ -11,6 +11,7 @@
 
 #include "aif_device.cuh"
 #include "aif_internal.h"
+#include "aif_tc_ptx.cuh"
 
 namespace aif {
 namespace {
@@ -89,13 +90,6 @@ __global__ void __launch_bounds__(256) k_item_bridge_weights(const T *__restrict
 // is read in the same order, once, into registers.  Lane 4 g + t of the accumulator holds bridges 2 t, 2 t + 1 of items g and
 // g + 8: the softmax over bridges is two shuffles inside a quad.  One warp per item with a warp reduction per bridge (the form
 // above) took 217 us for 262143 items at d = 128, n = 8.
-__device__ __forceinline__ void mma_16816(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1)
-{
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
-                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-                 : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-
 template <int VJ, int NT>
 __global__ void __launch_bounds__(256) k_item_bridge_weights_mma(const __nv_bfloat16 *__restrict__ I_id, int64_t n, int nb,
                                                                  const __nv_bfloat16 *__restrict__ Bm, __nv_bfloat16 *__restrict__ out)
@@ -124,8 +118,8 @@ __global__ void __launch_bounds__(256) k_item_bridge_weights_mma(const __nv_bflo
             c[j][0] = c[j][1] = c[j][2] = c[j][3] = 0.f;
 #pragma unroll
             for (int v = 0; v < VJ; ++v) {
-                mma_16816(c[j], a[0][v].x, a[1][v].x, a[0][v].y, a[1][v].y, b[j][v].x, b[j][v].y);
-                mma_16816(c[j], a[0][v].z, a[1][v].z, a[0][v].w, a[1][v].w, b[j][v].z, b[j][v].w);
+                mma_bf16(c[j], a[0][v].x, a[1][v].x, a[0][v].y, a[1][v].y, b[j][v].x, b[j][v].y);
+                mma_bf16(c[j], a[0][v].z, a[1][v].z, a[0][v].w, a[1][v].w, b[j][v].z, b[j][v].w);
             }
         }
 #pragma unroll

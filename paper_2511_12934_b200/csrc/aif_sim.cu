@@ -157,34 +157,33 @@ __global__ void __launch_bounds__(256) k_sim_count(ScoreLaunch sl, int64_t M, in
     }
 }
 
-// One block over the groups: first grouped position of every group (exclusive scan of the counts), the tile records, the
-// number of tiles; the counts go back to zero for the next launch (the ranks place the candidates: k_cross_buckets).
-// Beside the tiles, the jobs of the attention and LSH kernels: a tile's cost there is its number of key blocks, from none to
-// hundreds (a user's favourite category holds a fifth of the sequence), so tiles are cut into pieces of about half of what an
-// SM gets on average; a tile left whole made the launch as long as the longest sub-sequence (150 key blocks of one tile against
-// 22 per SM on average).  Jobs are laid out by size, largest first (in classes of a quarter octave), and every second row of 148
-// runs backwards: job j goes to CTA j mod 148, so the CTA with the largest job of one row gets the smallest of the next (4 x 10^4
-// candidates over 100 categories of 10^5 items: at most 29 blocks per SM for 22 on average; 38 in plain order).
+// One block over the groups: first grouped position of every group (exclusive scan of the counts), the jobs of the attention and
+// LSH kernels, their number; the counts go back to zero for the next launch (the ranks place the candidates: k_cross_buckets).
+// A group is ceil(candidates / 128) tiles.  A tile's cost is its number of key blocks, from none to hundreds (a user's favourite
+// category holds a fifth of the sequence), so tiles with more than an SM's share of the launch are cut into pieces of that share
+// (below); a tile left whole made the launch as long as the longest sub-sequence (150 key blocks of one tile against 22 per SM on
+// average).  Jobs are laid out by size, largest first (in classes of a quarter octave), and every second row of 148 runs backwards:
+// job j goes to CTA j mod 148, so the CTA with the largest job of one row gets the smallest of the next (4 x 10^4 candidates over
+// 100 categories of 10^5 items, with pieces of half a share: at most 29 blocks per SM for 22 on average; 38 in plain order).
 struct SimGroup {
-    int32_t cnt, start, slot, len, key0, np, t0, j0, p0;
+    int32_t cnt, start, slot, len, key0, np, j0, p0;
 };
 
 __global__ void __launch_bounds__(1024) k_sim_tiles(ScoreLaunch sl, int n_groups, int n_cat, int32_t *__restrict__ grp_cnt,
-                                                    int32_t *__restrict__ grp_start, TileDev *__restrict__ tiles, int tile_cap,
-                                                    JobDev *__restrict__ jobs, int job_cap, int32_t *__restrict__ joins,
-                                                    int32_t *__restrict__ n_out)
+                                                    int32_t *__restrict__ grp_start, JobDev *__restrict__ jobs, int job_cap,
+                                                    int32_t *__restrict__ joins, int32_t *__restrict__ n_out)
 {
     constexpr int kClasses = 128;
     __shared__ SimGroup grp[1024];
     __shared__ int32_t warp_sum_s[32];
     __shared__ long long warp_blocks_s[32];
-    __shared__ int32_t carry_c, tile_cur, pslot_cur, join_cur;
+    __shared__ int32_t carry_c, pslot_cur, join_cur;
     __shared__ int32_t cls_jobs[kClasses], cls_base[kClasses];
     __shared__ int32_t n_jobs_s;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     grid_dep_launch();
     grid_dep_wait();
-    if (tid == 0) carry_c = 0, tile_cur = 0, pslot_cur = 0, join_cur = 0;
+    if (tid == 0) carry_c = 0, pslot_cur = 0, join_cur = 0;
     if (tid < kClasses) cls_jobs[tid] = 0;
     __syncthreads();
     auto key_blocks = [](int len) { return len > 0 ? (len + 127) / 128 : 1; };
@@ -261,7 +260,7 @@ __global__ void __launch_bounds__(1024) k_sim_tiles(ScoreLaunch sl, int n_groups
             const int v = __shfl_up_sync(0xffffffffu, before, o);
             if (lane >= o) before += v;
         }
-        if (lane == 31) n_out[1] = n_jobs_s = min(before, job_cap);
+        if (lane == 31) n_out[0] = n_jobs_s = min(before, job_cap);
         before -= run;
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
@@ -287,7 +286,7 @@ __global__ void __launch_bounds__(1024) k_sim_tiles(ScoreLaunch sl, int n_groups
             grp_cnt[g] = 0;
             me.np = pieces_of(me.len);
             const int nt = (me.cnt + kTcTile - 1) / kTcTile, k = class_of(key_blocks(me.len) / me.np);
-            me.t0 = atomicAdd(&tile_cur, nt), me.j0 = cls_base[k] + atomicAdd(&cls_jobs[k], nt * me.np);
+            me.j0 = cls_base[k] + atomicAdd(&cls_jobs[k], nt * me.np);
             if (me.np > 1) me.p0 = atomicAdd(&pslot_cur, nt * me.np);
         }
         grp[tid] = me;
@@ -299,10 +298,8 @@ __global__ void __launch_bounds__(1024) k_sim_tiles(ScoreLaunch sl, int n_groups
             for (int e = lane; e < nt * q.np; e += 32) {
                 const int t = e / q.np, part = e - t * q.np, n = min(kTcTile, q.cnt - t * kTcTile);
                 const int64_t pos0 = (int64_t)q.start + (int64_t)t * kTcTile;
-                // (within the caps for a launch within the context's limits, sim_prepare)
-                if (part == 0 && q.t0 + t < tile_cap) tiles[q.t0 + t] = TileDev{q.slot, n, pos0, q.len, q.key0, {0, 0}};
                 const int b0 = nb * part / q.np, b1 = nb * (part + 1) / q.np;
-                if (q.j0 + e < job_cap) {
+                if (q.j0 + e < job_cap) {   // (it is for a launch within the context's limits, sim_prepare)
                     const int j = place_of(q.j0 + e);
                     jobs[j] = JobDev{q.slot, n, pos0, q.np == 1 ? q.len : min(q.len - b0 * 128, (b1 - b0) * 128), q.key0 + b0 * 128, part, q.np,
                                             q.p0 + t * q.np, q.len};
@@ -312,14 +309,13 @@ __global__ void __launch_bounds__(1024) k_sim_tiles(ScoreLaunch sl, int n_groups
         }
         __syncthreads();
     }
-    if (tid == 0) n_out[0] = min(tile_cur, tile_cap), n_out[2] = join_cur;
+    if (tid == 0) n_out[1] = join_cur;
 }
 
 struct SimPlan {
     int n_groups_max = 0;
     size_t tile_cap = 0, cap = 0;
-    int32_t *grp_cnt = nullptr, *grp_start = nullptr, *ids_sorted = nullptr, *out_index = nullptr, *n_tiles_dev = nullptr;   // [3]: tiles, jobs, split tiles
-    TileDev *tiles = nullptr;
+    int32_t *grp_cnt = nullptr, *grp_start = nullptr, *ids_sorted = nullptr, *out_index = nullptr, *n_jobs_dev = nullptr;   // [2]: jobs, split tiles
     int2 *where = nullptr;       // [cap] group and rank of every candidate
     JobDev *jobs = nullptr;      // [tile_cap + kSplitSlots]
     int32_t *joins = nullptr;    // [kSplitSlots] first pieces of the split tiles
@@ -356,8 +352,7 @@ cudaError_t sim_prepare(aif_ctx *ctx)
     if ((e = alloc((void **)&pl->ids_sorted, (pl->cap + kTcTile) * 4)) != cudaSuccess) return e;
     if ((e = alloc((void **)&pl->out_index, (pl->cap + kTcTile) * 4)) != cudaSuccess) return e;
     if ((e = alloc((void **)&pl->where, pl->cap * sizeof(int2))) != cudaSuccess) return e;
-    if ((e = alloc((void **)&pl->n_tiles_dev, 256)) != cudaSuccess) return e;
-    if ((e = alloc((void **)&pl->tiles, pl->tile_cap * sizeof(TileDev))) != cudaSuccess) return e;
+    if ((e = alloc((void **)&pl->n_jobs_dev, 256)) != cudaSuccess) return e;
     if ((e = alloc((void **)&pl->jobs, (pl->tile_cap + kSplitSlots) * sizeof(JobDev))) != cudaSuccess) return e;
     if ((e = alloc((void **)&pl->joins, kSplitSlots * 4)) != cudaSuccess) return e;
     return cudaSuccess;
@@ -368,8 +363,6 @@ void sim_destroy(aif_ctx *ctx)
     delete plan_of(ctx);
     ctx->sim_plan = nullptr;
 }
-
-size_t sim_tile_capacity(const aif_ctx *ctx) { return plan_of(ctx)->tile_cap; }
 
 cudaError_t sim_group_sequence(const aif_ctx *ctx, HostSlot &hs, const int32_t *seq_cat, int L, cudaStream_t st)
 {
@@ -408,16 +401,14 @@ cudaError_t sim_group_candidates(const aif_ctx *ctx, ScoreLaunch &sl, SimPlace &
     cudaError_t e = launch_pdl(k_sim_count, dim3(grid), dim3(256), 0, st, sl, c.M, c.n_categories, c.bucket_mode, pl->grp_cnt, pl->where,
                                c.mini_batch, row_tiles);
     if (e != cudaSuccess) return e;
-    e = launch_pdl(k_sim_tiles, dim3(1), dim3(1024), 0, st, sl, n_groups, c.n_categories, pl->grp_cnt, pl->grp_start, pl->tiles, (int)pl->tile_cap, pl->jobs,
-                   (int)pl->tile_cap + kSplitSlots, pl->joins, pl->n_tiles_dev);
+    e = launch_pdl(k_sim_tiles, dim3(1), dim3(1024), 0, st, sl, n_groups, c.n_categories, pl->grp_cnt, pl->grp_start, pl->jobs,
+                   (int)pl->tile_cap + kSplitSlots, pl->joins, pl->n_jobs_dev);
     if (e != cudaSuccess) return e;
     count_launch(2);
     place = SimPlace{pl->where, pl->grp_start, pl->ids_sorted, pl->out_index};
     const int64_t groups = (int64_t)n_groups < sl.total ? (int64_t)n_groups : sl.total;
     sl.n_tiles = (int32_t)(sl.total / kTcTile + groups + 1 < (int64_t)pl->tile_cap ? sl.total / kTcTile + groups + 1 : (int64_t)pl->tile_cap);
-    sl.tiles = pl->tiles;
-    sl.n_tiles_dev = pl->n_tiles_dev;
-    sl.joins = pl->joins, sl.jobs = pl->jobs, sl.n_jobs_dev = pl->n_tiles_dev + 1, sl.n_jobs = sl.n_tiles + (sl.split.slots >= kSplitSlots ? kSplitSlots : 0);
+    sl.joins = pl->joins, sl.jobs = pl->jobs, sl.n_jobs_dev = pl->n_jobs_dev, sl.n_jobs = sl.n_tiles + (sl.split.slots >= kSplitSlots ? kSplitSlots : 0);
     sl.out_index = pl->out_index;
     sl.grouped = 1;
     return cudaSuccess;

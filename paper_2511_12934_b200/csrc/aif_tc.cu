@@ -27,7 +27,6 @@ namespace aif {
 namespace {
 
 constexpr int kABytes = kTcTile * 128;    // one A chunk of one tile: 128 rows x 64 bf16
-constexpr int kBBytes = 256 * 128;        // one B chunk: up to 256 weight rows x 64 bf16
 constexpr int kMaxChunks = 64;
 constexpr int kFusedMaxTiles = 148;
 
@@ -47,7 +46,6 @@ struct LayerParams {
     const uint8_t *E;
     int64_t M;
     int32_t e_row_bytes;
-    int32_t x_row_bytes;
     const uint8_t *X;             // dense rows, indexed by candidate position in the launch
     const uint16_t *xb;           // cross-feature buckets [positions x F], written by k_cross_buckets
     const uint8_t *T0;            // cross pre-cache of slot 0; slot i's lies i * slot_bytes further
@@ -326,11 +324,8 @@ __global__ void __launch_bounds__(PairCfg::kThreads, 1) k_layer_pair(const __gri
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
     grid_dep_launch();
-    // The weights are older than any launch this one may overlap: where the number of tiles is known to the host, their lane
-    // starts at once.
-    const bool early = warp == C::kBWarp && !p.sl.n_tiles_dev;
-    if (!early) grid_dep_wait();
-    const int n_tiles = p.sl.n_tiles_dev ? *p.sl.n_tiles_dev : p.sl.n_tiles;
+    if (warp != C::kBWarp) grid_dep_wait();   // the weights are older than any launch this one may overlap
+    const int n_tiles = p.sl.n_tiles;
     const int n_items = ((n_tiles + 1) / 2) * p.n_nchunks;
     const int item0 = (int)(blockIdx.x >> 1), item_step = (int)(gridDim.x >> 1);
 
@@ -913,19 +908,13 @@ __global__ void __launch_bounds__(MlpCfg::kThreads, 1) k_mlp_pair(const __grid_c
     if (warp == C::kMmaWarp) tmem_dealloc_pair(tmem_base, 512);
 }
 
-// The tile of a block in the kernels below: from the launch's tile table when it was formed on the device, else from the
-// request table.
+// The tile of a block in the kernels below, from the request table.
 struct BlockTile {
     int slot, cnt;
     int64_t pos0;
 };
 __device__ __forceinline__ BlockTile block_tile(const ScoreLaunch &sl, int tile, int mini_batch)
 {
-    if (sl.n_tiles_dev) {
-        if (tile >= *sl.n_tiles_dev) return BlockTile{0, 0, 0};
-        const TileDev t = sl.tiles[tile];
-        return BlockTile{t.slot, t.cnt, t.pos0};
-    }
     const ReqDev rq = find_request(sl, tile);
     int start, cnt;
     tile_range(tile - rq.tile_begin, rq.n, kTcTile, mini_batch, start, cnt);
@@ -1440,7 +1429,7 @@ cudaError_t tc_dense_layer(const aif_ctx *ctx, const DenseLayer &L, int64_t rows
     p.sl.ids = nullptr, p.sl.logits = nullptr, p.sl.status = ctx->status;
     p.n_cols = slice_cols(L.H), p.n_nchunks = (L.H + p.n_cols - 1) / p.n_cols, p.n_out = L.H, p.n_k = L.in_w / 64, p.mini_batch = 0;
     p.E = (const uint8_t *)ctx->E, p.M = ctx->cfg.M, p.e_row_bytes = ctx->cfg.d * 2;
-    p.X = (const uint8_t *)L.A, p.x_row_bytes = L.in_w * 2;
+    p.X = (const uint8_t *)L.A;
     p.B = 1, p.dc = 8, p.F = 0, p.xb = nullptr, p.check_ids = 0;
     for (int i = 0; i < p.n_k; ++i) p.src[i].kind = SRC_DENSE, p.src[i].off = i * 128;
     p.epi = L.sign_bits ? EPI_SIGN : EPI_STORE;
@@ -1558,7 +1547,7 @@ cudaError_t launch_score_tc_scratch(const aif_ctx *ctx, const ScoreLaunch &sl_in
     // are its positions, in another order.  By the groups' tiles the layers ran on rows that were mostly padding (20 candidates per
     // category: 800 tiles instead of 130).
     ScoreLaunch sl_rows = sl;
-    if (c.n_categories > 0) sl_rows.n_tiles = sl_in.n_tiles, sl_rows.n_tiles_dev = nullptr, sl_rows.tiles = sl.reqs ? (const TileDev *)sc.tiles : nullptr;
+    if (c.n_categories > 0) sl_rows.n_tiles = sl_in.n_tiles, sl_rows.tiles = sl.reqs ? (const TileDev *)sc.tiles : nullptr;
     // few tiles with many keys: their keys over several CTAs each (the table of jobs does it where categories are on)
     if (!sl.jobs) sl.parts = split_parts(sl.n_tiles, (sl.max_L + (c.d == 128 ? 127 : 63)) / (c.d == 128 ? 128 : 64), sl.split.slots);
     JoinParams join_att{}, join_lsh{};
@@ -1631,10 +1620,10 @@ cudaError_t launch_score_tc_scratch(const aif_ctx *ctx, const ScoreLaunch &sl_in
         p.T0 = (const uint8_t *)ctx->slots[0].dev.T, p.slot_bytes = (int64_t)ctx->slot_bytes;
         p.check_ids = k == 0;
         if (k == 0) {
-            p.X = (const uint8_t *)sc.X, p.x_row_bytes = pl->x_cols * 2;
+            p.X = (const uint8_t *)sc.X;
             for (int i = 0; i < p.n_k; ++i) p.src[i] = pl->src0[i];
         } else {
-            p.X = (const uint8_t *)sc.H[k - 1], p.x_row_bytes = c.hidden[k - 1] * 2;
+            p.X = (const uint8_t *)sc.H[k - 1];
             for (int i = 0; i < p.n_k; ++i) p.src[i].kind = SRC_DENSE, p.src[i].off = i * 128;
         }
         const bool last = k + 1 == c.n_hidden;

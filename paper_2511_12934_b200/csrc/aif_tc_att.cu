@@ -682,13 +682,6 @@ void tc_att_destroy(aif_ctx *ctx)
     ctx->tc_att_plan = nullptr;
 }
 
-// Rows a user state's S must have zeroed beyond L so that the last key block reads no stale values.
-int tc_att_key_block(const aif_ctx *ctx)
-{
-    const AttPlan *pl = reinterpret_cast<const AttPlan *>(ctx->tc_att_plan);
-    return pl ? pl->bn : 0;
-}
-
 // Store target of the attention rows: X as a [rows x x_stride] bf16 tensor, 32 x 32 boxes, 64-byte swizzle.
 static cudaError_t encode_x_map(CUtensorMap *m, void *X, int x_stride, size_t rows)
 {

@@ -148,13 +148,6 @@ __global__ void __launch_bounds__(256) k_slot_begin(SlotPieces sp, BeaUser bea, 
 // memory, no pipeline to fill, one memory latency per 16 rows.  A tcgen05 tile needs 128 rows, tensor memory and a weight
 // ring set up before its first product; at the 50 to 10^4 rows of one user that costs more than the product.
 // (K, N) of one thread's fragments: lane 4 g + t holds rows g, g + 8 and columns 2 t, 2 t + 1 of every eight.
-__device__ __forceinline__ void mma_bf16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1)
-{
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
-                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-                 : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-
 template <int VJ, int NT>
 struct WeightSlice {
     uint4 b[NT][VJ];
@@ -402,12 +395,11 @@ __global__ void k_user_project(const T *__restrict__ seq, const T *__restrict__ 
     }
 }
 
-// eq. 2.  Warp g handles rows g, g + n_warps, ...: attention over the whole sequence (or the rows att_rows, if the tensor-core
-// kernel has computed them), FFN hidden layer, running sum; partial[g] holds the warp's sum.
+// eq. 2.  Warp g handles rows g, g + n_warps, ...: attention over the whole sequence, FFN hidden layer, running sum; partial[g] holds
+// the warp's sum.
 template <typename T>
 __global__ void __launch_bounds__(256) k_user_self(const T *__restrict__ S, int L, int d, const T *__restrict__ Wa_t,
-                                                   const float *__restrict__ b_a, float *__restrict__ partial, int n_warps,
-                                                   const T *__restrict__ att_rows)
+                                                   const float *__restrict__ b_a, float *__restrict__ partial, int n_warps)
 {
     extern __shared__ float sm[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = blockIdx.x * 8 + warp, dq = d >> 5;
@@ -417,17 +409,13 @@ __global__ void __launch_bounds__(256) k_user_self(const T *__restrict__ S, int 
     for (int c = 0; c < 8; ++c) pooled[c] = 0.f;
     const float scale = rsqrtf((float)d);
     for (int i = g; i < L; i += n_warps) {
-        if (att_rows) {
-            for (int k = lane; k < d; k += 32) ctx[k] = to_f(att_rows[(size_t)i * d + k]);
-        } else {
-            for (int k = lane; k < d; k += 32) q[k] = to_f(S[(size_t)i * d + k]);
-            __syncwarp();
-            float att[8], din[8];
-            warp_interact<T>(q, S, L, d, scale, true, false, false, nullptr, nullptr, 0, 0, nullptr, att, din);
+        for (int k = lane; k < d; k += 32) q[k] = to_f(S[(size_t)i * d + k]);
+        __syncwarp();
+        float att[8], din[8];
+        warp_interact<T>(q, S, L, d, scale, true, false, false, nullptr, nullptr, 0, 0, nullptr, att, din);
 #pragma unroll
-            for (int c = 0; c < 8; ++c)
-                if (c < dq) ctx[lane + 32 * c] = att[c];
-        }
+        for (int c = 0; c < 8; ++c)
+            if (c < dq) ctx[lane + 32 * c] = att[c];
         __syncwarp();
 #pragma unroll
         for (int c = 0; c < 8; ++c)
@@ -614,7 +602,7 @@ cudaError_t launch_pool(const aif_ctx *ctx, const HostSlot &hs, const void *att_
                           hs.partial, (const bf16 *)hs.dev.S, (const float *)hs.prof_hat, slice, n_slices, hs.ppart);
     };
     count_launch();
-    return d == 64 ? go(k_user_pool<2, 1>) : d == 128 ? go(k_user_pool<4, 2>) : go(k_user_pool<8, 4>);
+    return d == 128 ? go(k_user_pool<4, 2>) : go(k_user_pool<8, 4>);
 }
 
 template <typename T>
@@ -678,20 +666,19 @@ cudaError_t user_network_typed(const aif_ctx *ctx, HostSlot &hs, int slot_index,
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
             if ((e = launch_row_norm_max(ctx, S, L, const_cast<float *>(hs.dev.k_norm), st)) != cudaSuccess) return e;
         }
-        const void *att_rows = nullptr;   // eq. 2: the attention rows on the tensor cores where the shape allows, else in k_user_self
+        const void *att_rows = nullptr;   // eq. 2: the attention rows on the tensor cores where the shape allows (d = 128, 256), else in k_user_self
         if (bf && ctx->tc_att_plan && (e = launch_self_att_tc(ctx, slot_index, L, st, &att_rows)) != cudaSuccess) return e;
         // key slices of eq. 3: whole steps of a warp (256 / d rows per load, eight loads), at most kProfParts of them
         const int step = 8 * (d <= 64 ? 4 : d <= 128 ? 2 : 1);
         const int slice = ((L + kProfParts - 1) / kProfParts + step - 1) / step * step;
         n_slices = (L + slice - 1) / slice;
-        if (att_rows && mma_width(d)) {
+        if (att_rows) {
             n_parts = (L + 15) / 16 < 148 ? (L + 15) / 16 : 148;
             if ((e = launch_pool(ctx, hs, att_rows, L, n_parts, slice, n_slices, st)) != cudaSuccess) return e;
         } else {
             k_user_prof<T><<<(n_slices + 7) / 8, 256, 0, st>>>(S, L, d, hs.prof_hat, slice, n_slices, hs.ppart);
             n_parts = (L + 7) / 8 * 8 < kUserPartials ? (L + 7) / 8 * 8 : kUserPartials;
-            k_user_self<T><<<n_parts / 8, 256, 8 * 2 * d * sizeof(float), st>>>(S, L, d, (const T *)ctx->Wa_t, ctx->b_a, hs.partial, n_parts,
-                                                                               (const T *)att_rows);
+            k_user_self<T><<<n_parts / 8, 256, 8 * 2 * d * sizeof(float), st>>>(S, L, d, (const T *)ctx->Wa_t, ctx->b_a, hs.partial, n_parts);
             count_launch(2);
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
         }
