@@ -342,23 +342,15 @@ __global__ void __launch_bounds__(PairCfg::kThreads, 1) k_layer_pair(const __gri
         // a wait that ran out in an earlier kernel of this call left its outputs unwritten: logits computed from them are
         // replaced by NaN
         const bool poisoned = p.epi == EPI_DOT && (*reinterpret_cast<volatile const uint32_t *>(p.sl.status) & AIF_STATUS_TIMEOUT) != 0u;
-        // What an item's epilogue reads from memory, its tile's place and the ids there, is requested while the one before is at work,
-        // the place two items ahead; biases that are the same for all items stay.  A narrow layer's item is shorter than the reads
-        // (64 -> 32 units, 3.2 x 10^5 candidates: 32.8 -> 28.7 us).
-        auto tile_of = [&](int item) { return decode_tile(p, item < n_items ? item / p.n_nchunks * 2 + rank : n_tiles, n_tiles); };
-        auto id_of = [&](const TileInfo &t) { return p.epi == EPI_DOT && half == 0 && row < t.cnt ? p.sl.ids[t.pos0 + row] : -1; };
-        const float b_out = p.epi == EPI_DOT ? p.b_out[0] : 0.f;
-        const bool same_bias = !p.bias_from_slot && p.n_nchunks == 1;
-        TileInfo t = tile_of(item0), t_next = tile_of(item0 + item_step);
-        int id = id_of(t);
         int it = 0;
         for (int item = item0; item < n_items; item += item_step, ++it) {
             const int grp = item / p.n_nchunks, n0 = (item - grp * p.n_nchunks) * p.n_cols;
             const int buf = it & 1;
+            const TileInfo t = decode_tile(p, grp * 2 + rank, n_tiles);
             const bool valid = row < t.cnt;
-            const int id_next = id_of(t_next);
-            const TileInfo t_after = tile_of(item + 2 * item_step);
-            if (t.cnt > 0 && !(same_bias && it > 0)) {
+            int id = -1;
+            if (p.epi == EPI_DOT && half == 0 && valid) id = p.sl.ids[t.pos0 + row];
+            if (t.cnt > 0) {
                 const float *bias = p.bias_from_slot ? p.sl.slots[t.rq.slot].p_u : p.bias;
                 if (tid < p.n_cols) {
                     const bool is_out = n0 + tid < p.n_out;
@@ -477,7 +469,7 @@ __global__ void __launch_bounds__(PairCfg::kThreads, 1) k_layer_pair(const __gri
             if (got && lane == 0) mbar_arrive_cluster(empty_addr[buf]);
             const bool out = named_bar_or(1, 256, !got);   // also orders dot_s
             if (p.epi == EPI_DOT && half == 0 && valid) {
-                float logit = dot + dot_s[row] + b_out;
+                float logit = dot + dot_s[row] + p.b_out[0];
                 if (p.emit_sigmoid) logit = 1.0f / (1.0f + expf(-logit));
                 // no number for an id outside the table, nor for a tile whose inputs never arrived (here or in an earlier
                 // kernel of the call: the status word says so)
@@ -485,7 +477,6 @@ __global__ void __launch_bounds__(PairCfg::kThreads, 1) k_layer_pair(const __gri
                 p.sl.logits[p.sl.out_index ? (int64_t)p.sl.out_index[t.pos0 + row] : t.pos0 + row] = logit;
             }
             if (out) break;
-            t = t_next, id = id_next, t_next = t_after;
         }
         if (lane == 0) bulk_wait<0>();   // all tile stores of this warp have reached global memory
     } else if (warp == C::kMmaWarp) {
