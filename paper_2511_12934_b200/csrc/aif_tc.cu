@@ -95,9 +95,11 @@ __device__ __forceinline__ TileInfo decode_tile(const LayerParams &p, int tile, 
 // once per call so that the layer kernel's gather threads only look the bucket up.  Ids in mapped host memory are copied
 // to ids_copy on the way, for the kernels that follow; candidates that are grouped by category are placed on the way (pl.where:
 // pos becomes the grouped position; F = 0 does nothing else).
+// POW2: the number of buckets is a power of two (a mask, with nothing of the other form's multiplications beside it).
 constexpr uint32_t kNoBucket = 0xFFFFu;
+template <bool POW2>
 __global__ void __launch_bounds__(256) k_cross_buckets(const int32_t *__restrict__ ids, int64_t total, int64_t M, int F, int B,
-                                                        int b_mask, uint64_t b_inv, int mode, uint16_t *__restrict__ xb, int32_t *__restrict__ ids_copy, const SimPlace pl, int late)
+                                                        uint64_t b_inv, int mode, uint16_t *__restrict__ xb, int32_t *__restrict__ ids_copy, const SimPlace pl, int late)
 {
     if (!late) grid_dep_wait();
     grid_dep_launch();
@@ -132,7 +134,7 @@ __global__ void __launch_bounds__(256) k_cross_buckets(const int32_t *__restrict
                     if (mode == AIF_BUCKET_MOD) bk[q] = (uint32_t)(id % B);
                     else {
                         const uint64_t h = mix64((uint64_t)id, (uint64_t)(f + q));
-                        if (b_mask >= 0) bk[q] = (uint32_t)(h & (uint64_t)b_mask);
+                        if (POW2) bk[q] = (uint32_t)h & (uint32_t)(B - 1);
                         else {
                             // Barrett reduction with b_inv = floor(2^64 / B): the estimated quotient is the true one or one less, as
                             // h (2^64 / B - b_inv) / 2^64 < 1.  With a 64-bit remainder each, 2 x 10^7 hashes took 130 us, so 62.
@@ -1517,8 +1519,8 @@ cudaError_t launch_score_tc_scratch(const aif_ctx *ctx, const ScoreLaunch &sl_in
         // of the ids crosses the bus
         const int rounds = F == 0 ? 1 : F & 1 ? F : F / 2, want_y = sl.ids_copy ? 1 : 296 / grid;
         const int grid_y = want_y < 1 ? 1 : want_y > 8 ? (rounds < 8 ? rounds : 8) : want_y > rounds ? rounds : want_y;
-        cudaError_t e = launch_pdl(k_cross_buckets, dim3(grid, grid_y), dim3(256), 0, st, sl.ids, sl.total, c.M, F, c.B,
-                                   (c.B & (c.B - 1)) == 0 ? c.B - 1 : -1, c.B > 0 ? ~0ull / (uint64_t)c.B : 0ull, c.bucket_mode, (uint16_t *)sc.xb, sl.ids_copy, place, late);
+        auto kernel = (c.B & (c.B - 1)) == 0 ? k_cross_buckets<true> : k_cross_buckets<false>;
+        cudaError_t e = launch_pdl(kernel, dim3(grid, grid_y), dim3(256), 0, st, sl.ids, sl.total, c.M, F, c.B, c.B > 0 ? ~0ull / (uint64_t)c.B : 0ull, c.bucket_mode, (uint16_t *)sc.xb, sl.ids_copy, place, late);
         if (sl.ids_copy) sl.ids = sl.ids_copy;
         if (place.where) sl.ids = place.ids;
         count_launch();
