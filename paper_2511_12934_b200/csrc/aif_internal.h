@@ -220,6 +220,8 @@ struct aif_ctx {
     void *nearline_plan = nullptr;    // item-side weights and scratch of aif_item_nearline_compute
     void *tc_fused_plan = nullptr;    // single-launch scoring: the second layer's bias split into two bf16 rows
     void *tc_lsh_plan = nullptr;      // tensor-core LSH blocks: tensor maps over the arena's S and +-1 signature regions
+    void *tc_tier_plan = nullptr;     // tensor-core SimTier: tensor maps over the +-1 signature regions, constants of the tier arithmetic
+    void *tc_din_plan = nullptr;      // LSH-DIN through the requests' own sums: tensor map, partial sums, operands; nullptr: not to be had
     void *sim_plan = nullptr;         // categories on: scratch of the grouping passes (aif_sim.cu)
     size_t grouped_rows = 0;          // rows of a slot's grouped sequence
     aif::PinnedRing ring;
@@ -297,6 +299,18 @@ cudaError_t tc_lsh_prepare(aif_ctx *ctx);
 void tc_lsh_destroy(aif_ctx *ctx);
 cudaError_t launch_lsh_tc(const aif_ctx *ctx, const ScoreLaunch &sl, cudaStream_t st, void *X, int x_stride, size_t x_rows, int x_din,
                           int x_tier, JoinParams &join);
+// SimTier alone, up to eight tiers (aif_tc_tier.cu)
+bool tc_tiers_supported(const aif_config &cfg);
+cudaError_t tc_tiers_prepare(aif_ctx *ctx);
+void tc_tiers_destroy(aif_ctx *ctx);
+cudaError_t launch_tiers(const aif_ctx *ctx, const ScoreLaunch &sl, cudaStream_t st, void *X, int x_stride, int x_tier, JoinParams &join);
+// LSH-DIN through sums that depend on the request alone (aif_tc_din.cu)
+bool tc_din_supported(const aif_config &cfg);
+cudaError_t tc_din_prepare(aif_ctx *ctx);
+void tc_din_destroy(aif_ctx *ctx);
+bool tc_din_pays(const aif_ctx *ctx, const ScoreLaunch &sl);
+cudaError_t launch_din_sums(const aif_ctx *ctx, const ScoreLaunch &sl, cudaStream_t st);
+cudaError_t launch_din_apply(const aif_ctx *ctx, const ScoreLaunch &sl, cudaStream_t st, void *X, int x_stride, size_t x_rows, int x_din);
 // category sub-sequences (aif_sim.cu): the user-side grouping of a sequence, and the grouping of a launch's candidates by
 // (request, category) into tiles
 size_t sim_grouped_rows(int L_max, int n_categories);

@@ -1321,6 +1321,8 @@ cudaError_t tc_prepare_context(aif_ctx *ctx)
     if (tc_att_supported(c) && (e = tc_att_prepare(ctx)) != cudaSuccess) return e;
     if (tc_fused_supported(c) && (e = tc_fused_prepare(ctx)) != cudaSuccess) return e;
     if (tc_lsh_supported(c) && (e = tc_lsh_prepare(ctx)) != cudaSuccess) return e;
+    if (tc_tiers_supported(c) && (e = tc_tiers_prepare(ctx)) != cudaSuccess) return e;
+    if (tc_din_supported(c) && (e = tc_din_prepare(ctx)) != cudaSuccess) return e;
     if (c.n_categories > 0 && (e = sim_prepare(ctx)) != cudaSuccess) return e;
     return cudaSuccess;
 }
@@ -1353,6 +1355,8 @@ void tc_destroy_context(aif_ctx *ctx)
 {
     if (ctx->tc_att_plan) tc_att_destroy(ctx);
     if (ctx->tc_lsh_plan) tc_lsh_destroy(ctx);
+    if (ctx->tc_tier_plan) tc_tiers_destroy(ctx);
+    if (ctx->tc_din_plan) tc_din_destroy(ctx);
     delete plan_of(ctx);
     ctx->tc_plan = nullptr;
 }
@@ -1542,15 +1546,32 @@ cudaError_t launch_score_tc_scratch(const aif_ctx *ctx, const ScoreLaunch &sl_in
     ScoreLaunch sl_rows = sl;
     if (c.n_categories > 0) sl_rows.n_tiles = sl_in.n_tiles, sl_rows.tiles = sl.reqs ? (const TileDev *)sc.tiles : nullptr;
     // few tiles with many keys: their keys over several CTAs each (the table of jobs does it where categories are on)
+    // LSH-DIN through sums of the request's own, where that is the shorter way; SimTier then counts by itself.  The sums come first and
+    // need nothing of the call: what follows runs beside them.
+    const bool din = c.blocks & AIF_BLK_LSH_DIN, tier = c.blocks & AIF_BLK_SIMTIER;
+    const bool din_sums = lsh_tc && din && sc.split && (!tier || ctx->tc_tier_plan) && tc_din_pays(ctx, sl);
+    const bool tiers_alone = tier && ctx->tc_tier_plan && (din_sums || !din);
+    int late = 0;
+    if (din_sums) {
+        StageRange range("aif lsh sums");
+        ScoreLaunch sl_sums = sl;
+        sl_sums.late = buckets_first;
+        const cudaError_t e = launch_din_sums(ctx, sl_sums, st);
+        if (c.n_hidden <= 2) timing_mark(ctx, "lsh_sums", st);   // (a call has room for eight marks)
+        if (e != cudaSuccess) return e;
+        late = !buckets_first;   // (ids that the buckets bring are waited for)
+    }
     if (!sl.jobs) sl.parts = split_parts(sl.n_tiles, (sl.max_L + (c.d == 128 ? 127 : 63)) / (c.d == 128 ? 128 : 64), sl.split.slots);
     JoinParams join_att{}, join_lsh{};
     if (att_tc) {
         StageRange range("aif attention");
-        cudaError_t e = launch_att_tc(ctx, sl, st, sc.X, pl->x_cols, sc.rows, join_att);
+        ScoreLaunch sl_att = sl;
+        sl_att.late = late;
+        cudaError_t e = launch_att_tc(ctx, sl_att, st, sc.X, pl->x_cols, sc.rows, join_att);
         timing_mark(ctx, "attention", st);
         if (e != cudaSuccess) return e;
     }
-    int late = att_tc;
+    if (att_tc) late = 1;
     auto bea = [&]() -> cudaError_t {
         if (!(c.blocks & AIF_BLK_BEA)) return cudaSuccess;
         StageRange range("aif bea");
@@ -1564,32 +1585,38 @@ cudaError_t launch_score_tc_scratch(const aif_ctx *ctx, const ScoreLaunch &sl_in
         return e;
     };
     if (att_tc && (eb = bea()) != cudaSuccess) return eb;
-    if (lsh_tc) {
-        // columns of X: [ att | v_bea | lsh_din | simtier (64) ], enabled blocks only
-        int col = 0;
-        if (c.blocks & AIF_BLK_ATT) col += c.d;
-        if (c.blocks & AIF_BLK_BEA) col += c.d;
-        const int x_din = (c.blocks & AIF_BLK_LSH_DIN) ? col : -1;
-        if (c.blocks & AIF_BLK_LSH_DIN) col += c.d;
-        const int x_tier = (c.blocks & AIF_BLK_SIMTIER) ? col : -1;
+    // columns of X: [ att | v_bea | lsh_din | simtier (64) ], enabled blocks only
+    const int x_lsh = ((c.blocks & AIF_BLK_ATT) ? c.d : 0) + ((c.blocks & AIF_BLK_BEA) ? c.d : 0);
+    const int x_din = din ? x_lsh : -1, x_tier = tier ? x_lsh + (din ? c.d : 0) : -1;
+    if (lsh_tc && !(din_sums && !tier)) {
         StageRange range("aif lsh");
         ScoreLaunch sl_lsh = sl;
         sl_lsh.late = late;
         if (att_tc && sc.split) sl_lsh.split = ctx->split_lsh;   // records of its own: the attention's are not joined yet
-        cudaError_t e = launch_lsh_tc(ctx, sl_lsh, st, sc.X, pl->x_cols, sc.rows, x_din, x_tier, join_lsh);
+        cudaError_t e = tiers_alone ? launch_tiers(ctx, sl_lsh, st, sc.X, pl->x_cols, x_tier, join_lsh)
+                                    : launch_lsh_tc(ctx, sl_lsh, st, sc.X, pl->x_cols, sc.rows, x_din, x_tier, join_lsh);
         timing_mark(ctx, "lsh", st);
         if (e != cudaSuccess) return e;
         late = 1;
     }
     // the pieces of keys: the first join waits for both kernels, the second one runs beside it
+    join_att.sl.late = 0;
     if (join_att.d && (eb = launch_join_pieces(join_att, st)) != cudaSuccess) return eb;
     if (join_lsh.d) {
         join_lsh.sl.late = join_att.d != 0;
         if ((eb = launch_join_pieces(join_lsh, st)) != cudaSuccess) return eb;
     }
+    if (!buckets_first && (eb = buckets(late)) != cudaSuccess) return eb;
+    if (din_sums) {
+        StageRange range("aif lsh rows");
+        ScoreLaunch sl_din = sl;
+        sl_din.late = 0;
+        const cudaError_t e = launch_din_apply(ctx, sl_din, st, sc.X, pl->x_cols, sc.rows, x_din);
+        timing_mark(ctx, tier ? "lsh_rows" : "lsh", st);
+        if (e != cudaSuccess) return e;
+    }
     const bool need_att = (c.blocks & AIF_BLK_ATT) && !att_tc, need_lsh = lsh_blocks && !lsh_tc;
     if (!att_tc && (eb = bea()) != cudaSuccess) return eb;
-    if (!buckets_first && (eb = buckets(late)) != cudaSuccess) return eb;
     if (need_att || need_lsh) {
         StageRange range("aif interact");
         const size_t smem = (size_t)8 * c.d * 4 + 64 * 4 + 128 * 4;

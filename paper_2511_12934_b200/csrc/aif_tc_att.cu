@@ -133,7 +133,7 @@ __global__ void __launch_bounds__((AttCfg<D, BN>::kThreads), 1) k_att_tc(const _
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
-    grid_dep_wait();   // the set-up above overlapped the previous kernel; the request table and slots are read from here on
+    if (!p.sl.late) grid_dep_wait();   // the set-up above overlapped the previous kernel; the request table and slots are read from here on
     grid_dep_launch();   // (after the wait: see ScoreLaunch::late)
 
     const int n_tiles = key_jobs<SPLIT>(p.sl);   // tiles, or pieces of tiles
@@ -603,6 +603,7 @@ __global__ void __launch_bounds__((AttCfg<D, BN>::kThreads), 1) k_att_tc(const _
     tc_fence_before();
     __syncthreads();
     if (warp == C::kMmaWarp) tmem_dealloc(tmem_base, 512);
+    if (p.sl.late && blockIdx.x == 0) grid_dep_wait();
 }
 
 struct AttPlan {

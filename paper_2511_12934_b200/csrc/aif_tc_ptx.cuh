@@ -200,6 +200,9 @@ __host__ __device__ constexpr uint32_t umma_idesc_e4m3(int m, int n)
     return (1u << 4) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
 
+// The same with D fp16: one value in the low half of every 32-bit column.
+__host__ __device__ constexpr uint32_t umma_idesc_e4m3_f16(int m, int n) { return ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24); }
+
 __device__ __forceinline__ void umma_e4m3(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate)
 {
     asm volatile(
@@ -498,9 +501,9 @@ __device__ __forceinline__ float fast_exp2(float x)
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-// The same for a kernel of CTA pairs (clusters of two; the grid is even).
+// The same for a kernel of clusters of CTAs along x (the grid is a multiple of them).
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_pdl_pair(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args &&...args)
+inline cudaError_t launch_pdl_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, unsigned cluster, cudaStream_t st, Args &&...args)
 {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid, cfg.blockDim = block, cfg.dynamicSmemBytes = smem, cfg.stream = st;
@@ -508,9 +511,15 @@ inline cudaError_t launch_pdl_pair(void (*kernel)(KArgs...), dim3 grid, dim3 blo
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = 2, attr[1].val.clusterDim.y = 1, attr[1].val.clusterDim.z = 1;
+    attr[1].val.clusterDim.x = cluster, attr[1].val.clusterDim.y = 1, attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr, cfg.numAttrs = 2;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+// Of CTA pairs.
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_pdl_pair(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args &&...args)
+{
+    return launch_pdl_cluster(kernel, grid, block, smem, 2u, st, static_cast<Args &&>(args)...);
 }
 
 template <typename... KArgs, typename... Args>
