@@ -361,6 +361,7 @@ struct DenseLayer {
     int32_t in_w, H;
     int32_t relu;        // 0: linear output
     int32_t sign_bits;
+    int32_t late = 0;    // as in ScoreLaunch
 };
 cudaError_t tc_dense_layer(const aif_ctx *ctx, const DenseLayer &L, int64_t rows, cudaStream_t st);
 // the item-side tower in one kernel, hidden activations in tensor memory (aif_tc_tower.cu)

@@ -92,8 +92,10 @@ __global__ void __launch_bounds__(256) k_item_bridge_weights(const T *__restrict
 // above) took 217 us for 262143 items at d = 128, n = 8.
 template <int VJ, int NT>
 __global__ void __launch_bounds__(256) k_item_bridge_weights_mma(const __nv_bfloat16 *__restrict__ I_id, int64_t n, int nb,
-                                                                 const __nv_bfloat16 *__restrict__ Bm, __nv_bfloat16 *__restrict__ out)
+                                                                 const __nv_bfloat16 *__restrict__ Bm, __nv_bfloat16 *__restrict__ out, int late)
 {
+    if (!late) grid_dep_wait();
+    grid_dep_launch();
     constexpr int D = 32 * VJ;
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     const float scale = rsqrtf((float)D);
@@ -153,6 +155,7 @@ __global__ void __launch_bounds__(256) k_item_bridge_weights_mma(const __nv_bflo
             }
         }
     }
+    if (late && blockIdx.x == 0) grid_dep_wait();
 }
 
 // eq. 5 on CUDA cores: one warp per item, 32 bits per round; eight bits per byte, first bit most significant.
@@ -213,6 +216,9 @@ cudaError_t run_pass(aif_ctx *ctx, NearlinePlan *pl, int64_t m, const void *I_ra
     }
     // the table's norm bound from the rows just computed (whether or not their ids turn out to lie in the table)
     if (!(pl->tensor && pl->fused_tower) && (e = launch_row_norm_max(ctx, rows_out, m, ctx->e_norm, st)) != cudaSuccess) return e;
+    // The tower in one kernel waits for the stream's earlier work before it lets the next kernel start, so that what needs nothing of it
+    // runs beside it, in its tail and without the gaps between launches.
+    bool beside = pl->tensor && pl->fused_tower;
     if (c.blocks & AIF_BLK_BEA) {
         const void *id_rows = I_id ? I_id : rows_out;
         // matrix instructions for the d that divide into whole quads of 16-byte pieces; they read 16 bytes at a time
@@ -221,19 +227,25 @@ cudaError_t run_pass(aif_ctx *ctx, NearlinePlan *pl, int64_t m, const void *I_ra
             using bf = __nv_bfloat16;
             const int64_t blocks = (m + 127) / 128;
             const int grid = (int)(blocks < 148 * 6 ? blocks : 148 * 6);
-            auto go = [&](auto kernel) { kernel<<<grid, 256, 0, st>>>((const bf *)id_rows, m, c.n_bridge, (const bf *)pl->bridges, (bf *)bea_out); };
+            const int late = beside && I_id;   // (else it reads the rows just computed)
+            auto go = [&](auto kernel) {
+                e = launch_pdl(kernel, dim3(grid), dim3(256), 0, st, (const bf *)id_rows, m, c.n_bridge, (const bf *)pl->bridges, (bf *)bea_out, late);
+            };
             const bool two = c.n_bridge > 8;
             if (c.d == 64) two ? go(k_item_bridge_weights_mma<2, 2>) : go(k_item_bridge_weights_mma<2, 1>);
             else if (c.d == 128) two ? go(k_item_bridge_weights_mma<4, 2>) : go(k_item_bridge_weights_mma<4, 1>);
             else two ? go(k_item_bridge_weights_mma<8, 2>) : go(k_item_bridge_weights_mma<8, 1>);
-        } else
+            if (e != cudaSuccess) return e;
+        } else {
+            beside = false;
             k_item_bridge_weights<T><<<grid_for_items(m), 256, 0, st>>>((const T *)id_rows, m, c.d, c.n_bridge, (const T *)pl->bridges, (T *)bea_out);
+        }
         count_launch();
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     if (c.blocks & (AIF_BLK_LSH_DIN | AIF_BLK_SIMTIER)) {
         if (pl->tensor) {
-            DenseLayer lh{M_mm, pl->W_hash, pl->zeros, sig_out, pl->d_mm, c.lsh_bits, 0, 1};
+            DenseLayer lh{M_mm, pl->W_hash, pl->zeros, sig_out, pl->d_mm, c.lsh_bits, 0, 1, beside};
             if ((e = tc_dense_layer(ctx, lh, m, st)) != cudaSuccess) return e;
         } else {
             k_item_signatures<T><<<grid_for_items(m), 256, (size_t)8 * pl->d_mm * 4, st>>>((const T *)M_mm, m, pl->d_mm, c.lsh_bits,

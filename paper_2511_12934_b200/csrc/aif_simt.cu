@@ -49,6 +49,10 @@ __device__ __forceinline__ void move_side(const SideRows &s, int rows, int64_t r
     else move_side_units<uint8_t, SCATTER>((const uint8_t *)s.src, (uint8_t *)s.dst, s.bytes, rows, r0, n, my);
 }
 
+// Sidecar rows of one 16-byte unit (eight bf16 bridge weights, 128 signature bits): a lane moves its row's in one piece, so the loads of
+// both sidecars go out with the others of a step instead of after its stores.
+__device__ __forceinline__ bool one_unit(const SideRows &s) { return s.bytes == 16 && s.unit == 16; }
+
 static SideRows side_rows(const void *src, void *dst, size_t bytes)
 {
     SideRows s{src, dst, (int32_t)bytes, 16};
@@ -97,6 +101,10 @@ __global__ void __launch_bounds__(256) k_refresh_rows(uint4 *__restrict__ table,
         int64_t dst_row = -1;
         const bool has_id = lane < RPS && r0 + lane < n;
         if (has_id) dst_row = ids ? (int64_t)ids[r0 + lane] : r0 + lane;
+        const bool bea_one = one_unit(bea), sig_one = one_unit(sig);
+        uint4 bea_v = make_uint4(0, 0, 0, 0), sig_v = bea_v;
+        if (has_id && bea_one) bea_v = __ldcs(reinterpret_cast<const uint4 *>(bea.src) + r0 + lane);
+        if (has_id && sig_one) sig_v = __ldcs(reinterpret_cast<const uint4 *>(sig.src) + r0 + lane);
         float ss[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u) ss[u] = 0.f;
@@ -127,8 +135,10 @@ __global__ void __launch_bounds__(256) k_refresh_rows(uint4 *__restrict__ table,
                 best = max(best, __float_as_int(sqrtf(ss[u])) & 0x7fffffff);
             }
         }
-        move_side<true>(bea, RPS, r0, n, my);
-        move_side<true>(sig, RPS, r0, n, my);
+        if (!bea_one) move_side<true>(bea, RPS, r0, n, my);
+        else if (my >= 0) reinterpret_cast<uint4 *>(bea.dst)[my] = bea_v;
+        if (!sig_one) move_side<true>(sig, RPS, r0, n, my);
+        else if (my >= 0) reinterpret_cast<uint4 *>(sig.dst)[my] = sig_v;
     }
     if (norm_max) {
         best = __reduce_max_sync(0xffffffffu, best);
@@ -292,8 +302,14 @@ __global__ void __launch_bounds__(256) k_gather_sidecars(const int32_t *__restri
                 atomicOr(status, AIF_STATUS_BAD_ID);
             }
         }
-        move_side<false>(bea, 32, r0, n, my);
-        move_side<false>(sig, 32, r0, n, my);
+        const bool bea_one = one_unit(bea), sig_one = one_unit(sig);
+        uint4 bea_v = make_uint4(0, 0, 0, 0), sig_v = bea_v;
+        if (my >= 0 && bea_one) bea_v = reinterpret_cast<const uint4 *>(bea.src)[my];
+        if (my >= 0 && sig_one) sig_v = reinterpret_cast<const uint4 *>(sig.src)[my];
+        if (!bea_one) move_side<false>(bea, 32, r0, n, my);
+        else if (r0 + lane < n) __stcs(reinterpret_cast<uint4 *>(bea.dst) + r0 + lane, bea_v);
+        if (!sig_one) move_side<false>(sig, 32, r0, n, my);
+        else if (r0 + lane < n) __stcs(reinterpret_cast<uint4 *>(sig.dst) + r0 + lane, sig_v);
     }
 }
 

@@ -326,7 +326,7 @@ __global__ void __launch_bounds__(PairCfg::kThreads, 1) k_layer_pair(const __gri
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
     grid_dep_launch();
-    if (warp != C::kBWarp) grid_dep_wait();   // the weights are older than any launch this one may overlap
+    if (warp != C::kBWarp && !p.sl.late) grid_dep_wait();   // the weights are older than any launch this one may overlap
     const int n_tiles = p.sl.n_tiles;
     const int n_items = ((n_tiles + 1) / 2) * p.n_nchunks;
     const int item0 = (int)(blockIdx.x >> 1), item_step = (int)(gridDim.x >> 1);
@@ -608,6 +608,7 @@ __global__ void __launch_bounds__(PairCfg::kThreads, 1) k_layer_pair(const __gri
     __syncthreads();
     cluster_sync();
     if (warp == C::kMmaWarp) tmem_dealloc_pair(tmem_base, 512);
+    if (p.sl.late && blockIdx.x == 0) grid_dep_wait();
 }
 
 // ---- both layers of a two-layer MLP -------------------------------------------------------------------------------
@@ -1423,7 +1424,7 @@ cudaError_t tc_dense_layer(const aif_ctx *ctx, const DenseLayer &L, int64_t rows
     p.sl.slots = ctx->slots_dev, p.sl.reqs = nullptr, p.sl.n_req = 1;
     p.sl.single = ReqDev{0, (int32_t)rows, 0, 0, 0};
     p.sl.n_tiles = (int32_t)((rows + kTcTile - 1) / kTcTile), p.sl.total = rows, p.sl.max_L = 0;
-    p.sl.ids = nullptr, p.sl.logits = nullptr, p.sl.status = ctx->status;
+    p.sl.ids = nullptr, p.sl.logits = nullptr, p.sl.status = ctx->status, p.sl.late = L.late;
     p.n_cols = slice_cols(L.H), p.n_nchunks = (L.H + p.n_cols - 1) / p.n_cols, p.n_out = L.H, p.n_k = L.in_w / 64, p.mini_batch = 0;
     p.E = (const uint8_t *)ctx->E, p.M = ctx->cfg.M, p.e_row_bytes = ctx->cfg.d * 2;
     p.X = (const uint8_t *)L.A;

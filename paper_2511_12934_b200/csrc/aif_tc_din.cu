@@ -550,6 +550,16 @@ int din_parts(const DinPlan &pl, int n_req, int d, int max_L)
     return best;
 }
 
+// Where the two launches (about 10 us before and behind the others) are less than what the pass over the pairs saves without the product:
+// key blocks of 128 per SM.  d = 128, this way / the other, us: 64 x 5000 candidates of 300 keys (52 blocks) 658 / 675 with all blocks on, of
+// 1000 (138) 752 / 827; 32 x 5000 of 400 (35) 243 / 245; 8 x 5000 of 1000 (17) 91.1 / 91.6; 1 x 3000 of 10^4 (13) 48.5 / 47.2; one key
+// block each 458 / 447.  d = 256: 32 x 2000 of 1000 (28) 437 / 423, of 2000 (55) 451 / 479; 4 x 4000 of 2000 (14) 137 / 137, of 5000 (35) 149 / 173.
+bool din_pays(int d, int64_t n_tiles, int L)
+{
+    const int64_t blocks = ((int64_t)L + kDinBlock - 1) / kDinBlock;
+    return d == 128 ? blocks >= 3 && n_tiles * blocks >= 148 * 20 : blocks >= 8 && n_tiles * blocks >= 148 * 32;
+}
+
 }  // namespace
 
 bool tc_din_supported(const aif_config &c)
@@ -561,6 +571,7 @@ bool tc_din_supported(const aif_config &c)
 cudaError_t tc_din_prepare(aif_ctx *ctx)
 {
     const aif_config &c = ctx->cfg;
+    if (!din_pays(c.d, (int64_t)tc_tile_capacity(ctx), c.L_max)) return cudaSuccess;   // no launch of this context is large enough
     const size_t n = (size_t)c.max_user_states * (c.d / kDinCols), records = n < 148 ? 148 : n;   // din_parts: more than one part only within them
     const size_t rec_bytes = records * din_record_bytes(c.d), image_bytes = (size_t)c.max_user_states * din_image_bytes(c.d);
     void *rec = nullptr, *image = nullptr;
@@ -611,18 +622,11 @@ void tc_din_destroy(aif_ctx *ctx)
     ctx->tc_din_plan = nullptr;
 }
 
-// Where the two launches (about 10 us before and behind the others) are less than what the pass over the pairs saves without the product:
-// key blocks of 128 per SM.  d = 128, this way / the other, us: 64 x 5000 candidates of 300 keys (52 blocks) 658 / 675 with all blocks on, of
-// 1000 (138) 752 / 827; 32 x 5000 of 400 (35) 243 / 245; 8 x 5000 of 1000 (17) 91.1 / 91.6; 1 x 3000 of 10^4 (13) 48.5 / 47.2; one key
-// block each 458 / 447.  d = 256: 32 x 2000 of 1000 (28) 437 / 423, of 2000 (55) 451 / 479; 4 x 4000 of 2000 (14) 137 / 137, of 5000 (35) 149 / 173.
 bool tc_din_pays(const aif_ctx *ctx, const ScoreLaunch &sl)
 {
     const aif_config &c = ctx->cfg;
     const DinPlan *pl = reinterpret_cast<const DinPlan *>(ctx->tc_din_plan);
-    if (!pl || sl.grouped || sl.n_req > 65535) return false;
-    if ((int64_t)sl.n_req * (c.d / kDinCols) * din_parts(*pl, sl.n_req, c.d, sl.max_L) > pl->records_cap) return false;
-    const int64_t blocks = (sl.max_L + kDinBlock - 1) / kDinBlock;
-    return c.d == 128 ? blocks >= 3 && sl.n_tiles * blocks >= 148 * 20 : blocks >= 8 && sl.n_tiles * blocks >= 148 * 32;
+    return pl && !sl.grouped && sl.n_req <= 65535 && (int64_t)sl.n_req * (c.d / kDinCols) <= pl->records_cap && din_pays(c.d, sl.n_tiles, sl.max_L);
 }
 
 cudaError_t launch_din_sums(const aif_ctx *ctx, const ScoreLaunch &sl, cudaStream_t st)

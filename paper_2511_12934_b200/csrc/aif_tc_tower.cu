@@ -79,8 +79,8 @@ __global__ void __launch_bounds__(kTThreads, 1) k_item_tower_tc(const __grid_con
     cluster_sync();   // the other CTA's barriers exist
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
-    grid_dep_launch();
     grid_dep_wait();
+    grid_dep_launch();   // (after the wait: what follows in the call runs beside this kernel without one of its own)
     // layer 2 of an item comes in the middle of the next one's layer 1: by then its activations are packed, and its output leaves
     // under the other half (after the whole of it: 9.0 k cycles per item, 2.3 k of them waiting for the output)
     const int n_k2 = p.hI >> 6, mid = p.n_k1 >> 1;
