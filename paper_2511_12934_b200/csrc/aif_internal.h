@@ -219,6 +219,7 @@ struct aif_ctx {
     void *tc_att_plan = nullptr;      // tensor-core attention: tensor map over the arena's S regions
     void *nearline_plan = nullptr;    // item-side weights and scratch of aif_item_nearline_compute
     void *tc_fused_plan = nullptr;    // single-launch scoring: the second layer's bias split into two bf16 rows
+    int split_clusters = 0;           // clusters of four of the small-request kernel that the machine holds at once
     void *tc_lsh_plan = nullptr;      // tensor-core LSH blocks: tensor maps over the arena's S and +-1 signature regions
     void *tc_tier_plan = nullptr;     // tensor-core SimTier: tensor maps over the +-1 signature regions, constants of the tier arithmetic
     void *tc_din_plan = nullptr;      // LSH-DIN through the requests' own sums: tensor map, partial sums, operands; nullptr: not to be had
@@ -334,6 +335,12 @@ bool tc_fused_supported(const aif_config &cfg);
 cudaError_t tc_fused_prepare(aif_ctx *ctx);
 cudaError_t tc_fused_prepare_weights(aif_ctx *ctx, cudaStream_t st);
 cudaError_t launch_request_fused(const aif_ctx *ctx, const ScoreLaunch &sl, cudaStream_t st);
+// the same for a small request by clusters of four CTAs (aif_tc_split.cu)
+int tc_split_prepare();
+bool tc_split_fits(const aif_ctx *ctx, int n);
+cudaError_t launch_request_split(const aif_ctx *ctx, const ScoreLaunch &sl, cudaStream_t st);
+const void *tc_weight_half_tmap(const aif_ctx *ctx, int k);   // with boxes of half a slice's rows
+const void *tc_weight_quarter_tmap(const aif_ctx *ctx);       // second layer, boxes of a quarter of its units
 const void *tc_weight_tmap(const aif_ctx *ctx, int k);   // CUtensorMap over the packed weights of hidden layer k
 const void *tc_att_tmap(const aif_ctx *ctx);             // CUtensorMap over the S regions of the user-state arena
 cudaError_t tc_prepare_weights(aif_ctx *ctx, const aif_weights *w, cudaStream_t st);

@@ -1148,6 +1148,7 @@ struct TcPlan {
     ChunkSrc src0[kMaxChunks] = {};
     CUtensorMap tmap[kMaxHidden];
     CUtensorMap tmap_half[kMaxHidden];   // the same weights, boxes of half a slice's rows (layer kernel)
+    CUtensorMap tmap_quarter;            // the second layer's, boxes of a quarter of its units (small-request kernel)
     size_t cap_rows = 0;                 // rows of the context's own scratch arrays
     __nv_bfloat16 *W[kMaxHidden] = {};
     __nv_bfloat16 *H[kMaxHidden] = {};   // activations after layer k (k < last)
@@ -1288,6 +1289,12 @@ cudaError_t tc_prepare_context(aif_ctx *ctx)
                              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
             if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
         }
+        if (k == 1 && tc_fused_supported(c)) {
+            const cuuint32_t box[2] = {64, (cuuint32_t)c.hidden[1] / 4};
+            if (enc(&pl->tmap_quarter, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, pl->W[k], dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                    CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+                return cudaErrorInvalidValue;
+        }
         in_w = c.hidden[k];
     }
     pl->maps_ready = true;
@@ -1321,6 +1328,7 @@ cudaError_t tc_prepare_context(aif_ctx *ctx)
     if (att) take_split(ctx->split_user, records((c.L_max + kTcTile - 1) / kTcTile, kSplitSlotsUser), false);
     if (tc_att_supported(c) && (e = tc_att_prepare(ctx)) != cudaSuccess) return e;
     if (tc_fused_supported(c) && (e = tc_fused_prepare(ctx)) != cudaSuccess) return e;
+    if (tc_fused_supported(c)) ctx->split_clusters = tc_split_prepare();
     if (tc_lsh_supported(c) && (e = tc_lsh_prepare(ctx)) != cudaSuccess) return e;
     if (tc_tiers_supported(c) && (e = tc_tiers_prepare(ctx)) != cudaSuccess) return e;
     if (tc_din_supported(c) && (e = tc_din_prepare(ctx)) != cudaSuccess) return e;
@@ -1350,6 +1358,8 @@ cudaError_t launch_join_pieces(const JoinParams &p, cudaStream_t st)
     return e;
 }
 
+const void *tc_weight_half_tmap(const aif_ctx *ctx, int k) { return &plan_of(ctx)->tmap_half[k]; }
+const void *tc_weight_quarter_tmap(const aif_ctx *ctx) { return &plan_of(ctx)->tmap_quarter; }
 const void *tc_weight_tmap(const aif_ctx *ctx, int k) { return &plan_of(ctx)->tmap[k]; }
 
 void tc_destroy_context(aif_ctx *ctx)
@@ -1490,7 +1500,7 @@ cudaError_t launch_score_tc_scratch(const aif_ctx *ctx, const ScoreLaunch &sl_in
     // a launch that fits the machine in one round of tiles: the whole pass in one kernel, one CTA per tile
     if (c.n_categories == 0 && sl.n_tiles <= kFusedMaxTiles && sl.max_L <= 256 && tc_fused_supported(c)) {
         StageRange range("aif score_fused");
-        cudaError_t e = launch_request_fused(ctx, sl, st);
+        cudaError_t e = !sl.reqs && tc_split_fits(ctx, sl.single.n) ? launch_request_split(ctx, sl, st) : launch_request_fused(ctx, sl, st);
         timing_mark(ctx, "score_fused", st);
         return e;
     }

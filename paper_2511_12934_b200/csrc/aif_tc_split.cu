@@ -1,0 +1,496 @@
+// Scoring pass of a small request by clusters of four CTAs (sm_100a, bf16 storage), the same shapes as aif_tc_fused.cu.
+//
+// In the kernel of one CTA per tile every SM takes in all weights, 1.05 MB at 59 bytes per clock, and 1000 candidates are 8 tiles on 148 SMs:
+// 37 k cycles whatever the machine could do beside.  Here a request's candidates go in tiles of 16 to 48, as many as clusters of four find
+// room for at once, and the four CTAs of a cluster share the units: each forms 128 units of the first layer and a quarter of the
+// second for all candidates of the tile, 260 KB of weights.  The layers' products are units x candidates (M = 128 units, N = the tile),
+// so a narrow tile costs no padding.  Every CTA of a cluster gathers the tile's rows and does its attention (a few hundred keys for a few
+// candidates: less than handing the rows round); the first layer's activations, 128 units of every candidate, go to the other three from
+// shared memory to shared memory (8 KB each for 32 candidates), and the four partial logits to the first.
+// RESULT
+//
+// Products the other way round without sharing the units (a tile of up to 128 per CTA, all weights): 22.5 us for 1000 candidates, the weights'
+// way into the SM unchanged.
+//
+// 448 threads: warps 0-7 softmax and epilogues, 8 the issuing lane, 9-12 gather, 13 one lane of TMA, as there.
+// Tensor memory: attention as there (scores [0, 256), O [256, 384), probabilities [384, 512)); then the layers' accumulators, tile columns each, at 0
+// and 64.  Every wait is bounded.
+#include <cuda.h>
+
+#include "aif_device.cuh"
+#include "aif_internal.h"
+#include "aif_tc_ptx.cuh"
+
+namespace aif {
+namespace {
+
+constexpr int kFThreads = 448;
+constexpr int kFMmaWarp = 8, kFProdWarp0 = 9, kFBWarp = 13;
+constexpr int kChunk = 16384;                  // 128 rows x 64 bf16
+constexpr int kCtas = 4;                       // of a cluster
+constexpr int kMaxTile = 48;
+constexpr int kBStage = 16384, kMaxStages = 8;
+constexpr size_t kFSmem = 227 * 1024;
+constexpr int kMiscBytes = 1024 + 2048;        // barriers | 8 x 64 partial dots
+// shared memory behind the miscellany, with c = tile x 128 bytes a chunk of 64 columns: E 2 c | key/value blocks 64 KB, later the attention
+// chunks | cross chunks 8 c | activations 8 c | weight ring
+constexpr int stages_for(int tile) { return ((int)kFSmem - 1024 - kMiscBytes - 65536 - 18 * tile * 128) / kBStage < kMaxStages ? ((int)kFSmem - 1024 - kMiscBytes - 65536 - 18 * tile * 128) / kBStage : kMaxStages; }
+static_assert(stages_for(kMaxTile) >= 3, "weight ring");
+constexpr int kMaxCross = 8;                   // cross-feature chunks (64 columns each)
+constexpr int kH1 = 512;
+
+enum {
+    BAR_E_FULL = 0, BAR_KV_FULL, BAR_S_FULL = BAR_KV_FULL + 2, BAR_P_FULL = BAR_S_FULL + 2, BAR_O_FINAL, BAR_ATT_FULL, BAR_ACC1_FULL,
+    BAR_H1_FULL, BAR_ACC2_FULL, BAR_FULL_A, BAR_FULL_B = BAR_FULL_A + kMaxCross, BAR_EMPTY_B = BAR_FULL_B + kMaxStages, BAR_COUNT = BAR_EMPTY_B + kMaxStages
+};
+static_assert(BAR_COUNT * 8 + 16 <= 512, "barriers");
+
+struct SplitParams {
+    ScoreLaunch sl;
+    const uint8_t *E;
+    int64_t M;
+    int32_t tile;           // candidates per cluster, a multiple of 16, at most kMaxTile
+    int32_t stages;         // of the weight ring
+    int32_t B, dc, b_mask, bucket_mode, n_cross;
+    int32_t H2, emit_sigmoid;
+    float scale_log2;       // log2(e) / sqrt(d)
+    const float *b2;        // [H2] second-layer bias
+    const __nv_bfloat16 *w_out;
+    const float *b_out;
+};
+
+__global__ void __launch_bounds__(kFThreads, 1) k_request_split(const __grid_constant__ CUtensorMap tmapS,
+                                                                const __grid_constant__ CUtensorMap tmapW1,
+                                                                const __grid_constant__ CUtensorMap tmapW2, const SplitParams p)
+{
+    extern __shared__ unsigned char smem_dyn[];
+    unsigned char *misc = reinterpret_cast<unsigned char *>(((uintptr_t)smem_dyn + 1023) & ~(uintptr_t)1023);
+    uint64_t *bars = reinterpret_cast<uint64_t *>(misc);
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + BAR_COUNT);
+    volatile uint32_t *abort_flag = tmem_slot + 1;
+    float *xs = reinterpret_cast<float *>(misc + 512);         // [2][64]: row sums or maxima of the two softmax groups
+    float *dot_s = reinterpret_cast<float *>(misc + 1024);     // [4][64]: per warp of a group's rows, partial dots
+    float *red_s = dot_s + 256;                                // [4][64]: the CTAs' partial logits (first CTA), element 63 of each: all is well
+    const int cs = p.tile * 128;
+    unsigned char *smE = misc + kMiscBytes, *smKV = smE + 2 * cs, *smAtt = smKV, *smX = smKV + 65536, *smH = smX + 8 * cs, *smB = smH + 8 * cs;
+    auto bar = [&](int i) { return smem_u32(bars + i); };
+
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int rank = (int)cluster_rank(), cluster = (int)(blockIdx.x / kCtas);
+
+    if (tid == 0) {
+        mbar_init(bar(BAR_E_FULL), 128);
+        mbar_init(bar(BAR_KV_FULL), 1);
+        mbar_init(bar(BAR_KV_FULL + 1), 1);
+        mbar_init(bar(BAR_S_FULL), 1);
+        mbar_init(bar(BAR_S_FULL + 1), 1);
+        mbar_init(bar(BAR_P_FULL), 256);
+        mbar_init(bar(BAR_O_FINAL), 1);
+        mbar_init(bar(BAR_ATT_FULL), 256);
+        mbar_init(bar(BAR_ACC1_FULL), 1);
+        mbar_init(bar(BAR_H1_FULL), 1);
+        mbar_init(bar(BAR_ACC2_FULL), 1);
+        for (int i = 0; i < kMaxCross; ++i) mbar_init(bar(BAR_FULL_A + i), 128);
+        for (int s = 0; s < kMaxStages; ++s) mbar_init(bar(BAR_FULL_B + s), 1), mbar_init(bar(BAR_EMPTY_B + s), 1);
+        *abort_flag = 0u;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    // The gather threads fetch their candidate ids while barriers and tensor memory are being set up: the ids head the
+    // longest chain of dependent memory accesses of the kernel (ids -> item rows -> scores).
+    int mine = -1;
+    if (warp >= kFProdWarp0 && warp < kFBWarp) {
+        grid_dep_wait();
+        // (they may lie in host memory across the bus: a gather warp reads its rows' once and hands them round by shuffle, after the barrier)
+        const int w = warp - kFProdWarp0, r = 4 * w + (lane & 3) + 16 * (lane >> 2);
+        if (r < min(p.tile, p.sl.single.n - cluster * p.tile)) mine = p.sl.ids[p.sl.single.off + cluster * p.tile + r];
+    }
+    if (warp == kFMmaWarp) tmem_alloc(smem_u32(tmem_slot), 512);
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync();   // the other CTAs' barriers exist
+    tc_fence_after();
+    const uint32_t tmem_base = *tmem_slot;
+    grid_dep_launch();
+    grid_dep_wait();
+
+    const ReqDev rq = p.sl.single;
+    const int start = cluster * p.tile, cnt = min(p.tile, rq.n - start);
+    const int64_t pos0 = rq.off + start;
+    const SlotDev *slot = p.sl.slots + rq.slot;
+    const int L = slot->L;
+    const int nb = L > 128 ? 2 : 1;
+    const int n_k1 = 4 + p.n_cross;
+
+    if (warp < 8) {
+        // ===================== softmax, epilogues =====================
+        const int g = warp >> 2, wq = warp & 3, row = wq * 32 + lane;
+        const uint32_t lane_base = tmem_base + ((uint32_t)(wq * 32) << 16);
+        const float k2 = p.scale_log2;
+        bool ok = true;
+        // a wait of the whole warp: the tensor-memory loads and stores that follow need every lane to take the same branch
+        auto wait = [&](int b) {
+            const bool got = ok && mbar_wait(bar(b), 0u, abort_flag);
+            ok = __all_sync(0xffffffffu, got);
+        };
+        bool good = false;
+        if (row < cnt) {
+            const int id = p.sl.ids[pos0 + row];
+            good = id >= 0 && (int64_t)id < p.M;
+        }
+        // ---- attention: scores of key block g -> probabilities
+        // Softmax is invariant to the offset subtracted in the exponent, and bf16 keeps its relative precision over the
+        // whole fp32 exponent range.  The first attempt therefore subtracts nothing, p = 2^(s k2), and saves the pass
+        // over the scores that finds the row maxima; a row sum outside [2^-80, 2^80] (scores far from zero: overflow,
+        // or every term flushed to zero) makes the whole CTA repeat the step with the exact row maxima.  The
+        // probabilities go to columns of their own, so the scores are still there for the repeat.
+        const bool act = g < nb && wq * 32 < p.tile;   // rows beyond the tile: nobody's (the products read whatever lies there)
+        const int valid_cols = L - g * 128 < 128 ? L - g * 128 : 128;
+        const uint32_t p_col = 384u + (uint32_t)(g * 64);
+        auto probabilities = [&](float mt) {   // P = 2^(s k2 - mt) as packed bf16; returns the row sum over this block
+            float lsum = 0.f;
+#pragma unroll 1
+            for (int h = 0; h < 2; ++h) {
+                uint32_t sc[64];
+                tmem_ld32(lane_base + (uint32_t)(g * 128 + 64 * h), *reinterpret_cast<uint32_t(*)[32]>(&sc[0]));
+                tmem_ld32(lane_base + (uint32_t)(g * 128 + 64 * h + 32), *reinterpret_cast<uint32_t(*)[32]>(&sc[32]));
+                tmem_ld_wait();
+                uint32_t packed[32];
+                float ls4[4] = {0.f, 0.f, 0.f, 0.f};
+                const int left = valid_cols - 64 * h;   // valid columns among these 64
+#pragma unroll
+                for (int i = 0; i < 32; ++i) {
+                    float p0 = fast_exp2(fmaf(__uint_as_float(sc[2 * i]), k2, -mt));
+                    float p1 = fast_exp2(fmaf(__uint_as_float(sc[2 * i + 1]), k2, -mt));
+                    if (2 * i >= left) p0 = 0.f;
+                    if (2 * i + 1 >= left) p1 = 0.f;
+                    ls4[i & 3] += p0 + p1;
+                    const __nv_bfloat162 hh = __floats2bfloat162_rn(p0, p1);
+                    packed[i] = *reinterpret_cast<const uint32_t *>(&hh);
+                }
+                tmem_st32(lane_base + p_col + (uint32_t)(32 * h), packed);
+                lsum += (ls4[0] + ls4[1]) + (ls4[2] + ls4[3]);
+            }
+            tmem_st_wait();
+            return lsum;
+        };
+        float lsum = 0.f;
+        if (act) {
+            wait(BAR_S_FULL + g);   // of its own key block: the first group's exponentials run under the second block's products
+            tc_fence_after();
+            if (ok) lsum = probabilities(0.f);
+        }
+        if (row < 64) xs[g * 64 + row] = lsum;
+        const bool off_range = act && ok && row < p.tile && !(lsum > 0x1p-80f && lsum < 0x1p80f);
+        float l_other;
+        if (named_bar_or(1, 256, off_range)) {
+            // exact form: row maxima over both key blocks first
+            float mx = -INFINITY;
+            if (act && ok) {
+#pragma unroll 1
+                for (int c0 = 0; c0 < 128; c0 += 32) {
+                    uint32_t r[32];
+                    tmem_ld32(lane_base + (uint32_t)(g * 128 + c0), r);
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int i = 0; i < 32; ++i)
+                        if (c0 + i < valid_cols) mx = fmaxf(mx, __uint_as_float(r[i]));
+                }
+            }
+            if (row < 64) xs[g * 64 + row] = mx;
+            named_bar_sync(1, 256);
+            const float mt = fmaxf(mx, xs[(g ^ 1) * 64 + (row & 63)]) * k2;   // an inactive group has published -inf
+            named_bar_sync(1, 256);                                    // both maxima are read: xs may now take the sums
+            lsum = act && ok ? probabilities(mt) : 0.f;
+            if (row < 64) xs[g * 64 + row] = lsum;
+            named_bar_sync(1, 256);
+        }
+        l_other = xs[(g ^ 1) * 64 + (row & 63)];
+        tc_fence_before();
+        mbar_arrive(bar(BAR_P_FULL));
+        const float l_all = lsum + l_other;
+        // ---- O -> attention chunk g of the first layer's input (64 columns, 128B-swizzled K-major)
+        wait(BAR_O_FINAL);
+        tc_fence_after();
+        if (ok && wq * 32 < p.tile) {
+            const float inv = good ? 1.0f / l_all : 0.f;
+            unsigned char *dst = smAtt + g * cs + row * 128;
+#pragma unroll 1
+            for (int c0 = 0; c0 < 64; c0 += 32) {
+                uint32_t r[32];
+                tmem_ld32(lane_base + (uint32_t)(256 + 64 * g + c0), r);
+                tmem_ld_wait();
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    uint32_t w[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const __nv_bfloat162 hh = __floats2bfloat162_rn(__uint_as_float(r[8 * q + 2 * i]) * inv,
+                                                                        __uint_as_float(r[8 * q + 2 * i + 1]) * inv);
+                        w[i] = *reinterpret_cast<const uint32_t *>(&hh);
+                    }
+                    const int slot16 = (c0 >> 3) + q;
+                    if (row < p.tile) *reinterpret_cast<uint4 *>(dst + ((slot16 ^ (row & 7)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
+                }
+            }
+        }
+        fence_proxy_async();   // the MMA reads these chunks through the async proxy
+        tc_fence_before();
+        mbar_arrive(bar(BAR_ATT_FULL));
+        // ---- layer-1 epilogue: a thread owns a unit (lane) and, with the other group, every second sixteen candidates (columns); its bias is
+        // one value.  ReLU, bf16, and the activations go to shared memory as the second layer's operand: 64-unit chunks of 128-byte
+        // rows, one per candidate; this CTA's two chunks then go to the other three.
+        const int unit = rank * 128 + row, h2 = p.H2 / kCtas, unit2 = rank * h2 + row;
+        const bool has2 = row < h2;
+        const float bias = __ldg(slot->p_u + unit), b2 = has2 ? __ldg(p.b2 + unit2) : 0.f, w2 = has2 ? __bfloat162float(p.w_out[unit2]) : 0.f;
+        wait(BAR_ACC1_FULL);
+        tc_fence_after();
+        if (ok) {
+            unsigned char *dst = smH + (unit >> 6) * cs + (unit & 7) * 2;
+            const int piece = (unit & 63) >> 3;
+#pragma unroll 1
+            for (int c0 = 16 * g; c0 < p.tile; c0 += 32) {
+                uint32_t r[16];
+                tmem_ld16(lane_base + (uint32_t)c0, r);
+                tmem_ld_wait();
+#pragma unroll
+                for (int c = 0; c < 16; ++c)
+                    *reinterpret_cast<__nv_bfloat16 *>(dst + (c0 + c) * 128 + ((piece ^ (c & 7)) << 4)) = __float2bfloat16_rn(fmaxf(__uint_as_float(r[c]) + bias, 0.f));
+            }
+        }
+        fence_proxy_async();   // read by the copies and the MMA through the async proxy
+        tc_fence_before();
+        if (!named_bar_or(1, 256, !ok) && tid == 0) {
+            mbar_expect_tx(bar(BAR_H1_FULL), (uint32_t)((kCtas - 1) * 2 * cs));
+            const uint32_t src = smem_u32(smH + 2 * rank * cs);
+            for (int q = 1; q < kCtas; ++q) {
+                const uint32_t to = (uint32_t)((rank + q) % kCtas);
+                bulk_copy_cluster(cluster_addr(src, to), src, (uint32_t)(2 * cs), cluster_addr(bar(BAR_H1_FULL), to));
+            }
+        }
+        // ---- layer-2 epilogue: unit (lane) of this CTA's quarter, ReLU, times its output weight; then the sum over units: over a warp's 32
+        // lanes (every exchange halves the columns a lane still holds), over the warps through shared memory, over the CTAs in the first one's.
+        wait(BAR_ACC2_FULL);
+        tc_fence_after();
+        if (ok && wq * 32 < h2) {
+#pragma unroll 1
+            for (int c0 = 16 * g; c0 < p.tile; c0 += 32) {
+                uint32_t r[16];
+                tmem_ld16(lane_base + 64u + (uint32_t)c0, r);
+                tmem_ld_wait();
+                float v[16];
+#pragma unroll
+                for (int c = 0; c < 16; ++c) v[c] = has2 ? fmaxf(__uint_as_float(r[c]) + b2, 0.f) * w2 : 0.f;
+#pragma unroll
+                for (int w = 8; w > 0; w >>= 1) {   // lanes with bit 2 w keep the upper half
+                    const bool up = lane & (2 * w);
+#pragma unroll
+                    for (int c = 0; c < w; ++c) {
+                        const float give = up ? v[c] : v[c + w], keep = up ? v[c + w] : v[c];
+                        v[c] = keep + __shfl_xor_sync(0xffffffffu, give, 2 * w);
+                    }
+                }
+                v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+                if (!(lane & 1)) dot_s[wq * 64 + c0 + (lane >> 1)] = v[0];
+            }
+        }
+        const bool all_ok = !named_bar_or(1, 256, !ok);   // also orders dot_s; a wait that ran out anywhere in these warps
+        if (g == 0 && row < 64) {
+            float part = 0.f;
+            for (int w = 0; w < (h2 + 31) / 32; ++w) part += dot_s[w * 64 + row];
+            if (row == 63) part = all_ok ? 1.f : 0.f;
+            st_cluster_f32(cluster_addr(smem_u32(red_s + rank * 64 + row), 0u), part);
+        }
+        mine = good;   // (for the last step)
+    } else if (warp == kFMmaWarp) {
+        // ===================== MMA issuer =====================
+        if (lane == 0) {
+            constexpr uint32_t idesc_qk = umma_idesc_bf16(kTcTile, 128);
+            constexpr uint32_t idesc_pv = umma_idesc_bf16_bmn(kTcTile, 128);
+            const uint32_t idesc_l = umma_idesc_bf16(128, p.tile);   // of both layers: 128 units x the tile's candidates
+            bool ok = mbar_wait(bar(BAR_E_FULL), 0u, abort_flag);
+            fence_proxy_async();   // the item rows were written by cp.async
+            // scores = Q K^T, one key block after the other
+            const uint64_t qd = umma_desc_sw128(smem_u32(smE));
+            for (int j = 0; ok && j < nb; ++j) {
+                ok = mbar_wait(bar(BAR_KV_FULL + j), 0u, abort_flag);
+                tc_fence_after();
+                if (!ok) break;
+                const uint64_t kd = umma_desc_sw128(smem_u32(smKV + j * 32768));
+                const uint32_t d_tmem = tmem_base + (uint32_t)(j * 128);
+#pragma unroll
+                for (int kk = 0; kk < 8; ++kk)
+                    umma_bf16(d_tmem, qd + (uint64_t)(uint32_t)((kk >> 2) * (cs >> 4) + 2 * (kk & 3)), kd + (uint64_t)((kk >> 2) * (kChunk >> 4) + 2 * (kk & 3)), idesc_qk, kk > 0 ? 1u : 0u);
+                umma_commit(bar(BAR_S_FULL + j));
+            }
+            // O = P V: the probabilities from tensor memory, V = the key blocks read MN-major
+            ok = ok && mbar_wait(bar(BAR_P_FULL), 0u, abort_flag);
+            tc_fence_after();
+            if (ok) {
+                for (int j = 0; j < nb; ++j) {
+                    const uint64_t vd = umma_desc_mn_sw128(smem_u32(smKV + j * 32768), kChunk);
+#pragma unroll
+                    for (int kk = 0; kk < 8; ++kk)
+                        umma_bf16_ts(tmem_base + 256u, tmem_base + (uint32_t)(384 + j * 64 + kk * 8), vd + (uint64_t)(kk * (2048 >> 4)), idesc_pv,
+                                     (j > 0 || kk > 0) ? 1u : 0u);
+                }
+                umma_commit(bar(BAR_O_FINAL));
+            }
+            // layer 1: K chunks [ item 0-1 | attention 2-3 | cross 4.. ], this CTA's 128 units
+            ok = ok && mbar_wait(bar(BAR_ATT_FULL), 0u, abort_flag);
+            tc_fence_after();
+            int sb = 0;
+            uint32_t phase = 0;
+            auto product = [&](uint32_t d_tmem, uint64_t xd, bool first) {
+                if (!(ok = mbar_wait(bar(BAR_FULL_B + sb), phase, abort_flag))) return;
+                tc_fence_after();
+                const uint64_t wd = umma_desc_sw128(smem_u32(smB + sb * kBStage));
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk) umma_bf16(d_tmem, wd + (uint64_t)(2 * kk), xd + (uint64_t)(2 * kk), idesc_l, first && kk == 0 ? 0u : 1u);
+                umma_commit(bar(BAR_EMPTY_B + sb));
+                if (++sb == p.stages) sb = 0, phase ^= 1u;
+            };
+            for (int kc = 0; ok && kc < n_k1; ++kc) {
+                if (kc >= 4) {
+                    if (!(ok = mbar_wait(bar(BAR_FULL_A + kc - 4), 0u, abort_flag))) break;
+                    fence_proxy_async();
+                }
+                product(tmem_base, umma_desc_sw128(smem_u32(kc < 2 ? smE + kc * cs : kc < 4 ? smAtt + (kc - 2) * cs : smX + (kc - 4) * cs)), kc == 0);
+            }
+            if (ok) umma_commit(bar(BAR_ACC1_FULL));
+            // layer 2, this CTA's quarter of the units (lanes beyond it: whatever the stage held, nobody reads them)
+            ok = ok && mbar_wait(bar(BAR_H1_FULL), 0u, abort_flag);
+            tc_fence_after();
+            for (int kc = 0; ok && kc < kH1 / 64; ++kc) product(tmem_base + 64u, umma_desc_sw128(smem_u32(smH + kc * cs)), kc == 0);
+            if (ok) umma_commit(bar(BAR_ACC2_FULL));
+        }
+        __syncwarp();
+    } else if (warp < kFBWarp) {
+        // ===================== item-row and cross-feature gather (128 threads) =====================
+        const int pt = tid - kFProdWarp0 * 32;
+        const int sub = pt & 7, r0 = pt >> 3;   // 16-byte slot of the 128-byte chunk row; rows r0, r0 + 16, r0 + 32
+        constexpr int kR = kMaxTile / 16;
+        const uint32_t row_off = (uint32_t)(r0 * 128) + (uint32_t)((sub ^ (r0 & 7)) << 4);
+        int id[kR];
+#pragma unroll
+        for (int i = 0; i < kR; ++i) id[i] = __shfl_sync(0xffffffffu, mine, (lane >> 3) + 4 * i);
+#pragma unroll
+        for (int i = 0; i < kR; ++i)
+            if (r0 + 16 * i < cnt && (id[i] < 0 || (int64_t)id[i] >= p.M)) {
+                id[i] = -1;
+                if (sub == 0) atomicOr(p.sl.status, AIF_STATUS_BAD_ID);
+            }
+#pragma unroll
+        for (int i = 0; i < kR; ++i) {
+            if (16 * i >= p.tile) break;
+            const uint8_t *gsrc = p.E + (id[i] >= 0 ? (size_t)id[i] * 256 + sub * 16 : 0);
+            const uint32_t dst = smem_u32(smE) + row_off + (uint32_t)(i * 16 * 128);
+            cp_async16(dst, gsrc, id[i] >= 0 ? 16u : 0u);
+            cp_async16(dst + (uint32_t)cs, gsrc + 128, id[i] >= 0 ? 16u : 0u);
+        }
+        cp_async_arrive_noinc(bar(BAR_E_FULL));
+        // cross features (Section 3.3): the row of field f's user-side table that the candidate's bucket selects
+        const uint8_t *Tt = reinterpret_cast<const uint8_t *>(slot->T);
+        for (int n = 0; n < p.n_cross; ++n) {
+            const int col = 64 * n + 8 * sub, f = col / p.dc, kin = col - f * p.dc;
+            const uint32_t row16 = (uint32_t)(p.dc >> 3), base16 = (uint32_t)(f * p.B) * row16 + (uint32_t)(kin >> 3);
+            const uint32_t dst0 = smem_u32(smX + n * cs) + row_off;
+#pragma unroll
+            for (int i = 0; i < kR; ++i) {
+                if (16 * i >= p.tile) break;
+                uint32_t bk;
+                if (p.bucket_mode == AIF_BUCKET_MOD) bk = (uint32_t)(id[i] % p.B);
+                else {
+                    const uint64_t h = mix64((uint64_t)id[i], (uint64_t)f);
+                    bk = p.b_mask >= 0 ? (uint32_t)(h & (uint64_t)p.b_mask) : (uint32_t)(h % (uint64_t)p.B);
+                }
+                cp_async16(dst0 + (uint32_t)(i * 16 * 128), id[i] >= 0 ? Tt + ((size_t)(bk * row16 + base16) << 4) : p.E, id[i] >= 0 ? 16u : 0u);
+            }
+            cp_async_arrive_noinc(bar(BAR_FULL_A + n));
+        }
+        cp_async_wait_all();
+    } else {
+        // ===================== key/value blocks and weights (TMA) =====================
+        if (lane == 0) {
+            for (int j = 0; j < nb; ++j) {
+                mbar_expect_tx(bar(BAR_KV_FULL + j), 32768u);
+                tma_load_3d(smem_u32(smKV + j * 32768), &tmapS, bar(BAR_KV_FULL + j), 0, j * 128, rq.slot);
+                tma_load_3d(smem_u32(smKV + j * 32768 + kChunk), &tmapS, bar(BAR_KV_FULL + j), 64, j * 128, rq.slot);
+            }
+            int sb = 0;
+            uint32_t phase = 1;
+            for (int kc = 0; kc < n_k1 + kH1 / 64; ++kc) {
+                if (!mbar_wait(bar(BAR_EMPTY_B + sb), phase, abort_flag)) break;
+                const bool first = kc < n_k1;
+                mbar_expect_tx(bar(BAR_FULL_B + sb), first ? 16384u : (uint32_t)(p.H2 / kCtas) * 128u);
+                if (first) tma_load_2d(smem_u32(smB + sb * kBStage), &tmapW1, bar(BAR_FULL_B + sb), kc * 64, rank * 128);
+                else tma_load_2d(smem_u32(smB + sb * kBStage), &tmapW2, bar(BAR_FULL_B + sb), (kc - n_k1) * 64, rank * (p.H2 / kCtas));
+                if (++sb == p.stages) sb = 0, phase ^= 1u;
+            }
+        }
+        __syncwarp();
+    }
+
+    // ---- teardown: everybody arrives here, also after an abort
+    if (*abort_flag) {
+        if (tid == 0) atomicOr(p.sl.status, AIF_STATUS_TIMEOUT);
+        // let copies and MMAs that are still in flight land before shared memory and TMEM go away
+        const long long t0 = clock64();
+        while (clock64() - t0 < 2000000ll) __nanosleep(1000);
+    }
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync();   // all partial logits are with the first CTA; nobody leaves while another may still write to it
+    if (rank == 0 && tid < cnt) {   // (thread = row: `mine` is whether its id is in the table)
+        float logit = p.b_out[0];
+        bool all = true;
+        for (int q = 0; q < kCtas; ++q) logit += red_s[q * 64 + tid], all = all && red_s[q * 64 + 63] != 0.f;
+        if (p.emit_sigmoid) logit = 1.0f / (1.0f + expf(-logit));
+        p.sl.logits[pos0 + tid] = mine && all ? logit : __int_as_float(0x7fc00000);   // no number for a bad id, nor where a wait ran out
+    }
+    if (warp == kFMmaWarp) tmem_dealloc(tmem_base, 512);
+}
+
+}  // namespace
+
+// Clusters of four that the machine holds at once (0: not usable).
+int tc_split_prepare()
+{
+    if (cudaFuncSetAttribute(k_request_split, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFSmem) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(kCtas), cfg.blockDim = dim3(kFThreads), cfg.dynamicSmemBytes = kFSmem;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = kCtas, attr.val.clusterDim.y = 1, attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr, cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, k_request_split, &cfg) != cudaSuccess) cudaGetLastError(), n = 0;
+    return n;
+}
+
+// Whether a single request of n candidates is one round of clusters (the caller has checked tc_fused_supported and the sequence's length).
+bool tc_split_fits(const aif_ctx *ctx, int n) { return n <= ctx->split_clusters * kMaxTile; }
+
+cudaError_t launch_request_split(const aif_ctx *ctx, const ScoreLaunch &sl, cudaStream_t st)
+{
+    const aif_config &c = ctx->cfg;
+    SplitParams p{};
+    p.sl = sl, p.E = (const uint8_t *)ctx->E, p.M = c.M;
+    p.tile = ((sl.single.n + ctx->split_clusters - 1) / ctx->split_clusters + 15) / 16 * 16, p.stages = stages_for(p.tile);
+    p.B = c.B, p.dc = c.dc, p.b_mask = (c.B & (c.B - 1)) == 0 ? c.B - 1 : -1, p.bucket_mode = c.bucket_mode;
+    p.n_cross = c.F * c.dc / 64;
+    p.H2 = c.hidden[1], p.emit_sigmoid = c.emit_sigmoid;
+    p.scale_log2 = 1.4426950408889634f / sqrtf((float)c.d);
+    p.b2 = ctx->b[1], p.w_out = (const __nv_bfloat16 *)ctx->w_out, p.b_out = ctx->b_out;
+    const CUtensorMap *ms = reinterpret_cast<const CUtensorMap *>(tc_att_tmap(ctx));
+    const CUtensorMap *m1 = reinterpret_cast<const CUtensorMap *>(tc_weight_half_tmap(ctx, 0));
+    const CUtensorMap *m2 = reinterpret_cast<const CUtensorMap *>(tc_weight_quarter_tmap(ctx));
+    const int grid = (sl.single.n + p.tile - 1) / p.tile * kCtas;
+    cudaError_t e = launch_pdl_cluster(k_request_split, dim3(grid), dim3(kFThreads), kFSmem, kCtas, st, *ms, *m1, *m2, p);
+    count_launch();
+    return e;
+}
+
+}  // namespace aif
