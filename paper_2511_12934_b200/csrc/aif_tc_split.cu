@@ -12,9 +12,11 @@
 // Products the other way round without sharing the units (a tile of up to 128 per CTA, all weights): 22.5 us for 1000 candidates, the weights'
 // way into the SM unchanged.
 //
-// 448 threads: warps 0-7 softmax and epilogues, 8 the issuing lane, 9-12 gather, 13 one lane of TMA, as there.
-// Tensor memory: attention as there (scores [0, 256), O [256, 384), probabilities [384, 512)); then the layers' accumulators, tile columns each, at 0
-// and 64.  Every wait is bounded.
+// 480 threads: warps 0-7 softmax and epilogues, 8 the issuing lane, 9-12 gather, 13 one lane of TMA, as there; 14 a second issuing lane.  A chunk of
+// 64 columns is four products of 45 cycles, and its waits, descriptors and commit take the lane 450 more: two lanes take the chunks in
+// turn, each with accumulators of its own that the epilogue adds (one lane: 7900 and 3900 cycles for the layers).
+// Tensor memory: attention as there (scores [0, 256), O [256, 384), probabilities [384, 512)); then the layers' accumulators, 64 columns each.
+// Every wait is bounded.
 #include <cuda.h>
 
 #include "aif_device.cuh"
@@ -24,26 +26,29 @@
 namespace aif {
 namespace {
 
-constexpr int kFThreads = 448;
-constexpr int kFMmaWarp = 8, kFProdWarp0 = 9, kFBWarp = 13;
+constexpr int kFThreads = 480;
+constexpr int kFMmaWarp = 8, kFProdWarp0 = 9, kFBWarp = 13, kFMmaWarp2 = 14;
 constexpr int kChunk = 16384;                  // 128 rows x 64 bf16
+constexpr int kMaxCross = 8;                   // cross-feature chunks (64 columns each)
+constexpr int kH1 = 512;
 constexpr int kCtas = 4;                       // of a cluster
 constexpr int kMaxTile = 48;
 constexpr int kBStage = 16384, kMaxStages = 8;
+constexpr int kMaxWeights = 4 + kMaxCross + kH1 / 64;   // chunks of weights of both layers, a barrier pair each
 constexpr size_t kFSmem = 227 * 1024;
 constexpr int kMiscBytes = 1024 + 2048;        // barriers | 8 x 64 partial dots
 // shared memory behind the miscellany, with c = tile x 128 bytes a chunk of 64 columns: E 2 c | key/value blocks 64 KB, later the attention
 // chunks | cross chunks 8 c | activations 8 c | weight ring
 constexpr int stages_for(int tile) { return ((int)kFSmem - 1024 - kMiscBytes - 65536 - 18 * tile * 128) / kBStage < kMaxStages ? ((int)kFSmem - 1024 - kMiscBytes - 65536 - 18 * tile * 128) / kBStage : kMaxStages; }
 static_assert(stages_for(kMaxTile) >= 3, "weight ring");
-constexpr int kMaxCross = 8;                   // cross-feature chunks (64 columns each)
-constexpr int kH1 = 512;
 
 enum {
     BAR_E_FULL = 0, BAR_KV_FULL, BAR_S_FULL = BAR_KV_FULL + 2, BAR_P_FULL = BAR_S_FULL + 2, BAR_O_FINAL, BAR_ATT_FULL, BAR_ACC1_FULL,
-    BAR_H1_FULL, BAR_ACC2_FULL, BAR_FULL_A, BAR_FULL_B = BAR_FULL_A + kMaxCross, BAR_EMPTY_B = BAR_FULL_B + kMaxStages, BAR_COUNT = BAR_EMPTY_B + kMaxStages
+    BAR_H1_FULL, BAR_ACC2_FULL, BAR_FULL_A, BAR_FULL_B = BAR_FULL_A + kMaxCross, BAR_EMPTY_B = BAR_FULL_B + kMaxWeights, BAR_COUNT = BAR_EMPTY_B + kMaxWeights
 };
 static_assert(BAR_COUNT * 8 + 16 <= 512, "barriers");
+// D of the first layer at 0 and 64, of the second at 128 and 192, one per issuer
+static_assert(kMaxTile <= 64, "tensor memory");
 
 struct SplitParams {
     ScoreLaunch sl;
@@ -87,11 +92,11 @@ __global__ void __launch_bounds__(kFThreads, 1) k_request_split(const __grid_con
         mbar_init(bar(BAR_P_FULL), 256);
         mbar_init(bar(BAR_O_FINAL), 1);
         mbar_init(bar(BAR_ATT_FULL), 256);
-        mbar_init(bar(BAR_ACC1_FULL), 1);
+        mbar_init(bar(BAR_ACC1_FULL), 2);
         mbar_init(bar(BAR_H1_FULL), 1);
-        mbar_init(bar(BAR_ACC2_FULL), 1);
+        mbar_init(bar(BAR_ACC2_FULL), 2);
         for (int i = 0; i < kMaxCross; ++i) mbar_init(bar(BAR_FULL_A + i), 128);
-        for (int s = 0; s < kMaxStages; ++s) mbar_init(bar(BAR_FULL_B + s), 1), mbar_init(bar(BAR_EMPTY_B + s), 1);
+        for (int s = 0; s < kMaxWeights; ++s) mbar_init(bar(BAR_FULL_B + s), 1), mbar_init(bar(BAR_EMPTY_B + s), 1);
         *abort_flag = 0u;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -249,12 +254,12 @@ __global__ void __launch_bounds__(kFThreads, 1) k_request_split(const __grid_con
             const int piece = (unit & 63) >> 3;
 #pragma unroll 1
             for (int c0 = 16 * g; c0 < p.tile; c0 += 32) {
-                uint32_t r[16];
-                tmem_ld16(lane_base + (uint32_t)c0, r);
+                uint32_t r[16], r2[16];   // what either issuer has summed
+                tmem_ld16(lane_base + (uint32_t)c0, r), tmem_ld16(lane_base + 64u + (uint32_t)c0, r2);
                 tmem_ld_wait();
 #pragma unroll
                 for (int c = 0; c < 16; ++c)
-                    *reinterpret_cast<__nv_bfloat16 *>(dst + (c0 + c) * 128 + ((piece ^ (c & 7)) << 4)) = __float2bfloat16_rn(fmaxf(__uint_as_float(r[c]) + bias, 0.f));
+                    *reinterpret_cast<__nv_bfloat16 *>(dst + (c0 + c) * 128 + ((piece ^ (c & 7)) << 4)) = __float2bfloat16_rn(fmaxf(__uint_as_float(r[c]) + __uint_as_float(r2[c]) + bias, 0.f));
             }
         }
         fence_proxy_async();   // read by the copies and the MMA through the async proxy
@@ -274,12 +279,12 @@ __global__ void __launch_bounds__(kFThreads, 1) k_request_split(const __grid_con
         if (ok && wq * 32 < h2) {
 #pragma unroll 1
             for (int c0 = 16 * g; c0 < p.tile; c0 += 32) {
-                uint32_t r[16];
-                tmem_ld16(lane_base + 64u + (uint32_t)c0, r);
+                uint32_t r[16], r2[16];
+                tmem_ld16(lane_base + 128u + (uint32_t)c0, r), tmem_ld16(lane_base + 192u + (uint32_t)c0, r2);
                 tmem_ld_wait();
                 float v[16];
 #pragma unroll
-                for (int c = 0; c < 16; ++c) v[c] = has2 ? fmaxf(__uint_as_float(r[c]) + b2, 0.f) * w2 : 0.f;
+                for (int c = 0; c < 16; ++c) v[c] = has2 ? fmaxf(__uint_as_float(r[c]) + __uint_as_float(r2[c]) + b2, 0.f) * w2 : 0.f;
 #pragma unroll
                 for (int w = 8; w > 0; w >>= 1) {   // lanes with bit 2 w keep the upper half
                     const bool up = lane & (2 * w);
@@ -301,66 +306,72 @@ __global__ void __launch_bounds__(kFThreads, 1) k_request_split(const __grid_con
             st_cluster_f32(cluster_addr(smem_u32(red_s + rank * 64 + row), 0u), part);
         }
         mine = good;   // (for the last step)
-    } else if (warp == kFMmaWarp) {
-        // ===================== MMA issuer =====================
+    } else if (warp == kFMmaWarp || warp == kFMmaWarp2) {
+        // ===================== MMA issuers: even and odd chunks of the layers; the attention is the first one's =====================
         if (lane == 0) {
             constexpr uint32_t idesc_qk = umma_idesc_bf16(kTcTile, 128);
             constexpr uint32_t idesc_pv = umma_idesc_bf16_bmn(kTcTile, 128);
             const uint32_t idesc_l = umma_idesc_bf16(128, p.tile);   // of both layers: 128 units x the tile's candidates
-            bool ok = mbar_wait(bar(BAR_E_FULL), 0u, abort_flag);
-            fence_proxy_async();   // the item rows were written by cp.async
-            // scores = Q K^T, one key block after the other
-            const uint64_t qd = umma_desc_sw128(smem_u32(smE));
-            for (int j = 0; ok && j < nb; ++j) {
-                ok = mbar_wait(bar(BAR_KV_FULL + j), 0u, abort_flag);
-                tc_fence_after();
-                if (!ok) break;
-                const uint64_t kd = umma_desc_sw128(smem_u32(smKV + j * 32768));
-                const uint32_t d_tmem = tmem_base + (uint32_t)(j * 128);
-#pragma unroll
-                for (int kk = 0; kk < 8; ++kk)
-                    umma_bf16(d_tmem, qd + (uint64_t)(uint32_t)((kk >> 2) * (cs >> 4) + 2 * (kk & 3)), kd + (uint64_t)((kk >> 2) * (kChunk >> 4) + 2 * (kk & 3)), idesc_qk, kk > 0 ? 1u : 0u);
-                umma_commit(bar(BAR_S_FULL + j));
-            }
-            // O = P V: the probabilities from tensor memory, V = the key blocks read MN-major
-            ok = ok && mbar_wait(bar(BAR_P_FULL), 0u, abort_flag);
-            tc_fence_after();
-            if (ok) {
-                for (int j = 0; j < nb; ++j) {
-                    const uint64_t vd = umma_desc_mn_sw128(smem_u32(smKV + j * 32768), kChunk);
+            const int mine2 = warp == kFMmaWarp2;
+            bool ok = true;
+            if (mine2 == 0) {
+                ok = mbar_wait(bar(BAR_E_FULL), 0u, abort_flag);
+                fence_proxy_async();   // the item rows were written by cp.async
+                // scores = Q K^T, one key block after the other
+                const uint64_t qd = umma_desc_sw128(smem_u32(smE));
+                for (int j = 0; ok && j < nb; ++j) {
+                    ok = mbar_wait(bar(BAR_KV_FULL + j), 0u, abort_flag);
+                    tc_fence_after();
+                    if (!ok) break;
+                    const uint64_t kd = umma_desc_sw128(smem_u32(smKV + j * 32768));
+                    const uint32_t d_tmem = tmem_base + (uint32_t)(j * 128);
 #pragma unroll
                     for (int kk = 0; kk < 8; ++kk)
-                        umma_bf16_ts(tmem_base + 256u, tmem_base + (uint32_t)(384 + j * 64 + kk * 8), vd + (uint64_t)(kk * (2048 >> 4)), idesc_pv,
-                                     (j > 0 || kk > 0) ? 1u : 0u);
+                        umma_bf16(d_tmem, qd + (uint64_t)(uint32_t)((kk >> 2) * (cs >> 4) + 2 * (kk & 3)), kd + (uint64_t)((kk >> 2) * (kChunk >> 4) + 2 * (kk & 3)), idesc_qk, kk > 0 ? 1u : 0u);
+                    umma_commit(bar(BAR_S_FULL + j));
                 }
-                umma_commit(bar(BAR_O_FINAL));
+                // O = P V: the probabilities from tensor memory, V = the key blocks read MN-major
+                ok = ok && mbar_wait(bar(BAR_P_FULL), 0u, abort_flag);
+                tc_fence_after();
+                if (ok) {
+                    for (int j = 0; j < nb; ++j) {
+                        const uint64_t vd = umma_desc_mn_sw128(smem_u32(smKV + j * 32768), kChunk);
+#pragma unroll
+                        for (int kk = 0; kk < 8; ++kk)
+                            umma_bf16_ts(tmem_base + 256u, tmem_base + (uint32_t)(384 + j * 64 + kk * 8), vd + (uint64_t)(kk * (2048 >> 4)), idesc_pv,
+                                         (j > 0 || kk > 0) ? 1u : 0u);
+                    }
+                    umma_commit(bar(BAR_O_FINAL));
+                }
             }
             // layer 1: K chunks [ item 0-1 | attention 2-3 | cross 4.. ], this CTA's 128 units
             ok = ok && mbar_wait(bar(BAR_ATT_FULL), 0u, abort_flag);
             tc_fence_after();
-            int sb = 0;
-            uint32_t phase = 0;
-            auto product = [&](uint32_t d_tmem, uint64_t xd, bool first) {
-                if (!(ok = mbar_wait(bar(BAR_FULL_B + sb), phase, abort_flag))) return;
+            if (ok && mine2 && (ok = mbar_wait(bar(BAR_E_FULL), 0u, abort_flag))) fence_proxy_async();   // (the item rows, as above)
+            int sb = mine2 % p.stages;
+            auto product = [&](int c, uint32_t d_tmem, uint64_t xd, bool first) {   // weight chunk c, of both layers in their order
+                if (!(ok = mbar_wait(bar(BAR_FULL_B + c), 0u, abort_flag))) return;
                 tc_fence_after();
                 const uint64_t wd = umma_desc_sw128(smem_u32(smB + sb * kBStage));
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk) umma_bf16(d_tmem, wd + (uint64_t)(2 * kk), xd + (uint64_t)(2 * kk), idesc_l, first && kk == 0 ? 0u : 1u);
-                umma_commit(bar(BAR_EMPTY_B + sb));
-                if (++sb == p.stages) sb = 0, phase ^= 1u;
+                umma_commit(bar(BAR_EMPTY_B + c));
             };
-            for (int kc = 0; ok && kc < n_k1; ++kc) {
+            auto ahead = [&](int n) { sb += n; while (sb >= p.stages) sb -= p.stages; };
+            const uint32_t d1 = tmem_base + (uint32_t)(64 * mine2), d2 = tmem_base + 128u + (uint32_t)(64 * mine2);
+            for (int kc = mine2; ok && kc < n_k1; kc += 2, ahead(2)) {
                 if (kc >= 4) {
                     if (!(ok = mbar_wait(bar(BAR_FULL_A + kc - 4), 0u, abort_flag))) break;
                     fence_proxy_async();
                 }
-                product(tmem_base, umma_desc_sw128(smem_u32(kc < 2 ? smE + kc * cs : kc < 4 ? smAtt + (kc - 2) * cs : smX + (kc - 4) * cs)), kc == 0);
+                product(kc, d1, umma_desc_sw128(smem_u32(kc < 2 ? smE + kc * cs : kc < 4 ? smAtt + (kc - 2) * cs : smX + (kc - 4) * cs)), kc == mine2);
             }
             if (ok) umma_commit(bar(BAR_ACC1_FULL));
             // layer 2, this CTA's quarter of the units (lanes beyond it: whatever the stage held, nobody reads them)
             ok = ok && mbar_wait(bar(BAR_H1_FULL), 0u, abort_flag);
             tc_fence_after();
-            for (int kc = 0; ok && kc < kH1 / 64; ++kc) product(tmem_base + 64u, umma_desc_sw128(smem_u32(smH + kc * cs)), kc == 0);
+            sb = 0, ahead(n_k1 + mine2);
+            for (int kc = mine2; ok && kc < kH1 / 64; kc += 2, ahead(2)) product(n_k1 + kc, d2, umma_desc_sw128(smem_u32(smH + kc * cs)), kc == mine2);
             if (ok) umma_commit(bar(BAR_ACC2_FULL));
         }
         __syncwarp();
@@ -417,14 +428,13 @@ __global__ void __launch_bounds__(kFThreads, 1) k_request_split(const __grid_con
                 tma_load_3d(smem_u32(smKV + j * 32768 + kChunk), &tmapS, bar(BAR_KV_FULL + j), 64, j * 128, rq.slot);
             }
             int sb = 0;
-            uint32_t phase = 1;
             for (int kc = 0; kc < n_k1 + kH1 / 64; ++kc) {
-                if (!mbar_wait(bar(BAR_EMPTY_B + sb), phase, abort_flag)) break;
+                if (kc >= p.stages && !mbar_wait(bar(BAR_EMPTY_B + kc - p.stages), 0u, abort_flag)) break;
                 const bool first = kc < n_k1;
-                mbar_expect_tx(bar(BAR_FULL_B + sb), first ? 16384u : (uint32_t)(p.H2 / kCtas) * 128u);
-                if (first) tma_load_2d(smem_u32(smB + sb * kBStage), &tmapW1, bar(BAR_FULL_B + sb), kc * 64, rank * 128);
-                else tma_load_2d(smem_u32(smB + sb * kBStage), &tmapW2, bar(BAR_FULL_B + sb), (kc - n_k1) * 64, rank * (p.H2 / kCtas));
-                if (++sb == p.stages) sb = 0, phase ^= 1u;
+                mbar_expect_tx(bar(BAR_FULL_B + kc), first ? 16384u : (uint32_t)(p.H2 / kCtas) * 128u);
+                if (first) tma_load_2d(smem_u32(smB + sb * kBStage), &tmapW1, bar(BAR_FULL_B + kc), kc * 64, rank * 128);
+                else tma_load_2d(smem_u32(smB + sb * kBStage), &tmapW2, bar(BAR_FULL_B + kc), (kc - n_k1) * 64, rank * (p.H2 / kCtas));
+                if (++sb == p.stages) sb = 0;
             }
         }
         __syncwarp();
