@@ -606,3 +606,44 @@ def test_contexts_take_no_more_room_for_partial_results_than_their_sequences_can
     ctx = B.Aif(cfg)
     assert ctx.get_stats().device_bytes <= most << 20
     ctx.close()
+
+
+@pytest.mark.parametrize("H2,L", [(256, 200), (64, 128), (192, 129), (256, 1)])
+def test_small_requests_at_the_edges_of_their_tiles(H2, L):
+    """Requests by themselves go in tiles of 16, 32 or 48 candidates on clusters of four CTAs, larger ones by the kernel of one CTA per tile:
+    numbers of candidates on either side of every change, an id outside the table among them, and the widths of the second layer that
+    a cluster splits into quarters of 16 to 64 units."""
+    sizes = [1, 15, 16, 17, 33, 560, 577, 592, 593, 1000, 1153, 1185, 1729, 1777, 1900]
+    wl = helpers.MINI["c2"].with_(name=f"split_{H2}_{L}", N=max(sizes), M=20_000, mini_batch=0, L=L, hidden=(512, H2))
+    weights, table = synth.make_weights(wl, zero_bias=False), synth.make_item_table(wl)
+    srv = serving.Server(wl, weights, table, path=B.PATH_TENSOR)
+    oracle = helpers.make_oracle(wl, weights, M=wl.M)
+    rq = synth.make_request(wl, 0)
+    st = srv.precompute(0, srv.upload_request(rq, B.USER_PROJECTED))
+    sampler = synth.IdSampler(wl)
+    for n in sizes:
+        ids = sampler.request_ids(0, n)
+        if n > 20:
+            ids[n // 2] = wl.M
+        got = srv.score_ids(st, ids)
+        pick = np.unique(np.r_[0:min(n, 50), max(0, n - 50):n, n // 2])
+        _check(got[pick], oracle.score(table, helpers.projected_request(wl, rq), ids[pick]))
+        assert int(np.isnan(got).sum()) == int(n > 20)
+    srv.close()
+
+
+def test_request_of_one_tile_per_cta_with_scores_that_overflow():
+    """The kernel of one CTA per tile (too many candidates for the clusters) where 2^score leaves fp32: it repeats the softmax with exact row
+    maxima, as the clusters do (the sharp-softmax test's single launch).  Activations of magnitude A carry about 2^-9 A of rounding error."""
+    wl = helpers.MINI["c2"].with_(name="sharp_tiles", R=1, N=2000, L=200, mini_batch=0)
+    weights, table = synth.make_weights(wl, zero_bias=False), synth.make_item_table(wl)
+    table["E"] = synth.to_bf16_bits(synth.bf16_bits_to_f32(table["E"]) * 32.0)
+    rq = synth.make_request(wl, 0)
+    rq["S"] = synth.to_bf16_bits(synth.bf16_bits_to_f32(rq["S"]) * 1024.0)
+    srv = serving.Server(wl, weights, table)
+    st = srv.precompute(1, srv.upload_request(rq, B.USER_PROJECTED))
+    ids = synth.IdSampler(wl).request_ids(0)
+    got = srv.score_ids(st, ids)[::9]
+    want = helpers.make_oracle(wl, weights, M=table["E"].shape[0]).score(table, helpers.projected_request(wl, rq), ids[::9])
+    _check(got, want, 1e-2 * max(1.0, float(np.abs(want).max())))
+    srv.close()
