@@ -60,7 +60,7 @@ def flops_per_candidate(wl: synth.Workload, keys=None) -> dict:
     """keys: mean number of sequence items a candidate interacts with (the whole sequence unless the workload has
     category sub-sequences)."""
     k1 = wl.input_width() - wl.d                       # the user columns are done once per request
-    keys = float(wl.L if keys is None else keys)
+    keys = keys_of(wl, keys)
     f = {"attention": 4.0 * keys * wl.d if wl.blocks & synth.BLK_ATT else 0.0}
     f["lsh_din"] = 2.0 * keys * wl.d if wl.blocks & synth.BLK_LSH_DIN else 0.0
     f["bea"] = 2.0 * wl.n_bridge * wl.d if wl.blocks & synth.BLK_BEA else 0.0
@@ -72,6 +72,10 @@ def flops_per_candidate(wl: synth.Workload, keys=None) -> dict:
     return f
 
 
+def keys_of(wl: synth.Workload, keys) -> float:
+    return float(wl.L if keys is None else keys)
+
+
 def kernel_flops(name: str, wl: synth.Workload, n: int, keys=None) -> float:
     f = flops_per_candidate(wl, keys)
     if name in ("score_simt", "score_fused"):
@@ -80,7 +84,9 @@ def kernel_flops(name: str, wl: synth.Workload, n: int, keys=None) -> float:
         return (f["attention"] + f["lsh_din"] + f["bea"]) * n
     if name == "lsh":          # eq. 8's contraction; the match counts of eqs. 6-7 ride in the same kernel (see lsh_note)
         return f["lsh_din"] * n
-    if name in ("buckets", "group"):
+    if name == "simtier":      # eq. 6's counts as a +-1 fp8 product; eq. 8 then goes through sums of the request's own
+        return 2.0 * keys_of(wl, keys) * wl.lsh_bits * n
+    if name in ("buckets", "group", "lsh_sums", "lsh_rows"):
         return 0.0
     return f.get(name, 0.0) * n
 
@@ -541,6 +547,9 @@ def measure(args, wl, steps, warmup, dist, world, rank, full):
         roof["lsh_note"] = (f"eqs. 6-7 need {wl.lsh_bits // 32} xor + popc on 32-bit words per (candidate, key) pair by the definition; "
                             f"the kernel gets the counts from a +-1 fp8 product ({2 * wl.lsh_bits} tensor flop per pair, not counted "
                             "in `achieved`) and spends about five integer / fp32 instructions per pair on conversion and tiers")
+    if top == "simtier":
+        roof["lsh_note"] = ("`achieved` counts the +-1 product behind the match counts, at most twice the bf16 rate; the kernel is bound by "
+                            "the issue slots of the tier counts, about three instructions per pair")
     if tensor:
         roof["frac_nominal"] = roof["achieved"] / NOMINAL_BF16_TFLOPS
         roof["peak_nominal"] = NOMINAL_BF16_TFLOPS

@@ -1606,7 +1606,7 @@ cudaError_t launch_score_tc_scratch(const aif_ctx *ctx, const ScoreLaunch &sl_in
         if (att_tc && sc.split) sl_lsh.split = ctx->split_lsh;   // records of its own: the attention's are not joined yet
         cudaError_t e = tiers_alone ? launch_tiers(ctx, sl_lsh, st, sc.X, pl->x_cols, x_tier, join_lsh)
                                     : launch_lsh_tc(ctx, sl_lsh, st, sc.X, pl->x_cols, sc.rows, x_din, x_tier, join_lsh);
-        timing_mark(ctx, "lsh", st);
+        timing_mark(ctx, din_sums ? "simtier" : "lsh", st);
         if (e != cudaSuccess) return e;
         late = 1;
     }
@@ -1623,7 +1623,7 @@ cudaError_t launch_score_tc_scratch(const aif_ctx *ctx, const ScoreLaunch &sl_in
         ScoreLaunch sl_din = sl;
         sl_din.late = 0;
         const cudaError_t e = launch_din_apply(ctx, sl_din, st, sc.X, pl->x_cols, sc.rows, x_din);
-        timing_mark(ctx, tier ? "lsh_rows" : "lsh", st);
+        timing_mark(ctx, "lsh_rows", st);
         if (e != cudaSuccess) return e;
     }
     const bool need_att = (c.blocks & AIF_BLK_ATT) && !att_tc, need_lsh = lsh_blocks && !lsh_tc;
