@@ -264,6 +264,7 @@ __global__ void __launch_bounds__((TierCfg<D>::kThreads), 1) k_tiers(const __gri
         const int wq = warp & 3, h = warp >> 2;
         const int row = wq * 32 + lane;
         const uint32_t lane_base = tmem_base + ((uint32_t)(wq * 32) << 16);
+        const uint32_t s_col = lane_base + (uint32_t)(h * kUnit);
         const __half2 scale = as_half2(p.scale);
         if (lane == 0) mbar_arrive(smem_u32(ready + h));   // the buffers are free for the first units
         bool ok = true;
@@ -293,22 +294,17 @@ __global__ void __launch_bounds__((TierCfg<D>::kThreads), 1) k_tiers(const __gri
             int n_valid = 0, n_pad = 0, since = 0;
             const int nu = units_of(t.L);
             int u = skip;
-            for (; u < nu; u += kT) {
-                if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(s_full + h), phase, abort_flag))) {
-                    ok = false;
-                    break;
-                }
+            // Keys are counted by 64.  Columns between the end of the sequence and the next multiple of 64 have zero signatures (the user side
+            // pads to 128): their matches read d' / 2, and they are taken out at the end.
+            auto unit = [&](int here) {
+                if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(s_full + h), phase, abort_flag))) return false;
                 phase ^= 1u;
                 tc_fence_after();
-                // Keys are counted by 64.  Columns between the end of the sequence and the next multiple of 64 have zero signatures (the
-                // user side pads to 128): their matches read d' / 2, and they are taken out at the end.
-                const int here = min(kUnit, t.L - u * kUnit);
-                const uint32_t s_col = lane_base + (uint32_t)(h * kUnit);
                 // (96 registers to a thread: 64 columns at a time)
-                uint32_t v[32];
+                uint32_t v[32], c = 0u, c1 = 0u;
                 tmem_ld64_pack16(s_col, v);
                 tmem_ld_wait();
-                uint32_t c = here > 0 ? count_tiers(v, scale, digit) : 0u;
+                if (here > 0) c = count_tiers(v, scale, digit);
                 if (here > 64) {
                     tmem_ld64_pack16(s_col + 64u, v);
                     tmem_ld_wait();
@@ -316,17 +312,20 @@ __global__ void __launch_bounds__((TierCfg<D>::kThreads), 1) k_tiers(const __gri
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(ready + h));   // for the unit four further
-                if (here > 64) {
-                    const uint32_t c1 = count_tiers(v, scale, digit);
-                    carried |= carry_up<5>(digit, csa(digit[4], c, c1));
-                } else
-                    carried |= carry_up<4>(digit, c);
-                if (here > 0) n_valid += here, n_pad += (-here) & 63;
+                if (here > 64) c1 = count_tiers(v, scale, digit);
+                carried |= carry_up<5>(digit, csa(digit[4], c, c1));
                 if ((++since & 7) == 0) {
                     carry_up<0>(upper, carried);
                     carried = 0u;
                     if (since == kTierUnits) flush_tiers(digit, cnt, 0), flush_tiers(upper, cnt, 8), since = 0;
                 }
+                return true;
+            };
+            const int whole_units = t.L / kUnit;
+            for (; ok && u < whole_units; u += kT) ok = unit(kUnit), n_valid += kUnit;
+            if (ok && u < nu) {   // the last one, ragged
+                const int here = t.L - u * kUnit;
+                ok = unit(here), u += kT, n_valid += here, n_pad = (-here) & 63;
             }
             skip = u - nu;
             if (ok) {
