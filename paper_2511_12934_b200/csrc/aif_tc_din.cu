@@ -5,7 +5,7 @@
 //     sum_k (2 matches_k) S_k = d' sum_k S_k + sum_i q_i A_i,   A_i = sum_k s_ki S_k.
 // A and the sum of the rows depend on the request alone: [d' + 1 x d] numbers.  What a candidate costs then does not grow with the
 // sequence: [1 x d'] . [d' x d] instead of [1 x L] . [L x d] and the conversion of L match counts into an operand.  16 requests of 10^4
-// candidates and 10^4 keys, d 128: 15 + 12 us, and 225 for SimTier's counts alone (aif_tc_tier.cu), in place of 650 for the pass over the pairs that
+// candidates and 10^4 keys, d 128: 15 + 12 us, and 215 for SimTier's counts alone (aif_tc_tier.cu), in place of 650 for the pass over the pairs that
 // yields both.
 //
 //   k_din_sums    A and the row sums per request, on the tensor cores: a cluster of up to eight CTAs shares a request's key blocks,
