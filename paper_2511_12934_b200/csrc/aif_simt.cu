@@ -85,8 +85,10 @@ __device__ __forceinline__ float sum_squares(const uint4 &v, __nv_bfloat16)
 // integers; a NaN row yields a pattern above every finite one and stays.
 // Measured, 10^5 rows of 256 bytes with two 16-byte sidecars: 13 us (4.5 TB/s, the ids scatter the writes); as three scatter
 // launches, a 64-bit division per vector, and a norm pass over the table 45 us from first to last.
-template <typename T, int G>
-__global__ void __launch_bounds__(256) k_refresh_rows(uint4 *__restrict__ table, const uint4 *__restrict__ rows, const int32_t *__restrict__ ids,
+// SIDE: the table has sidecars.  Three blocks to an SM in either copy (3 x 10^5 rows and their gather: 48.4 us, with sidecars 62.4; with the 122
+// registers that the compiler would take for rows alone 52.1; sidecars asked for behind the row stores 68.9).
+template <typename T, int G, bool SIDE>
+__global__ void __launch_bounds__(256, 3) k_refresh_rows(uint4 *__restrict__ table, const uint4 *__restrict__ rows, const int32_t *__restrict__ ids,
                                                       int64_t n, int vpr, int64_t M, SideRows bea, SideRows sig, float *norm_max,
                                                       uint32_t *status)
 {
@@ -101,7 +103,7 @@ __global__ void __launch_bounds__(256) k_refresh_rows(uint4 *__restrict__ table,
         int64_t dst_row = -1;
         const bool has_id = lane < RPS && r0 + lane < n;
         if (has_id) dst_row = ids ? (int64_t)ids[r0 + lane] : r0 + lane;
-        const bool bea_one = one_unit(bea), sig_one = one_unit(sig);
+        const bool bea_one = SIDE && one_unit(bea), sig_one = SIDE && one_unit(sig);
         uint4 bea_v = make_uint4(0, 0, 0, 0), sig_v = bea_v;
         if (has_id && bea_one) bea_v = __ldcs(reinterpret_cast<const uint4 *>(bea.src) + r0 + lane);
         if (has_id && sig_one) sig_v = __ldcs(reinterpret_cast<const uint4 *>(sig.src) + r0 + lane);
@@ -135,10 +137,12 @@ __global__ void __launch_bounds__(256) k_refresh_rows(uint4 *__restrict__ table,
                 best = max(best, __float_as_int(sqrtf(ss[u])) & 0x7fffffff);
             }
         }
-        if (!bea_one) move_side<true>(bea, RPS, r0, n, my);
-        else if (my >= 0) reinterpret_cast<uint4 *>(bea.dst)[my] = bea_v;
-        if (!sig_one) move_side<true>(sig, RPS, r0, n, my);
-        else if (my >= 0) reinterpret_cast<uint4 *>(sig.dst)[my] = sig_v;
+        if (SIDE) {
+            if (!bea_one) move_side<true>(bea, RPS, r0, n, my);
+            else if (my >= 0) reinterpret_cast<uint4 *>(bea.dst)[my] = bea_v;
+            if (!sig_one) move_side<true>(sig, RPS, r0, n, my);
+            else if (my >= 0) reinterpret_cast<uint4 *>(sig.dst)[my] = sig_v;
+        }
     }
     if (norm_max) {
         best = __reduce_max_sync(0xffffffffu, best);
@@ -211,7 +215,11 @@ static cudaError_t refresh_typed(const aif_ctx *ctx, const int32_t *ids, int64_t
     auto go = [&](auto kernel) {
         return launch_pdl(kernel, dim3(grid), dim3(256), 0, st, (uint4 *)ctx->E, (const uint4 *)rows, ids, n, vpr, c.M, bea, sig, norm_max, ctx->status);
     };
-    const cudaError_t e = G == 8 ? go(k_refresh_rows<T, 8>) : G == 16 ? go(k_refresh_rows<T, 16>) : go(k_refresh_rows<T, 32>);
+    auto pick = [&](auto side) {
+        constexpr bool kSide = decltype(side)::value;
+        return G == 8 ? go(k_refresh_rows<T, 8, kSide>) : G == 16 ? go(k_refresh_rows<T, 16, kSide>) : go(k_refresh_rows<T, 32, kSide>);
+    };
+    const cudaError_t e = bea.bytes || sig.bytes ? pick(std::true_type{}) : pick(std::false_type{});
     count_launch();
     return e;
 }
