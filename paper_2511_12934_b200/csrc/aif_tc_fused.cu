@@ -320,7 +320,7 @@ __global__ void __launch_bounds__(kFThreads, 1) k_request_fused(const __grid_con
         }
         tc_fence_before();
         mbar_arrive(bar(BAR_H1_FULL));
-        // ---- layer-2 epilogue: half g of the units, ReLU, reduced against w_out
+        // ---- layer-2 epilogue: half g of the units, ReLU, reduced against w_out (four sums per half, in the order that aif_tc_split.cu keeps to)
         wait(BAR_ACC2_FULL);
         tc_fence_after();
         float dot = 0.f;

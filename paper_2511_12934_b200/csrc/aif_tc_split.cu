@@ -6,19 +6,20 @@
 // second for all candidates of the tile, 260 KB of weights.  The layers' products are units x candidates (M = 128 units, N = the tile),
 // so a narrow tile costs no padding.  Every CTA of a cluster gathers the tile's rows and does its attention (a few hundred keys for a few
 // candidates: less than handing the rows round); the first layer's activations, 128 units of every candidate, go to the other three from
-// shared memory to shared memory (8 KB each for 32 candidates), and the four partial logits to the first.
-// 1000 candidates, 200 behaviours: 20.25 us by the other kernel, 13.9 so; 200 candidates of 50: 19.5 and 12.1; 1500 of 200: 20.6 and 16.2.  Of
-// 25 k cycles the set-up is 1.8 k, rows and scores 2.7 k, the softmax 3.6 k (a tile's rows lie in one or two warps' tensor-memory lanes), O and its rows
-// 2.6 k, the layers 4.4 k and 2.3 k, their epilogues and the exchange 4 k.
+// shared memory to shared memory (8 KB each for 32 candidates), and the second layer's outputs to the first.
+// Every sum is in the order of aif_tc_fused.cu (one accumulator over a layer's chunks and, last, its biases; the output layer's eight partial sums), so a
+// candidate's logit is the same bits whichever kernel its call takes and whoever shares it.
+// 1000 candidates, 200 behaviours: 20.2 us by the other kernel, 13.7 so; 200 candidates: 20.4 and 12.4; 1500: 20.5 and 15.8.
 //
 // Tried: products the other way round without sharing the units (a tile of 16 to 128 per CTA, all weights): 22.5 us for 1000 candidates, 41.5 for 10^4 with
-// host buffers (37.0), three 32 KB stages of weights in flight being 43 bytes per clock; four issuing lanes: 12.6 us for 200 candidates (13.0), 14.2 for
-// 1000 (14.1), 16.5 for 1500 (16.2), where the weights' way in is what is left.
+// host buffers (37.0), three 32 KB stages of weights in flight being 43 bytes per clock; accumulators of its own for either issuing warp, which the
+// epilogue adds (another order of sums): 13.9 for 1000; one issuing lane that asks for the next chunk's barrier ahead: 15.4; two chunks to a turn:
+// 16.4, and 22 where the ring has three stages.
 //
-// 480 threads: warps 0-7 softmax and epilogues, 8 the issuing lane, 9-12 gather, 13 one lane of TMA, as there; 14 a second issuing lane.  A chunk of
-// 64 columns is four products of 45 cycles, and its waits, descriptors and commit take the lane 450 more: two lanes take the chunks in
-// turn, each with accumulators of its own that the epilogue adds (one lane: 7900 and 3900 cycles for the layers).
-// Tensor memory: attention as there (scores [0, 256), O [256, 384), probabilities [384, 512)); then the layers' accumulators, 64 columns each.
+// 480 threads: warps 0-7 softmax and epilogues, 8 and 14 the issuers, 9-12 gather, 13 one lane of TMA, as there.  A chunk of 64 columns is four
+// products of 45 cycles; the wait for its weights takes 140 cycles even where they are there, the hand-over between the issuers 180, the commit 100.
+// Tensor memory: attention as there (scores [0, 256), O [256, 384), probabilities [384, 512)); then the layers' accumulators, D of the first at 0, of
+// the second at 128.
 // Every wait is bounded.
 #include <cuda.h>
 
@@ -39,7 +40,8 @@ constexpr int kMaxTile = 48;
 constexpr int kBStage = 16384, kMaxStages = 8;
 constexpr int kMaxWeights = 4 + kMaxCross + kH1 / 64;   // chunks of weights of both layers, a barrier pair each
 constexpr size_t kFSmem = 227 * 1024;
-constexpr int kMiscBytes = 1024 + 2048;        // barriers | 8 x 64 partial dots
+constexpr int kMiscBytes = 3072;               // barriers | row sums | output weights, flags
+constexpr int kBias1 = 4096, kOnes = kMaxTile * 32, kBias = 2 * kBias1 + kOnes;   // bias operands: of either layer, and what they are multiplied by
 // shared memory behind the miscellany, with c = tile x 128 bytes a chunk of 64 columns: E 2 c | key/value blocks 64 KB, later the attention
 // chunks | cross chunks 8 c | activations 8 c | weight ring
 constexpr int stages_for(int tile) { return ((int)kFSmem - 1024 - kMiscBytes - 65536 - 18 * tile * 128) / kBStage < kMaxStages ? ((int)kFSmem - 1024 - kMiscBytes - 65536 - 18 * tile * 128) / kBStage : kMaxStages; }
@@ -47,11 +49,15 @@ static_assert(stages_for(kMaxTile) >= 3, "weight ring");
 
 enum {
     BAR_E_FULL = 0, BAR_KV_FULL, BAR_S_FULL = BAR_KV_FULL + 2, BAR_P_FULL = BAR_S_FULL + 2, BAR_O_FINAL, BAR_ATT_FULL, BAR_ACC1_FULL,
-    BAR_H1_FULL, BAR_ACC2_FULL, BAR_FULL_A, BAR_FULL_B = BAR_FULL_A + kMaxCross, BAR_EMPTY_B = BAR_FULL_B + kMaxWeights, BAR_COUNT = BAR_EMPTY_B + kMaxWeights
+    BAR_H1_FULL, BAR_ACC2_FULL, BAR_TURN, BAR_FULL_A = BAR_TURN + 2, BAR_FULL_B = BAR_FULL_A + kMaxCross, BAR_EMPTY_B = BAR_FULL_B + kMaxWeights, BAR_COUNT = BAR_EMPTY_B + kMaxWeights
 };
 static_assert(BAR_COUNT * 8 + 16 <= 512, "barriers");
-// D of the first layer at 0 and 64, of the second at 128 and 192, one per issuer
-static_assert(kMaxTile <= 64, "tensor memory");
+static_assert(2 * kMaxTile * 128 + kBias <= 32768, "attention rows and bias operands where the key blocks were");
+// The second layer's outputs of all units, [candidate][row_floats], as the first CTA sums them up: in front of the activations.  Eight floats
+// of padding, four of them in the middle: eight threads of a candidate and four candidates are on 32 banks.
+__host__ __device__ constexpr int row_floats(int H2) { return H2 + 8; }
+static_assert(kMaxTile * row_floats(256) * 4 <= 8 * kMaxTile * 128 + 32768 && 16 * row_floats(256) * 4 <= 8 * 16 * 128 + 32768, "second layer's outputs");
+static_assert(kMaxTile * 8 <= kFThreads, "eight threads per candidate");
 
 struct SplitParams {
     ScoreLaunch sl;
@@ -62,7 +68,7 @@ struct SplitParams {
     int32_t B, dc, b_mask, bucket_mode, n_cross;
     int32_t H2, emit_sigmoid;
     float scale_log2;       // log2(e) / sqrt(d)
-    const float *b2;        // [H2] second-layer bias
+    const __nv_bfloat16 *b2_hl;   // [2][H2]: second-layer bias, high parts then remainders
     const __nv_bfloat16 *w_out;
     const float *b_out;
 };
@@ -77,13 +83,16 @@ __global__ void __launch_bounds__(kFThreads, 1) k_request_split(const __grid_con
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + BAR_COUNT);
     volatile uint32_t *abort_flag = tmem_slot + 1;
     float *xs = reinterpret_cast<float *>(misc + 512);         // [2][64]: row sums or maxima of the two softmax groups
-    float *dot_s = reinterpret_cast<float *>(misc + 1024);     // [4][64]: per warp of a group's rows, partial dots
-    float *red_s = dot_s + 256;                                // [4][64]: the CTAs' partial logits (first CTA), element 63 of each: all is well
+    float *wout_s = reinterpret_cast<float *>(misc + 1024);    // [H2] output weights
+    float *ok_s = wout_s + 256;                                // [4]: all is well with a CTA (the first CTA's)
+    uint32_t *good_s = reinterpret_cast<uint32_t *>(ok_s + 4); // [tile]: a candidate's id is in the table
     const int cs = p.tile * 128;
     unsigned char *smE = misc + kMiscBytes, *smKV = smE + 2 * cs, *smAtt = smKV, *smX = smKV + 65536, *smH = smX + 8 * cs, *smB = smH + 8 * cs;
+    unsigned char *smBias1 = smAtt + 2 * cs, *smBias2 = smBias1 + kBias1, *smOnes = smBias2 + kBias1;
+    float *smOut = reinterpret_cast<float *>(smH) - p.tile * row_floats(p.H2);
     auto bar = [&](int i) { return smem_u32(bars + i); };
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;   // (a role is a whole warp's, and the compiler sees it)
     const int rank = (int)cluster_rank(), cluster = (int)(blockIdx.x / kCtas);
 
     if (tid == 0) {
@@ -98,6 +107,8 @@ __global__ void __launch_bounds__(kFThreads, 1) k_request_split(const __grid_con
         mbar_init(bar(BAR_ACC1_FULL), 2);
         mbar_init(bar(BAR_H1_FULL), 1);
         mbar_init(bar(BAR_ACC2_FULL), 2);
+        mbar_init(bar(BAR_TURN), 1);
+        mbar_init(bar(BAR_TURN + 1), 1);
         for (int i = 0; i < kMaxCross; ++i) mbar_init(bar(BAR_FULL_A + i), 128);
         for (int s = 0; s < kMaxWeights; ++s) mbar_init(bar(BAR_FULL_B + s), 1), mbar_init(bar(BAR_EMPTY_B + s), 1);
         *abort_flag = 0u;
@@ -128,6 +139,7 @@ __global__ void __launch_bounds__(kFThreads, 1) k_request_split(const __grid_con
     const int L = slot->L;
     const int nb = L > 128 ? 2 : 1;
     const int n_k1 = 4 + p.n_cross;
+    const float b_out = __ldg(p.b_out);   // (for the last step)
 
     if (warp < 8) {
         // ===================== softmax, epilogues =====================
@@ -144,6 +156,17 @@ __global__ void __launch_bounds__(kFThreads, 1) k_request_split(const __grid_con
         if (row < cnt) {
             const int id = p.sl.ids[pos0 + row];
             good = id >= 0 && (int64_t)id < p.M;
+        }
+        if (g == 0 && row < p.tile) good_s[row] = good ? 1u : 0u;
+        if (tid < p.H2) wout_s[tid] = __bfloat162float(p.w_out[tid]);
+        // bias of this thread's unit, of the first layer (group 0: the request's cached user partial) or the second
+        const int unit = rank * 128 + row, h2 = p.H2 / kCtas;
+        const bool has2 = row < h2;
+        uint32_t bias_hl = 0u;
+        {
+            const __nv_bfloat16 *hl = g == 0 ? reinterpret_cast<const __nv_bfloat16 *>(slot->pu_hl) : p.b2_hl;
+            const int at = g == 0 ? unit : rank * h2 + row, n = g == 0 ? kH1 : p.H2;
+            if (g == 0 || has2) bias_hl = (uint32_t)__bfloat16_as_ushort(hl[at]) | (uint32_t)__bfloat16_as_ushort(hl[n + at]) << 16;
         }
         // ---- attention: scores of key block g -> probabilities
         // Softmax is invariant to the offset subtracted in the exponent, and bf16 keeps its relative precision over the
@@ -241,15 +264,23 @@ __global__ void __launch_bounds__(kFThreads, 1) k_request_split(const __grid_con
                 }
             }
         }
+        // The biases are added by the tensor cores, as in aif_tc_fused.cu: one more step of K = 16 whose operands are, per unit, the bias in two
+        // bf16 values (high part, remainder) and, per candidate, two ones (no swizzle: 16-byte columns, the second ones zero).
+        if (ok) {
+            const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+            uint4 *b = reinterpret_cast<uint4 *>(g == 0 ? smBias1 : smBias2);
+            b[row] = make_uint4(bias_hl, 0u, 0u, 0u), b[128 + row] = zero;
+            if (g == 0 && row < p.tile) {
+                uint4 *one = reinterpret_cast<uint4 *>(smOnes);
+                one[row] = make_uint4(0x3F803F80u, 0u, 0u, 0u), one[p.tile + row] = zero;
+            }
+        }
         fence_proxy_async();   // the MMA reads these chunks through the async proxy
         tc_fence_before();
         mbar_arrive(bar(BAR_ATT_FULL));
-        // ---- layer-1 epilogue: a thread owns a unit (lane) and, with the other group, every second sixteen candidates (columns); its bias is
-        // one value.  ReLU, bf16, and the activations go to shared memory as the second layer's operand: 64-unit chunks of 128-byte
-        // rows, one per candidate; this CTA's two chunks then go to the other three.
-        const int unit = rank * 128 + row, h2 = p.H2 / kCtas, unit2 = rank * h2 + row;
-        const bool has2 = row < h2;
-        const float bias = __ldg(slot->p_u + unit), b2 = has2 ? __ldg(p.b2 + unit2) : 0.f, w2 = has2 ? __bfloat162float(p.w_out[unit2]) : 0.f;
+        // ---- layer-1 epilogue: a thread owns a unit (lane) and, with the other group, every second sixteen candidates (columns).  ReLU, bf16, and
+        // the activations go to shared memory as the second layer's operand: 64-unit chunks of 128-byte rows, one per candidate; this
+        // CTA's two chunks then go to the other three.
         wait(BAR_ACC1_FULL);
         tc_fence_after();
         if (ok) {
@@ -257,12 +288,12 @@ __global__ void __launch_bounds__(kFThreads, 1) k_request_split(const __grid_con
             const int piece = (unit & 63) >> 3;
 #pragma unroll 1
             for (int c0 = 16 * g; c0 < p.tile; c0 += 32) {
-                uint32_t r[16], r2[16];   // what either issuer has summed
-                tmem_ld16(lane_base + (uint32_t)c0, r), tmem_ld16(lane_base + 64u + (uint32_t)c0, r2);
+                uint32_t r[16];
+                tmem_ld16(lane_base + (uint32_t)c0, r);
                 tmem_ld_wait();
 #pragma unroll
                 for (int c = 0; c < 16; ++c)
-                    *reinterpret_cast<__nv_bfloat16 *>(dst + (c0 + c) * 128 + ((piece ^ (c & 7)) << 4)) = __float2bfloat16_rn(fmaxf(__uint_as_float(r[c]) + __uint_as_float(r2[c]) + bias, 0.f));
+                    *reinterpret_cast<__nv_bfloat16 *>(dst + (c0 + c) * 128 + ((piece ^ (c & 7)) << 4)) = __float2bfloat16_rn(fmaxf(__uint_as_float(r[c]), 0.f));
             }
         }
         fence_proxy_async();   // read by the copies and the MMA through the async proxy
@@ -275,108 +306,106 @@ __global__ void __launch_bounds__(kFThreads, 1) k_request_split(const __grid_con
                 bulk_copy_cluster(cluster_addr(src, to), src, (uint32_t)(2 * cs), cluster_addr(bar(BAR_H1_FULL), to));
             }
         }
-        // ---- layer-2 epilogue: unit (lane) of this CTA's quarter, ReLU, times its output weight; then the sum over units: over a warp's 32
-        // lanes (every exchange halves the columns a lane still holds), over the warps through shared memory, over the CTAs in the first one's.
+        // ---- layer-2 epilogue: unit (lane) of this CTA's quarter, ReLU, into the first CTA's shared memory
         wait(BAR_ACC2_FULL);
         tc_fence_after();
         if (ok && wq * 32 < h2) {
+            const int unit2 = rank * h2 + row, stride = row_floats(p.H2);
+            const uint32_t out = cluster_addr(smem_u32(smOut + unit2 + (unit2 >= p.H2 / 2 ? 4 : 0)), 0u);
 #pragma unroll 1
             for (int c0 = 16 * g; c0 < p.tile; c0 += 32) {
-                uint32_t r[16], r2[16];
-                tmem_ld16(lane_base + 128u + (uint32_t)c0, r), tmem_ld16(lane_base + 192u + (uint32_t)c0, r2);
+                uint32_t r[16];
+                tmem_ld16(lane_base + 128u + (uint32_t)c0, r);
                 tmem_ld_wait();
-                float v[16];
+                if (has2)
 #pragma unroll
-                for (int c = 0; c < 16; ++c) v[c] = has2 ? fmaxf(__uint_as_float(r[c]) + __uint_as_float(r2[c]) + b2, 0.f) * w2 : 0.f;
-#pragma unroll
-                for (int w = 8; w > 0; w >>= 1) {   // lanes with bit 2 w keep the upper half
-                    const bool up = lane & (2 * w);
-#pragma unroll
-                    for (int c = 0; c < w; ++c) {
-                        const float give = up ? v[c] : v[c + w], keep = up ? v[c + w] : v[c];
-                        v[c] = keep + __shfl_xor_sync(0xffffffffu, give, 2 * w);
-                    }
-                }
-                v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
-                if (!(lane & 1)) dot_s[wq * 64 + c0 + (lane >> 1)] = v[0];
+                    for (int c = 0; c < 16; ++c) st_cluster_f32(out + (uint32_t)((c0 + c) * stride * 4), fmaxf(__uint_as_float(r[c]), 0.f));
             }
         }
-        const bool all_ok = !named_bar_or(1, 256, !ok);   // also orders dot_s; a wait that ran out anywhere in these warps
-        if (g == 0 && row < 64) {
-            float part = 0.f;
-            for (int w = 0; w < (h2 + 31) / 32; ++w) part += dot_s[w * 64 + row];
-            if (row == 63) part = all_ok ? 1.f : 0.f;
-            st_cluster_f32(cluster_addr(smem_u32(red_s + rank * 64 + row), 0u), part);
-        }
-        mine = good;   // (for the last step)
+        const bool all_ok = !named_bar_or(1, 256, !ok);   // a wait that ran out anywhere in these warps
+        if (tid == 0) st_cluster_f32(cluster_addr(smem_u32(ok_s + rank), 0u), all_ok ? 1.f : 0.f);
     } else if (warp == kFMmaWarp || warp == kFMmaWarp2) {
         // ===================== MMA issuers: even and odd chunks of the layers; the attention is the first one's =====================
-        if (lane == 0) {
-            constexpr uint32_t idesc_qk = umma_idesc_bf16(kTcTile, 128);
-            constexpr uint32_t idesc_pv = umma_idesc_bf16_bmn(kTcTile, 128);
-            const uint32_t idesc_l = umma_idesc_bf16(128, p.tile);   // of both layers: 128 units x the tile's candidates
-            const int mine2 = warp == kFMmaWarp2;
-            bool ok = true;
-            if (mine2 == 0) {
-                ok = mbar_wait(bar(BAR_E_FULL), 0u, abort_flag);
-                fence_proxy_async();   // the item rows were written by cp.async
-                // scores = Q K^T, one key block after the other
-                const uint64_t qd = umma_desc_sw128(smem_u32(smE));
-                for (int j = 0; ok && j < nb; ++j) {
-                    ok = mbar_wait(bar(BAR_KV_FULL + j), 0u, abort_flag);
-                    tc_fence_after();
-                    if (!ok) break;
-                    const uint64_t kd = umma_desc_sw128(smem_u32(smKV + j * 32768));
-                    const uint32_t d_tmem = tmem_base + (uint32_t)(j * 128);
+        // The whole warp walks through, one lane issues.  (With the walk in one lane, behind a branch, its descriptors are no uniform values
+        // to the compiler and a product takes 75 cycles to issue: 15.9 us for 1000 candidates.)
+        const bool one = elect_one();
+        constexpr uint32_t idesc_qk = umma_idesc_bf16(kTcTile, 128);
+        constexpr uint32_t idesc_pv = umma_idesc_bf16_bmn(kTcTile, 128);
+        const uint32_t idesc_l = umma_idesc_bf16(128, p.tile);   // of both layers: 128 units x the tile's candidates
+        const int second = warp == kFMmaWarp2;
+        bool ok = mbar_wait(bar(BAR_E_FULL), 0u, abort_flag);
+        fence_proxy_async();   // the item rows were written by cp.async
+        if (!second) {
+            // scores = Q K^T, one key block after the other
+            const uint64_t qd = umma_desc_sw128(smem_u32(smE));
+            for (int j = 0; ok && j < nb; ++j) {
+                ok = mbar_wait(bar(BAR_KV_FULL + j), 0u, abort_flag);
+                tc_fence_after();
+                if (!ok) break;
+                const uint64_t kd = umma_desc_sw128(smem_u32(smKV + j * 32768));
+                const uint32_t d_tmem = tmem_base + (uint32_t)(j * 128);
+                if (one) {
 #pragma unroll
                     for (int kk = 0; kk < 8; ++kk)
                         umma_bf16(d_tmem, qd + (uint64_t)(uint32_t)((kk >> 2) * (cs >> 4) + 2 * (kk & 3)), kd + (uint64_t)((kk >> 2) * (kChunk >> 4) + 2 * (kk & 3)), idesc_qk, kk > 0 ? 1u : 0u);
                     umma_commit(bar(BAR_S_FULL + j));
                 }
-                // O = P V: the probabilities from tensor memory, V = the key blocks read MN-major
-                ok = ok && mbar_wait(bar(BAR_P_FULL), 0u, abort_flag);
-                tc_fence_after();
-                if (ok) {
-                    for (int j = 0; j < nb; ++j) {
-                        const uint64_t vd = umma_desc_mn_sw128(smem_u32(smKV + j * 32768), kChunk);
-#pragma unroll
-                        for (int kk = 0; kk < 8; ++kk)
-                            umma_bf16_ts(tmem_base + 256u, tmem_base + (uint32_t)(384 + j * 64 + kk * 8), vd + (uint64_t)(kk * (2048 >> 4)), idesc_pv,
-                                         (j > 0 || kk > 0) ? 1u : 0u);
-                    }
-                    umma_commit(bar(BAR_O_FINAL));
-                }
             }
-            // layer 1: K chunks [ item 0-1 | attention 2-3 | cross 4.. ], this CTA's 128 units
-            ok = ok && mbar_wait(bar(BAR_ATT_FULL), 0u, abort_flag);
+            // O = P V: the probabilities from tensor memory, V = the key blocks read MN-major
+            ok = ok && mbar_wait(bar(BAR_P_FULL), 0u, abort_flag);
             tc_fence_after();
-            if (ok && mine2 && (ok = mbar_wait(bar(BAR_E_FULL), 0u, abort_flag))) fence_proxy_async();   // (the item rows, as above)
-            int sb = mine2 % p.stages;
-            auto product = [&](int c, uint32_t d_tmem, uint64_t xd, bool first) {   // weight chunk c, of both layers in their order
-                if (!(ok = mbar_wait(bar(BAR_FULL_B + c), 0u, abort_flag))) return;
-                tc_fence_after();
-                const uint64_t wd = umma_desc_sw128(smem_u32(smB + sb * kBStage));
+            if (ok && one) {
+                for (int j = 0; j < nb; ++j) {
+                    const uint64_t vd = umma_desc_mn_sw128(smem_u32(smKV + j * 32768), kChunk);
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk) umma_bf16(d_tmem, wd + (uint64_t)(2 * kk), xd + (uint64_t)(2 * kk), idesc_l, first && kk == 0 ? 0u : 1u);
-                umma_commit(bar(BAR_EMPTY_B + c));
-            };
-            auto ahead = [&](int n) { sb += n; while (sb >= p.stages) sb -= p.stages; };
-            const uint32_t d1 = tmem_base + (uint32_t)(64 * mine2), d2 = tmem_base + 128u + (uint32_t)(64 * mine2);
-            for (int kc = mine2; ok && kc < n_k1; kc += 2, ahead(2)) {
-                if (kc >= 4) {
-                    if (!(ok = mbar_wait(bar(BAR_FULL_A + kc - 4), 0u, abort_flag))) break;
-                    fence_proxy_async();
+                    for (int kk = 0; kk < 8; ++kk)
+                        umma_bf16_ts(tmem_base + 256u, tmem_base + (uint32_t)(384 + j * 64 + kk * 8), vd + (uint64_t)(kk * (2048 >> 4)), idesc_pv,
+                                     (j > 0 || kk > 0) ? 1u : 0u);
                 }
-                product(kc, d1, umma_desc_sw128(smem_u32(kc < 2 ? smE + kc * cs : kc < 4 ? smAtt + (kc - 2) * cs : smX + (kc - 4) * cs)), kc == mine2);
+                umma_commit(bar(BAR_O_FINAL));
             }
-            if (ok) umma_commit(bar(BAR_ACC1_FULL));
-            // layer 2, this CTA's quarter of the units (lanes beyond it: whatever the stage held, nobody reads them)
-            ok = ok && mbar_wait(bar(BAR_H1_FULL), 0u, abort_flag);
-            tc_fence_after();
-            sb = 0, ahead(n_k1 + mine2);
-            for (int kc = mine2; ok && kc < kH1 / 64; kc += 2, ahead(2)) product(n_k1 + kc, d2, umma_desc_sw128(smem_u32(smH + kc * cs)), kc == mine2);
-            if (ok) umma_commit(bar(BAR_ACC2_FULL));
         }
+        // The chunks of a layer in their order, then its biases, into one accumulator: a candidate's sums are those of the kernel of one CTA per
+        // tile, bit for bit.  The two warps take turns, so the order of their products is that of the hand-overs between them; what comes
+        // before a chunk's products (waits, descriptors) and behind them (commits) is in nobody's way.
+        ok = ok && mbar_wait(bar(BAR_ATT_FULL), 0u, abort_flag);
+        tc_fence_after();
+        uint32_t turn = 0;   // of this warp: every second chunk of both layers
+        int sb = second % p.stages;
+        auto product = [&](int c, uint32_t d_tmem, uint64_t xd, bool first, const unsigned char *bias) {   // weight chunk c, of both layers in their order
+            if (!(ok = mbar_wait(bar(BAR_FULL_B + c), 0u, abort_flag))) return;
+            tc_fence_after();
+            const uint64_t wd = umma_desc_sw128(smem_u32(smB + sb * kBStage));
+            if (c > 0 && !(ok = mbar_wait(bar(BAR_TURN + second), (turn - (uint32_t)!second) & 1u, abort_flag))) return;
+            ++turn;
+            tc_fence_after();
+            if (one) {
+                umma_bf16(d_tmem, wd, xd, idesc_l, first ? 0u : 1u);
+#pragma unroll
+                for (int kk = 1; kk < 4; ++kk) umma_bf16_acc(d_tmem, wd + (uint64_t)(2 * kk), xd + (uint64_t)(2 * kk), idesc_l);
+                if (bias) umma_bf16_acc(d_tmem, umma_desc_plain(smem_u32(bias), 2048), umma_desc_plain(smem_u32(smOnes), (uint32_t)p.tile * 16u), idesc_l);
+                tc_fence_before();
+                mbar_arrive(bar(BAR_TURN + (second ^ 1)));
+                umma_commit(bar(BAR_EMPTY_B + c));
+            }
+            for (sb += 2; sb >= p.stages;) sb -= p.stages;
+        };
+        // layer 1: K chunks [ item 0-1 | attention 2-3 | cross 4.. ], this CTA's 128 units
+        int c = second;
+        for (; ok && c < n_k1; c += 2) {
+            if (c >= 4) {
+                if (!(ok = mbar_wait(bar(BAR_FULL_A + c - 4), 0u, abort_flag))) break;
+                fence_proxy_async();
+            }
+            product(c, tmem_base, umma_desc_sw128(smem_u32(c < 2 ? smE + c * cs : c < 4 ? smAtt + (c - 2) * cs : smX + (c - 4) * cs)), c == 0, c == n_k1 - 1 ? smBias1 : nullptr);
+        }
+        if (ok && one) umma_commit(bar(BAR_ACC1_FULL));
+        // layer 2, this CTA's quarter of the units (lanes beyond it: whatever the stage held, nobody reads them)
+        ok = ok && mbar_wait(bar(BAR_H1_FULL), 0u, abort_flag);
+        tc_fence_after();
+        for (; ok && c < n_k1 + kH1 / 64; c += 2)
+            product(c, tmem_base + 128u, umma_desc_sw128(smem_u32(smH + (c - n_k1) * cs)), c == n_k1, c == n_k1 + kH1 / 64 - 1 ? smBias2 : nullptr);
+        if (ok && one) umma_commit(bar(BAR_ACC2_FULL));
         __syncwarp();
     } else if (warp < kFBWarp) {
         // ===================== item-row and cross-feature gather (128 threads) =====================
@@ -453,12 +482,24 @@ __global__ void __launch_bounds__(kFThreads, 1) k_request_split(const __grid_con
     tc_fence_before();
     __syncthreads();
     cluster_sync();   // all partial logits are with the first CTA; nobody leaves while another may still write to it
-    if (rank == 0 && tid < cnt) {   // (thread = row: `mine` is whether its id is in the table)
-        float logit = p.b_out[0];
-        bool all = true;
-        for (int q = 0; q < kCtas; ++q) logit += red_s[q * 64 + tid], all = all && red_s[q * 64 + 63] != 0.f;
-        if (p.emit_sigmoid) logit = 1.0f / (1.0f + expf(-logit));
-        p.sl.logits[pos0 + tid] = mine && all ? logit : __int_as_float(0x7fc00000);   // no number for a bad id, nor where a wait ran out
+    if (rank == 0) {
+        // The output layer, in the order of the kernel of one CTA per tile: eight threads per candidate, each every fourth unit of one half
+        const int cand = tid >> 3, half = (tid >> 2) & 1, i = tid & 3, hn = p.H2 / 2;
+        float dot = 0.f;
+        if (cand < cnt) {
+            const float *v = smOut + cand * row_floats(p.H2) + half * (hn + 4) + i, *w = wout_s + half * hn + i;
+#pragma unroll 16
+            for (int k = 0; k < hn; k += 4) dot = fmaf(v[k], w[k], dot);
+        }
+        dot += __shfl_xor_sync(0xffffffffu, dot, 1);
+        dot += __shfl_xor_sync(0xffffffffu, dot, 2);
+        dot += __shfl_xor_sync(0xffffffffu, dot, 4);
+        if (cand < cnt && (tid & 7) == 0) {
+            float logit = dot + b_out;
+            const bool all = ok_s[0] != 0.f && ok_s[1] != 0.f && ok_s[2] != 0.f && ok_s[3] != 0.f;
+            if (p.emit_sigmoid) logit = 1.0f / (1.0f + expf(-logit));
+            p.sl.logits[pos0 + cand] = good_s[cand] && all ? logit : __int_as_float(0x7fc00000);   // no number for a bad id, nor where a wait ran out
+        }
     }
     if (warp == kFMmaWarp) tmem_dealloc(tmem_base, 512);
 }
@@ -496,7 +537,7 @@ cudaError_t launch_request_split(const aif_ctx *ctx, const ScoreLaunch &sl, cuda
     p.n_cross = c.F * c.dc / 64;
     p.H2 = c.hidden[1], p.emit_sigmoid = c.emit_sigmoid;
     p.scale_log2 = 1.4426950408889634f / sqrtf((float)c.d);
-    p.b2 = ctx->b[1], p.w_out = (const __nv_bfloat16 *)ctx->w_out, p.b_out = ctx->b_out;
+    p.b2_hl = reinterpret_cast<const __nv_bfloat16 *>(ctx->tc_fused_plan), p.w_out = (const __nv_bfloat16 *)ctx->w_out, p.b_out = ctx->b_out;
     const CUtensorMap *ms = reinterpret_cast<const CUtensorMap *>(tc_att_tmap(ctx));
     const CUtensorMap *m1 = reinterpret_cast<const CUtensorMap *>(tc_weight_half_tmap(ctx, 0));
     const CUtensorMap *m2 = reinterpret_cast<const CUtensorMap *>(tc_weight_quarter_tmap(ctx));

@@ -86,17 +86,6 @@ struct TierCfg {
     static_assert(kStages == kScores && (kStages + 2 * kScores + 5) * 8 + 8 <= 512, "barriers");
 };
 
-// K-major operand without swizzle (8 rows x 16 bytes contiguous, 8-row groups 128 bytes apart, 16-byte columns `col_bytes` apart).
-__device__ __forceinline__ uint64_t umma_desc_plain(uint32_t smem_addr, uint32_t col_bytes)
-{
-    uint64_t d = 0;
-    d |= (uint64_t)((smem_addr & 0x3FFFFu) >> 4);
-    d |= (uint64_t)(col_bytes >> 4) << 16;
-    d |= (uint64_t)(128u >> 4) << 32;
-    d |= (uint64_t)1 << 46;
-    return d;
-}
-
 // 32 lanes x 64 columns, the low halves of two adjacent columns in one register.
 __device__ __forceinline__ void tmem_ld64_pack16(uint32_t taddr, uint32_t (&r)[32])
 {

@@ -647,3 +647,21 @@ def test_request_of_one_tile_per_cta_with_scores_that_overflow():
     want = helpers.make_oracle(wl, weights, M=table["E"].shape[0]).score(table, helpers.projected_request(wl, rq), ids[::9])
     _check(got, want, 1e-2 * max(1.0, float(np.abs(want).max())))
     srv.close()
+
+
+@pytest.mark.parametrize("H2,L,sigmoid", [(256, 200, 0), (64, 128, 0), (192, 129, 1), (128, 1, 0)])
+def test_a_request_in_one_call_or_in_several_gives_the_same_bits(H2, L, sigmoid):
+    """A candidate's logit does not depend on how many share its call: clusters of four CTAs (small calls) and one CTA per tile (large ones, and
+    batches) sum in the same order, so a request cut into calls on either side of every change is ranked by the bits of the whole."""
+    wl = helpers.MINI["c2"].with_(name=f"cut_{H2}_{L}", R=2, N=3000, M=20_000, mini_batch=0, L=L, hidden=(512, H2), emit_sigmoid=sigmoid)
+    srv = serving.Server(wl, synth.make_weights(wl, zero_bias=False), synth.make_item_table(wl), path=B.PATH_TENSOR)
+    st = srv.precompute(0, srv.upload_request(synth.make_request(wl, 0), B.USER_PROJECTED))
+    ids = synth.IdSampler(wl).request_ids(0, 3000)
+    whole = srv.score_ids(st, ids)
+    assert len(np.unique(whole)) > 1000
+    for first in (1, 15, 16, 17, 33, 200, 577, 592, 593, 1000, 1184, 1185, 1728, 1729, 1800):
+        assert np.array_equal(srv.score_ids(st, ids[:first]).view(np.uint32), whole[:first].view(np.uint32)), first
+        assert np.array_equal(srv.score_ids(st, ids[first:]).view(np.uint32), whole[first:].view(np.uint32)), first
+    a, b = srv.score_many([st, st], [ids[:700], ids[700:]])
+    assert np.array_equal(np.concatenate([a, b]).view(np.uint32), whole.view(np.uint32))
+    srv.close()
