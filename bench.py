@@ -78,7 +78,7 @@ def keys_of(wl: synth.Workload, keys) -> float:
 
 def kernel_flops(name: str, wl: synth.Workload, n: int, keys=None) -> float:
     f = flops_per_candidate(wl, keys)
-    if name in ("score_simt", "score_fused"):
+    if name in ("score_simt", "score_fused", "score_split"):
         return f["total"] * n
     if name == "interact":
         return (f["attention"] + f["lsh_din"] + f["bea"]) * n

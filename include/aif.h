@@ -274,6 +274,9 @@ int aif_user_state_export(aif_ctx *ctx, const aif_user_state *state, float *u_ou
  * per request or once per mini-batch; the result of a candidate does not depend on which (but for the order of fp32 sums on the
  * tensor-core path: where a call has few tiles, the keys of a long sequence are summed in pieces).  n = 0 is a no-op.
  * An id outside [0, M) gives NaN and sets AIF_STATUS_BAD_ID.  No host-device copy happens inside.
+ * Small requests of the base shape (up to about 1700 candidates) spread over most of the GPU for a short time, except where the device's last
+ * eight such calls, of any context, came on so many streams that they would stand in each other's way; their logits are the same bits either way.
+ * A captured call keeps what was chosen when it was captured.
  * Errors: AIF_ERR_VERSION, AIF_ERR_NOT_READY, AIF_ERR_SHAPE (n > max_batch_candidates), AIF_ERR_ARG. */
 int aif_score(aif_ctx *ctx, const aif_user_state *state, const int32_t *cand_ids, int32_t n, float *logits,
               aif_stream stream);

@@ -337,8 +337,8 @@ cudaError_t tc_fused_prepare_weights(aif_ctx *ctx, cudaStream_t st);
 cudaError_t launch_request_fused(const aif_ctx *ctx, const ScoreLaunch &sl, cudaStream_t st);
 // the same for a small request by clusters of four CTAs (aif_tc_split.cu)
 int tc_split_prepare();
-bool tc_split_fits(const aif_ctx *ctx, int n);
-cudaError_t launch_request_split(const aif_ctx *ctx, const ScoreLaunch &sl, cudaStream_t st);
+int tc_split_tile(const aif_ctx *ctx, int n, cudaStream_t st);
+cudaError_t launch_request_split(const aif_ctx *ctx, const ScoreLaunch &sl, int tile, cudaStream_t st);
 const void *tc_weight_half_tmap(const aif_ctx *ctx, int k);   // with boxes of half a slice's rows
 const void *tc_weight_quarter_tmap(const aif_ctx *ctx);       // second layer, boxes of a quarter of its units
 const void *tc_weight_tmap(const aif_ctx *ctx, int k);   // CUtensorMap over the packed weights of hidden layer k

@@ -1500,8 +1500,9 @@ cudaError_t launch_score_tc_scratch(const aif_ctx *ctx, const ScoreLaunch &sl_in
     // a launch that fits the machine in one round of tiles: the whole pass in one kernel, one CTA per tile
     if (c.n_categories == 0 && sl.n_tiles <= kFusedMaxTiles && sl.max_L <= 256 && tc_fused_supported(c)) {
         StageRange range("aif score_fused");
-        cudaError_t e = !sl.reqs && tc_split_fits(ctx, sl.single.n) ? launch_request_split(ctx, sl, st) : launch_request_fused(ctx, sl, st);
-        timing_mark(ctx, "score_fused", st);
+        const int tile = sl.reqs ? 0 : tc_split_tile(ctx, sl.single.n, st);
+        cudaError_t e = tile ? launch_request_split(ctx, sl, tile, st) : launch_request_fused(ctx, sl, st);
+        timing_mark(ctx, tile ? "score_split" : "score_fused", st);
         return e;
     }
     // ids across the bus: on the way through the bucket kernel where that one comes first, else by a copy of their own

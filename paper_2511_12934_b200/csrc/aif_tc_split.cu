@@ -1,8 +1,8 @@
 // Scoring pass of a small request by clusters of four CTAs (sm_100a, bf16 storage), the same shapes as aif_tc_fused.cu.
 //
 // In the kernel of one CTA per tile every SM takes in all weights, 1.05 MB at 59 bytes per clock, and 1000 candidates are 8 tiles on 148 SMs:
-// 37 k cycles whatever the machine could do beside.  Here a request's candidates go in tiles of 16 to 48, as many as clusters of four find
-// room for at once, and the four CTAs of a cluster share the units: each forms 128 units of the first layer and a quarter of the
+// 37 k cycles whatever the machine could do beside.  Here a request's candidates go in tiles of 16 to 48, so many that all clusters of four find
+// room at once, and the four CTAs of a cluster share the units: each forms 128 units of the first layer and a quarter of the
 // second for all candidates of the tile, 260 KB of weights.  The layers' products are units x candidates (M = 128 units, N = the tile),
 // so a narrow tile costs no padding.  Every CTA of a cluster gathers the tile's rows and does its attention (a few hundred keys for a few
 // candidates: less than handing the rows round); the first layer's activations, 128 units of every candidate, go to the other three from
@@ -22,6 +22,8 @@
 // the second at 128.
 // Every wait is bounded.
 #include <cuda.h>
+
+#include <mutex>
 
 #include "aif_device.cuh"
 #include "aif_internal.h"
@@ -524,15 +526,49 @@ int tc_split_prepare()
     return n;
 }
 
-// Whether a single request of n candidates is one round of clusters (the caller has checked tc_fused_supported and the sequence's length).
-bool tc_split_fits(const aif_ctx *ctx, int n) { return n <= ctx->split_clusters * kMaxTile; }
+// The streams of a device's last small requests, of all contexts: how many of them run beside each other as far as a call can know.  A hint
+// that decides on speed alone; a handle is compared, never used.
+struct RecentStreams {
+    static constexpr int kCalls = 8;
+    std::mutex lock;
+    cudaStream_t stream[kCalls];
+    int calls = 0;
+    int note(cudaStream_t st)   // different streams among the last calls, this one included
+    {
+        const std::lock_guard<std::mutex> guard(lock);
+        stream[calls++ % kCalls] = st;
+        if (calls == 2 * kCalls) calls = kCalls;
+        int different = 0;
+        for (int i = 0, n = calls < kCalls ? calls : kCalls; i < n; ++i) {
+            bool seen = false;
+            for (int j = 0; j < i; ++j) seen = seen || stream[j] == stream[i];
+            different += !seen;
+        }
+        return different;
+    }
+};
+static RecentStreams g_recent[16];
 
-cudaError_t launch_request_split(const aif_ctx *ctx, const ScoreLaunch &sl, cudaStream_t st)
+// Candidates per cluster for a single request of n, 0: the kernel of one CTA per tile is the better one (the caller has checked tc_fused_supported
+// and the sequence's length).  Clusters make a call shorter by taking more of the machine: 1000 candidates hold 128 SMs for 14 us in place of 8
+// for 20.  So they are taken where as many calls as there are streams at work are one round of clusters together.  1000 candidates on
+// 1, 2, 4 and 8 streams, us per call: clusters 13.5, 12.2, 12.1, 12.1, one CTA per tile 20.1, 10.4, 5.4, 2.9; 200 candidates 12.0, 6.3, 4.8, 4.7
+// and 20.4, 10.3, 5.3, 2.8.
+int tc_split_tile(const aif_ctx *ctx, int n, cudaStream_t st)
+{
+    if (n > ctx->split_clusters * kMaxTile) return 0;
+    const int calls = ctx->device < 16 ? g_recent[ctx->device].note(st) : 1;
+    for (int tile = 16; tile <= kMaxTile; tile += 16)
+        if ((n + tile - 1) / tile * calls <= ctx->split_clusters) return tile;
+    return 0;
+}
+
+cudaError_t launch_request_split(const aif_ctx *ctx, const ScoreLaunch &sl, int tile, cudaStream_t st)
 {
     const aif_config &c = ctx->cfg;
     SplitParams p{};
     p.sl = sl, p.E = (const uint8_t *)ctx->E, p.M = c.M;
-    p.tile = ((sl.single.n + ctx->split_clusters - 1) / ctx->split_clusters + 15) / 16 * 16, p.stages = stages_for(p.tile);
+    p.tile = tile, p.stages = stages_for(tile);
     p.B = c.B, p.dc = c.dc, p.b_mask = (c.B & (c.B - 1)) == 0 ? c.B - 1 : -1, p.bucket_mode = c.bucket_mode;
     p.n_cross = c.F * c.dc / 64;
     p.H2 = c.hidden[1], p.emit_sigmoid = c.emit_sigmoid;

@@ -665,3 +665,47 @@ def test_a_request_in_one_call_or_in_several_gives_the_same_bits(H2, L, sigmoid)
     a, b = srv.score_many([st, st], [ids[:700], ids[700:]])
     assert np.array_equal(np.concatenate([a, b]).view(np.uint32), whole.view(np.uint32))
     srv.close()
+
+
+def _route(ctx, st, ids, stream):
+    """One scoring call on `stream`: the kernels that it took, and its logits."""
+    out = torch.empty(ids.numel(), dtype=torch.float32, device="cuda")
+    stream.wait_stream(torch.cuda.current_stream())
+    ctx.set_kernel_timing(True)
+    with torch.cuda.stream(stream):
+        ctx.score(st, ids, out)
+    names = list(ctx.get_kernel_timing())
+    ctx.set_kernel_timing(False)
+    torch.cuda.synchronize()
+    return names, out.cpu().numpy()
+
+
+def test_small_requests_on_several_streams_leave_room_for_each_other():
+    """Clusters shorten a call by holding most of the machine.  Calls that alternate between streams, of one context or of two, take them only
+    where all fit side by side: 1000 candidates on two streams go by the kernel that holds 8 SMs, 200 on two by clusters, 200 on eight
+    not; and by clusters again once the calls are on one stream.  The logits are the same bits by any way."""
+    wl = helpers.MINI["c2"].with_(name="streams", R=2, N=1000, M=20_000, mini_batch=0, L=200)
+    weights, table = synth.make_weights(wl, zero_bias=False), synth.make_item_table(wl)
+    srvs = [serving.Server(wl, weights, table, path=B.PATH_TENSOR) for _ in range(2)]
+    sts = [s.precompute(0, s.upload_request(synth.make_request(wl, 0), B.USER_PROJECTED)) for s in srvs]
+    torch.cuda.synchronize()
+    ids = torch.from_numpy(np.ascontiguousarray(synth.IdSampler(wl).request_ids(0, 1000), dtype=np.int32)).cuda()
+    streams = [torch.cuda.Stream() for _ in range(8)]
+
+    def go(which, n, stream):
+        return _route(srvs[which].ctx, sts[which], ids[:n], streams[stream])
+
+    alone = [go(0, 1000, 0) for _ in range(8)][-1]   # eight calls later nothing of what ran before counts
+    assert alone[0] == ["score_split"]
+    for two in (0, 1):
+        beside = [go(two * (i & 1), 1000, i & 1) for i in range(9)][1:]
+        for names, out in beside:
+            assert names == ["score_fused"] and np.array_equal(out.view(np.uint32), alone[1].view(np.uint32))
+        for i in range(9):
+            names, out = go(two * (i & 1), 200, i & 1)
+            assert names == ["score_split"] and np.array_equal(out.view(np.uint32), alone[1][:200].view(np.uint32))
+    many = [go(0, 200, i) for i in range(8)]
+    assert many[-1][0] == ["score_fused"] and np.array_equal(many[-1][1].view(np.uint32), alone[1][:200].view(np.uint32))
+    assert [go(0, 1000, 0)[0] for _ in range(8)][-1] == ["score_split"]
+    for s in srvs:
+        s.close()
