@@ -703,7 +703,7 @@ static int score_batch(aif_ctx *ctx, int32_t n_req, const aif_user_state *const 
     }
     AIF_CUDA(cudaMemcpyAsync(ring.dev[slot], ring.host[slot], sizeof(ReqDev) * (size_t)n_req, cudaMemcpyHostToDevice, st));
     ScoreLaunch sl{};
-    sl.slots = ctx->slots_dev, sl.reqs = ring.dev[slot], sl.n_req = n_req, sl.n_tiles = tiles, sl.total = total, sl.max_L = max_L;
+    sl.slots = ctx->slots_dev, sl.reqs = ring.dev[slot], sl.reqs_host = ring.host[slot], sl.n_req = n_req, sl.n_tiles = tiles, sl.total = total, sl.max_L = max_L;
     sl.ids = cand_ids, sl.logits = logits, sl.status = ctx->status, sl.ids_copy = ids_copy;
     int rc = run_score(ctx, sl, total, st);
     if (rc != AIF_OK) return rc;

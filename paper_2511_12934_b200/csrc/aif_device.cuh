@@ -184,25 +184,28 @@ __device__ inline void tile_range(int lt, int n, int tile, int mb, int &start, i
     cnt = end - start;
 }
 
-__device__ inline ReqDev find_request(const ScoreLaunch &sl, int t)
+__device__ inline int find_request_index(const ScoreLaunch &sl, int t)
 {
-    if (sl.reqs == nullptr) return sl.single;
+    if (sl.reqs == nullptr) return 0;
     int lo = 0, hi = sl.n_req - 1;
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
         if (sl.reqs[mid].tile_begin <= t) lo = mid;
         else hi = mid - 1;
     }
-    return sl.reqs[lo];
+    return lo;
 }
+
+__device__ inline ReqDev find_request(const ScoreLaunch &sl, int t) { return sl.reqs ? sl.reqs[find_request_index(sl, t)] : sl.single; }
 
 // Record of tile `tile` of the launch's requests.
 __device__ inline TileDev tile_entry(const ScoreLaunch &sl, int tile, int mini_batch)
 {
-    const ReqDev rq = find_request(sl, tile);
+    const int r = find_request_index(sl, tile);
+    const ReqDev rq = sl.reqs ? sl.reqs[r] : sl.single;
     int start, cnt;
     tile_range(tile - rq.tile_begin, rq.n, kTcTile, mini_batch, start, cnt);
-    return TileDev{rq.slot, cnt, rq.off + start, sl.slots[rq.slot].L, {0, 0, 0}};
+    return TileDev{rq.slot, cnt, rq.off + start, sl.slots[rq.slot].L, r, {0, 0}};
 }
 
 // One tile, or (SPLIT) one piece of a tile's keys, as every role of the attention and LSH kernels needs it.

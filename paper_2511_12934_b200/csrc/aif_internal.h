@@ -69,7 +69,8 @@ struct TileDev {
     int32_t cnt;     // candidates in the tile
     int64_t pos0;    // position of its first candidate in ids / logits
     int32_t L;       // keys of the tile: the request's sequence length
-    int32_t pad_[3];
+    int32_t req;     // its place among the launch's requests
+    int32_t pad_[2];
 };
 
 // A piece of a tile's keys, the unit of the attention and LSH kernels where tiles are formed by category (their keys are a part of
@@ -97,6 +98,7 @@ constexpr int kSplitSlotsUser = 2 * 148;   // of the user side's self-attention
 struct ScoreLaunch {
     const SlotDev *slots;   // device array of all slots
     const ReqDev *reqs;     // device array [n_req], or nullptr: use `single`
+    const ReqDev *reqs_host;   // the same on the host, for the launching side
     ReqDev single;
     int32_t n_req;
     int32_t n_tiles;
@@ -310,8 +312,10 @@ bool tc_din_supported(const aif_config &cfg);
 cudaError_t tc_din_prepare(aif_ctx *ctx);
 void tc_din_destroy(aif_ctx *ctx);
 bool tc_din_pays(const aif_ctx *ctx, const ScoreLaunch &sl);
-cudaError_t launch_din_sums(const aif_ctx *ctx, const ScoreLaunch &sl, cudaStream_t st);
-cudaError_t launch_din_apply(const aif_ctx *ctx, const ScoreLaunch &sl, cudaStream_t st, void *X, int x_stride, size_t x_rows, int x_din);
+// requests of a launch whose sums there is room for at a time; either call is for that many from request r0 on
+int din_requests_at_once(const aif_ctx *ctx);
+cudaError_t launch_din_sums(const aif_ctx *ctx, const ScoreLaunch &sl, int r0, cudaStream_t st);
+cudaError_t launch_din_apply(const aif_ctx *ctx, const ScoreLaunch &sl, int r0, cudaStream_t st, void *X, int x_stride, size_t x_rows, int x_din);
 // category sub-sequences (aif_sim.cu): the user-side grouping of a sequence, and the grouping of a launch's candidates by
 // (request, category) into tiles
 size_t sim_grouped_rows(int L_max, int n_categories);

@@ -1568,7 +1568,7 @@ cudaError_t launch_score_tc_scratch(const aif_ctx *ctx, const ScoreLaunch &sl_in
         StageRange range("aif lsh sums");
         ScoreLaunch sl_sums = sl;
         sl_sums.late = buckets_first;
-        const cudaError_t e = launch_din_sums(ctx, sl_sums, st);
+        const cudaError_t e = launch_din_sums(ctx, sl_sums, 0, st);
         if (c.n_hidden <= 2) timing_mark(ctx, "lsh_sums", st);   // (a call has room for eight marks)
         if (e != cudaSuccess) return e;
         late = !buckets_first;   // (ids that the buckets bring are waited for)
@@ -1623,7 +1623,11 @@ cudaError_t launch_score_tc_scratch(const aif_ctx *ctx, const ScoreLaunch &sl_in
         StageRange range("aif lsh rows");
         ScoreLaunch sl_din = sl;
         sl_din.late = 0;
-        const cudaError_t e = launch_din_apply(ctx, sl_din, st, sc.X, pl->x_cols, sc.rows, x_din);
+        cudaError_t e = cudaSuccess;
+        for (int r0 = 0; e == cudaSuccess && r0 < sl.n_req; r0 += din_requests_at_once(ctx)) {   // (the first round's sums are there)
+            if (r0 > 0) e = launch_din_sums(ctx, sl_din, r0, st);
+            if (e == cudaSuccess) e = launch_din_apply(ctx, sl_din, r0, st, sc.X, pl->x_cols, sc.rows, x_din);
+        }
         timing_mark(ctx, "lsh_rows", st);
         if (e != cudaSuccess) return e;
     }

@@ -28,9 +28,10 @@ namespace {
 constexpr int kDinBlock = 128;    // keys per block
 constexpr int kDinCols = 128;     // columns of S per CTA (k_din_sums) or item (k_din_apply)
 constexpr int kDinCluster = 8;    // most CTAs that share a request's keys
+constexpr int kDinRequests = 256; // requests at a time (29 MB of operands at d = 128, 109 at 256): a launch of more goes in rounds of as many
 
 __host__ __device__ constexpr int din_chunks(int D) { return 3 * (D / 64) + 1; }                     // 64-wide K chunks of the operand
-__host__ __device__ constexpr size_t din_image_bytes(int D) { return (size_t)din_chunks(D) * D * 128; }   // of a slot
+__host__ __device__ constexpr size_t din_image_bytes(int D) { return (size_t)din_chunks(D) * D * 128; }   // of a request
 __host__ __device__ constexpr int din_record_groups(int D) { return D / 4 + 1; }                     // float4 groups of a partial record, the last one the row sum
 __host__ __device__ constexpr size_t din_record_bytes(int D) { return (size_t)din_record_groups(D) * kDinCols * 16; }
 
@@ -39,13 +40,13 @@ __host__ __device__ constexpr uint32_t umma_idesc_bf16_mn_mn(int m, int n) { ret
 
 struct DinSums {
     const SlotDev *slots;
-    const ReqDev *reqs;     // [n_req], or nullptr: single
+    const ReqDev *reqs;     // of this round, or nullptr: single
     ReqDev single;
     int32_t parts;          // CTAs per request and column half = cluster size
     int32_t late;
     uint32_t *status;
     float4 *records;        // [request][column half][part] records
-    unsigned char *image;   // [slot] operands
+    unsigned char *image;   // [request] operands
 };
 
 template <int D>
@@ -233,7 +234,7 @@ __global__ void __launch_bounds__((DinSumsCfg<D>::kThreads), 1) k_din_sums(const
     // this CTA's share of the operand: eight bits of one column per thread and round
     const int units = D / 8 * kDinCols;
     const size_t piece = (size_t)(din_record_groups(D) * kDinCols);
-    unsigned char *image = p.image + (size_t)slot * din_image_bytes(D);
+    unsigned char *image = p.image + (size_t)r * din_image_bytes(D);
     for (int u = part * C::kThreads + tid; u < units + kDinCols; u += p.parts * C::kThreads) {
         const int c = u % kDinCols, g = u / kDinCols;   // g < D / 8: bits 8 g ..; g == D / 8: the row sum
         const float4 *src = rec0 + c;
@@ -281,6 +282,7 @@ struct DinApply {
     ScoreLaunch sl;
     const uint8_t *sig;
     const unsigned char *image;
+    int32_t req0, tile0, n_tiles;   // the round's first request, its tiles
     int64_t M;
     int32_t mini_batch, x_stride, x_din, din_mean;
     __nv_bfloat16 *X;
@@ -341,8 +343,9 @@ __global__ void __launch_bounds__((DinApplyCfg<D>::kThreads), 1) k_din_apply(con
     if (!p.sl.late) grid_dep_wait();
     grid_dep_launch();
 
-    const int tile0 = (int)((int64_t)p.sl.n_tiles * blockIdx.x / gridDim.x), tile1 = (int)((int64_t)p.sl.n_tiles * (blockIdx.x + 1) / gridDim.x);
+    const int tile0 = p.tile0 + (int)((int64_t)p.n_tiles * blockIdx.x / gridDim.x), tile1 = p.tile0 + (int)((int64_t)p.n_tiles * (blockIdx.x + 1) / gridDim.x);
     auto tile_of = [&](int tile) { return key_tile<kDinBlock, false>(p.sl, tile, p.mini_batch); };
+    auto req_of = [&](int tile) { return p.sl.tiles ? p.sl.tiles[tile].req - p.req0 : 0; };   // (a single request has no table)
 
     if (warp < C::kOutWarps) {
         // ===================== rows out =====================
@@ -411,10 +414,10 @@ __global__ void __launch_bounds__((DinApplyCfg<D>::kThreads), 1) k_din_apply(con
             uint64_t ones = umma_desc_sw128(smem_u32(smOne));   // without swizzle: 16-byte columns 2048 bytes apart, 8-row groups 128
             ones = (ones & ~((uint64_t)7 << 61) & ~((uint64_t)0x3FFF << 32)) | ((uint64_t)(128u >> 4) << 32) | ((uint64_t)(2048u >> 4) << 16);
             uint32_t it = 0, chunk = 0;   // chunk: chunks so far (d = 256), requests so far (d = 128)
-            int k = 0, slot = tile0 < tile1 ? tile_of(tile0).slot : -1;
+            int k = 0, req = tile0 < tile1 ? req_of(tile0) : -1;
             bool ok = true, fresh = true;
             for (int tile = tile0; ok && tile < tile1; ++tile, ++k) {
-                const int ab = k & 1, slot_next = tile + 1 < tile1 ? tile_of(tile + 1).slot : -1;
+                const int ab = k & 1, req_next = tile + 1 < tile1 ? req_of(tile + 1) : -1;
                 if (!(ok = mbar_wait(smem_u32(a_full + ab), (uint32_t)((k >> 1) & 1), abort_flag))) break;
                 if (C::kResident && fresh && !(ok = mbar_wait(smem_u32(b_full), chunk & 1u, abort_flag))) break;
                 const uint64_t a = umma_desc_sw128(smem_u32(smA + ab * C::kABytes));
@@ -444,8 +447,8 @@ __global__ void __launch_bounds__((DinApplyCfg<D>::kThreads), 1) k_din_apply(con
                     umma_commit(smem_u32(o_full + b));
                     if (half == kH - 1) umma_commit(smem_u32(a_empty + ab));
                 }
-                fresh = slot_next != slot;
-                slot = slot_next;
+                fresh = req_next != req;
+                req = req_next;
                 if (C::kResident && ok && fresh) umma_commit(smem_u32(b_empty)), ++chunk;   // the request's last product
             }
         }
@@ -454,12 +457,12 @@ __global__ void __launch_bounds__((DinApplyCfg<D>::kThreads), 1) k_din_apply(con
         if (lane == 0) {
             uint32_t chunk = 0;
             bool ok = true;
-            int slot = -1, slot_next = tile0 < tile1 ? tile_of(tile0).slot : 0;
+            int req = -1, req_next = tile0 < tile1 ? req_of(tile0) : 0;
             for (int tile = tile0; ok && tile < tile1; ++tile) {
-                const bool fresh = slot_next != slot;
-                slot = slot_next;
-                if (tile + 1 < tile1) slot_next = tile_of(tile + 1).slot;   // a tile ahead of its use
-                const unsigned char *image = p.image + (size_t)slot * din_image_bytes(D);
+                const bool fresh = req_next != req;
+                req = req_next;
+                if (tile + 1 < tile1) req_next = req_of(tile + 1);   // a tile ahead of its use
+                const unsigned char *image = p.image + (size_t)req * din_image_bytes(D);
                 if constexpr (C::kResident) {
                     if (!fresh) continue;
                     if (!(ok = mbar_wait(smem_u32(b_empty), (chunk & 1u) ^ 1u, abort_flag))) break;
@@ -530,7 +533,7 @@ struct DinPlan {
     CUtensorMap tmap_s;
     float4 *records = nullptr;
     unsigned char *image = nullptr;
-    int records_cap = 0;
+    int records_cap = 0, requests = 0;
     int at_once[4] = {};   // clusters of 1, 2, 4, 8 CTAs of k_din_sums that the machine holds
 };
 
@@ -567,13 +570,14 @@ bool tc_din_supported(const aif_config &c)
     return c.dtype == AIF_BF16 && (c.blocks & AIF_BLK_LSH_DIN) && (c.d == 128 || c.d == 256) && c.lsh_bits == c.d && c.n_categories == 0 && encode_fn() != nullptr;
 }
 
-// Scratch for every state of the context; without room for it the context does with the pass over the pairs.
+// Scratch for the requests of a round; without room for it the context does with the pass over the pairs.
 cudaError_t tc_din_prepare(aif_ctx *ctx)
 {
     const aif_config &c = ctx->cfg;
     if (!din_pays(c.d, (int64_t)tc_tile_capacity(ctx), c.L_max)) return cudaSuccess;   // no launch of this context is large enough
-    const size_t n = (size_t)c.max_user_states * (c.d / kDinCols), records = n < 148 ? 148 : n;   // din_parts: more than one part only within them
-    const size_t rec_bytes = records * din_record_bytes(c.d), image_bytes = (size_t)c.max_user_states * din_image_bytes(c.d);
+    const int requests = c.max_user_states < kDinRequests ? c.max_user_states : kDinRequests;
+    const size_t n = (size_t)requests * (c.d / kDinCols), records = n < 148 ? 148 : n;   // din_parts: more than one part only within them
+    const size_t rec_bytes = records * din_record_bytes(c.d), image_bytes = (size_t)requests * din_image_bytes(c.d);
     void *rec = nullptr, *image = nullptr;
     if (cudaMalloc(&rec, rec_bytes) != cudaSuccess || cudaMalloc(&image, image_bytes) != cudaSuccess) {
         if (rec) cudaFree(rec);
@@ -584,7 +588,7 @@ cudaError_t tc_din_prepare(aif_ctx *ctx)
     ctx->device_bytes += (int64_t)(rec_bytes + image_bytes);
     DinPlan *pl = new DinPlan();
     ctx->tc_din_plan = pl;
-    pl->records = (float4 *)rec, pl->image = (unsigned char *)image, pl->records_cap = (int)records;
+    pl->records = (float4 *)rec, pl->image = (unsigned char *)image, pl->records_cap = (int)records, pl->requests = requests;
     const cuuint64_t dims[3] = {(cuuint64_t)c.d, (cuuint64_t)c.L_max, (cuuint64_t)c.max_user_states};
     const cuuint64_t strides[2] = {(cuuint64_t)c.d * 2, (cuuint64_t)ctx->slot_bytes};
     const cuuint32_t box[3] = {64, kDinBlock, 1}, estr[3] = {1, 1, 1};
@@ -626,19 +630,24 @@ bool tc_din_pays(const aif_ctx *ctx, const ScoreLaunch &sl)
 {
     const aif_config &c = ctx->cfg;
     const DinPlan *pl = reinterpret_cast<const DinPlan *>(ctx->tc_din_plan);
-    return pl && !sl.grouped && sl.n_req <= 65535 && (int64_t)sl.n_req * (c.d / kDinCols) <= pl->records_cap && din_pays(c.d, sl.n_tiles, sl.max_L);
+    return pl && !sl.grouped && din_pays(c.d, sl.n_tiles, sl.max_L);
 }
 
-cudaError_t launch_din_sums(const aif_ctx *ctx, const ScoreLaunch &sl, cudaStream_t st)
+int din_requests_at_once(const aif_ctx *ctx) { return reinterpret_cast<const DinPlan *>(ctx->tc_din_plan)->requests; }
+
+static int round_of(const DinPlan &pl, const ScoreLaunch &sl, int r0) { return sl.n_req - r0 < pl.requests ? sl.n_req - r0 : pl.requests; }
+
+cudaError_t launch_din_sums(const aif_ctx *ctx, const ScoreLaunch &sl, int r0, cudaStream_t st)
 {
     const aif_config &c = ctx->cfg;
     const DinPlan *pl = reinterpret_cast<const DinPlan *>(ctx->tc_din_plan);
     DinSums p{};
-    p.slots = sl.slots, p.reqs = sl.reqs, p.single = sl.single, p.late = sl.late, p.status = sl.status;
-    p.parts = din_parts(*pl, sl.n_req, c.d, sl.max_L), p.records = pl->records, p.image = pl->image;
-    if ((int64_t)p.parts * sl.n_req * (c.d / kDinCols) > pl->records_cap) return cudaErrorInvalidValue;
+    const int n_req = round_of(*pl, sl, r0);
+    p.slots = sl.slots, p.reqs = sl.reqs ? sl.reqs + r0 : nullptr, p.single = sl.single, p.late = sl.late, p.status = sl.status;
+    p.parts = din_parts(*pl, n_req, c.d, sl.max_L), p.records = pl->records, p.image = pl->image;
+    if ((int64_t)p.parts * n_req * (c.d / kDinCols) > pl->records_cap) return cudaErrorInvalidValue;
     auto go = [&](auto kernel, int threads, size_t smem) {
-        return launch_pdl_cluster(kernel, dim3(p.parts, c.d / kDinCols, sl.n_req), dim3(threads), smem, (unsigned)p.parts, st, pl->tmap_s, p);
+        return launch_pdl_cluster(kernel, dim3(p.parts, c.d / kDinCols, n_req), dim3(threads), smem, (unsigned)p.parts, st, pl->tmap_s, p);
     };
     const cudaError_t e = c.d == 128 ? go(k_din_sums<128>, DinSumsCfg<128>::kThreads, DinSumsCfg<128>::kSmem)
                                      : go(k_din_sums<256>, DinSumsCfg<256>::kThreads, DinSumsCfg<256>::kSmem);
@@ -646,8 +655,8 @@ cudaError_t launch_din_sums(const aif_ctx *ctx, const ScoreLaunch &sl, cudaStrea
     return e;
 }
 
-// LSH-DIN rows into columns [x_din, x_din + d) of X, after launch_din_sums of the same launch.
-cudaError_t launch_din_apply(const aif_ctx *ctx, const ScoreLaunch &sl, cudaStream_t st, void *X, int x_stride, size_t x_rows, int x_din)
+// LSH-DIN rows into columns [x_din, x_din + d) of X, after launch_din_sums of the same round.
+cudaError_t launch_din_apply(const aif_ctx *ctx, const ScoreLaunch &sl, int r0, cudaStream_t st, void *X, int x_stride, size_t x_rows, int x_din)
 {
     const aif_config &c = ctx->cfg;
     const DinPlan *pl = reinterpret_cast<const DinPlan *>(ctx->tc_din_plan);
@@ -663,7 +672,10 @@ cudaError_t launch_din_apply(const aif_ctx *ctx, const ScoreLaunch &sl, cudaStre
     DinApply p{};
     p.sl = sl, p.sig = ctx->sig, p.image = pl->image, p.M = c.M, p.mini_batch = c.mini_batch;
     p.x_stride = x_stride, p.x_din = x_din, p.din_mean = c.lsh_din_norm == AIF_NORM_MEAN, p.X = (__nv_bfloat16 *)X;
-    const int grid = sl.n_tiles < 148 ? sl.n_tiles : 148;
+    const int r1 = r0 + round_of(*pl, sl, r0);
+    p.req0 = r0, p.tile0 = r0 > 0 ? sl.reqs_host[r0].tile_begin : 0, p.n_tiles = (r1 < sl.n_req ? sl.reqs_host[r1].tile_begin : sl.n_tiles) - p.tile0;
+    if (p.n_tiles == 0) return cudaSuccess;   // requests without candidates
+    const int grid = p.n_tiles < 148 ? p.n_tiles : 148;
     const cudaError_t e = c.d == 128 ? launch_pdl(k_din_apply<128>, dim3(grid), dim3(DinApplyCfg<128>::kThreads), DinApplyCfg<128>::kSmem, st, tmap_x, p)
                                      : launch_pdl(k_din_apply<256>, dim3(grid), dim3(DinApplyCfg<256>::kThreads), DinApplyCfg<256>::kSmem, st, tmap_x, p);
     count_launch();

@@ -75,6 +75,165 @@ def test_more_requests_than_sms(base, L):
     _run(base, synth.BLK_CROSS | LSH, [L] + [40 + r for r in range(n - 1)], [3 + r % 5 for r in range(n)], one_by_one=(0,))
 
 
+# ---- the columns themselves -------------------------------------------------------------------------------------------
+# One hidden layer of which two units pass sum_c r_c x_c on, its positive and its negative part: the logit is that sum over the LSH-DIN
+# or SimTier columns as the layer reads them (bf16).  Rounding them and the unit costs at most 2^-9 of each, which is the tolerance; a scoring
+# network of random weights hides most of what can be wrong in a few of its inputs.
+BF16 = 2.0 ** -9
+
+
+def _columns(wl, blk):
+    at = 2 * wl.d + (wl.d if wl.blocks & synth.BLK_ATT else 0) + (wl.F * wl.dc if wl.blocks & synth.BLK_CROSS else 0)
+    at += wl.d if wl.blocks & synth.BLK_BEA else 0
+    if blk == synth.BLK_LSH_DIN:
+        return at, wl.d
+    return at + (wl.d if wl.blocks & synth.BLK_LSH_DIN else 0), wl.n_tiers
+
+
+def _probe(wl, blk, which):
+    """Row of factors over the input columns: random signs over the block's (different ones per `which`); first, over tiers, a ramp about
+    zero, which every pair that is in the next tier moves by two."""
+    at, n = _columns(wl, blk)
+    r = np.zeros(wl.input_width(), np.float32)
+    r[at:at + n] = np.random.default_rng(100 * n + which).choice([-1.0, 1.0], n)
+    if blk == synth.BLK_SIMTIER and which == 0 and n > 1:
+        r[at:at + n] = 2.0 * np.arange(n) - (n - 1)
+    return r
+
+
+def _load(ctx, r):
+    W = torch.zeros(64, r.size, dtype=torch.bfloat16, device="cuda")
+    W[0], W[1] = torch.from_numpy(r).cuda(), -torch.from_numpy(r).cuda()
+    w_out = torch.zeros(64, dtype=torch.bfloat16, device="cuda")
+    w_out[0], w_out[1] = 1, -1
+    ctx.load_weights({"W": [W], "b": [torch.zeros(64, device="cuda")], "w_out": w_out, "b_out": torch.zeros(1, device="cuda")})
+
+
+def _sums(x, r):
+    """What the logit has to be and how far off it may be."""
+    a = x @ r.astype(np.float64)
+    return a, 1.25 * BF16 * (np.abs(x) @ np.abs(r).astype(np.float64) + np.abs(a)) + 1e-6
+
+
+def _without_block(rq, b):
+    """The request with the rows of key block b (of 128) at zero."""
+    out = dict(rq, S=rq["S"].copy())
+    out["S"][128 * b:128 * b + 128] = 0.0
+    return out
+
+
+def _tiers_shifted(wl, table, rq, ids):
+    """SimTier columns with every tier's edge one match lower."""
+    bits = lambda a: np.unpackbits(a, axis=1).astype(np.float32) * 2 - 1
+    m = ((bits(table["sig"][ids]) @ bits(rq["sig_seq"]).T + wl.d) / 2).astype(np.int64)
+    t = np.minimum((m + 1) * wl.n_tiers // wl.d, wl.n_tiers - 1)
+    x = np.stack([(t == k).sum(1) for k in range(wl.n_tiers)], 1).astype(np.float64)
+    return x / (m.shape[1] if wl.simtier_norm == synth.NORM_MEAN else 1)
+
+
+class Columns:
+    """A context over a workload's requests whose LSH columns are read by probes."""
+
+    def __init__(self, base, blocks, Ls, sizes, M=5000, change=None, **kw):
+        self.wl = wl = helpers.MINI[base].with_(name=f"lsh_cols_{base}", R=len(Ls), N=max(sizes), M=M, L=max(Ls), mini_batch=0, blocks=blocks,
+                                                hidden=(64,), **{"n_cross_tables": 2, **kw})
+        weights = synth.make_weights(wl)
+        self.table = synth.make_item_table(wl)
+        self.rqs = [synth.make_request(wl, r, L=L) for r, L in enumerate(Ls)]
+        sampler = synth.IdSampler(wl)
+        self.ids = [sampler.request_ids(r, n) for r, n in enumerate(sizes)]
+        if change:
+            change(self)
+        self.srv = serving.Server(wl, weights, self.table, path=B.PATH_TENSOR, max_batch_candidates=sum(sizes))
+        self.up = [self.srv.upload_request(rq, B.USER_PROJECTED) for rq in self.rqs]
+        oracle = helpers.make_oracle(wl, weights, M=M)
+        self.oracle = lambda r, rq=None: oracle.score(self.table, rq or helpers.projected_request(wl, self.rqs[r]), self.ids[r], return_inputs=True)[1]
+        self.x = [self.oracle(r) for r in range(len(Ls))]
+
+    def read(self, r, states=None, alone=False):
+        """Logits of every request under the probe r, and the kernels of the (last) call."""
+        _load(self.srv.ctx, r)
+        st = [self.srv.precompute(k, u) for k, u in enumerate(self.up)]
+        self.srv.ctx.set_kernel_timing(True)
+        outs = [self.srv.score_ids(s, i) for s, i in zip(st, self.ids)] if alone else self.srv.score_many(st, self.ids)
+        names = set(self.srv.ctx.get_kernel_timing())
+        self.srv.ctx.set_kernel_timing(False)
+        for s in st:
+            s.release()
+        return outs, names
+
+    def check(self, blk, route, probes=(0, 1, 2), alone=False, sharp=()):
+        """Every request's block against the oracle, by the kernels `route`; for the requests `sharp` the oracle's values for a wrong answer (a key
+        block left out: the last where it holds eight keys of a thousand, else the first; tiers one match off) lie outside the tolerance."""
+        seen = np.zeros(len(self.ids), bool)
+        for which in probes:
+            r = _probe(self.wl, blk, which)
+            outs, names = self.read(r, alone=alone)
+            assert route <= names, names
+            for k, (o, x) in enumerate(zip(outs, self.x)):
+                want, tol = _sums(x, r)
+                err = np.abs(o.astype(np.float64) - want)
+                assert (err <= tol).all(), (k, which, float((err / tol).max()))
+                if blk == synth.BLK_LSH_DIN and k in sharp:
+                    L = len(self.rqs[k]["S"])
+                    last = (L - 1) // 128 if 125 * ((L - 1) % 128 + 1) >= L or L > 10_000 else 0
+                    wrong = _sums(self.oracle(k, _without_block(helpers.projected_request(self.wl, self.rqs[k]), last)), r)[0]
+                elif k in sharp:
+                    wrong = _tiers_shifted(self.wl, self.table, self.rqs[k], self.ids[k]) @ r[slice(*np.cumsum(_columns(self.wl, blk)))].astype(np.float64)
+                else:
+                    continue
+                seen[k] |= bool((np.abs(wrong - want) > 2 * tol).any())
+        assert all(seen[k] for k in sharp), seen
+        return self
+
+
+SUMS, TIERS = {"lsh_sums", "lsh_rows"}, {"simtier"}
+
+
+@pytest.mark.parametrize("base,blocks", [("c2", LSH), ("c2", helpers.ALL_BLOCKS), ("c2", synth.BLK_LSH_DIN), ("c5", LSH), ("c5", synth.BLK_ATT | LSH)])
+def test_columns_at_the_edges_of_blocks_and_units(base, blocks):
+    """The launch of many key blocks above, its columns read by probes: a dropped key block shows in every request of more than one, the
+    last of 313 (over eight CTAs) included; so does a tier's edge that is off by one match."""
+    Ls = [1, 63, 65, 127, 128, 129, 255, 256, 257, 385, 640, 1025, 40_001]
+    sizes = [1, 127, 128, 129, 33, 300, 64, 31, 256, 40, 130, 700, 24]
+    c = Columns(base, blocks, Ls, sizes)
+    c.check(synth.BLK_LSH_DIN, SUMS, sharp=(5, 6, 7, 8, 9, 10, 11, 12))
+    if blocks & synth.BLK_SIMTIER:
+        c.check(synth.BLK_SIMTIER, SUMS | TIERS, sharp=(3, 4, 5, 6, 7, 8, 9, 10, 11, 12))
+    c.srv.close()
+
+
+def test_a_launch_of_more_requests_than_a_round_of_sums():
+    """300 requests, of none to a few hundred candidates, go in a round of 256 and one of the rest; one state serves two of them."""
+    n = 300
+    sizes = [(3 + 7 * k % 260) if k % 11 else 0 for k in range(n)]
+    sizes[255], sizes[256], sizes[299] = 0, 130, 129
+    c = Columns("c2", synth.BLK_LSH_DIN, [1500] + [40 + k for k in range(n - 1)], [max(1, k) for k in sizes], n_cross_tables=1)
+    c.ids = [i[:k] for i, k in zip(c.ids, sizes)]
+    r = _probe(c.wl, synth.BLK_LSH_DIN, 0)
+    _load(c.srv.ctx, r)
+    st = [c.srv.precompute(k, u) for k, u in enumerate(c.up)]
+    st[257], c.ids[257], c.x[257] = st[256], c.ids[256], c.x[256]   # (and a state twice)
+    c.srv.ctx.set_kernel_timing(True)
+    outs = c.srv.score_many(st, c.ids)
+    assert SUMS <= set(c.srv.ctx.get_kernel_timing())
+    for k, o in enumerate(outs):
+        want, tol = _sums(c.x[k][:len(o)], r)
+        assert (np.abs(o - want) <= tol).all(), k
+    c.srv.close()
+
+
+def test_room_for_the_sums_does_not_grow_with_the_states_of_a_context():
+    """Sums are a request's of a launch, not a state's: 2000 states take the room of a round of requests."""
+    def held(blocks):
+        ctx = B.Aif(B.make_config(dtype=B.BF16, M=1000, d=128, L_max=384, hidden=(64,), blocks=blocks, n_tiers=8, lsh_bits=128, max_user_states=2000,
+                                  max_batch_candidates=4096))
+        n = ctx.get_stats().device_bytes
+        ctx.close()
+        return n
+    assert held(LSH) - held(synth.BLK_SIMTIER) < 50 << 20
+
+
 @pytest.mark.parametrize("value", [np.inf, -np.inf, np.nan])
 def test_rows_that_are_not_finite(value):
     """A sequence row with one infinite or missing value: the scores are what the pass over the pairs makes of it."""
