@@ -354,7 +354,8 @@ int aif_get_stats(aif_ctx *ctx, aif_stats *out);
 /* Per-kernel timing of scoring calls, for roofline measurements.  While on, every scoring call brackets each of
  * its kernels with CUDA events on the call's stream (a few microseconds of overhead per kernel, so leave it off
  * for throughput runs).  aif_get_kernel_timing synchronises on the last scoring call and returns, for that call,
- * the number of kernels (<= 8), their names (static strings) and their durations in milliseconds.
+ * the number of kernels (<= 8), their names (static strings) and their durations in milliseconds.  Where a call has more, the
+ * kernels of the LSH blocks are reported as one, "lsh".
  * names / ms: host arrays of 8 entries. */
 int aif_set_kernel_timing(aif_ctx *ctx, int on);
 int aif_get_kernel_timing(aif_ctx *ctx, int32_t *n, const char **names, float *ms);

@@ -148,7 +148,7 @@ constexpr int kProfParts = 256;       // most key slices of the profile attentio
 
 // Optional per-kernel timing of the last scoring call (events on the call's stream).
 struct KernelTiming {
-    static constexpr int kMax = 8;
+    static constexpr int kMax = 12, kReported = 8;   // marks of a call; entries that the caller's arrays have
     bool on = false;
     int n = 0;
     cudaEvent_t ev[kMax + 1] = {};

@@ -1569,7 +1569,7 @@ cudaError_t launch_score_tc_scratch(const aif_ctx *ctx, const ScoreLaunch &sl_in
         ScoreLaunch sl_sums = sl;
         sl_sums.late = buckets_first;
         const cudaError_t e = launch_din_sums(ctx, sl_sums, 0, st);
-        if (c.n_hidden <= 2) timing_mark(ctx, "lsh_sums", st);   // (a call has room for eight marks)
+        timing_mark(ctx, "lsh_sums", st);
         if (e != cudaSuccess) return e;
         late = !buckets_first;   // (ids that the buckets bring are waited for)
     }

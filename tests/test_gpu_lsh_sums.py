@@ -234,6 +234,27 @@ def test_room_for_the_sums_does_not_grow_with_the_states_of_a_context():
     assert held(LSH) - held(synth.BLK_SIMTIER) < 50 << 20
 
 
+def test_marks_of_a_call_with_four_layers_and_every_block():
+    """Ten kernels and eight entries: the LSH blocks' are reported as one, the others by themselves, nothing is lost."""
+    wl = helpers.MINI["c2"].with_(name="lsh_marks", R=1, N=6000, L=9000, mini_batch=0, blocks=helpers.ALL_BLOCKS, hidden=(512, 256, 128, 64))
+    srv = serving.Server(wl, synth.make_weights(wl), synth.make_item_table(wl), path=B.PATH_TENSOR)
+    st = srv.precompute(0, srv.upload_request(synth.make_request(wl, 0), B.USER_PROJECTED))
+    ids = synth.IdSampler(wl).request_ids(0)
+    srv.ctx.set_kernel_timing(True)
+    a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    srv.score_ids(st, ids)
+    a.record()
+    srv.score_ids(st, ids)
+    b.record()
+    torch.cuda.synchronize()
+    marks = srv.ctx.get_kernel_timing()
+    assert set(marks) == {"lsh", "attention", "bea", "buckets", "layer1", "layer2", "layer3", "layer4"}
+    assert 0.0 < sum(marks.values()) <= a.elapsed_time(b)
+    # what the scores hang on most, the pass over the pairs, is under "lsh"
+    assert marks["lsh"] > max(marks[k] for k in ("layer2", "layer3", "layer4"))
+    srv.close()
+
+
 @pytest.mark.parametrize("value", [np.inf, -np.inf, np.nan])
 def test_rows_that_are_not_finite(value):
     """A sequence row with one infinite or missing value: the scores are what the pass over the pairs makes of it."""
