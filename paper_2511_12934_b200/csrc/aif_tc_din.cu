@@ -14,8 +14,11 @@
 //                 (24 bits: nothing of the fp32 sum is lost), K-major, in the swizzled layout of shared memory.
 //   k_din_apply   rows = [q, q, q, 1 1 1] . [A parts; d' sum parts], q exact in bf16, fp32 accumulation; scaled and stored.
 //
-// A sequence row that is not finite makes the row sums of its columns infinite or NaN.  Every match count but zero hands that on, so such
-// a column of the operand keeps the row sum (unscaled by sign) and drops A, whose mixed signs would turn an infinity into NaN.
+// A sequence row that is not finite makes the row sums of its columns infinite or NaN, and the A of its columns infinite with either sign.  A NaN
+// sum is the column's value for every candidate.  Where the sum is an infinity, every match count but zero hands that on, and zero times it is
+// NaN: A_i's sign is the row's bit, so the operand takes signs (0 where several such rows differ in a bit) and d' in place of the sum, the
+// product is twice the row's match count (positive if rows with different bits are behind it), and the rows' columns are multiplied by the
+// infinity when they leave.  (Several infinite rows of different bits, one of them the complement of the candidate's: the infinity.)
 #include <type_traits>
 
 #include "aif_device.cuh"
@@ -32,6 +35,7 @@ constexpr int kDinRequests = 256; // requests at a time (29 MB of operands at d 
 
 __host__ __device__ constexpr int din_chunks(int D) { return 3 * (D / 64) + 1; }                     // 64-wide K chunks of the operand
 __host__ __device__ constexpr size_t din_image_bytes(int D) { return (size_t)din_chunks(D) * D * 128; }   // of a request
+__host__ __device__ constexpr size_t din_image_step(int D) { return din_image_bytes(D) + 128; }   // behind it: per 32 columns, which are infinite, and negative
 __host__ __device__ constexpr int din_record_groups(int D) { return D / 4 + 1; }                     // float4 groups of a partial record, the last one the row sum
 __host__ __device__ constexpr size_t din_record_bytes(int D) { return (size_t)din_record_groups(D) * kDinCols * 16; }
 
@@ -234,7 +238,7 @@ __global__ void __launch_bounds__((DinSumsCfg<D>::kThreads), 1) k_din_sums(const
     // this CTA's share of the operand: eight bits of one column per thread and round
     const int units = D / 8 * kDinCols;
     const size_t piece = (size_t)(din_record_groups(D) * kDinCols);
-    unsigned char *image = p.image + (size_t)r * din_image_bytes(D);
+    unsigned char *image = p.image + (size_t)r * din_image_step(D);
     for (int u = part * C::kThreads + tid; u < units + kDinCols; u += p.parts * C::kThreads) {
         const int c = u % kDinCols, g = u / kDinCols;   // g < D / 8: bits 8 g ..; g == D / 8: the row sum
         const float4 *src = rec0 + c;
@@ -254,10 +258,11 @@ __global__ void __launch_bounds__((DinSumsCfg<D>::kThreads), 1) k_din_sums(const
         for (int q = 0; q < kDinCluster; ++q) sum += part_sum[q];
         unsigned char *row = image + (size_t)(half * kDinCols + c) * 128;
         const int swz = (half * kDinCols + c) & 7;
-        if (g == D / 8) {
-            const bool fin = isfinite(sum);
-            const float t[8] = {fin ? sum * (float)D : sum, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-            const uint32_t hi = bf16_parts8(t, 0).x & 0xFFFFu, mid = fin ? bf16_parts8(t, 1).x & 0xFFFFu : 0u, lo = fin ? bf16_parts8(t, 2).x & 0xFFFFu : 0u;
+        if (g == D / 8) {   // (a whole warp: 32 columns)
+            const uint32_t inf = __ballot_sync(0xffffffffu, isinf(sum)), neg = __ballot_sync(0xffffffffu, sum < 0.f);
+            if (lane == 0) reinterpret_cast<uint2 *>(image + din_image_bytes(D))[(half * kDinCols + c) >> 5] = make_uint2(inf, neg);
+            const float t[8] = {isinf(sum) ? (float)D : sum * (float)D, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+            const uint32_t hi = bf16_parts8(t, 0).x & 0xFFFFu, mid = bf16_parts8(t, 1).x & 0xFFFFu, lo = bf16_parts8(t, 2).x & 0xFFFFu;
             unsigned char *dst = row + (size_t)(3 * (D / 64)) * D * 128;
             *reinterpret_cast<uint4 *>(dst + (swz << 4)) = make_uint4(hi | mid << 16, lo, 0u, 0u);
             *reinterpret_cast<uint4 *>(dst + ((1 ^ swz) << 4)) = make_uint4(0u, 0u, 0u, 0u);
@@ -269,7 +274,7 @@ __global__ void __launch_bounds__((DinSumsCfg<D>::kThreads), 1) k_din_sums(const
             v[0] += a[q].x, v[1] += a[q].y, v[2] += a[q].z, v[3] += a[q].w, v[4] += b[q].x, v[5] += b[q].y, v[6] += b[q].z, v[7] += b[q].w;
         if (!isfinite(sum))
 #pragma unroll
-            for (int i = 0; i < 8; ++i) v[i] = 0.f;
+            for (int i = 0; i < 8; ++i) v[i] = isinf(sum) && isinf(v[i]) ? ((v[i] > 0.f) == (sum > 0.f) ? 1.f : -1.f) : 0.f;
 #pragma unroll
         for (int h = 0; h < 3; ++h)
             *reinterpret_cast<uint4 *>(row + (size_t)(h * (D / 64) + (g >> 3)) * D * 128 + (((g & 7) ^ swz) << 4)) = bf16_parts8(v, h);
@@ -364,8 +369,12 @@ __global__ void __launch_bounds__((DinApplyCfg<D>::kThreads), 1) k_din_apply(con
             }
             const float scale = (0.5f / (float)D) * (p.din_mean ? 1.0f / (float)t.L : 1.0f);
             const bool whole = wq * 32 + 32 <= t.cnt;
+            const uint2 *flags = reinterpret_cast<const uint2 *>(p.image + (size_t)req_of(tile) * din_image_step(D) + din_image_bytes(D));
             for (int half = 0; half < kH; ++half, ++it) {
                 const int b = (int)(it & 1u);
+                uint32_t infinite = 0u;
+#pragma unroll
+                for (int c0 = 0; c0 < kCols; c0 += 32) infinite |= __ldcg(&flags[(half * kDinCols + col0 + c0) >> 5].x);
                 if (!(ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(o_full + b), (it >> 1) & 1u, abort_flag)))) break;
                 tc_fence_after();
 #pragma unroll 1
@@ -377,6 +386,12 @@ __global__ void __launch_bounds__((DinApplyCfg<D>::kThreads), 1) k_din_apply(con
                         tc_fence_before();
                         __syncwarp();
                         if (lane == 0) mbar_arrive(smem_u32(o_empty + b));
+                    }
+                    if (infinite) {
+                        const uint2 f = __ldcg(&flags[(half * kDinCols + c0) >> 5]);
+#pragma unroll
+                        for (int i = 0; i < 32; ++i)
+                            if ((f.x >> i) & 1u) r[i] = __float_as_uint(__uint_as_float(r[i]) * __uint_as_float(0x7F800000u | ((f.y >> i) & 1u) << 31));
                     }
 #pragma unroll
                     for (int i = 0; i < 16; ++i) {
@@ -462,7 +477,7 @@ __global__ void __launch_bounds__((DinApplyCfg<D>::kThreads), 1) k_din_apply(con
                 const bool fresh = req_next != req;
                 req = req_next;
                 if (tile + 1 < tile1) req_next = req_of(tile + 1);   // a tile ahead of its use
-                const unsigned char *image = p.image + (size_t)req * din_image_bytes(D);
+                const unsigned char *image = p.image + (size_t)req * din_image_step(D);
                 if constexpr (C::kResident) {
                     if (!fresh) continue;
                     if (!(ok = mbar_wait(smem_u32(b_empty), (chunk & 1u) ^ 1u, abort_flag))) break;
@@ -577,7 +592,7 @@ cudaError_t tc_din_prepare(aif_ctx *ctx)
     if (!din_pays(c.d, (int64_t)tc_tile_capacity(ctx), c.L_max)) return cudaSuccess;   // no launch of this context is large enough
     const int requests = c.max_user_states < kDinRequests ? c.max_user_states : kDinRequests;
     const size_t n = (size_t)requests * (c.d / kDinCols), records = n < 148 ? 148 : n;   // din_parts: more than one part only within them
-    const size_t rec_bytes = records * din_record_bytes(c.d), image_bytes = (size_t)requests * din_image_bytes(c.d);
+    const size_t rec_bytes = records * din_record_bytes(c.d), image_bytes = (size_t)requests * din_image_step(c.d);
     void *rec = nullptr, *image = nullptr;
     if (cudaMalloc(&rec, rec_bytes) != cudaSuccess || cudaMalloc(&image, image_bytes) != cudaSuccess) {
         if (rec) cudaFree(rec);
