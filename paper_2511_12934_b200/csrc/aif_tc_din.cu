@@ -568,14 +568,33 @@ int din_parts(const DinPlan &pl, int n_req, int d, int max_L)
     return best;
 }
 
-// Where the two launches (about 10 us before and behind the others) are less than what the pass over the pairs saves without the product:
-// key blocks of 128 per SM.  d = 128, this way / the other, us: 64 x 5000 candidates of 300 keys (52 blocks) 658 / 675 with all blocks on, of
-// 1000 (138) 752 / 827; 32 x 5000 of 400 (35) 243 / 245; 8 x 5000 of 1000 (17) 91.1 / 91.6; 1 x 3000 of 10^4 (13) 48.5 / 47.2; one key
-// block each 458 / 447.  d = 256: 32 x 2000 of 1000 (28) 437 / 423, of 2000 (55) 451 / 479; 4 x 4000 of 2000 (14) 137 / 137, of 5000 (35) 149 / 173.
-bool din_pays(int d, int64_t n_tiles, int L)
+// A launch's work in key blocks of 128: of its tiles, and of its requests, each with eight blocks' worth of start and end.
+struct DinWork {
+    int64_t tile_blocks = 0, request_blocks = 0;
+    int requests = 0;
+    void add(int64_t tiles, int L)
+    {
+        const int64_t b = ((int64_t)L + kDinBlock - 1) / kDinBlock;
+        tile_blocks += tiles * b, request_blocks += b + 8, requests += 1;
+    }
+};
+
+// The sums save of every tile's pass over the keys what the product costs there (0.7 us per 148 tiles and block), and cost two launches (about
+// 10 us before and behind the others; a round more 25) and a pass over the keys of every request with d output columns, whether the request has one
+// tile or a hundred.  This way / the other, us:
+// d = 128, LSH-DIN and SimTier: 64 x 5000 candidates of 300 keys 658 / 675 with all blocks on, of 1000 752 / 827; 8 x 5000 of 1000 91.1 / 91.6;
+// 1 x 3000 of 10^4 48.5 / 47.2; 8 x 1000 of 6000 57.9 / 60.3; 16 x 500 of 8000 68.8 / 70.0; 32 x 256 of 7000 74.6 / 69.9; 148 x 128 of 4000
+// 103 / 83; 256 x 100 of 1500 127 / 103; 1024 x 30 of 400 337 / 192.  One key block each 458 / 447.
+// d = 128, LSH-DIN alone: 8 x 1000 of 6000 41.5 / 53.6; 32 x 256 of 7000 52.0 / 62.8; 64 x 128 of 10^4 84.2 / 87.2; 148 x 128 of 4000 87.5 / 80.1.
+// d = 256, both: 32 x 2000 of 1000 437 / 423, of 2000 451 / 479; 4 x 4000 of 2000 137 / 137, of 5000 149 / 173; 16 x 500 of 10^4 122 / 123; 32 x 256
+// of 10^4 152 / 125; 148 x 128 of 4200 247 / 160.  LSH-DIN alone: 16 x 500 of 10^4 99.4 / 115; 32 x 256 of 10^4 127 / 119.
+bool din_pays(const aif_config &c, const DinWork &w, int max_L)
 {
-    const int64_t blocks = ((int64_t)L + kDinBlock - 1) / kDinBlock;
-    return d == 128 ? blocks >= 3 && n_tiles * blocks >= 148 * 20 : blocks >= 8 && n_tiles * blocks >= 148 * 32;
+    const bool tiers = c.blocks & AIF_BLK_SIMTIER;
+    const int blocks = (max_L + kDinBlock - 1) / kDinBlock, rounds = (w.requests + kDinRequests - 1) / kDinRequests;
+    const int64_t tiles = w.tile_blocks - 5500ll * (rounds - 1);
+    if (c.d == 128) return blocks >= 3 && w.tile_blocks >= 148 * 20 && 10 * tiles - (tiers ? 13 : 8) * w.request_blocks >= (tiers ? 23700 : 4000);
+    return blocks >= 8 && w.tile_blocks >= 148 * 32 && 10 * tiles >= (tiers ? 35 : 22) * w.request_blocks;
 }
 
 }  // namespace
@@ -589,7 +608,9 @@ bool tc_din_supported(const aif_config &c)
 cudaError_t tc_din_prepare(aif_ctx *ctx)
 {
     const aif_config &c = ctx->cfg;
-    if (!din_pays(c.d, (int64_t)tc_tile_capacity(ctx), c.L_max)) return cudaSuccess;   // no launch of this context is large enough
+    DinWork most;
+    most.add((int64_t)tc_tile_capacity(ctx), c.L_max);
+    if (!din_pays(c, most, c.L_max)) return cudaSuccess;   // no launch of this context is large enough
     const int requests = c.max_user_states < kDinRequests ? c.max_user_states : kDinRequests;
     const size_t n = (size_t)requests * (c.d / kDinCols), records = n < 148 ? 148 : n;   // din_parts: more than one part only within them
     const size_t rec_bytes = records * din_record_bytes(c.d), image_bytes = (size_t)requests * din_image_step(c.d);
@@ -645,7 +666,13 @@ bool tc_din_pays(const aif_ctx *ctx, const ScoreLaunch &sl)
 {
     const aif_config &c = ctx->cfg;
     const DinPlan *pl = reinterpret_cast<const DinPlan *>(ctx->tc_din_plan);
-    return pl && !sl.grouped && din_pays(c.d, sl.n_tiles, sl.max_L);
+    if (!pl || sl.grouped) return false;
+    DinWork w;
+    for (int r = 0; r < sl.n_req; ++r) {
+        const ReqDev &rq = sl.reqs_host ? sl.reqs_host[r] : sl.single;
+        w.add(tiles_of(rq.n, kTcTile, c.mini_batch), ctx->slots[(size_t)rq.slot].L);
+    }
+    return din_pays(c, w, sl.max_L);
 }
 
 int din_requests_at_once(const aif_ctx *ctx) { return reinterpret_cast<const DinPlan *>(ctx->tc_din_plan)->requests; }

@@ -20,11 +20,13 @@ def _built():
     B.load_library()
 
 
-def _run(base, blocks, Ls, sizes, one_by_one=(), **kw):
+def _run(base, blocks, Ls, sizes, one_by_one=(), more=None, route=(), **kw):
+    """more: (request, candidates that it has besides, which make the launch a large one); route: kernels that the launch has to take."""
+    extra = more[1] if more else 0
     wl = helpers.MINI[base].with_(name=f"lsh_sums_{base}_{blocks}", R=len(Ls), N=max(sizes), L=max(Ls), mini_batch=0, blocks=blocks, **kw)
     weights, table = synth.make_weights(wl, zero_bias=False), None
     table = synth.make_item_table(wl)
-    srv = serving.Server(wl, weights, table, path=B.PATH_TENSOR, max_batch_candidates=sum(sizes))
+    srv = serving.Server(wl, weights, table, path=B.PATH_TENSOR, max_batch_candidates=sum(sizes) + extra)
     oracle = helpers.make_oracle(wl, weights, M=table["E"].shape[0])
     sampler = synth.IdSampler(wl)
     states, ids, want = [], [], []
@@ -33,7 +35,11 @@ def _run(base, blocks, Ls, sizes, one_by_one=(), **kw):
         states.append(srv.precompute(r, srv.upload_request(rq, B.USER_PROJECTED)))
         ids.append(sampler.request_ids(r, n))
         want.append(oracle.score(table, helpers.projected_request(wl, rq), ids[-1]))
-    outs = srv.score_many(states, ids)
+    whole = [np.concatenate([i, np.resize(ids[0], extra)]) if more and r == more[0] else i for r, i in enumerate(ids)]
+    srv.ctx.set_kernel_timing(True)
+    outs = [o[:len(i)] for o, i in zip(srv.score_many(states, whole), ids)]
+    assert set(route) <= set(srv.ctx.get_kernel_timing())
+    srv.ctx.set_kernel_timing(False)
     for r in one_by_one:
         outs.append(srv.score_ids(states[r], ids[r])), want.append(want[r])
     for r, (o, w) in enumerate(zip(outs, want)):
@@ -50,7 +56,7 @@ def test_numbers_of_tiers(n_tiers):
     _run("c2", synth.BLK_CROSS | synth.BLK_SIMTIER, [700, 130], [130, 77], n_tiers=n_tiers)
 
 
-# One long sequence makes the launch one of many key blocks, which is what takes LSH-DIN to the sums; the others are at the edges.
+# One long sequence with many candidates makes the launch a large one, which is what takes LSH-DIN to the sums; the others are at the edges.
 @pytest.mark.parametrize("base,blocks", [("c2", synth.BLK_CROSS | LSH), ("c2", helpers.ALL_BLOCKS), ("c2", synth.BLK_CROSS | synth.BLK_LSH_DIN),
                                          ("c5", synth.BLK_CROSS | LSH), ("c5", synth.BLK_ATT | synth.BLK_CROSS | LSH)])
 def test_sequences_at_the_edges_of_blocks_and_units(base, blocks):
@@ -58,12 +64,12 @@ def test_sequences_at_the_edges_of_blocks_and_units(base, blocks):
     one candidate and of a whole number of tiles, scored together and, a few, alone (the pass over the pairs)."""
     Ls = [1, 63, 65, 127, 128, 129, 255, 256, 257, 385, 640, 1025, 40_001]
     sizes = [1, 127, 128, 129, 33, 300, 64, 31, 256, 1, 130, 700, 2]
-    _run(base, blocks, Ls, sizes, one_by_one=(9, 10, 11))
+    _run(base, blocks, Ls, sizes, one_by_one=(9, 10, 11), more=(12, 2500), route=("lsh_sums", "lsh_rows"))
 
 
 def test_pieces_of_long_sequences():
     """Fewer tiles than SMs: SimTier's counts in pieces of the keys; one tile over a sequence that a counter's lower digits do not hold."""
-    _run("c2", synth.BLK_CROSS | LSH, [9001, 4096], [5300, 128], one_by_one=(1,))
+    _run("c2", synth.BLK_CROSS | LSH, [9001, 4096], [5300, 128], one_by_one=(1,), route=("lsh_sums", "simtier"))
     _run("c2", synth.BLK_CROSS | synth.BLK_SIMTIER, [70_000], [3])
     _run("c5", synth.BLK_CROSS | synth.BLK_SIMTIER, [3001], [100])
 
@@ -72,7 +78,7 @@ def test_pieces_of_long_sequences():
 def test_more_requests_than_sms(base, L):
     """One CTA per request and column half."""
     n = 160
-    _run(base, synth.BLK_CROSS | LSH, [L] + [40 + r for r in range(n - 1)], [3 + r % 5 for r in range(n)], one_by_one=(0,))
+    _run(base, synth.BLK_CROSS | LSH, [L] + [40 + r for r in range(n - 1)], [3 + r % 5 for r in range(n)], one_by_one=(0,), more=(0, 26_000), route=("lsh_sums", "simtier"))
 
 
 # ---- the columns themselves -------------------------------------------------------------------------------------------
@@ -132,9 +138,9 @@ def _tiers_shifted(wl, table, rq, ids):
 
 
 class Columns:
-    """A context over a workload's requests whose LSH columns are read by probes."""
+    """A context over a workload's requests whose LSH columns are read by probes.  more: as for _run."""
 
-    def __init__(self, base, blocks, Ls, sizes, M=5000, change=None, **kw):
+    def __init__(self, base, blocks, Ls, sizes, M=5000, change=None, more=None, **kw):
         self.wl = wl = helpers.MINI[base].with_(name=f"lsh_cols_{base}", R=len(Ls), N=max(sizes), M=M, L=max(Ls), mini_batch=0, blocks=blocks,
                                                 hidden=(64,), **{"n_cross_tables": 2, **kw})
         weights = synth.make_weights(wl)
@@ -144,18 +150,23 @@ class Columns:
         self.ids = [sampler.request_ids(r, n) for r, n in enumerate(sizes)]
         if change:
             change(self)
-        self.srv = serving.Server(wl, weights, self.table, path=B.PATH_TENSOR, max_batch_candidates=sum(sizes))
+        self.more = more or (0, 0)
+        self.srv = serving.Server(wl, weights, self.table, path=B.PATH_TENSOR, max_batch_candidates=sum(sizes) + self.more[1])
         self.up = [self.srv.upload_request(rq, B.USER_PROJECTED) for rq in self.rqs]
         oracle = helpers.make_oracle(wl, weights, M=M)
         self.oracle = lambda r, rq=None: oracle.score(self.table, rq or helpers.projected_request(wl, self.rqs[r]), self.ids[r], return_inputs=True)[1]
         self.x = [self.oracle(r) for r in range(len(Ls))]
 
-    def read(self, r, states=None, alone=False):
+    def score(self, states):
+        whole = [np.concatenate([i, np.resize(self.ids[0], self.more[1])]) if k == self.more[0] else i for k, i in enumerate(self.ids)]
+        return [o[:len(i)] for o, i in zip(self.srv.score_many(states, whole), self.ids)]
+
+    def read(self, r, alone=False):
         """Logits of every request under the probe r, and the kernels of the (last) call."""
         _load(self.srv.ctx, r)
         st = [self.srv.precompute(k, u) for k, u in enumerate(self.up)]
         self.srv.ctx.set_kernel_timing(True)
-        outs = [self.srv.score_ids(s, i) for s, i in zip(st, self.ids)] if alone else self.srv.score_many(st, self.ids)
+        outs = [self.srv.score_ids(s, i) for s, i in zip(st, self.ids)] if alone else self.score(st)
         names = set(self.srv.ctx.get_kernel_timing())
         self.srv.ctx.set_kernel_timing(False)
         for s in st:
@@ -198,7 +209,7 @@ def test_columns_at_the_edges_of_blocks_and_units(base, blocks):
     last of 313 (over eight CTAs) included; so does a tier's edge that is off by one match."""
     Ls = [1, 63, 65, 127, 128, 129, 255, 256, 257, 385, 640, 1025, 40_001]
     sizes = [1, 127, 128, 129, 33, 300, 64, 31, 256, 40, 130, 700, 24]
-    c = Columns(base, blocks, Ls, sizes)
+    c = Columns(base, blocks, Ls, sizes, more=(12, 2500))
     c.check(synth.BLK_LSH_DIN, SUMS, sharp=(5, 6, 7, 8, 9, 10, 11, 12))
     if blocks & synth.BLK_SIMTIER:
         c.check(synth.BLK_SIMTIER, SUMS | TIERS, sharp=(3, 4, 5, 6, 7, 8, 9, 10, 11, 12))
@@ -209,15 +220,15 @@ def test_a_launch_of_more_requests_than_a_round_of_sums():
     """300 requests, of none to a few hundred candidates, go in a round of 256 and one of the rest; one state serves two of them."""
     n = 300
     sizes = [(3 + 7 * k % 260) if k % 11 else 0 for k in range(n)]
-    sizes[255], sizes[256], sizes[299] = 0, 130, 129
-    c = Columns("c2", synth.BLK_LSH_DIN, [1500] + [40 + k for k in range(n - 1)], [max(1, k) for k in sizes], n_cross_tables=1)
+    sizes[0], sizes[255], sizes[256], sizes[299] = 5, 0, 130, 129
+    c = Columns("c2", synth.BLK_LSH_DIN, [9000] + [40 + k for k in range(n - 1)], [max(1, k) for k in sizes], more=(0, 20_000), n_cross_tables=1)
     c.ids = [i[:k] for i, k in zip(c.ids, sizes)]
     r = _probe(c.wl, synth.BLK_LSH_DIN, 0)
     _load(c.srv.ctx, r)
     st = [c.srv.precompute(k, u) for k, u in enumerate(c.up)]
     st[257], c.ids[257], c.x[257] = st[256], c.ids[256], c.x[256]   # (and a state twice)
     c.srv.ctx.set_kernel_timing(True)
-    outs = c.srv.score_many(st, c.ids)
+    outs = c.score(st)
     assert SUMS <= set(c.srv.ctx.get_kernel_timing())
     for k, o in enumerate(outs):
         want, tol = _sums(c.x[k][:len(o)], r)
@@ -234,6 +245,24 @@ def test_room_for_the_sums_does_not_grow_with_the_states_of_a_context():
         ctx.close()
         return n
     assert held(LSH) - held(synth.BLK_SIMTIER) < 50 << 20
+
+
+@pytest.mark.parametrize("base,blocks,R,n,L,sums", [
+    ("c2", LSH, 8, 1000, 6000, True), ("c2", LSH, 148, 128, 4000, False), ("c2", LSH, 300, 60, 1500, False),
+    ("c2", synth.BLK_LSH_DIN, 32, 256, 7000, True), ("c2", synth.BLK_LSH_DIN, 148, 128, 4000, False),
+    ("c5", LSH, 4, 4000, 5000, True), ("c5", LSH, 32, 256, 10_000, False), ("c5", synth.BLK_LSH_DIN, 148, 128, 4200, False)])
+def test_sums_are_for_requests_of_many_candidates(base, blocks, R, n, L, sums):
+    """The sums are a pass over every request's keys: requests of a tile or two go by the pass over the pairs, which is one as well and needs no other
+    launch, however many they are."""
+    wl = helpers.MINI[base].with_(name="lsh_route", R=R, N=n, M=5000, L=L, mini_batch=0, blocks=blocks, hidden=(64,))
+    srv = serving.Server(wl, synth.make_weights(wl), synth.make_item_table(wl), path=B.PATH_TENSOR)
+    up = srv.upload_request(synth.make_request(wl, 0), B.USER_PROJECTED)
+    states = [srv.precompute(r, up) for r in range(R)]
+    srv.ctx.set_kernel_timing(True)
+    srv.score_many(states, [synth.IdSampler(wl).request_ids(0)] * R)
+    names = set(srv.ctx.get_kernel_timing())
+    assert (SUMS <= names) == sums and ("lsh" in names) == (not sums)
+    srv.close()
 
 
 def test_marks_of_a_call_with_four_layers_and_every_block():
@@ -270,7 +299,7 @@ def test_rows_that_are_not_finite(base, value, long):
         bits = np.array([value], np.float32).view(np.uint32)[0] >> 16
         c.rqs[0]["S"][row, col] = bits
         c.table["sig"][c.ids[0][3]] = ~c.rqs[0]["sig_seq"][row]   # candidate 3 shares no bit with the row
-    c = Columns(base, LSH, [300, 200] + [40_001] * long, [2000, 300] + [30] * long, change=poison)
+    c = Columns(base, LSH, [300, 200] + [40_001] * long, [2000, 300] + [30] * long, change=poison, more=(2, 2500) if long else None)
     at = _columns(c.wl, synth.BLK_LSH_DIN)[0]
     r = np.zeros(c.wl.input_width(), np.float32)
     r[at + col] = 1.0
