@@ -57,8 +57,8 @@ def ncu_traffic_table():
 # algorithmic work (what the method itself has to do; padding and recomputation are not counted)
 # ----------------------------------------------------------------------------------------------------------------
 def flops_per_candidate(wl: synth.Workload, keys=None) -> dict:
-    """keys: mean number of sequence items a candidate interacts with (the whole sequence unless the workload has
-    category sub-sequences)."""
+    """By the definition of the blocks.  keys: mean number of sequence items a candidate interacts with (the whole sequence
+    unless the workload has category sub-sequences)."""
     k1 = wl.input_width() - wl.d                       # the user columns are done once per request
     keys = keys_of(wl, keys)
     f = {"attention": 4.0 * keys * wl.d if wl.blocks & synth.BLK_ATT else 0.0}
@@ -86,9 +86,23 @@ def kernel_flops(name: str, wl: synth.Workload, n: int, keys=None) -> float:
         return f["lsh_din"] * n
     if name == "simtier":      # eq. 6's counts as a +-1 fp8 product; eq. 8 then goes through sums of the request's own
         return 2.0 * keys_of(wl, keys) * wl.lsh_bits * n
-    if name in ("buckets", "group", "lsh_sums", "lsh_rows"):
+    if name == "lsh_sums":     # [d' + 1 x L] . [L x d] per request
+        return 2.0 * keys_of(wl, keys) * (wl.lsh_bits + 1) * wl.d * wl.R
+    if name == "lsh_rows":     # [1 x d'] . [d' x d] in three bf16 parts, and the row sum's
+        return 2.0 * 3 * (wl.lsh_bits + 1) * wl.d * n
+    if name in ("buckets", "group"):
         return 0.0
     return f.get(name, 0.0) * n
+
+
+def flops_done(wl: synth.Workload, kernels, n: int, keys=None) -> float:
+    """bf16 operations of a step of n candidates as these kernels carry it out: where LSH-DIN goes through sums of the request's
+    own, those and their product with the signatures stand in for eq. 8's pass over the pairs.  (The +-1 fp8 product behind the
+    match counts is in neither.)"""
+    f = flops_per_candidate(wl, keys)
+    if "lsh_rows" not in kernels:
+        return f["total"] * n
+    return (f["total"] - f["lsh_din"]) * n + sum(kernel_flops(k, wl, n, keys) for k in ("lsh_sums", "lsh_rows"))
 
 
 def load_peaks():
@@ -542,17 +556,19 @@ def measure(args, wl, steps, warmup, dist, world, rank, full):
     else:
         roof = {"bound": "alu", "kernel": top, "achieved": kf / (kavg[top] * 1e-3) / 1e12, "peak": FP32_FMA_PEAK_TFLOPS,
                 "unit": "TFLOP/s", "peak_kind": "fp32 FMA: 148 SMs x 128 lanes x 2 x 1.965 GHz"}
+    if top == "simtier":
+        roof["peak"], roof["peak_kind"] = 2 * roof["peak"], f"fp8, as twice the bf16 burst, {peak_kind}"
     roof["frac"] = roof["achieved"] / roof["peak"]
     if top == "lsh":
         roof["lsh_note"] = (f"eqs. 6-7 need {wl.lsh_bits // 32} xor + popc on 32-bit words per (candidate, key) pair by the definition; "
                             f"the kernel gets the counts from a +-1 fp8 product ({2 * wl.lsh_bits} tensor flop per pair, not counted "
                             "in `achieved`) and spends about five integer / fp32 instructions per pair on conversion and tiers")
     if top == "simtier":
-        roof["lsh_note"] = ("`achieved` counts the +-1 product behind the match counts, at most twice the bf16 rate; the kernel is bound by "
-                            "the issue slots of the tier counts, about three instructions per pair")
+        roof["lsh_note"] = ("`achieved` counts the +-1 fp8 product behind the match counts; the kernel is bound by the issue slots of the tier "
+                            "counts, about three instructions per pair")
     if tensor:
-        roof["frac_nominal"] = roof["achieved"] / NOMINAL_BF16_TFLOPS
-        roof["peak_nominal"] = NOMINAL_BF16_TFLOPS
+        roof["peak_nominal"] = NOMINAL_BF16_TFLOPS * (2 if top == "simtier" else 1)
+        roof["frac_nominal"] = roof["achieved"] / roof["peak_nominal"]
     traffic = ncu_traffic_table().get((wl.name, top))
     roof["traffic"] = None if traffic is None else int(traffic[1] * (cands if traffic[0] == "per_candidate" else 1))
     roof["traffic_source"] = None if traffic is None else f"ncu dram bytes read + write, {traffic[0].replace('_', ' ')}"
@@ -560,6 +576,7 @@ def measure(args, wl, steps, warmup, dist, world, rank, full):
 
     value = world * cands * steps / (total_ms * 1e-3)
     per_request_ms = [t / (wl.R if batch else 1) for t in lat_times]
+    step_tflops = flops_done(wl, kavg, cands, keys) * steps / (total_ms * 1e-3) / 1e12
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": steps, "warmup": max(3, warmup),
         "ms_per_step": total_ms / steps, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
@@ -574,9 +591,8 @@ def measure(args, wl, steps, warmup, dist, world, rank, full):
         "p99_ms_per_request": float(np.percentile(per_request_ms, 99)),
         "latency_samples": {"scoring_calls": len(lat_times), "requests_per_call": wl.R if batch else 1},
         "flops_per_candidate": flops_per_candidate(wl, keys)["total"],
-        "step_tflops": flops_per_candidate(wl, keys)["total"] * cands * steps / (total_ms * 1e-3) / 1e12,
-        "step_frac": {"of_measured_peak": flops_per_candidate(wl, keys)["total"] * cands * steps / (total_ms * 1e-3) / 1e12 / float(peaks["bf16_tflops"]),
-                      "of_nominal_peak": flops_per_candidate(wl, keys)["total"] * cands * steps / (total_ms * 1e-3) / 1e12 / NOMINAL_BF16_TFLOPS}
+        "step_tflops": step_tflops,
+        "step_frac": {"of_measured_peak": step_tflops / float(peaks["bf16_tflops"]), "of_nominal_peak": step_tflops / NOMINAL_BF16_TFLOPS}
         if wl.dtype == "bf16" else None,
         "e2e": {"value": world * cands * e2e_steps / (e2e_ms * 1e-3), "unit": UNIT, "h2d_bytes_per_step": 4 * cands,
                 "d2h_bytes_per_step": 4 * cands, "steps": e2e_steps},

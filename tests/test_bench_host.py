@@ -41,6 +41,20 @@ def test_flop_model_matches_the_scope_table():
     assert bench.kernel_flops("layer1", synth.C2, 10) == 10 * f["layer1"]
 
 
+def test_step_flops_are_those_of_the_kernels_that_ran():
+    """Long sequences, LSH blocks: by the definition eq. 8 is 2.6 MFLOP of a candidate's 3.9; through the request's sums it is 0.1."""
+    wl = synth.C4_LSH
+    n = wl.R * wl.N
+    f = bench.flops_per_candidate(wl)
+    assert bench.flops_done(wl, {"lsh", "buckets", "layer1", "layer2"}, n) == f["total"] * n
+    done = bench.flops_done(wl, {"lsh_sums", "simtier", "buckets", "lsh_rows", "layer1", "layer2"}, n)
+    layers = (f["layer1"] + f["layer2"]) * n
+    assert f["lsh_din"] == 2 * 10_000 * 128
+    assert abs(done - layers - 16 * 2 * 10_000 * 129 * 128 - n * 6 * 129 * 128) < 1e-6 * done
+    assert bench.kernel_flops("simtier", wl, 10) == 10 * 2 * 10_000 * 128
+    assert bench.kernel_flops("score_split", synth.C2, 10) == bench.kernel_flops("score_fused", synth.C2, 10) == 10 * bench.flops_per_candidate(synth.C2)["total"]
+
+
 def test_replica_plan_and_max_over_ranks_with_two_gloo_ranks(tmp_path):
     script = tmp_path / "worker.py"
     script.write_text(WORKER)
