@@ -184,25 +184,26 @@ __device__ inline void tile_range(int lt, int n, int tile, int mb, int &start, i
     cnt = end - start;
 }
 
-__device__ inline int find_request_index(const ScoreLaunch &sl, int t)
+// index (may be null): its place among the launch's requests.
+__device__ inline ReqDev find_request(const ScoreLaunch &sl, int t, int *index = nullptr)
 {
-    if (sl.reqs == nullptr) return 0;
+    if (index) *index = 0;
+    if (sl.reqs == nullptr) return sl.single;
     int lo = 0, hi = sl.n_req - 1;
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
         if (sl.reqs[mid].tile_begin <= t) lo = mid;
         else hi = mid - 1;
     }
-    return lo;
+    if (index) *index = lo;
+    return sl.reqs[lo];
 }
-
-__device__ inline ReqDev find_request(const ScoreLaunch &sl, int t) { return sl.reqs ? sl.reqs[find_request_index(sl, t)] : sl.single; }
 
 // Record of tile `tile` of the launch's requests.
 __device__ inline TileDev tile_entry(const ScoreLaunch &sl, int tile, int mini_batch)
 {
-    const int r = find_request_index(sl, tile);
-    const ReqDev rq = sl.reqs ? sl.reqs[r] : sl.single;
+    int r;
+    const ReqDev rq = find_request(sl, tile, &r);
     int start, cnt;
     tile_range(tile - rq.tile_begin, rq.n, kTcTile, mini_batch, start, cnt);
     return TileDev{rq.slot, cnt, rq.off + start, sl.slots[rq.slot].L, r, {0, 0}};
