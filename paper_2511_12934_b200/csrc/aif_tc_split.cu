@@ -25,9 +25,7 @@
 
 #include <mutex>
 
-#include "aif_device.cuh"
-#include "aif_internal.h"
-#include "aif_tc_ptx.cuh"
+#include "aif_tc_request.cuh"
 
 namespace aif {
 namespace {
@@ -67,7 +65,8 @@ struct SplitParams {
     int64_t M;
     int32_t tile;           // candidates per cluster, a multiple of 16, at most kMaxTile
     int32_t stages;         // of the weight ring
-    int32_t B, dc, b_mask, bucket_mode, n_cross;
+    CrossTables cross;
+    int32_t n_cross;
     int32_t H2, emit_sigmoid;
     float scale_log2;       // log2(e) / sqrt(d)
     const __nv_bfloat16 *b2_hl;   // [2][H2]: second-layer bias, high parts then remainders
@@ -147,7 +146,6 @@ __global__ void __launch_bounds__(kFThreads, 1) k_request_split(const __grid_con
         // ===================== softmax, epilogues =====================
         const int g = warp >> 2, wq = warp & 3, row = wq * 32 + lane;
         const uint32_t lane_base = tmem_base + ((uint32_t)(wq * 32) << 16);
-        const float k2 = p.scale_log2;
         bool ok = true;
         // a wait of the whole warp: the tensor-memory loads and stores that follow need every lane to take the same branch
         auto wait = [&](int b) {
@@ -171,101 +169,15 @@ __global__ void __launch_bounds__(kFThreads, 1) k_request_split(const __grid_con
             if (g == 0 || has2) bias_hl = (uint32_t)__bfloat16_as_ushort(hl[at]) | (uint32_t)__bfloat16_as_ushort(hl[n + at]) << 16;
         }
         // ---- attention: scores of key block g -> probabilities
-        // Softmax is invariant to the offset subtracted in the exponent, and bf16 keeps its relative precision over the
-        // whole fp32 exponent range.  The first attempt therefore subtracts nothing, p = 2^(s k2), and saves the pass
-        // over the scores that finds the row maxima; a row sum outside [2^-80, 2^80] (scores far from zero: overflow,
-        // or every term flushed to zero) makes the whole CTA repeat the step with the exact row maxima.  The
-        // probabilities go to columns of their own, so the scores are still there for the repeat.
-        const bool act = g < nb && wq * 32 < p.tile;   // rows beyond the tile: nobody's (the products read whatever lies there)
-        const int valid_cols = L - g * 128 < 128 ? L - g * 128 : 128;
-        const uint32_t p_col = 384u + (uint32_t)(g * 64);
-        auto probabilities = [&](float mt) {   // P = 2^(s k2 - mt) as packed bf16; returns the row sum over this block
-            float lsum = 0.f;
-#pragma unroll 1
-            for (int h = 0; h < 2; ++h) {
-                uint32_t sc[64];
-                tmem_ld32(lane_base + (uint32_t)(g * 128 + 64 * h), *reinterpret_cast<uint32_t(*)[32]>(&sc[0]));
-                tmem_ld32(lane_base + (uint32_t)(g * 128 + 64 * h + 32), *reinterpret_cast<uint32_t(*)[32]>(&sc[32]));
-                tmem_ld_wait();
-                uint32_t packed[32];
-                float ls4[4] = {0.f, 0.f, 0.f, 0.f};
-                const int left = valid_cols - 64 * h;   // valid columns among these 64
-#pragma unroll
-                for (int i = 0; i < 32; ++i) {
-                    float p0 = fast_exp2(fmaf(__uint_as_float(sc[2 * i]), k2, -mt));
-                    float p1 = fast_exp2(fmaf(__uint_as_float(sc[2 * i + 1]), k2, -mt));
-                    if (2 * i >= left) p0 = 0.f;
-                    if (2 * i + 1 >= left) p1 = 0.f;
-                    ls4[i & 3] += p0 + p1;
-                    const __nv_bfloat162 hh = __floats2bfloat162_rn(p0, p1);
-                    packed[i] = *reinterpret_cast<const uint32_t *>(&hh);
-                }
-                tmem_st32(lane_base + p_col + (uint32_t)(32 * h), packed);
-                lsum += (ls4[0] + ls4[1]) + (ls4[2] + ls4[3]);
-            }
-            tmem_st_wait();
-            return lsum;
-        };
-        float lsum = 0.f;
-        if (act) {
-            wait(BAR_S_FULL + g);   // of its own key block: the first group's exponentials run under the second block's products
-            tc_fence_after();
-            if (ok) lsum = probabilities(0.f);
-        }
-        if (row < 64) xs[g * 64 + row] = lsum;
-        const bool off_range = act && ok && row < p.tile && !(lsum > 0x1p-80f && lsum < 0x1p80f);
-        float l_other;
-        if (named_bar_or(1, 256, off_range)) {
-            // exact form: row maxima over both key blocks first
-            float mx = -INFINITY;
-            if (act && ok) {
-#pragma unroll 1
-                for (int c0 = 0; c0 < 128; c0 += 32) {
-                    uint32_t r[32];
-                    tmem_ld32(lane_base + (uint32_t)(g * 128 + c0), r);
-                    tmem_ld_wait();
-#pragma unroll
-                    for (int i = 0; i < 32; ++i)
-                        if (c0 + i < valid_cols) mx = fmaxf(mx, __uint_as_float(r[i]));
-                }
-            }
-            if (row < 64) xs[g * 64 + row] = mx;
-            named_bar_sync(1, 256);
-            const float mt = fmaxf(mx, xs[(g ^ 1) * 64 + (row & 63)]) * k2;   // an inactive group has published -inf
-            named_bar_sync(1, 256);                                    // both maxima are read: xs may now take the sums
-            lsum = act && ok ? probabilities(mt) : 0.f;
-            if (row < 64) xs[g * 64 + row] = lsum;
-            named_bar_sync(1, 256);
-        }
-        l_other = xs[(g ^ 1) * 64 + (row & 63)];
+        // (rows beyond the tile: nobody's; the products read whatever lies there)
+        const RequestRow rr{lane_base, g, row, L - g * 128 < 128 ? L - g * 128 : 128, g < nb && wq * 32 < p.tile, p.scale_log2};
+        const float l_all = request_softmax<64>(rr, xs, ok, row < p.tile, [&] { wait(BAR_S_FULL + g); });
         tc_fence_before();
         mbar_arrive(bar(BAR_P_FULL));
-        const float l_all = lsum + l_other;
         // ---- O -> attention chunk g of the first layer's input (64 columns, 128B-swizzled K-major)
         wait(BAR_O_FINAL);
         tc_fence_after();
-        if (ok && wq * 32 < p.tile) {
-            const float inv = good ? 1.0f / l_all : 0.f;
-            unsigned char *dst = smAtt + g * cs + row * 128;
-#pragma unroll 1
-            for (int c0 = 0; c0 < 64; c0 += 32) {
-                uint32_t r[32];
-                tmem_ld32(lane_base + (uint32_t)(256 + 64 * g + c0), r);
-                tmem_ld_wait();
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    uint32_t w[4];
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const __nv_bfloat162 hh = __floats2bfloat162_rn(__uint_as_float(r[8 * q + 2 * i]) * inv,
-                                                                        __uint_as_float(r[8 * q + 2 * i + 1]) * inv);
-                        w[i] = *reinterpret_cast<const uint32_t *>(&hh);
-                    }
-                    const int slot16 = (c0 >> 3) + q;
-                    if (row < p.tile) *reinterpret_cast<uint4 *>(dst + ((slot16 ^ (row & 7)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
-                }
-            }
-        }
+        if (ok && wq * 32 < p.tile) request_attention_row(rr, good ? 1.0f / l_all : 0.f, smAtt + g * cs + row * 128, row < p.tile);
         // The biases are added by the tensor cores, as in aif_tc_fused.cu: one more step of K = 16 whose operands are, per unit, the bias in two
         // bf16 values (high part, remainder) and, per candidate, two ones (no swizzle: 16-byte columns, the second ones zero).
         if (ok) {
@@ -416,14 +328,7 @@ __global__ void __launch_bounds__(kFThreads, 1) k_request_split(const __grid_con
         constexpr int kR = kMaxTile / 16;
         const uint32_t row_off = (uint32_t)(r0 * 128) + (uint32_t)((sub ^ (r0 & 7)) << 4);
         int id[kR];
-#pragma unroll
-        for (int i = 0; i < kR; ++i) id[i] = __shfl_sync(0xffffffffu, mine, (lane >> 3) + 4 * i);
-#pragma unroll
-        for (int i = 0; i < kR; ++i)
-            if (r0 + 16 * i < cnt && (id[i] < 0 || (int64_t)id[i] >= p.M)) {
-                id[i] = -1;
-                if (sub == 0) atomicOr(p.sl.status, AIF_STATUS_BAD_ID);
-            }
+        request_ids(id, mine, cnt, p.M, p.sl.status, lane, sub, r0);
 #pragma unroll
         for (int i = 0; i < kR; ++i) {
             if (16 * i >= p.tile) break;
@@ -436,19 +341,13 @@ __global__ void __launch_bounds__(kFThreads, 1) k_request_split(const __grid_con
         // cross features (Section 3.3): the row of field f's user-side table that the candidate's bucket selects
         const uint8_t *Tt = reinterpret_cast<const uint8_t *>(slot->T);
         for (int n = 0; n < p.n_cross; ++n) {
-            const int col = 64 * n + 8 * sub, f = col / p.dc, kin = col - f * p.dc;
-            const uint32_t row16 = (uint32_t)(p.dc >> 3), base16 = (uint32_t)(f * p.B) * row16 + (uint32_t)(kin >> 3);
+            const CrossColumns at = cross_columns(p.cross, 64 * n + 8 * sub);
             const uint32_t dst0 = smem_u32(smX + n * cs) + row_off;
 #pragma unroll
             for (int i = 0; i < kR; ++i) {
                 if (16 * i >= p.tile) break;
-                uint32_t bk;
-                if (p.bucket_mode == AIF_BUCKET_MOD) bk = (uint32_t)(id[i] % p.B);
-                else {
-                    const uint64_t h = mix64((uint64_t)id[i], (uint64_t)f);
-                    bk = p.b_mask >= 0 ? (uint32_t)(h & (uint64_t)p.b_mask) : (uint32_t)(h % (uint64_t)p.B);
-                }
-                cp_async16(dst0 + (uint32_t)(i * 16 * 128), id[i] >= 0 ? Tt + ((size_t)(bk * row16 + base16) << 4) : p.E, id[i] >= 0 ? 16u : 0u);
+                const uint32_t off = cross_offset16(p.cross, at, id[i]);
+                cp_async16(dst0 + (uint32_t)(i * 16 * 128), id[i] >= 0 ? Tt + ((size_t)off << 4) : p.E, id[i] >= 0 ? 16u : 0u);
             }
             cp_async_arrive_noinc(bar(BAR_FULL_A + n));
         }
@@ -569,7 +468,7 @@ cudaError_t launch_request_split(const aif_ctx *ctx, const ScoreLaunch &sl, int 
     SplitParams p{};
     p.sl = sl, p.E = (const uint8_t *)ctx->E, p.M = c.M;
     p.tile = tile, p.stages = stages_for(tile);
-    p.B = c.B, p.dc = c.dc, p.b_mask = (c.B & (c.B - 1)) == 0 ? c.B - 1 : -1, p.bucket_mode = c.bucket_mode;
+    p.cross = CrossTables{c.B, c.dc, (c.B & (c.B - 1)) == 0 ? c.B - 1 : -1, c.bucket_mode};
     p.n_cross = c.F * c.dc / 64;
     p.H2 = c.hidden[1], p.emit_sigmoid = c.emit_sigmoid;
     p.scale_log2 = 1.4426950408889634f / sqrtf((float)c.d);
