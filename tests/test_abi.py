@@ -80,3 +80,24 @@ def test_binding_refuses_to_run_without_cuda():
         B.Aif(B.make_config(dtype=B.BF16, M=10, d=128, L_max=10, hidden=(512, 256)))
     with pytest.raises(FileNotFoundError):
         B.load_library(os.path.join(ROOT, "no_such_dir", "libaif.so"))
+
+
+def test_a_change_of_any_source_or_header_asks_for_a_build(tmp_path, monkeypatch):
+    for folder in ("csrc", "pkg", "include"):
+        (tmp_path / folder).mkdir()
+    names = ["a.cu", "a.h", "a.cuh"]
+    for name in names:
+        (tmp_path / "csrc" / name).write_text("")
+        os.utime(tmp_path / "csrc" / name, (1000, 1000))
+    (tmp_path / "lib.so").write_text("")
+    now = os.path.getmtime(tmp_path / "lib.so")
+    monkeypatch.setattr(libbuild, "CSRC", str(tmp_path / "csrc"))
+    monkeypatch.setattr(libbuild, "LIB", str(tmp_path / "lib.so"))
+    monkeypatch.setattr(libbuild, "HERE", str(tmp_path / "pkg"))
+    (tmp_path / "include" / "aif.h").write_text("")
+    os.utime(tmp_path / "include" / "aif.h", (1000, 1000))
+    assert not libbuild._stale()
+    for name in names:
+        os.utime(tmp_path / "csrc" / name, (now + 10, now + 10))
+        assert libbuild._stale(), name
+        os.utime(tmp_path / "csrc" / name, (1000, 1000))
