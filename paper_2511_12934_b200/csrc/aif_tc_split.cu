@@ -16,6 +16,9 @@
 // epilogue adds (another order of sums): 13.9 for 1000; one issuing lane that asks for the next chunk's barrier ahead: 15.4; two chunks to a turn:
 // 16.4, and 22 where the ring has three stages.
 //
+// Of 23 k cycles for 1000 candidates the set-up is 1.8 k, rows and scores 2.9 k, the softmax 3.3 k (a tile's rows lie in one or two warps'
+// tensor-memory lanes), O and its rows 2.2 k, the layers 4.5 k and 3.8 k, their epilogues and the exchange 1.9 k, the CTAs' meeting 1.3 k, the
+// output layer 1.5 k.
 // 480 threads: warps 0-7 softmax and epilogues, 8 and 14 the issuers, 9-12 gather, 13 one lane of TMA, as there.  A chunk of 64 columns is four
 // products of 45 cycles; the wait for its weights takes 140 cycles even where they are there, the hand-over between the issuers 180, the commit 100.
 // Tensor memory: attention as there (scores [0, 256), O [256, 384), probabilities [384, 512)); then the layers' accumulators, D of the first at 0, of

@@ -16,9 +16,10 @@
 //   * The bytes are summed bit-sliced: eight words hold the binary digits of 32 counters (7 tiers x 4 byte positions), a carry-save
 //     adder (two three-input logic instructions) takes in two words, halving with every digit.  The digits are transposed into bytes and
 //     added to 32-bit counters when the tile ends.
-// Per pair 2.1 instructions (3.1 with everything around the loop), on two half-rate pipes (integer, and the fp16 half of the FMA pipe) in equal
-// shares, against 5.0 where the counts also become the operand of eq. 8's product: 520 cycles per 128 keys for 320 of products (16 requests of
-// 10^4 candidates, 10^4 keys: 215 us; both blocks in one pass over the pairs: 1600 cycles, 650 us).  What bounds it: issue slots, 0.66 of them taken.
+// Per pair 2.1 instructions (2.9 with everything around the loop), on two half-rate pipes (integer, and the fp16 half of the FMA pipe) in equal
+// shares, against 5.0 where the counts also become the operand of eq. 8's product: 592 cycles per 128 keys for 320 of products (means over the SMs,
+// 4 requests of 10^4 candidates, 10^4 keys; 16 of them: 215 us; both blocks in one pass over the pairs: 1600 cycles, 650 us).  What bounds it:
+// issue slots, 0.62 of them taken.
 // Tried: sixteen warps over two buffers of 256 columns with one issuing lane (673 cycles, the lane), twelve warps with all 128 columns of a unit
 // in registers (617 to 640: three warps to a scheduler do not cover each other's waits of 200 cycles for scores and 200 for their load), the
 // counters emptied every seven units (490 cycles of a warp each time; now carried into eight more digits), 32 columns at a time with the next ones
