@@ -44,7 +44,7 @@ __host__ __device__ constexpr uint32_t umma_idesc_bf16_mn_mn(int m, int n) { ret
 
 struct DinSums {
     const SlotDev *slots;
-    const ReqDev *reqs;     // of this round, or nullptr: single
+    const ReqDev *reqs;     // the requests at hand, or nullptr: single
     ReqDev single;
     int32_t parts;          // CTAs per request and column half = cluster size
     int32_t late;
